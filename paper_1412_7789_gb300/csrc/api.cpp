@@ -262,12 +262,33 @@ namespace {
 
 using pfac::scratch_pool;
 
+// The streaming form of one long text, its walk list from the pool.
+cudaError_t run_stream(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st) {
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = scratch_pool(h->device, &pool);
+    if (e != cudaSuccess) return e;
+    r.walk_cap = pfac::stream_walk_cap(r.n);
+    void *scratch = nullptr;
+    e = cudaMallocFromPoolAsync(&scratch, pfac::stream_bytes(r.walk_cap), pool, st);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(scratch, 0, 32, st);
+    if (e == cudaSuccess) {
+        r.list_count = static_cast<unsigned int *>(scratch);
+        r.walks = reinterpret_cast<uint2 *>(static_cast<uint8_t *>(scratch) + 32);
+        e = pfac::launch_stream(h->dev, r, mode, h->tuning, st);
+    }
+    const cudaError_t e2 = cudaFreeAsync(scratch, st);
+    return e != cudaSuccess ? e : e2;
+}
+
 // A tiled launch (dense ids or count) with its zeroed scratch (the tile
 // counter) in stream-ordered memory, so calls on different streams never share it.
 // A text short enough that every tile is some warp's first needs no counter:
 // the launchers accept no scratch then, which saves the allocation and the
 // clearing of small calls.
 cudaError_t run_tiled(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st) {
+    if (!r.batch && pfac::at_serves(h->dev, h->tuning, r.n)) return pfac::launch_at(h->dev, r, mode, st);
+    if (!r.batch && pfac::stream_serves(h->dev, h->tuning, r.n)) return run_stream(h, r, mode, st);
     // 8-bit codes, long text: the phased form's lists after the counter
     pfac::SurvivorLists sl;
     if (!r.batch && pfac::uses_filter(h->dev, h->tuning)) sl = pfac::survivor_lists(h->dev, h->tuning, r.n);
@@ -485,6 +506,8 @@ ac_status ac_compile(const uint8_t *const *patterns, const uint32_t *lens, uint3
     d.hash_shift = t.hash_shift;
     d.full_max_clen = t.full_max_clen;
     d.nkw = t.nkw;
+    d.stream = t.stream;
+    d.stream_f2bytes = static_cast<uint32_t>(t.stream_F2.size() * sizeof(uint32_t));
     std::memcpy(d.hash_code, t.hash_code, 8);
     std::memcpy(d.hash_byte, t.hash_byte, 8);
     d.direct_shift = t.direct_shift;
@@ -512,6 +535,12 @@ ac_status ac_compile(const uint8_t *const *patterns, const uint32_t *lens, uint3
             s = upload(h, t.F.data(), t.F.size() * sizeof(uint32_t), reinterpret_cast<const void **>(&d.F));
         if (s == AC_OK && !t.JK.empty())
             s = upload(h, t.JK.data(), t.JK.size() * sizeof(int32_t), reinterpret_cast<const void **>(&d.JK));
+        if (s == AC_OK && !t.stream_F1.empty())
+            s = upload(h, t.stream_F1.data(), t.stream_F1.size() * sizeof(uint32_t),
+                       reinterpret_cast<const void **>(&d.stream_F1));
+        if (s == AC_OK && !t.stream_F2.empty())
+            s = upload(h, t.stream_F2.data(), t.stream_F2.size() * sizeof(uint32_t),
+                       reinterpret_cast<const void **>(&d.stream_F2));
         if (s == AC_OK && !t.HK.empty())
             s = upload(h, t.HK.data(), t.HK.size() * sizeof(uint32_t), reinterpret_cast<const void **>(&d.HK));
         if (s == AC_OK && !t.J2.empty())
@@ -569,7 +598,8 @@ ac_status ac_info(ac_handle h, ac_info_t *info) {
     info->table_bytes = t.G.size() + t.J.size() * sizeof(int16_t) + t.J2.size() * sizeof(int32_t) +
                         t.F.size() * sizeof(uint32_t) + t.JK.size() * sizeof(int32_t) +
                         t.skip.size() * sizeof(uint32_t) + t.chain.size() + 768 +
-                        (t.full_rec.size() + t.full_dups.size()) * sizeof(uint32_t);
+                        (t.full_rec.size() + t.full_dups.size()) * sizeof(uint32_t) +
+                        (t.stream_F1.size() + t.stream_F2.size()) * sizeof(uint32_t);
     info->depth_base_jump = t.base_k;
     info->count_jump = t.count_k;
     info->class_hash_shift = t.hash_shift;
@@ -1063,6 +1093,11 @@ ac_status ac_autotune(ac_handle h, const uint8_t *d_sample, uint64_t n, uint32_t
     // with the hashed filter (when built) and the three 8-bit kernels
     std::vector<int> variants{0};
     if (!h->dev.filter) variants = h->dev.hashed ? std::vector<int>{0, 3, 2, 1} : std::vector<int>{3, 2, 1};
+    {  // as built: the forms for short and long texts
+        pfac::Tuning tu;
+        tu.wait_ns = keep.wait_ns;
+        time_one(tu);
+    }
     for (int v : variants) {
         pfac::Tuning tu = keep;
         tu.variant = v;

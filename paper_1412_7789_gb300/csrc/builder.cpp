@@ -25,7 +25,8 @@
 //      codes from every depth-k state;
 //   8. chain records for the deep, mostly unbranched states;
 //   9. the full-output records: for each keyword, the keywords that are
-//      prefixes of it (its sub-patterns on any walk that reaches it).
+//      prefixes of it (its sub-patterns on any walk that reaches it);
+//  10. the streaming form's filters, from the keywords alone.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -265,6 +266,104 @@ void hashed_filter(const HostTables &h, uint32_t fbits, RootTables *rt) {
         if (h.HK[b + 1] == 0u) continue;  // an empty entry
         const uint32_t f = (h.HK[b] * kFilterHashMul) >> (32u - fbits);
         rt->F[f >> 5] |= 1u << (31u - (f & 31u));
+    }
+}
+
+void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTables *hp) {
+    HostTables &h = *hp;
+    StreamTables &st = h.stream;
+    st = StreamTables{};
+    h.stream_F1.clear();
+    h.stream_F2.clear();
+    constexpr uint32_t kWords = (1u << kFilterBits) / 32u;
+    auto set_bit = [](uint32_t *F, uint32_t i) { F[i >> 5] |= 1u << (31u - (i & 31u)); };
+    if (h.filter && h.B == 2 && h.direct_shift == 1 && h.B * h.k == kFilterBits) {
+        const uint32_t k = h.k;
+        auto codes = [&](uint32_t id, uint32_t o, uint32_t len) {  // len <= 16 codes from offset o
+            uint32_t w = 0;
+            for (uint32_t j = 0; j < len; ++j) w |= static_cast<uint32_t>(h.cls8[patterns[id][o + j]]) << (2u * j);
+            return w;
+        };
+        // the fewest lookups whose filter stays sparse: with it too dense, the
+        // candidates of the chance hits cost more than the lookups saved
+        for (uint32_t step : {4u, 2u}) {
+            if (h.minlen < step + 4u) continue;  // at most 4^6 completions a window
+            std::vector<uint32_t> F(kWords, 0u);
+            for (uint32_t id = 0; id < h.nkw; ++id)
+                for (uint32_t o = 0; o < step; ++o) {
+                    const uint32_t len = std::min(k, lens[id] - o);
+                    const uint32_t w = codes(id, o, len);
+                    for (uint32_t v = w; v < (1u << (2u * k)); v += 1u << (2u * len)) set_bit(F.data(), v);
+                }
+            uint64_t bits = 0;
+            for (uint32_t x : F) bits += static_cast<uint64_t>(__builtin_popcount(x));
+            if (bits * 25u > (1ull << kFilterBits)) continue;  // over 4 %
+            st.step = step;
+            h.stream_F1 = std::move(F);
+            // windows longer than the filter's, where every keyword has them
+            const uint32_t win2 = std::min(16u, h.minlen - (step - 1u));
+            if (win2 >= k + 2u) {
+                constexpr uint32_t kWords2 = 8192u;  // 32 KiB
+                st.win2 = win2;
+                h.stream_F2.assign(kWords2, 0u);
+                for (uint32_t id = 0; id < h.nkw; ++id)
+                    for (uint32_t o = 0; o < step; ++o) {
+                        const uint32_t x = (codes(id, o, win2) << (32u - 2u * win2)) * kFilterHashMul;
+                        h.stream_F2[(static_cast<uint64_t>(x) * kWords2) >> 32] |= 1u << ((x >> 12) & 31u);
+                    }
+            }
+            break;
+        }
+        st.form = 2;
+        st.win1 = k;
+        st.root = k;
+    } else if (h.hashed && h.minlen >= kHashWindow && h.fbits == kFilterBits) {
+        st.form = 8;
+        st.root = h.fbits;
+        // the window: the shortest keyword's length, at most 8 bytes, then as
+        // many bits of the next bytes as keep the filter sparse (a keyword that
+        // ends before them has all its completions set)
+        constexpr uint64_t kMostBits = (1ull << kFilterBits) / 40u;  // 2.5 %
+        uint32_t win = std::min(64u, 8u * h.minlen);
+        for (; win < 64u; ++win) {
+            uint64_t bits = 0;
+            for (uint32_t id = 0; id < h.nkw && bits <= kMostBits; ++id)
+                bits += 8u * lens[id] > win ? 1u : 1ull << (win + 1u - 8u * lens[id]);
+            if (bits > kMostBits) break;
+        }
+        st.win1 = win;
+        st.m1 = kFilterHashMul;
+        st.m2 = win > 32u ? kStreamMul2 << (64u - win) : 0u;
+        auto bytes4 = [&](uint32_t id, uint32_t o) {  // 4 bytes from offset o, zero past the end
+            uint32_t w = 0;
+            for (uint32_t j = 0; j < 4 && o + j < lens[id]; ++j) w |= static_cast<uint32_t>(patterns[id][o + j]) << (8u * j);
+            return w;
+        };
+        h.stream_F1.assign(kWords, 0u);
+        for (uint32_t id = 0; id < h.nkw; ++id) {
+            const uint32_t w0 = bytes4(id, 0), w1 = bytes4(id, 4);
+            const uint32_t own = 8u * lens[id] < win ? 8u * lens[id] : win;  // >= 32
+            for (uint32_t v = 0; v < (1u << (win - own)); ++v) {
+                const uint64_t x = static_cast<uint64_t>(w0) * st.m1;
+                const uint32_t y = static_cast<uint32_t>(x) + (own < win ? w1 | (v << (own - 32u)) : w1) * st.m2;
+                set_bit(h.stream_F1.data(), ((y >> 17) << 5) | (static_cast<uint32_t>(x >> 32) & 31u));
+            }
+        }
+        if (win < 48u) {
+            constexpr uint32_t kWords2 = 4096u;  // 16 KiB
+            st.win2 = 6u;
+            h.stream_F2.assign(kWords2 + kStreamShortBytes / 4u, 0u);
+            for (uint32_t id = 0; id < h.nkw; ++id) {
+                const uint32_t w = bytes4(id, 0);
+                if (lens[id] < 6u) {
+                    const uint32_t x = w * kStateHashMul;
+                    h.stream_F2[kWords2 + (x >> 22)] |= 1u << ((x >> 17) & 31u);
+                } else {
+                    const uint32_t x = w * kFilterHashMul + (bytes4(id, 4) << 16) * kStreamMul2;
+                    h.stream_F2[(static_cast<uint64_t>(x) * kWords2) >> 32] |= 1u << ((x >> 12) & 31u);
+                }
+            }
+        }
     }
 }
 
@@ -831,6 +930,11 @@ int build_tables(const uint8_t *const *patterns, const uint32_t *lens, uint32_t 
                 i = j;
             }
         }
+    } catch (const std::bad_alloc &) {
+        return AC_ERR_OOM;
+    }
+    try {
+        stream_filters(patterns, lens, &h);  // 10. the streaming form's filters
     } catch (const std::bad_alloc &) {
         return AC_ERR_OOM;
     }

@@ -33,7 +33,8 @@ uint32_t staged_bytes(const DevTables &t, const Tuning &tu) {
 cudaError_t fill_params(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu, FilterParams &p) {
     if (!served(t)) return cudaErrorInvalidValue;
     const bool hashed = t.B == 8;
-    if (mode != OUT_DENSE && mode != OUT_COUNT && mode != OUT_SLOTS) return cudaErrorInvalidValue;
+    if (mode != OUT_DENSE && mode != OUT_COUNT && mode != OUT_SLOTS && mode != OUT_BITS) return cudaErrorInvalidValue;
+    if (mode == OUT_BITS && (!r.bits.bits || !r.bits.ids)) return cudaErrorInvalidValue;
     const bool batch = r.batch != nullptr;
     if (batch && (mode == OUT_COUNT || !r.lists)) return cudaErrorInvalidValue;
     if (mode == OUT_SLOTS && (!r.slots.counts || !r.slots.slots)) return cudaErrorInvalidValue;
@@ -101,6 +102,7 @@ cudaError_t fill_params(const DevTables &t, const MatchRequest &r, OutMode mode,
     p.out = r.out;
     p.count = r.count;
     p.sl = r.slots;
+    p.bo = r.bits;
     if (!batch && r.list && r.list_count && r.list_cap && p.ntiles < (1u << 22)) {
         p.list = r.list;
         p.list_count = r.list_count;
@@ -163,6 +165,19 @@ cudaError_t device_shape(DeviceShape *out) {
 }
 
 }  // namespace
+
+cudaError_t filter_params(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
+                          FilterParams &p) {
+    return fill_params(t, r, mode, tu, p);
+}
+
+cudaError_t filter_device_shape(int *sms, int *max_smem) {
+    DeviceShape ds;
+    const cudaError_t e = device_shape(&ds);
+    *sms = ds.sms;
+    *max_smem = ds.max_smem;
+    return e;
+}
 
 bool filter_phased(const DevTables &t, const Tuning &tu, uint64_t n, bool slots) {
     if (!served(t) || n / kTile >= (1ull << 22) - 1 || tu.survivor_list == 2) return false;

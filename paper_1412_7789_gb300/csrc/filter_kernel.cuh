@@ -106,6 +106,8 @@ struct FilterParams {
     int32_t *out;
     unsigned long long *count;
     SlotOut sl;
+    BitsOut bo;
+    uint32_t bits_head;  // OUT_BITS: text position i is position i + bits_head there
     unsigned int *counter;
     unsigned int *err;
     uint32_t off_neg1, off_warp, warp_bytes, off_packed, off_inv, off_queue, off_meta, off_help;
@@ -2078,6 +2080,13 @@ cudaError_t launch_modes(OutMode mode, const FilterParams &p, uint32_t grid, uin
 }
 
 }  // namespace filt
+
+// The parameters of a launch for automaton t and request r, all but the shared-
+// memory layout, and the current device's SM count and largest shared memory
+// per CTA (filter.cu).
+cudaError_t filter_params(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
+                          filt::FilterParams &p);
+cudaError_t filter_device_shape(int *sms, int *max_smem);
 
 // Launch of the forms that share heavy tiles (one text only), filter_help.cu.
 cudaError_t launch_filter_help(OutMode mode, const filt::FilterParams &p, uint32_t B, uint32_t gbits, uint32_t grid,

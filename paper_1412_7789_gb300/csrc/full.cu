@@ -46,16 +46,6 @@ struct FullParams : RootWalk {
     CompactOut out;
 };
 
-// Chain length of result id (an id outside the keyword set, which no matching
-// kernel writes, latches kErrWalk and counts as none).
-__device__ __forceinline__ uint32_t chain_len(const FullParams &p, uint32_t id) {
-    if (id >= p.nkw) {
-        atomicOr(p.err, static_cast<unsigned>(kErrWalk));
-        return 0;
-    }
-    return __ldg(reinterpret_cast<const uint32_t *>(p.rec) + 4ull * id + 3u);
-}
-
 // The dense id of tile position i of unit u (-1 outside the text): kept by
 // the matching kernel, or (no dense ids) the walk from the root again.
 template <typename GT>
@@ -102,28 +92,6 @@ __global__ void __launch_bounds__(kFullThreads) full_count(const FullParams p) {
             sum = __reduce_add_sync(kFull, sum);
             if (lane == 0) p.fcounts[u] = sum;
         }
-    }
-}
-
-// One lane: the occurrences of result r at start `pos`, from list index `at`:
-// the chain from r down to its shortest prefix keyword fills the range from
-// its end backwards, each string's equal keywords in ascending id.
-__device__ __forceinline__ void put_chain(const FullParams &p, unsigned long long at, uint32_t pos, uint32_t r) {
-    if (r >= p.nkw) return;  // latched by chain_len
-    uint4 rx = __ldg(p.rec + r);
-    for (uint32_t guard = 0; guard < p.max_clen; ++guard) {  // a chain has at most max_clen strings
-        uint4 ru = make_uint4(kNoKeyword, 0u, 0u, 0u);
-        if (rx.x != kNoKeyword && rx.x < p.nkw) ru = __ldg(p.rec + rx.x);
-        const uint32_t end = pos + rx.y - 1u;
-        for (uint32_t j = ru.w; j < rx.w; ++j) {
-            const unsigned long long o = at + j;
-            if (o < p.out.cap) {
-                p.out.pos[o] = end;
-                p.out.ids[o] = __ldg(p.dups + rx.z + (j - ru.w));
-            }
-        }
-        if (rx.x == kNoKeyword) break;
-        rx = ru;
     }
 }
 

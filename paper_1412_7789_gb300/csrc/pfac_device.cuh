@@ -406,4 +406,41 @@ __device__ int walk_from_root(const RootWalk &p, const uint8_t *text, uint64_t n
     return -1;
 }
 
+// The full output's expansion of a result (P: the launch's parameters, with the
+// full-output records rec and dups, max_clen, nkw, err and the list out).
+
+// Chain length of result id (an id outside the keyword set, which no matching
+// kernel writes, latches kErrWalk and counts as none).
+template <typename P>
+__device__ __forceinline__ uint32_t chain_len(const P &p, uint32_t id) {
+    if (id >= p.nkw) {
+        atomicOr(p.err, static_cast<unsigned>(kErrWalk));
+        return 0;
+    }
+    return __ldg(reinterpret_cast<const uint32_t *>(p.rec) + 4ull * id + 3u);
+}
+
+// One lane: the occurrences of result r at start `pos`, from list index `at`:
+// the chain from r down to its shortest prefix keyword fills the range from
+// its end backwards, each string's equal keywords in ascending id.
+template <typename P>
+__device__ __forceinline__ void put_chain(const P &p, unsigned long long at, uint32_t pos, uint32_t r) {
+    if (r >= p.nkw) return;  // latched by chain_len
+    uint4 rx = __ldg(p.rec + r);
+    for (uint32_t guard = 0; guard < p.max_clen; ++guard) {  // a chain has at most max_clen strings
+        uint4 ru = make_uint4(kNoKeyword, 0u, 0u, 0u);
+        if (rx.x != kNoKeyword && rx.x < p.nkw) ru = __ldg(p.rec + rx.x);
+        const uint32_t end = pos + rx.y - 1u;
+        for (uint32_t j = ru.w; j < rx.w; ++j) {
+            const unsigned long long o = at + j;
+            if (o < p.out.cap) {
+                p.out.pos[o] = end;
+                p.out.ids[o] = __ldg(p.dups + rx.z + (j - ru.w));
+            }
+        }
+        if (rx.x == kNoKeyword) break;
+        rx = ru;
+    }
+}
+
 }  // namespace pfac

@@ -45,6 +45,14 @@ constexpr uint32_t kHashWindow = 4;  // codes per hashed window (at most)
 // State-hash entry field `child` of a depth-kh state with several children.
 constexpr uint32_t kHkBranch = 0xFFFFFFFFu;
 
+// The streaming form for one long text (stream_kernel.cuh): positions a warp
+// takes at a time, positions per unit of a walk-list entry, multiplier of a
+// window's second word, and the short-keyword part of the second filter.
+constexpr uint32_t kStreamTile = 2048;
+constexpr uint32_t kStreamUnit = 1024;
+constexpr uint32_t kStreamMul2 = 0xC2B2AE35u;
+constexpr uint32_t kStreamShortBytes = 4096;
+
 // Longest halo staged in shared memory; walks that run past it read global memory.
 constexpr uint32_t kHaloCap = 256;
 
@@ -69,6 +77,24 @@ struct RawBytes {
         p.reset(new uint8_t[m]);
         n = m;
     }
+};
+
+// The filters of the streaming form (form 0: the automaton has none).
+//   form 2 (2-bit codes (byte >> 1) & 3, root windows of 10 codes): F1 has the
+//     bit of every window of 10 codes at offsets 0 .. step - 1 of a keyword
+//     (all completions where the keyword ends inside it); F2 (none when empty)
+//     that of every window of win2 codes there, hashed.
+//   form 8 (8-bit codes, no keyword shorter than 4): F1 the hashed windows of
+//     every keyword's first win1 bits (all completions where the keyword ends
+//     inside them); F2 (none when empty) those of its first 6 bytes, then, in
+//     its last kStreamShortBytes, the first 4 bytes of the keywords shorter
+//     than 6.
+struct StreamTables {
+    uint32_t form = 0;
+    uint32_t step = 1;             // form 2: every step-th position is looked up
+    uint32_t win1 = 0, win2 = 0;   // windows in codes (form 2); win1 in bits (form 8)
+    uint32_t m1 = 0, m2 = 0;       // form 8: multipliers of the window's words
+    uint32_t root = 0;             // the root tables' depth it was built with (k, or the filter's bits)
 };
 
 // Host-side automaton: everything the kernels need, in the layout they use.
@@ -126,6 +152,8 @@ struct HostTables {
     bool hashed = false;
     uint32_t kh = 0, fbits = 0, hk_bits = 0, hk_probes = 0;
     std::vector<uint32_t> HK;
+    StreamTables stream;
+    std::vector<uint32_t> stream_F1, stream_F2;  // F1 empty: the root filter F itself
     // Full output: 4 words per keyword id {up, len, dup_off, clen} (set for
     // the lowest id of each keyword string, the id a walk reports), the ids
     // grouped by string, and the largest clen.
@@ -173,6 +201,9 @@ void hashed_filter(const HostTables &h, uint32_t fbits, RootTables *out);
 // The widest window of B-bit codes whose filter fits `bytes`.
 uint32_t filter_window(uint32_t B, uint32_t maxlen, uint32_t bytes);
 
+// The streaming form's filters of a built automaton (h.stream, h.stream_F1/F2).
+void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTables *h);
+
 // Device view of a compiled automaton.
 struct DevTables {
     const void *G = nullptr;         // goto table
@@ -189,6 +220,9 @@ struct DevTables {
     const uint4 *skip = nullptr;     // chain records (states from s_chain on), or none
     const uint8_t *chain = nullptr;  // chain bytes
     uint32_t s_chain = 0xFFFFFFFFu;  // first state with a chain record
+    StreamTables stream;
+    const uint32_t *stream_F1 = nullptr, *stream_F2 = nullptr;
+    uint32_t stream_f2bytes = 0;
     const uint4 *full_rec = nullptr;    // full-output records (one per keyword id)
     const uint32_t *full_dups = nullptr;
     uint32_t full_max_clen = 0;
@@ -209,7 +243,9 @@ struct DevTables {
 // OUT_SLOTS: per work unit, the number of matches and the first kSlotCap of
 // them in any order (SlotOut); the compacted list is then made by the scan
 // and gather steps (compact.cu).  OUT_COMPACT names that whole sequence.
-enum OutMode : int { OUT_DENSE = 0, OUT_COUNT = 1, OUT_COMPACT = 2, OUT_SLOTS = 3 };
+// OUT_BITS (bits.cu): one bit per position with a match, the ids of those
+// positions in an array that is not filled elsewhere, a match count per tile.
+enum OutMode : int { OUT_DENSE = 0, OUT_COUNT = 1, OUT_COMPACT = 2, OUT_SLOTS = 3, OUT_BITS = 4 };
 
 // Matches a unit keeps in its slots; for a unit with more, the gather step
 // reads the unit's dense ids (SlotOut::dense), or matches it again.
@@ -227,6 +263,17 @@ struct SlotOut {
     // than kSlotCap matches, so the gather step reads them instead of matching
     // the unit again.
     int32_t *dense = nullptr;
+};
+
+// OUT_BITS: position g (its index from the text's 16-byte aligned base in the
+// streaming form, in the text in the short-text form) has bit g & 31 of
+// bits[g >> 5], its id ids[g], and counts in counts[g / kStreamTile] (the
+// streaming form alone).  Every bit and count is written; ids only where a
+// bit is set.
+struct BitsOut {
+    uint32_t *bits = nullptr;
+    int32_t *ids = nullptr;
+    uint32_t *counts = nullptr;
 };
 
 // Where one text's compacted list goes (ac_match_compact's arguments).
@@ -261,6 +308,7 @@ struct MatchRequest {
     const BatchItemDev *lists = nullptr;     // batch: the planned list (device)
     unsigned long long *count = nullptr;     // count
     SlotOut slots;                           // OUT_SLOTS
+    BitsOut bits;                            // OUT_BITS
     void *scratch = nullptr;                 // zeroed: tile counter (16 bytes)
     size_t scratch_bytes = 0;
     // One long text: the lists of the phased form (survivor_lists); list =
@@ -352,6 +400,29 @@ struct Tuning {
     unsigned long long wait_ns = 0;  // bounded waits give up after this (0 = kWaitNs)
     int stall_help = 0;   // test aid: owners wait for one chunk more than their heavy tile has
 };
+
+// One short text (dense ids or count): one thread per position, everything
+// from global memory (stream.cu).  Needs no scratch.
+bool at_serves(const DevTables &t, const Tuning &tu, uint64_t n);
+cudaError_t launch_at(const DevTables &t, const MatchRequest &r, OutMode mode, cudaStream_t stream);
+
+// The streaming form (stream.cu) of one long text: whether it serves the text
+// with this tuning (any knob set asks for the filter kernel's own forms), the
+// room of its walk list, and the launch (r.list_count: two words, zeroed;
+// r.walks, r.walk_cap).
+bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n);
+uint32_t stream_walk_cap(uint64_t n);
+inline size_t stream_bytes(uint32_t walk_cap) { return 32 + 8ull * walk_cap; }
+cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
+                          cudaStream_t stream);
+
+// The compacted list (full: every occurrence) of one text through OUT_BITS
+// (bits.cu): the short-text or the streaming form, then the lists.  Whether it
+// serves the text, its scratch, and the launches.
+bool bits_serve(const DevTables &t, const Tuning &tu, uint64_t n);
+size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full);
+cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, const CompactOut &out,
+                         bool full, void *scratch, size_t scratch_bytes, cudaStream_t stream);
 
 // The scan and gather steps of the compacted output (compact.cu).
 //   units: launch units (host count), or, when units_dev is set, read there.

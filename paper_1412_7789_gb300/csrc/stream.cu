@@ -1,0 +1,211 @@
+// One text in two launches, or one: the streaming form (stream_kernel.cuh) and
+// its walk step, and the form for short texts (one thread per position).
+
+#include "stream_kernel.cuh"
+
+namespace pfac {
+
+using namespace strm;
+
+namespace {
+
+// Texts up to this length take one thread per position: no filter to load
+// into every SM, no list, one launch.  4 KiB of the sweep set, where every
+// position walks to a match: 10 us a call against 70 in the filter kernel,
+// whose few tiles kept a handful of warps busy.  The line against the
+// streaming form (us a call from an idle GPU, host time included): ACGT 2 MiB
+// 30 / 32, 4 MiB 42 / 33; Zipf bytes 2 MiB 40 / 43, 4 MiB 57 / 45.
+constexpr uint64_t kAtMax = 2u << 20;
+constexpr int kAtBlock = 128;
+
+// One thread per position (a text this short and the tables it touches stay in
+// L2).  A warp reads its 32 bytes and the 16 after them once, one byte a lane,
+// and joins their codes into windows with log2(window) shuffles, so a position
+// costs two byte loads and one load per table level.
+template <int B, typename GT, int MODE>
+__global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ FilterParams p) {
+    __shared__ uint8_t cls8[256];
+    const int lane = threadIdx.x & 31;
+    const uint64_t gi = static_cast<uint64_t>(blockIdx.x) * kAtBlock + threadIdx.x;
+    const bool in = gi < p.n, in2 = lane < 16 && gi + 32u < p.n;
+    const uint32_t b0 = in ? __ldg(p.text + gi) : 0u, b1 = in2 ? __ldg(p.text + gi + 32u) : 0u;
+    for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
+    __syncthreads();
+    // codes, and which positions hold none (a byte in no keyword, or the text's end)
+    const bool id = B == 8 && p.identity;
+    uint32_t lo = id ? b0 : cls8[b0], hi = id ? b1 : cls8[b1];
+    const bool bad0 = !in || (!id && lo == 0xFFu), bad1 = !in2 || (!id && hi == 0xFFu);
+    const uint32_t m0 = __ballot_sync(kFull, bad0), m1 = __ballot_sync(kFull, bad1);
+    const uint32_t bad = __funnelshift_r(m0, m1, lane);  // bit j: position gi + j
+    lo &= (1u << B) - 1u;
+    hi &= (1u << B) - 1u;
+    uint32_t after = 0;  // 8-bit codes: the code after the window
+    if (B == 8) {
+        const uint32_t x = static_cast<uint32_t>(lane) + p.k;
+        const uint32_t y = __shfl_sync(kFull, lo, x & 31u), z = __shfl_sync(kFull, hi, x & 31u);
+        after = x < 32u ? y : z;
+    }
+#pragma unroll
+    for (uint32_t d = 1; d * B < 32u; d *= 2u) {  // windows of d codes -> 2 d
+        const uint32_t x = static_cast<uint32_t>(lane) + d;
+        const uint32_t y = __shfl_sync(kFull, lo, x & 31u), z = __shfl_sync(kFull, hi, x & 31u);
+        lo |= (x < 32u ? y : z) << (B * d);
+        hi |= z << (B * d);  // the last lanes' are never read
+    }
+    uint32_t cnt = 0;
+    if (in) {
+        const TileText tt = make_text(p.text, p.out, p.n, 0u);
+        const uint32_t need = B == 8 ? p.k : p.k + p.k2;
+        int r = -1;
+        uint32_t s = 0, q = 0;
+        bool walk = true;
+        if (!(bad & ((1u << need) - 1u))) {
+            if (B == 8) {
+                const uint32_t w = lo & p.wmask;
+                walk = !filt::hk_outcome(p, filt::hk_find(p, w, __ldg(p.HK + filt::hk_slot(p, w))), 0u, after,
+                                         !((bad >> p.k) & 1u), r, s, q);
+            } else {
+                const int e = __ldg(p.JK + (lo & ((1u << (B * p.k)) - 1u)));
+                walk = e >= 0;
+                if (walk) {
+                    s = static_cast<uint32_t>(e);
+                    q = p.k;
+                    if (p.k2) {
+                        const int e2 = __ldg(p.J2 + ((static_cast<uint64_t>(s - p.base_k) << (B * p.k2)) |
+                                                     ((lo >> (B * p.k)) & ((1u << (B * p.k2)) - 1u))));
+                        walk = e2 >= 0;
+                        if (walk) {
+                            s = static_cast<uint32_t>(e2);
+                            q += p.k2;
+                        } else {
+                            r = decode_dead(e2);
+                        }
+                    }
+                } else {
+                    r = decode_dead(e);
+                }
+            }
+        } else if (B == 8) {
+            walk = false;  // no keyword is shorter than the state hash's window
+        }
+        if (walk) r = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s, q);
+        if (MODE == OUT_DENSE)
+            p.out[gi] = r;
+        else
+            cnt = r >= 0 ? 1u : 0u;
+        if (MODE == OUT_BITS && r >= 0) p.bo.ids[gi] = r;
+    }
+    if (MODE == OUT_BITS) {
+        const uint32_t bits = __ballot_sync(kFull, cnt != 0u);
+        if (lane == 0 && in) p.bo.bits[gi >> 5] = bits;
+    }
+    add_count<MODE>(p, cnt, lane);
+}
+
+template <int B, typename GT>
+cudaError_t launch_at_modes(OutMode mode, const FilterParams &p, cudaStream_t stream) {
+    const uint32_t grid = static_cast<uint32_t>((p.n + kAtBlock - 1) / kAtBlock);
+    switch (mode) {
+        case OUT_DENSE: pfac_at<B, GT, OUT_DENSE><<<grid, kAtBlock, 0, stream>>>(p); break;
+        case OUT_COUNT: pfac_at<B, GT, OUT_COUNT><<<grid, kAtBlock, 0, stream>>>(p); break;
+        case OUT_BITS: pfac_at<B, GT, OUT_BITS><<<grid, kAtBlock, 0, stream>>>(p); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+template <int B, typename GT>
+cudaError_t launch_walk_modes(OutMode mode, const FilterParams &p, uint32_t sms, cudaStream_t stream) {
+    const uint32_t grid = sms * kWalkCtas;
+    switch (mode) {
+        case OUT_DENSE: pfac_stream_walks<B, GT, OUT_DENSE><<<grid, kWalkBlock, 0, stream>>>(p); break;
+        case OUT_COUNT: pfac_stream_walks<B, GT, OUT_COUNT><<<grid, kWalkBlock, 0, stream>>>(p); break;
+        case OUT_BITS: pfac_stream_walks<B, GT, OUT_BITS><<<grid, kWalkBlock, 0, stream>>>(p); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+// Every knob as built: the caller asks for no particular form.
+bool untuned(const Tuning &tu) {
+    return tu.block == 0 && tu.stages == 0 && tu.grid == 0 && tu.variant == 0 && tu.per_thread == 0 &&
+           tu.halo <= 16 && tu.survivor_list == 0 && !tu.stall_help;
+}
+
+}  // namespace
+
+bool at_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
+
+    return untuned(tu) && n <= kAtMax && (t.filter || (t.hashed && t.HK));
+}
+
+cudaError_t launch_at(const DevTables &t, const MatchRequest &r, OutMode mode, cudaStream_t stream) {
+    if (r.batch || r.n == 0) return cudaErrorInvalidValue;
+    FilterParams p;
+    const cudaError_t e = filter_params(t, r, mode, Tuning{}, p);
+    if (e != cudaSuccess) return e;
+    const bool g16 = t.gbits == 16;
+    if (t.B == 2) return g16 ? launch_at_modes<2, int16_t>(mode, p, stream) : launch_at_modes<2, int32_t>(mode, p, stream);
+    if (t.B == 4) return g16 ? launch_at_modes<4, int16_t>(mode, p, stream) : launch_at_modes<4, int32_t>(mode, p, stream);
+    return g16 ? launch_at_modes<8, int16_t>(mode, p, stream) : launch_at_modes<8, int32_t>(mode, p, stream);
+}
+
+bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
+    if (!t.stream.form || !untuned(tu) || n / kStreamUnit >= (1ull << 22) - 2) return false;
+    return t.stream.root == (t.stream.form == 2 ? t.k : t.fbits);
+}
+
+uint32_t stream_walk_cap(uint64_t n) {
+    // a walk for every eighth position, and each warp's last reservation
+    // (positions past that are settled where they are found)
+    return static_cast<uint32_t>(n / 8) + device_sm_count() * static_cast<uint32_t>(kWarps) * kWalkChunkEntries;
+}
+
+cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
+                          cudaStream_t stream) {
+    if (!stream_serves(t, tu, r.n) || r.batch || r.n == 0 || !r.walks || !r.list_count || r.walk_cap == 0)
+        return cudaErrorInvalidValue;
+    int sms = 0, max_smem = 0;
+    cudaError_t e = filter_device_shape(&sms, &max_smem);
+    if (e != cudaSuccess) return e;
+    StreamParams p{};
+    e = filter_params(t, r, mode, tu, p.f);
+    if (e != cudaSuccess) return e;
+    p.f.walks = r.walks;
+    p.f.walk_cap = r.walk_cap;
+    p.f.list_count = r.list_count;
+    p.F1 = t.stream_F1 ? t.stream_F1 : t.F;
+    p.f1bytes = (1u << kFilterBits) / 8u;
+    p.F2 = t.stream_F2;
+    p.f2bytes = t.stream_F2 ? t.stream_f2bytes : 0u;
+    p.head = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(r.text) & 15u);
+    p.f.bits_head = p.head;
+    if (mode == OUT_BITS && !r.bits.counts) return cudaErrorInvalidValue;
+    p.ntiles = static_cast<uint32_t>((r.n + p.head + kTile - 1) / kTile);
+    p.m1 = t.stream.m1;
+    p.m2 = t.stream.m2;
+    p.l2shift = t.stream.form == 2 ? 32u - 2u * t.stream.win2 : 0u;
+    // the tiles whose bytes, and the 16 after them, are all in the text's
+    // 16-byte aligned part
+    p.in_lo = p.f.a1 ? 1u : 0u;
+    p.in_hi = p.f.a2 >= 16u ? static_cast<uint32_t>((p.f.a2 - 16u) / kTile) : 0u;
+    p.off_none = (p.f1bytes + p.f2bytes + 127u) & ~127u;
+    p.off_warp = p.off_none + 4u * kNone;
+    const uint32_t smem =
+        p.off_warp + static_cast<uint32_t>(kWarps) * (t.stream.form == 2 ? kWarpBytes2 : kWarpBytes8);
+    if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
+    const uint32_t need = (p.ntiles + kWarps - 1) / kWarps;
+    const uint32_t grid = need < static_cast<uint32_t>(sms) ? need : static_cast<uint32_t>(sms);
+    e = t.stream.form == 2 ? launch_stream2(mode, p, t.stream.step, grid, smem, max_smem, stream)
+                           : launch_stream8(mode, p, grid, smem, max_smem, stream);
+    if (e != cudaSuccess) return e;
+    const uint32_t n_sm = static_cast<uint32_t>(sms);
+    const bool g16 = t.gbits == 16;
+    if (t.B == 2)
+        return g16 ? launch_walk_modes<2, int16_t>(mode, p.f, n_sm, stream)
+                   : launch_walk_modes<2, int32_t>(mode, p.f, n_sm, stream);
+    return g16 ? launch_walk_modes<8, int16_t>(mode, p.f, n_sm, stream)
+               : launch_walk_modes<8, int32_t>(mode, p.f, n_sm, stream);
+}
+
+}  // namespace pfac

@@ -1,0 +1,171 @@
+"""The forms a single text takes with the tuning left as built, against the
+oracle, where they can go wrong: the short-text form (one thread per position,
+up to 2 MiB) at warp and CTA edges, the streaming form (tiles of 2,048
+positions, longer texts) at tile edges, texts and outputs off 16-byte
+boundaries, every filter it can have, bytes in no keyword, and texts with more
+walks than the walk list holds."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1412_7789_gb300 import api, workloads
+from tests import _gpu
+
+pytestmark = pytest.mark.gpu
+
+AT_MAX = 2 << 20  # the short-text form's longest text
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_1412_7789_gb300 import build
+
+    build.build()
+    api.lib()
+    yield
+    assert api.ac_device_status() == api.AC_OK
+
+
+def _letters(n, alphabet, seed):
+    a = np.frombuffer(alphabet, dtype=np.uint8)
+    return a[workloads.rng(seed).integers(0, a.size, size=n)]
+
+
+def _cut(text, seed, count, lmin, lmax):
+    """Half copied from the text, half random over its letters."""
+    r = workloads.rng(seed)
+    out = []
+    for i in range(count):
+        m = int(r.integers(lmin, lmax + 1))
+        if i % 2:
+            at = int(r.integers(0, text.size - m))
+            out.append(bytes(text[at:at + m]))
+        else:
+            out.append(bytes(r.permutation(text[:4 * m])[:m]))
+    return out
+
+
+# name: (alphabet, keywords, shortest, longest)
+SETS = {
+    "dna16": (b"ACGT", 600, 16, 40),    # every 4th position looked up, a second filter
+    "dna8": (b"ACGT", 300, 8, 32),      # every 2nd
+    "dna4": (b"ACGT", 200, 4, 40),      # every one
+    "dna1": (b"ACGT", 60, 1, 30),       # keywords shorter than any window
+    "iupac": (b"ACGTNRYKM", 200, 6, 20),  # 4-bit codes: no streaming form
+    "bytes4": (bytes(range(256)), 4000, 4, 30),
+    "bytes5": (bytes(range(256)), 4000, 5, 30),
+    "bytes9": (bytes(range(256)), 4000, 9, 30),
+    "bytes2": (bytes(range(256)), 3000, 2, 12),  # keywords shorter than the hashed window
+    "words4": (b"abcdefghijklmnopqrstuvwxyz ", 400, 4, 12),  # classes, not bytes
+    "words7": (b"abcdefghijklmnopqrstuvwxyz ", 400, 7, 20),
+}
+
+
+def _workload(name, n):
+    alphabet, count, lmin, lmax = SETS[name]
+    if len(alphabet) == 256:
+        text = workloads.zipf_text(n, 11)
+    else:
+        text = _letters(n, alphabet, 11)
+    pats = _cut(text, 12, count, lmin, lmax)
+    text = text.copy()
+    if len(alphabet) < 256:  # bytes in no keyword, alone and in a run
+        r = workloads.rng(13)
+        text[r.integers(0, n, size=n // 500 + 1)] = ord("#")
+        text[n // 3:n // 3 + 40] = ord("#")
+    return text, pats
+
+
+def _check(a, text, want, shift, out_shift):
+    import torch
+
+    n = text.size
+    buf = torch.zeros(n + shift, dtype=torch.uint8, device="cuda")
+    buf[shift:] = torch.from_numpy(text)
+    t = buf[shift:]
+    out = torch.full((n + out_shift + 8,), -7, dtype=torch.int32, device="cuda")
+    api.ac_match(a.handle, t, n, out[out_shift:])
+    got = out.cpu().numpy()
+    assert np.array_equal(got[out_shift:out_shift + n], want)
+    assert (got[:out_shift] == -7).all() and (got[out_shift + n:] == -7).all()  # nothing beside it
+    _gpu.check_all_modes(a.handle, text, want, t=t, modes=("count", "compact"))
+
+
+@pytest.mark.parametrize("name", sorted(SETS))
+def test_short_texts(name):
+    text, pats = _workload(name, 5000)
+    with api.Automaton(pats) as a:
+        for n in (1, 2, 15, 16, 17, 31, 32, 33, 47, 48, 127, 128, 129, 2047, 2048, 2049, 5000):
+            want = oracle.pfac_ids(pats, text[:n])
+            for shift in (0, 7):
+                _check(a, text[:n], want, shift, 0)
+
+
+@pytest.mark.parametrize("name", sorted(SETS))
+def test_streaming_edges(name):
+    """Lengths on both sides of the short-text limit and of tile edges, text
+    and output at several offsets from a 16-byte boundary."""
+    top = AT_MAX + 6144
+    text, pats = _workload(name, top)
+    want_all = oracle.pfac_ids(pats, text)
+    longest = max(len(p) for p in pats)
+    with api.Automaton(pats) as a:
+        for n, shift, out_shift in ((AT_MAX, 0, 0), (AT_MAX + 1, 0, 0), (AT_MAX + 2047, 1, 0), (AT_MAX + 2048, 0, 1),
+                                    (AT_MAX + 2049, 15, 3), (AT_MAX + 4096 + 13, 3, 2), (top, 8, 0)):
+            want = want_all[:n].copy()
+            tail = max(0, n - longest)  # a keyword may not reach past n
+            want[tail:] = oracle.pfac_ids(pats, text[tail:n])
+            _check(a, text[:n], want, shift, out_shift)
+
+
+@pytest.mark.parametrize("name", ["dna16", "dna8", "dna4", "bytes4", "bytes9", "words7"])
+def test_full_list(name):
+    for n in (3000, AT_MAX + 777):
+        text, pats = _workload(name, n)
+        ends, ids = oracle.full_occurrences(pats, text)
+        import torch
+
+        cap = len(ends) + 1
+        t = torch.from_numpy(text).cuda()
+        with api.Automaton(pats) as a:
+            e, i, c = a.match_full(t, cap=cap)
+        assert int(c.item()) == len(ends)
+        got = np.stack([e.cpu().numpy()[:len(ends)], i.cpu().numpy()[:len(ends)]], axis=1)
+        want = np.stack([np.asarray(ends), np.asarray(ids)], axis=1).astype(got.dtype)
+        assert np.array_equal(got[np.lexsort((got[:, 1], got[:, 0]))], want[np.lexsort((want[:, 1], want[:, 0]))])
+
+
+@pytest.mark.parametrize("letters,lens", [(b"A", (16, 20, 60)), (b"A", (4, 33)), (b"x", (6, 9, 40)), (b"x", (4, 50))])
+def test_more_walks_than_listed(letters, lens):
+    """A text of one letter: every position is a survivor and a long walk, far
+    more than the walk list holds; the rest are settled where they are found."""
+    n = AT_MAX + 3000
+    text = np.full(n, letters[0], dtype=np.uint8)
+    text[5000] = ord("C") if letters == b"A" else ord("y")
+    others = [b"ACGT" * 10, b"TTGACCA" * 3] if letters == b"A" else [bytes(range(40, 120)), b"xyzw" * 3]
+    pats = [letters * m for m in lens] + others
+    want = oracle.pfac_ids(pats, text)
+    assert (want >= 0).sum() > n // 2
+    with api.Automaton(pats) as a:
+        _check(a, text, want, 3, 0)
+
+
+def test_list_capacity_is_kept():
+    """A compacted list longer than its capacity: the first entries and the
+    whole count, and nothing written past the capacity."""
+    import torch
+
+    for n in (4096, AT_MAX + 4096):
+        text, pats = _workload("dna4", n)
+        wpos, wids = oracle.compact(oracle.pfac_ids(pats, text))
+        t = torch.from_numpy(text).cuda()
+        with api.Automaton(pats) as a:
+            for cap in (0, 1, wpos.size // 2):
+                pos = torch.full((wpos.size,), -7, dtype=torch.int32, device="cuda")
+                ids = torch.full((wpos.size,), -7, dtype=torch.int32, device="cuda")
+                c = torch.zeros(1, dtype=torch.int64, device="cuda")
+                api.ac_match_compact(a.handle, t, n, pos, ids, cap, c)
+                assert int(c.item()) == wpos.size
+                assert np.array_equal(pos[:cap].cpu().numpy(), wpos[:cap])
+                assert np.array_equal(ids[:cap].cpu().numpy(), wids[:cap])
+                assert bool((pos[cap:] == -7).all()) and bool((ids[cap:] == -7).all())
