@@ -318,9 +318,26 @@ cudaError_t run_tiled(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode,
     return e != cudaSuccess ? e : e2;
 }
 
+// The compacted or full list of one text through the bit-per-position output,
+// its scratch from the pool.
+cudaError_t run_bits(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out, bool full,
+                     cudaStream_t st) {
+    const size_t bytes = pfac::bits_scratch_bytes(h->dev, h->tuning, text, n, full);
+    cudaMemPool_t pool = nullptr;
+    cudaError_t e = scratch_pool(h->device, &pool);
+    if (e != cudaSuccess) return e;
+    void *scratch = nullptr;
+    e = cudaMallocFromPoolAsync(&scratch, bytes, pool, st);
+    if (e != cudaSuccess) return e;
+    e = pfac::enqueue_bits(h->dev, h->tuning, text, n, out, full, scratch, bytes, st);
+    const cudaError_t e2 = cudaFreeAsync(scratch, st);
+    return e != cudaSuccess ? e : e2;
+}
+
 // The compacted match of one text with its scratch from the pool.
 cudaError_t run_compact(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out,
                         cudaStream_t st) {
+    if (pfac::bits_serve(h->dev, h->tuning, n)) return run_bits(h, text, n, out, false, st);
     const uint32_t units = pfac::compact_units(h->dev, h->tuning, text, n);
     if (units == 0xFFFFFFFFu) return cudaErrorInvalidValue;
     // the phased form's lists instead of the dense fallback when it applies
@@ -343,6 +360,7 @@ cudaError_t run_compact(ac_automaton *h, const uint8_t *text, uint64_t n, const 
 // The full output of one text with its scratch from the pool.
 cudaError_t run_full(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out,
                      cudaStream_t st) {
+    if (pfac::bits_serve(h->dev, h->tuning, n)) return run_bits(h, text, n, out, true, st);
     const uint32_t units = pfac::compact_units(h->dev, h->tuning, text, n);
     if (units == 0xFFFFFFFFu) return cudaErrorInvalidValue;
     const size_t bytes = pfac::full_scratch_bytes(h->dev, h->tuning, units, n);

@@ -1,0 +1,292 @@
+// Compacted and full output of one text from a bit per position: after the
+// short-text or the streaming form has left, for every position with a match,
+// its bit and its id (OUT_BITS), the lists are made here:
+//   streaming form, compacted:  the scan of the tiles' match counts
+//                               (compact.cu), then bits_gather;
+//   streaming form, full:       full_bits_count (per tile, the occurrences its
+//                               results stand for), their scan, bits_gather;
+//   short texts:                bits_gather alone (full: full_bits_count
+//                               first), each CTA adding up what lies before
+//                               its own tiles.
+// bits_gather takes a tile with one warp: the tile's positions with a match go
+// to shared memory in ascending order, then one lane takes each, so a tile
+// dense in matches costs no more per match than a sparse one (the per-tile
+// slots and dense fallback of compact.cu rank 32 matches at most, and a fuller
+// tile's positions are all read back).
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "pfac_device.cuh"
+
+namespace pfac {
+
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kThreads = 256;
+constexpr uint32_t kWarps = kThreads / 32;
+constexpr uint32_t kTile = kStreamTile;
+constexpr uint32_t kWords = kTile / 32;  // bit words of a tile: two a lane
+
+struct BitsParams {
+    const uint32_t *bits;
+    const int32_t *ids;
+    uint32_t words, ntiles;  // bit words written, tiles
+    uint32_t head;           // bit position of the text's first byte
+    const uint32_t *counts;             // per tile: what it adds to the list (small, compacted: null)
+    const unsigned long long *prefix;   // its exclusive sum (small: null)
+    uint32_t *fcounts;                  // full_bits_count's output
+    // full output
+    const uint4 *rec;
+    const uint32_t *dups;
+    uint32_t max_clen, nkw;
+    unsigned int *err;
+    CompactOut out;
+};
+
+// A lane's two bit words of tile t (words past the last are 0).
+__device__ __forceinline__ uint2 tile_bits(const BitsParams &p, uint32_t t, int lane) {
+    const uint32_t w = t * kWords + 2u * static_cast<uint32_t>(lane);
+    uint2 b = make_uint2(0u, 0u);
+    if (w < p.words) b.x = __ldg(p.bits + w);
+    if (w + 1u < p.words) b.y = __ldg(p.bits + w + 1u);
+    return b;
+}
+
+// The tile positions of the set bits, in ascending order, to list; returns
+// how many there are.
+__device__ __forceinline__ uint32_t list_bits(uint2 b, uint16_t *list, int lane) {
+    const uint32_t c = static_cast<uint32_t>(__popc(b.x) + __popc(b.y));
+    uint32_t inc = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, d);
+        if (lane >= d) inc += y;
+    }
+    const uint32_t total = __shfl_sync(kFull, inc, 31);
+    uint32_t o = inc - c;
+    __syncwarp();  // the previous tile's readers are done
+    for (uint32_t m = b.x; m; m &= m - 1u) list[o++] = static_cast<uint16_t>(64u * lane + (__ffs(m) - 1));
+    for (uint32_t m = b.y; m; m &= m - 1u) list[o++] = static_cast<uint16_t>(64u * lane + 32u + (__ffs(m) - 1));
+    __syncwarp();
+    return total;
+}
+
+// One warp: tile t's part of the list, from index at on.
+template <bool FULL>
+__device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint2 b, unsigned long long at, uint16_t *list,
+                                         int lane) {
+    const uint32_t total = list_bits(b, list, lane);
+    const size_t g0 = static_cast<size_t>(t) * kTile;
+    for (uint32_t k0 = 0; k0 < total; k0 += 32u) {
+        const uint32_t k = k0 + static_cast<uint32_t>(lane);
+        const uint32_t i = k < total ? list[k] : 0u;
+        const uint32_t pos = static_cast<uint32_t>(g0) + i - p.head;
+        if (!FULL) {
+            if (k < total && at + k < p.out.cap) {
+                p.out.pos[at + k] = pos;
+                p.out.ids[at + k] = static_cast<uint32_t>(__ldg(p.ids + g0 + i));
+            }
+        } else {
+            uint32_t id = 0, cl = 0;
+            if (k < total) {
+                id = static_cast<uint32_t>(__ldg(p.ids + g0 + i));
+                cl = chain_len(p, id);
+            }
+            uint32_t inc = cl;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, inc, d);
+                if (lane >= d) inc += y;
+            }
+            if (k < total) put_chain(p, at + (inc - cl), pos, id);
+            at += __shfl_sync(kFull, inc, 31);
+        }
+    }
+}
+
+// The occurrences of each tile's results, one warp per tile.
+__global__ void __launch_bounds__(kThreads) full_bits_count(const BitsParams p) {
+    __shared__ uint16_t lists[kWarps][kTile];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t t = blockIdx.x * kWarps + static_cast<uint32_t>(warp); t < p.ntiles; t += gridDim.x * kWarps) {
+        const uint32_t total = list_bits(tile_bits(p, t, lane), lists[warp], lane);
+        uint32_t sum = 0;
+        for (uint32_t k = static_cast<uint32_t>(lane); k < total; k += 32u)
+            sum += chain_len(p, static_cast<uint32_t>(__ldg(p.ids + static_cast<size_t>(t) * kTile + lists[warp][k])));
+        sum = __reduce_add_sync(kFull, sum);
+        if (lane == 0) p.fcounts[t] = sum;
+    }
+}
+
+// The lists.  SMALL: a CTA has kWarps consecutive tiles, one a warp, and adds
+// up what lies before them; else warps take tiles in grid stride, at their
+// prefix, and skip the empty ones by their counts.
+template <bool FULL, bool SMALL>
+__global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
+    __shared__ uint16_t lists[kWarps][kTile];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (SMALL) {
+        __shared__ unsigned long long before[kWarps];
+        __shared__ uint32_t own[kWarps];
+        const uint32_t t0 = blockIdx.x * kWarps, t = t0 + static_cast<uint32_t>(warp);
+        unsigned long long sum = 0;
+        if (FULL) {
+            for (uint32_t i = threadIdx.x; i < t0; i += kThreads) sum += __ldg(p.counts + i);
+        } else {  // the words before the CTA's tiles, 16 bytes a thread
+            const uint4 *b = reinterpret_cast<const uint4 *>(p.bits);
+            for (uint32_t i = threadIdx.x; i < t0 * (kWords / 4u); i += kThreads) {
+                const uint4 v = __ldg(b + i);
+                sum += static_cast<uint32_t>(__popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
+            }
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(kFull, sum, d);
+        uint2 b = make_uint2(0u, 0u);
+        if (t < p.ntiles) b = tile_bits(p, t, lane);
+        uint32_t mine = 0;
+        if (FULL)
+            mine = t < p.ntiles ? __ldg(p.counts + t) : 0u;
+        else
+            mine = __reduce_add_sync(kFull, static_cast<uint32_t>(__popc(b.x) + __popc(b.y)));
+        if (lane == 0) {
+            before[warp] = sum;
+            own[warp] = mine;
+        }
+        __syncthreads();
+        unsigned long long at = 0, all = 0;
+        for (uint32_t w = 0; w < kWarps; ++w) all += before[w];
+        at = all;
+        for (uint32_t w = 0; w < kWarps; ++w) {
+            if (w < static_cast<uint32_t>(warp)) at += own[w];
+            all += own[w];
+        }
+        if (t < p.ntiles) put_tile<FULL>(p, t, b, at, lists[warp], lane);
+        if (t0 + kWarps >= p.ntiles && threadIdx.x == 0) *p.out.count = all;
+    } else {
+        const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
+        for (uint64_t u0 = gw; u0 < p.ntiles; u0 += 32ull * nw) {
+            const uint64_t u = u0 + static_cast<uint64_t>(lane) * nw;
+            const uint32_t c = u < p.ntiles ? __ldg(p.counts + u) : 0u;
+            for (uint32_t todo = __ballot_sync(kFull, c != 0u); todo; todo &= todo - 1u) {
+                const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
+                put_tile<FULL>(p, t, tile_bits(p, t, lane), __ldg(p.prefix + t), lists[warp], lane);
+            }
+        }
+        if (gw == 0 && lane == 0)
+            *p.out.count = __ldg(p.prefix + p.ntiles - 1u) + __ldg(p.counts + p.ntiles - 1u);
+    }
+}
+
+inline size_t round256(size_t v) { return (v + 255u) & ~static_cast<size_t>(255u); }
+
+// Scratch: walk counters (32) | per tile: matches, occurrences (4 each),
+// prefix (8) | partial sums | bits | walk list | ids.
+struct Layout {
+    size_t counts, fcounts, prefix, partials, bits, walks, ids, bytes;
+    uint32_t ntiles, walk_cap;
+    bool small;
+};
+
+Layout layout_of(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full) {
+    Layout l{};
+    l.small = at_serves(t, tu, n);
+    const uint64_t head = l.small ? 0u : reinterpret_cast<uintptr_t>(text) & 15u;
+    l.ntiles = static_cast<uint32_t>((n + head + kTile - 1) / kTile);
+    l.walk_cap = l.small ? 0u : stream_walk_cap(n);
+    size_t at = 256;
+    auto take = [&](size_t bytes) {
+        const size_t o = at;
+        at += round256(bytes);
+        return o;
+    };
+    l.counts = take(l.small ? 0 : 4ull * l.ntiles);
+    l.fcounts = take(full ? 4ull * l.ntiles : 0);
+    l.prefix = take(l.small ? 0 : 8ull * l.ntiles);
+    l.partials = take(l.small ? 0 : 8ull * kScanCtas);
+    l.bits = take(4ull * kWords * l.ntiles);
+    l.walks = take(8ull * l.walk_cap);
+    l.ids = take(4ull * kTile * l.ntiles);
+    l.bytes = at;
+    return l;
+}
+
+}  // namespace
+
+bool bits_serve(const DevTables &t, const Tuning &tu, uint64_t n) {
+    return at_serves(t, tu, n) || stream_serves(t, tu, n);
+}
+
+size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full) {
+    return layout_of(t, tu, text, n, full).bytes;
+}
+
+cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, const CompactOut &out,
+                         bool full, void *scratch, size_t scratch_bytes, cudaStream_t stream) {
+    if (!bits_serve(t, tu, n) || n == 0 || n > 0xFFFFFFFFull || !scratch || (full && (!t.full_rec || !t.full_dups)))
+        return cudaErrorInvalidValue;
+    const Layout l = layout_of(t, tu, text, n, full);
+    if (scratch_bytes < l.bytes) return cudaErrorInvalidValue;
+    uint8_t *b = static_cast<uint8_t *>(scratch);
+    MatchRequest r;
+    r.text = text;
+    r.n = n;
+    r.bits.bits = reinterpret_cast<uint32_t *>(b + l.bits);
+    r.bits.ids = reinterpret_cast<int32_t *>(b + l.ids);
+    cudaError_t e = cudaSuccess;
+    if (l.small) {
+        e = launch_at(t, r, OUT_BITS, stream);
+    } else {
+        r.bits.counts = reinterpret_cast<uint32_t *>(b + l.counts);
+        r.list_count = reinterpret_cast<unsigned int *>(b);
+        r.walks = reinterpret_cast<uint2 *>(b + l.walks);
+        r.walk_cap = l.walk_cap;
+        e = cudaMemsetAsync(b, 0, 32, stream);
+        if (e == cudaSuccess) e = launch_stream(t, r, OUT_BITS, tu, stream);
+    }
+    if (e != cudaSuccess) return e;
+
+    BitsParams p{};
+    p.bits = r.bits.bits;
+    p.ids = r.bits.ids;
+    p.head = l.small ? 0u : static_cast<uint32_t>(reinterpret_cast<uintptr_t>(text) & 15u);
+    p.words = l.small ? static_cast<uint32_t>((n + 31u) / 32u) : l.ntiles * kWords;
+    p.ntiles = l.ntiles;
+    p.counts = full ? reinterpret_cast<uint32_t *>(b + l.fcounts) : r.bits.counts;
+    p.fcounts = reinterpret_cast<uint32_t *>(b + l.fcounts);
+    unsigned long long *prefix = reinterpret_cast<unsigned long long *>(b + l.prefix);
+    p.prefix = l.small ? nullptr : prefix;
+    p.rec = t.full_rec;
+    p.dups = t.full_dups;
+    p.max_clen = t.full_max_clen;
+    p.nkw = t.nkw;
+    p.out = out;
+    e = device_error_word(&p.err);
+    if (e != cudaSuccess) return e;
+    const uint32_t need = (l.ntiles + kWarps - 1) / kWarps, sms = device_sm_count();
+    if (sms == 0) return cudaErrorInvalidDevice;
+    const uint32_t grid = need < sms * 6u ? need : sms * 6u;
+    if (full) {
+        full_bits_count<<<grid, kThreads, 0, stream>>>(p);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    if (l.small) {
+        if (full)
+            bits_gather<true, true><<<need, kThreads, 0, stream>>>(p);
+        else
+            bits_gather<false, true><<<need, kThreads, 0, stream>>>(p);
+        return cudaGetLastError();
+    }
+    e = launch_compact_scan(p.counts, l.ntiles, nullptr, prefix, reinterpret_cast<unsigned long long *>(b + l.partials),
+                            stream);
+    if (e != cudaSuccess) return e;
+    if (full)
+        bits_gather<true, false><<<grid, kThreads, 0, stream>>>(p);
+    else
+        bits_gather<false, false><<<grid, kThreads, 0, stream>>>(p);
+    return cudaGetLastError();
+}
+
+}  // namespace pfac
