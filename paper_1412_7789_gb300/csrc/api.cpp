@@ -53,6 +53,8 @@ struct ac_batch_plan {
     void *scratch = nullptr;
     void *lists = nullptr;  // the phased form's lists (ac_batch_reserve_lists)
     uint32_t list_cap = 0;
+    void *walks = nullptr;  // the streaming form's walk list (with the lists)
+    uint32_t walk_cap = 0;
     cudaStream_t capture = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -398,43 +400,25 @@ ac_status check_handles(const ac_handle *hs, uint32_t nh) {
 }
 
 // Enqueue a batch on `st`: clear the tile counters, plan on the device, then
-// match: when the filter kernel serves every automaton, one persistent launch
-// for all of them (each CTA takes the automata in turn, so they overlap and no
-// launch boundary drains the GPU between them); otherwise one persistent
-// launch per automaton, one after another.
+// match: with a walk list (walks), the automata the streaming form serves in
+// its launches; the others (without one: all), when the filter kernel serves
+// them, in one persistent launch (each CTA takes the automata in turn, so they
+// overlap and no launch boundary drains the GPU between them); otherwise one
+// persistent launch per automaton, one after another.
 cudaError_t enqueue_batch(const ac_handle *hs, uint32_t nh, void *scratch, const uint8_t *texts,
                           const ac_batch_item *items, uint32_t nitems, int32_t *out, cudaStream_t st,
-                          void *surv_lists = nullptr, uint32_t list_cap = 0) {
+                          void *surv_lists = nullptr, uint32_t list_cap = 0, void *walks = nullptr,
+                          uint32_t walk_cap = 0) {
     uint8_t *base = static_cast<uint8_t *>(scratch);
     pfac::BatchHead *heads = reinterpret_cast<pfac::BatchHead *>(base);
     uint8_t *counters = base + static_cast<size_t>(nh) * 16u;
     pfac::BatchItemDev *lists = reinterpret_cast<pfac::BatchItemDev *>(base + static_cast<size_t>(nh) * 32u);
-    std::vector<const pfac::DevTables *> ts(nh);
-    for (uint32_t a = 0; a < nh; ++a) ts[a] = &hs[a]->dev;
-    const bool multi = pfac::filter_multi_serves(ts.data(), nh);
-    std::vector<uint32_t> tile_len(nh);
-    for (uint32_t a = 0; a < nh; ++a)
-        tile_len[a] = multi ? pfac::filter_tile_positions() : pfac::unit_positions(hs[a]->dev, hs[a]->tuning);
-    cudaError_t e = cudaMemsetAsync(counters, 0, static_cast<size_t>(nh) * 16u, st);
-    if (e == cudaSuccess) e = pfac::launch_batch_plan(items, nitems, nh, texts, tile_len.data(), heads, lists, st);
-    if (multi) {
-        std::vector<pfac::MatchRequest> rs(nh);
-        for (uint32_t a = 0; a < nh; ++a) {
-            rs[a].text = texts;
-            rs[a].out = out;
-            rs[a].batch = heads + a;
-            rs[a].lists = lists;
-            rs[a].scratch = counters + 16u * a;
-            rs[a].scratch_bytes = 16;
-        }
-        if (e == cudaSuccess && surv_lists && list_cap) e = cudaMemsetAsync(surv_lists, 0, 32, st);
-        if (e == cudaSuccess)
-            e = pfac::launch_filter_multi(ts.data(), rs.data(), nh, pfac::OUT_DENSE, hs[0]->tuning.wait_ns, st,
-                                          list_cap ? surv_lists : nullptr, list_cap);
-        return e;
-    }
-    for (uint32_t a = 0; a < nh && e == cudaSuccess; ++a) {
-        cudaStream_t sa = st;
+    const bool streams = walks && walk_cap && nh <= pfac::kStreamBatchMax;
+    std::vector<const pfac::DevTables *> ts, sts;   // the filter kernel's, the streaming form's
+    std::vector<pfac::MatchRequest> rs, srs;
+    std::vector<uint32_t> rest;                     // the filter kernel's automata
+    std::vector<uint32_t> tile_len(nh, pfac::kStreamTile);
+    for (uint32_t a = 0; a < nh; ++a) {
         pfac::MatchRequest r;
         r.text = texts;
         r.out = out;
@@ -442,9 +426,32 @@ cudaError_t enqueue_batch(const ac_handle *hs, uint32_t nh, void *scratch, const
         r.lists = lists;
         r.scratch = counters + 16u * a;
         r.scratch_bytes = 16;
-        ac_automaton *h = hs[a];
-        e = pfac::launch_match(h->dev, r, pfac::OUT_DENSE, h->tuning, sa);
+        const bool s = streams && pfac::stream_batch_serves(hs[a]->dev, hs[a]->tuning);
+        (s ? sts : ts).push_back(&hs[a]->dev);
+        (s ? srs : rs).push_back(r);
+        if (!s) rest.push_back(a);
     }
+    const uint32_t nr = static_cast<uint32_t>(rest.size());
+    const bool multi = pfac::filter_multi_serves(ts.data(), nr);
+    for (uint32_t a : rest)
+        tile_len[a] = multi ? pfac::filter_tile_positions() : pfac::unit_positions(hs[a]->dev, hs[a]->tuning);
+    cudaError_t e = cudaMemsetAsync(counters, 0, static_cast<size_t>(nh) * 16u, st);
+    if (e == cudaSuccess) e = pfac::launch_batch_plan(items, nitems, nh, texts, tile_len.data(), heads, lists, st);
+    if (e == cudaSuccess && !sts.empty()) {
+        e = cudaMemsetAsync(walks, 0, 32, st);
+        if (e == cudaSuccess)
+            e = pfac::launch_stream_batch(sts.data(), srs.data(), static_cast<uint32_t>(sts.size()), pfac::OUT_DENSE,
+                                          hs[0]->tuning.wait_ns, walks, walk_cap, st);
+    }
+    if (multi) {
+        if (e == cudaSuccess && surv_lists && list_cap) e = cudaMemsetAsync(surv_lists, 0, 32, st);
+        if (e == cudaSuccess)
+            e = pfac::launch_filter_multi(ts.data(), rs.data(), nr, pfac::OUT_DENSE, hs[0]->tuning.wait_ns, st,
+                                          list_cap ? surv_lists : nullptr, list_cap);
+        return e;
+    }
+    for (uint32_t i = 0; i < nr && e == cudaSuccess; ++i)
+        e = pfac::launch_match(*ts[i], rs[i], pfac::OUT_DENSE, hs[rest[i]]->tuning, st);
     return e;
 }
 
@@ -922,6 +929,7 @@ ac_status ac_batch_destroy(ac_batch b) {
     if (b->capture) cudaStreamDestroy(b->capture);
     if (b->scratch) cudaFree(b->scratch);
     if (b->lists) cudaFree(b->lists);
+    if (b->walks) cudaFree(b->walks);
     delete b;
     return AC_OK;
 }
@@ -967,15 +975,35 @@ ac_status ac_batch_reserve_lists(ac_batch b, uint64_t text_bytes) {
         b->list_cap = 0;
         if (e != cudaSuccess) return cuda_status(e);
     }
+    if (b->walks) {
+        cudaError_t e = cudaFree(b->walks);
+        b->walks = nullptr;
+        b->walk_cap = 0;
+        if (e != cudaSuccess) return cuda_status(e);
+    }
     if (cap == 0) return AC_OK;
-    void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, pfac::multi_lists_bytes(static_cast<uint32_t>(cap)));
+    // the filter kernel's lists for the automata it matches, the streaming
+    // form's walk list for the others
+    uint32_t streamed = 0;
+    for (ac_handle h : b->hs) streamed += pfac::stream_batch_serves(h->dev, h->tuning) ? 1u : 0u;
+    cudaError_t e = cudaSuccess;
+    // (a handle tuned later goes to the other kernel without a list)
+    if (streamed < b->hs.size() || b->hs.size() > pfac::kStreamBatchMax) {
+        e = cudaMalloc(&b->lists, pfac::multi_lists_bytes(static_cast<uint32_t>(cap)));
+        if (e == cudaSuccess) b->list_cap = static_cast<uint32_t>(cap);
+    }
+    if (e == cudaSuccess && streamed && b->hs.size() <= pfac::kStreamBatchMax) {
+        const uint32_t wc = pfac::stream_batch_cap(text_bytes);
+        e = cudaMalloc(&b->walks, pfac::stream_batch_bytes(wc));
+        if (e == cudaSuccess) b->walk_cap = wc;
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
+        if (b->lists) cudaFree(b->lists);
+        b->lists = b->walks = nullptr;  // a failed allocation leaves its pointer unset
+        b->list_cap = b->walk_cap = 0;
         return e == cudaErrorMemoryAllocation ? AC_ERR_OOM : cuda_status(e);
     }
-    b->lists = p;
-    b->list_cap = static_cast<uint32_t>(cap);
     return AC_OK;
 }
 
@@ -983,7 +1011,7 @@ namespace {
 ac_status batch_enqueue(ac_batch b, const uint8_t *d_texts, const ac_batch_item *d_items, uint32_t nitems,
                         int32_t *d_out, cudaStream_t st) {
     return cuda_status(enqueue_batch(b->hs.data(), static_cast<uint32_t>(b->hs.size()), b->scratch, d_texts, d_items,
-                                     nitems, d_out, st, b->lists, b->list_cap));
+                                     nitems, d_out, st, b->lists, b->list_cap, b->walks, b->walk_cap));
 }
 
 ac_status check_plan_args(ac_batch b, const uint8_t *d_texts, const ac_batch_item *d_items, uint32_t nitems,

@@ -284,36 +284,56 @@ void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTa
             for (uint32_t j = 0; j < len; ++j) w |= static_cast<uint32_t>(h.cls8[patterns[id][o + j]]) << (2u * j);
             return w;
         };
-        // the fewest lookups whose filter stays sparse: with it too dense, the
-        // candidates of the chance hits cost more than the lookups saved
-        for (uint32_t step : {4u, 2u}) {
+        // every 4th, 2nd or single position looked up, by the warp
+        // instructions that costs per 32 positions, lookups and candidates:
+        // about 7 a lookup; 150 a round of 32 candidates, and half as much
+        // again for its two dependent loads; 60 a round in the second filter.
+        // A set bit makes `step` candidates, less those the second filter
+        // drops; that exists where every keyword has win2 codes from every
+        // offset, more than the first filter's.  (Batch sets of 8 to 64
+        // letters: 1,000 keywords 8.3 / 4.2 / 7.3 for steps 4 / 2 / 1, 9,500
+        // keywords - / 11.3 / 9.7.)
+        constexpr uint32_t kWords2 = 8192u;  // 32 KiB
+        auto bits_of = [](const std::vector<uint32_t> &F) {
+            uint64_t bits = 0;
+            for (uint32_t x : F) bits += static_cast<uint64_t>(__builtin_popcount(x));
+            return static_cast<double>(bits) / (32.0 * static_cast<double>(F.size()));
+        };
+        const double dense = bits_of(h.F);
+        double best = 7.0 + 225.0 * dense;
+        for (uint32_t step : {2u, 4u}) {
             if (h.minlen < step + 4u) continue;  // at most 4^6 completions a window
-            std::vector<uint32_t> F(kWords, 0u);
+            std::vector<uint32_t> F(kWords, 0u), F2;
             for (uint32_t id = 0; id < h.nkw; ++id)
                 for (uint32_t o = 0; o < step; ++o) {
                     const uint32_t len = std::min(k, lens[id] - o);
                     const uint32_t w = codes(id, o, len);
                     for (uint32_t v = w; v < (1u << (2u * k)); v += 1u << (2u * len)) set_bit(F.data(), v);
                 }
-            uint64_t bits = 0;
-            for (uint32_t x : F) bits += static_cast<uint64_t>(__builtin_popcount(x));
-            if (bits * 25u > (1ull << kFilterBits)) continue;  // over 4 %
-            st.step = step;
-            h.stream_F1 = std::move(F);
-            // windows longer than the filter's, where every keyword has them
+            const double d = bits_of(F);
+            double cost = 7.0 / step + 225.0 * d;
             const uint32_t win2 = std::min(16u, h.minlen - (step - 1u));
             if (win2 >= k + 2u) {
-                constexpr uint32_t kWords2 = 8192u;  // 32 KiB
-                st.win2 = win2;
-                h.stream_F2.assign(kWords2, 0u);
+                F2.assign(kWords2, 0u);
                 for (uint32_t id = 0; id < h.nkw; ++id)
                     for (uint32_t o = 0; o < step; ++o) {
                         const uint32_t x = (codes(id, o, win2) << (32u - 2u * win2)) * kFilterHashMul;
-                        h.stream_F2[(static_cast<uint64_t>(x) * kWords2) >> 32] |= 1u << ((x >> 12) & 31u);
+                        F2[(static_cast<uint64_t>(x) * kWords2) >> 32] |= 1u << ((x >> 12) & 31u);
                     }
+                cost = 7.0 / step + 60.0 * d / step + 225.0 * d * bits_of(F2);
             }
-            break;
+            if (cost >= best) continue;
+            best = cost;
+            st.step = step;
+            st.win2 = F2.empty() ? 0u : win2;
+            h.stream_F1 = std::move(F);
+            h.stream_F2 = std::move(F2);
         }
+        // every position looked up and the root filter over 10 % full: the
+        // rounds that resolve the survivors cost more than the filter kernel's
+        // in-warp pipeline (64 MiB of uniform text, dense ids: at 6 % of the
+        // windows ending a keyword 163 against 182 us, at 20 % 330 against 240)
+        if (st.step == 1u && dense > 0.1) return;
         st.form = 2;
         st.win1 = k;
         st.root = k;

@@ -401,6 +401,18 @@ struct Tuning {
     int stall_help = 0;   // test aid: owners wait for one chunk more than their heavy tile has
 };
 
+// The streaming form over a batch: whether it serves the automaton, and the
+// launches for nh (<= 32) automata it serves (rs: as launch_filter_multi's, the
+// units being tiles of kStreamTile positions).  walks: stream_batch_bytes(cap)
+// bytes whose first 32 are zeroed; walks past cap are settled where they are
+// found.
+bool stream_batch_serves(const DevTables &t, const Tuning &tu);
+uint32_t stream_batch_cap(uint64_t text_bytes);
+inline size_t stream_batch_bytes(uint32_t cap) { return 32 + 16ull * cap; }
+constexpr uint32_t kStreamBatchMax = 32;
+cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *rs, uint32_t nh, OutMode mode,
+                                unsigned long long wait_ns, void *walks, uint32_t walk_cap, cudaStream_t stream);
+
 // One short text (dense ids or count): one thread per position, everything
 // from global memory (stream.cu).  Needs no scratch.
 bool at_serves(const DevTables &t, const Tuning &tu, uint64_t n);

@@ -1,6 +1,8 @@
 // One text in two launches, or one: the streaming form (stream_kernel.cuh) and
 // its walk step, and the form for short texts (one thread per position).
 
+#include <mutex>
+
 #include "stream_kernel.cuh"
 
 namespace pfac {
@@ -128,7 +130,7 @@ cudaError_t launch_walk_modes(OutMode mode, const FilterParams &p, uint32_t sms,
 
 // Every knob as built: the caller asks for no particular form.
 bool untuned(const Tuning &tu) {
-    return tu.block == 0 && tu.stages == 0 && tu.grid == 0 && tu.variant == 0 && tu.per_thread == 0 &&
+    return tu.block == 0 && tu.stages == 0 && tu.grid == 0 && tu.variant == 0 && tu.per_thread != 4 &&
            tu.halo <= 16 && tu.survivor_list == 0 && !tu.stall_help;
 }
 
@@ -158,8 +160,39 @@ bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
 uint32_t stream_walk_cap(uint64_t n) {
     // a walk for every eighth position, and each warp's last reservation
     // (positions past that are settled where they are found)
-    return static_cast<uint32_t>(n / 8) + device_sm_count() * static_cast<uint32_t>(kWarps) * kWalkChunkEntries;
+    return static_cast<uint32_t>(n / 8) + device_sm_count() * static_cast<uint32_t>(kMostWarps) * kWalkChunkEntries;
 }
+
+namespace {
+
+// The streaming form's parameters of one automaton, all but the places in
+// shared memory.
+cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu, StreamParams &p) {
+    const cudaError_t e = filter_params(t, r, mode, tu, p.f);
+    if (e != cudaSuccess) return e;
+    if (mode == OUT_BITS && !r.bits.counts) return cudaErrorInvalidValue;
+    p.f.walks = r.walks;
+    p.f.walk_cap = r.walk_cap;
+    p.f.list_count = r.list_count;
+    p.F1 = t.stream_F1 ? t.stream_F1 : t.F;
+    p.f1bytes = (1u << kFilterBits) / 8u;
+    p.F2 = t.stream_F2;
+    p.f2bytes = t.stream_F2 ? t.stream_f2bytes : 0u;
+    p.m1 = t.stream.m1;
+    p.m2 = t.stream.m2;
+    p.l2shift = t.stream.form == 2 ? 32u - 2u * t.stream.win2 : 0u;
+    return cudaSuccess;
+}
+
+// Shared memory of a launch: the filters, the -1 buffer (and 128 bytes for the
+// CTA), the warps' areas.
+uint32_t stream_smem(uint32_t form, uint32_t filters, uint32_t *off_none, uint32_t *off_warp) {
+    *off_none = (filters + 127u) & ~127u;
+    *off_warp = *off_none + 4u * kNone + 128u;
+    return *off_warp + static_cast<uint32_t>(block_of(form) / 32) * (form == 2 ? kWarpBytes2 : kWarpBytes8);
+}
+
+}  // namespace
 
 cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
                           cudaStream_t stream) {
@@ -169,32 +202,13 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
     cudaError_t e = filter_device_shape(&sms, &max_smem);
     if (e != cudaSuccess) return e;
     StreamParams p{};
-    e = filter_params(t, r, mode, tu, p.f);
+    e = stream_params(t, r, mode, tu, p);
     if (e != cudaSuccess) return e;
-    p.f.walks = r.walks;
-    p.f.walk_cap = r.walk_cap;
-    p.f.list_count = r.list_count;
-    p.F1 = t.stream_F1 ? t.stream_F1 : t.F;
-    p.f1bytes = (1u << kFilterBits) / 8u;
-    p.F2 = t.stream_F2;
-    p.f2bytes = t.stream_F2 ? t.stream_f2bytes : 0u;
-    p.head = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(r.text) & 15u);
-    p.f.bits_head = p.head;
-    if (mode == OUT_BITS && !r.bits.counts) return cudaErrorInvalidValue;
-    p.ntiles = static_cast<uint32_t>((r.n + p.head + kTile - 1) / kTile);
-    p.m1 = t.stream.m1;
-    p.m2 = t.stream.m2;
-    p.l2shift = t.stream.form == 2 ? 32u - 2u * t.stream.win2 : 0u;
-    // the tiles whose bytes, and the 16 after them, are all in the text's
-    // 16-byte aligned part
-    p.in_lo = p.f.a1 ? 1u : 0u;
-    p.in_hi = p.f.a2 >= 16u ? static_cast<uint32_t>((p.f.a2 - 16u) / kTile) : 0u;
-    p.off_none = (p.f1bytes + p.f2bytes + 127u) & ~127u;
-    p.off_warp = p.off_none + 4u * kNone;
-    const uint32_t smem =
-        p.off_warp + static_cast<uint32_t>(kWarps) * (t.stream.form == 2 ? kWarpBytes2 : kWarpBytes8);
+    const uint64_t head = reinterpret_cast<uintptr_t>(r.text) & 15u;
+    p.ntiles = static_cast<uint32_t>((r.n + head + kTile - 1) / kTile);
+    const uint32_t smem = stream_smem(t.stream.form, p.f1bytes + p.f2bytes, &p.off_none, &p.off_warp);
     if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
-    const uint32_t need = (p.ntiles + kWarps - 1) / kWarps;
+    const uint32_t nw = static_cast<uint32_t>(block_of(t.stream.form) / 32), need = (p.ntiles + nw - 1) / nw;
     const uint32_t grid = need < static_cast<uint32_t>(sms) ? need : static_cast<uint32_t>(sms);
     e = t.stream.form == 2 ? launch_stream2(mode, p, t.stream.step, grid, smem, max_smem, stream)
                            : launch_stream8(mode, p, grid, smem, max_smem, stream);
@@ -206,6 +220,67 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
                    : launch_walk_modes<2, int32_t>(mode, p.f, n_sm, stream);
     return g16 ? launch_walk_modes<8, int16_t>(mode, p.f, n_sm, stream)
                : launch_walk_modes<8, int32_t>(mode, p.f, n_sm, stream);
+}
+
+bool stream_batch_serves(const DevTables &t, const Tuning &tu) { return stream_serves(t, tu, 0); }
+
+uint32_t stream_batch_cap(uint64_t text_bytes) { return stream_walk_cap(text_bytes); }
+
+cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *rs, uint32_t nh, OutMode mode,
+                                unsigned long long wait_ns, void *walks, uint32_t walk_cap, cudaStream_t stream) {
+    if (nh == 0 || nh > kStreamMultiMax || !walks || walk_cap == 0 || (mode != OUT_DENSE && mode != OUT_BITS))
+        return cudaErrorInvalidValue;
+    int sms = 0, max_smem = 0;
+    cudaError_t e = filter_device_shape(&sms, &max_smem);
+    if (e != cudaSuccess) return e;
+    // some 20 KiB of parameters a launch: kept off the stack, filled and
+    // launched under a lock
+    static StreamMulti mp;
+    static WalkMulti wm;
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    Tuning tu;
+    tu.wait_ns = wait_ns;
+    uint8_t *b = static_cast<uint8_t *>(walks);
+    wm.nh = nh;
+    // one launch per form and step, then the walks of all
+    for (uint32_t group = 0; group < 4; ++group) {
+        const uint32_t form = group < 3 ? 2u : 8u, step = group < 3 ? 1u << group : 1u;
+        uint32_t filters = 0;
+        mp.nh = 0;
+        for (uint32_t a = 0; a < nh; ++a) {
+            const DevTables &t = *ts[a];
+            if (t.stream.form != form || t.stream.step != step) continue;
+            const MatchRequest &r = rs[a];
+            if (!stream_batch_serves(t, tu) || !r.batch || !r.lists || !r.scratch || r.scratch_bytes < 16)
+                return cudaErrorInvalidValue;
+            StreamParams &p = mp.a[mp.nh++];
+            p = StreamParams{};
+            e = stream_params(t, r, mode, tu, p);
+            if (e != cudaSuccess) return e;
+            p.f.sl.ubase = r.slots.ubase;
+            p.f.aidx = a;
+            p.f.list_count = reinterpret_cast<unsigned int *>(b);
+            p.f.walks4 = reinterpret_cast<uint4 *>(b + 32);
+            p.f.walk_cap = walk_cap;
+            wm.a[a] = p.f;
+            filters = filters > p.f1bytes + p.f2bytes ? filters : p.f1bytes + p.f2bytes;
+        }
+        if (mp.nh == 0) continue;
+        const uint32_t smem = stream_smem(form, filters, &mp.off_none, &mp.off_warp);
+        if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
+        const uint32_t grid = static_cast<uint32_t>(sms);
+        e = form == 2 ? launch_stream2_multi(mode, mp, step, grid, smem, max_smem, stream)
+                      : launch_stream8_multi(mode, mp, grid, smem, max_smem, stream);
+        if (e != cudaSuccess) return e;
+    }
+    const uint32_t grid = static_cast<uint32_t>(sms) * 8u;
+    const uint32_t smem = nh * (static_cast<uint32_t>(sizeof(FilterParams)) + 256u);
+    if (mode == OUT_DENSE)
+        pfac_stream_walks_multi<OUT_DENSE><<<grid, kWalkBlock, smem, stream>>>(wm);
+    else
+        pfac_stream_walks_multi<OUT_BITS><<<grid, kWalkBlock, smem, stream>>>(wm);
+    return cudaGetLastError();
 }
 
 }  // namespace pfac

@@ -47,10 +47,14 @@ namespace strm {
 using filt::FilterParams;
 using filt::kFull;
 
-constexpr int kBlock = 768;
-constexpr int kWarps = kBlock / 32;
+// Threads per CTA, one CTA per SM (GB300, 1 GiB: with 2-bit codes 640 / 768
+// threads count in 288 / 275 us; with 8-bit codes 512 / 640 / 768 write dense
+// ids in 1155 / 1064 / 1178 us, 768 spilling at 80 registers).
+constexpr int kBlock2 = 768;
+constexpr int kBlock8 = 640;
+constexpr int kMostWarps = (kBlock2 > kBlock8 ? kBlock2 : kBlock8) / 32;
+__host__ __device__ constexpr int block_of(uint32_t form) { return form == 2 ? kBlock2 : kBlock8; }
 constexpr uint32_t kTile = kStreamTile;  // positions a warp takes at a time
-constexpr uint32_t kUnit = kStreamUnit;  // positions per unit of a walk entry
 constexpr uint32_t kChunk = 512;         // positions per warp-wide 16-byte load
 constexpr uint32_t kQueue = 256;         // survivors of a tile kept in shared memory at a time
 constexpr uint32_t kNone = 1024;          // ids of -1 in shared memory
@@ -66,8 +70,6 @@ struct StreamParams {
     const uint32_t *F2;    // second filter (f2bytes; 0: none), with 8-bit codes then its short-keyword part
     uint32_t f1bytes, f2bytes;
     uint32_t ntiles;
-    uint32_t in_lo, in_hi;  // the tiles wholly inside the text, with the 16 bytes after them
-    uint32_t head;         // text - f.gbase
     uint32_t m1, m2;       // 8-bit codes: multipliers of the window's words
     uint32_t l2shift;      // 2-bit codes: left shift that drops the codes past the second filter's window
     uint32_t off_none, off_warp;
@@ -84,11 +86,46 @@ __device__ __forceinline__ uint4 ldg_stream(const uint8_t *p, uint64_t pol) {
 
 // The 16 bytes at gbase + off with the bytes outside the text zero.
 static __device__ __noinline__ uint4 load_fringe(const uint8_t *gbase, uint64_t off, uint64_t head, uint64_t end) {
+    if (off >= head && off + 16u <= end) return __ldg(reinterpret_cast<const uint4 *>(gbase + off));
     uint32_t v[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (uint32_t j = 0; j < 16; ++j)
         if (off + j >= head && off + j < end) v[j >> 2] |= static_cast<uint32_t>(__ldg(gbase + off + j)) << (8u * (j & 3u));
     return make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+// The text a warp's tiles belong to.  Positions are named by g, their index
+// from the first position of tile t0: the text's position t0 * kTile + g - head.
+// (One text: t0 = 0.  A batch: a few consecutive tiles of one text.)
+struct Seg {
+    const uint8_t *text;   // first byte
+    const uint8_t *gbase;  // the same, rounded down to 16 bytes
+    int32_t *out;          // dense ids
+    uint64_t n;
+    uint32_t head;         // text - gbase
+    uint32_t t0;
+    uint32_t in_lo, in_hi;  // the tiles wholly inside the text, with the 16 bytes after them
+    uint32_t bit0;         // OUT_BITS: g + bit0 is the position's bit
+    uint32_t unit0, item;  // a batch: work unit of tile t0, the text's entry in the planned list
+};
+
+__device__ __forceinline__ uint64_t text_pos(const Seg &sg, uint32_t g) {  // before the text wraps
+    return static_cast<uint64_t>(sg.t0) * kTile + g - sg.head;
+}
+
+// The text's part of a segment.
+__device__ __forceinline__ Seg make_seg(const uint8_t *text, int32_t *out, uint64_t n) {
+    Seg sg;
+    sg.text = text;
+    sg.out = out;
+    sg.n = n;
+    sg.head = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(text) & 15u);
+    sg.gbase = text - sg.head;
+    const uint64_t a2 = (sg.head + n) & ~15ull;  // end of the text's 16-byte aligned part
+    sg.in_lo = sg.head ? 1u : 0u;
+    sg.in_hi = a2 >= 16u ? static_cast<uint32_t>((a2 - 16u) / kTile) : 0u;
+    sg.t0 = sg.bit0 = sg.unit0 = sg.item = 0;
+    return sg;
 }
 
 // A tile's registers: lane l's 16 bytes of chunks 0-3, and (lane 0) the 16
@@ -98,29 +135,32 @@ struct TileRegs {
     uint4 look;
 };
 
-// The loads of a warp's tiles: lane l's address in tile 0.
-struct Loader {
-    const uint8_t *base;
-    uint64_t pol;
-    // chunk C (4: the look-ahead) of tile t (< ntiles)
-    template <int C>
-    __device__ __forceinline__ void load(const StreamParams &p, uint32_t t, int lane, TileRegs &r) const {
-        const uint64_t lo = static_cast<uint64_t>(t) * kTile;
-        if (t >= p.in_lo && t < p.in_hi) {
-            if constexpr (C < 4)
-                r.c[C] = ldg_stream(base + lo + static_cast<uint32_t>(C) * kChunk, pol);
-            else if (lane == 0)
-                r.look = ldg_stream(base + lo + kTile, pol);
-        } else {
-            const uint64_t end = p.head + p.f.n;
-            if constexpr (C < 4)
-                r.c[C] = load_fringe(p.f.gbase, lo + static_cast<uint32_t>(C) * kChunk + 16u * static_cast<uint32_t>(lane),
-                                     p.head, end);
-            else if (lane == 0)
-                r.look = load_fringe(p.f.gbase, lo + kTile, p.head, end);
-        }
+// Issue the loads of chunk C (4: the look-ahead) of the text's tile t.
+template <int C>
+__device__ __forceinline__ void load_chunk(const Seg &sg, uint32_t t, uint64_t pol, int lane, TileRegs &r) {
+    const uint64_t lo = static_cast<uint64_t>(t) * kTile;
+    if (t >= sg.in_lo && t < sg.in_hi) {
+        if constexpr (C < 4)
+            r.c[C] = ldg_stream(sg.gbase + lo + static_cast<uint32_t>(C) * kChunk + 16u * static_cast<uint32_t>(lane), pol);
+        else if (lane == 0)
+            r.look = ldg_stream(sg.gbase + lo + kTile, pol);
+    } else {
+        const uint64_t end = sg.head + sg.n;
+        if constexpr (C < 4)
+            r.c[C] = load_fringe(sg.gbase, lo + static_cast<uint32_t>(C) * kChunk + 16u * static_cast<uint32_t>(lane),
+                                 sg.head, end);
+        else if (lane == 0)
+            r.look = load_fringe(sg.gbase, lo + kTile, sg.head, end);
     }
-};
+}
+
+__device__ __forceinline__ void load_tile(const Seg &sg, uint32_t t, uint64_t pol, int lane, TileRegs &r) {
+    load_chunk<0>(sg, t, pol, lane, r);
+    load_chunk<1>(sg, t, pol, lane, r);
+    load_chunk<2>(sg, t, pol, lane, r);
+    load_chunk<3>(sg, t, pol, lane, r);
+    load_chunk<4>(sg, t, pol, lane, r);
+}
 
 // The id of the longest keyword starting at text position gi, all from global
 // memory: the window and stride tables, or the state hash, then the walk.
@@ -184,26 +224,40 @@ static __device__ __noinline__ int match_at_far(const FilterParams &p, const uin
     return match_at<GT>(p, cls8, tt, gi, B);
 }
 
-// An id found at text position gi.
+// An id found at position g.
 template <int MODE>
-__device__ __forceinline__ void put_id(const FilterParams &p, uint64_t gi, int r, uint32_t &cnt) {
+__device__ __forceinline__ void put_id(const FilterParams &p, const Seg &sg, uint32_t g, int r, uint32_t &cnt) {
     if (r < 0) return;
     if (MODE == OUT_DENSE) {
-        p.out[gi] = r;
+        sg.out[text_pos(sg, g)] = r;
     } else if (MODE == OUT_COUNT) {
         ++cnt;
     } else {
-        const uint32_t g = static_cast<uint32_t>(gi) + p.bits_head;
-        p.bo.ids[g] = r;
-        atomicOr(p.bo.bits + (g >> 5), 1u << (g & 31u));
-        atomicAdd(p.bo.counts + g / kTile, 1u);
+        const uint32_t b = g + sg.bit0;
+        p.bo.ids[b] = r;
+        atomicOr(p.bo.bits + (b >> 5), 1u << (b & 31u));
+        atomicAdd(p.bo.counts + b / kTile, 1u);
     }
 }
 
-// Positions are named by g, their index from gbase (text position + head).
-// Walk-list entry: {g, state | d << 31}: the walk goes on from the state with
-// the byte k + k2 + d after the position; state 0: not resolved at all.  An
-// empty entry's g is 0xFFFFFFFF.
+// Walk-list entries.  One text: {g, state | d << 31}: the walk goes on from the
+// state with the byte k + k2 + d after the position; state 0: not resolved at
+// all.  A batch: {work unit, state | d << 31, automaton << 11 | position in the
+// unit, planned-list entry}.  An empty entry's first word is 0xFFFFFFFF.
+template <bool BATCH>
+__device__ __forceinline__ void store_walk(const FilterParams &p, const Seg &sg, uint32_t slot, uint32_t g, uint32_t s) {
+    if (BATCH)
+        p.walks4[slot] = make_uint4(sg.unit0 + g / kTile, s, (p.aidx << 11) | (g & (kTile - 1u)), sg.item);
+    else
+        p.walks[slot] = make_uint2(g, s);
+}
+template <bool BATCH>
+__device__ __forceinline__ void blank_walk(const FilterParams &p, uint32_t slot) {
+    if (BATCH)
+        p.walks4[slot] = make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
+    else
+        p.walks[slot] = make_uint2(0xFFFFFFFFu, 0u);
+}
 
 // Walks to the walk list (all lanes of the warp; want: this lane has one).
 // Space is reserved in chunks; when one runs out its rest takes the first
@@ -212,7 +266,9 @@ struct WalkRoom {
     uint32_t next, end;  // the warp's chunk
     bool full;           // nothing more to reserve (the counter is left alone then)
 };
-__device__ __forceinline__ bool push_walk(const StreamParams &p, WalkRoom &room, bool want, uint2 e, int lane) {
+template <bool BATCH>
+__device__ __forceinline__ bool push_walk(const StreamParams &p, const Seg &sg, WalkRoom &room, bool want, uint32_t g,
+                                          uint32_t s, int lane) {
     const unsigned m = __ballot_sync(kFull, want);
     if (!m) return true;
     const uint32_t need = __popc(m), rank = __popc(m & ((1u << lane) - 1u)), rest = room.end - room.next;
@@ -236,14 +292,14 @@ __device__ __forceinline__ bool push_walk(const StreamParams &p, WalkRoom &room,
     } else {
         room.next += need;
     }
-    if (stored) p.f.walks[slot] = e;
+    if (stored) store_walk<BATCH>(p.f, sg, slot, g, s);
     return !want || stored;
 }
 
 // The warp's unused walk-list entries are empty.
-__device__ __forceinline__ void close_room(const StreamParams &p, const WalkRoom &room, int lane) {
-    for (uint32_t j = room.next + static_cast<uint32_t>(lane); j < room.end; j += 32u)
-        p.f.walks[j] = make_uint2(0xFFFFFFFFu, 0u);
+template <bool BATCH>
+__device__ __forceinline__ void close_room(const FilterParams &f, const WalkRoom &room, int lane) {
+    for (uint32_t j = room.next + static_cast<uint32_t>(lane); j < room.end; j += 32u) blank_walk<BATCH>(f, j);
 }
 
 // -1 for every position of tile t inside the text.  BULK (8-bit codes): bulk
@@ -256,11 +312,11 @@ __device__ __forceinline__ void close_room(const StreamParams &p, const WalkRoom
 // the output's own alignment: a tile whose first id is m ids past a boundary
 // writes its first 4 - m and last m ids one by one.
 template <bool BULK>
-__device__ __forceinline__ void fill_none(const StreamParams &p, const int32_t *none, uint32_t t, int lane) {
-    const int64_t lo = static_cast<int64_t>(static_cast<uint64_t>(t) * kTile) - p.head;
-    int32_t *o = p.f.out + lo;
-    if (t >= p.in_lo && t < p.in_hi) {
-        if (BULK && p.f.vec_ok) {
+__device__ __forceinline__ void fill_none(const Seg &sg, const int32_t *none, uint32_t t, int lane) {
+    const int64_t lo = static_cast<int64_t>(static_cast<uint64_t>(t) * kTile) - sg.head;
+    int32_t *o = sg.out + lo;
+    if (t >= sg.in_lo && t < sg.in_hi) {
+        if (BULK && (reinterpret_cast<uintptr_t>(o) & 15u) == 0u) {
             if (lane == 0) {
 #pragma unroll
                 for (uint32_t j = 0; j < kTile; j += kNone) bulk_store(o + j, none, kNone * 4u);
@@ -283,15 +339,16 @@ __device__ __forceinline__ void fill_none(const StreamParams &p, const int32_t *
     } else {
         for (uint32_t i = static_cast<uint32_t>(lane); i < kTile; i += 32u) {
             const int64_t g = lo + static_cast<int64_t>(i);
-            if (g >= 0 && g < static_cast<int64_t>(p.f.n)) o[i] = -1;
+            if (g >= 0 && g < static_cast<int64_t>(sg.n)) o[i] = -1;
         }
     }
 }
 
 // OUT_BITS: no bits and no matches yet in tile t.
-__device__ __forceinline__ void clear_bits(const StreamParams &p, uint32_t t, int lane) {
-    reinterpret_cast<uint2 *>(p.f.bo.bits + static_cast<size_t>(t) * (kTile / 32u))[lane] = make_uint2(0u, 0u);
-    if (lane == 0) p.f.bo.counts[t] = 0u;
+__device__ __forceinline__ void clear_bits(const FilterParams &f, const Seg &sg, uint32_t t, int lane) {
+    const size_t u = sg.bit0 / kTile + (t - sg.t0);
+    reinterpret_cast<uint2 *>(f.bo.bits + u * (kTile / 32u))[lane] = make_uint2(0u, 0u);
+    if (lane == 0) f.bo.counts[u] = 0u;
 }
 
 // Before ids are written over the fill: the bulk stores have completed (found:
@@ -305,22 +362,27 @@ __device__ __forceinline__ void fill_done(bool found, int lane) {
 
 // The id at position g, all here: the walk list is full.
 template <int MODE>
-__device__ __forceinline__ void settle_here(const StreamParams &p, uint32_t g, uint32_t B, uint32_t &cnt) {
-    const TileText tt = make_text(p.f.text, p.f.out, p.f.n, 0u);
-    const uint64_t gi = static_cast<uint64_t>(g) - p.head;
-    const int r = (p.f.kind & 0xFFu) == 16u ? match_at_far<int16_t>(p.f, p.f.cls8g, tt, gi, B)
-                                            : match_at_far<int32_t>(p.f, p.f.cls8g, tt, gi, B);
-    put_id<MODE>(p.f, gi, r, cnt);
+__device__ __forceinline__ void settle_here(const StreamParams &p, const Seg &sg, uint32_t g, uint32_t B, uint32_t &cnt) {
+    const TileText tt = make_text(sg.text, sg.out, sg.n, 0u);
+    const int r = (p.f.kind & 0xFFu) == 16u ? match_at_far<int16_t>(p.f, p.f.cls8g, tt, text_pos(sg, g), B)
+                                            : match_at_far<int32_t>(p.f, p.f.cls8g, tt, text_pos(sg, g), B);
+    put_id<MODE>(p.f, sg, g, r, cnt);
 }
 
 // Walks (want: this lane has one) to the list, or settled here when it is full.
-template <int B, int MODE>
-__device__ __forceinline__ void list_walk(const StreamParams &p, WalkRoom &room, bool want, uint2 e, int lane,
-                                          uint32_t &cnt) {
-    const bool stored = push_walk(p, room, want, e, lane);
+template <int B, int MODE, bool BATCH>
+__device__ __forceinline__ void list_walk(const StreamParams &p, const Seg &sg, WalkRoom &room, bool want, uint32_t g,
+                                          uint32_t s, int lane, uint32_t &cnt) {
+    const bool stored = push_walk<BATCH>(p, sg, room, want, g, s, lane);
     if (!room.full || __all_sync(kFull, stored)) return;
     fill_done<MODE, B == 8>(true, lane);
-    if (!stored) settle_here<MODE>(p, e.x, B, cnt);
+    if (!stored) settle_here<MODE>(p, sg, g, B, cnt);
+}
+
+// The -1 buffer (all threads; a CTA barrier follows).
+__device__ __forceinline__ void fill_constant(uint8_t *at) {
+    for (uint32_t i = threadIdx.x; i < kNone / 4u; i += blockDim.x) reinterpret_cast<int4 *>(at)[i] = make_int4(-1, -1, -1, -1);
+    fence_proxy_async_smem();  // read by bulk stores
 }
 
 // One CTA's filters into shared memory (all threads; a CTA barrier follows).
@@ -328,12 +390,9 @@ __device__ __forceinline__ void load_filters(const StreamParams &p, uint8_t *sme
     uint4 *d = reinterpret_cast<uint4 *>(smem);
     const uint4 *a = reinterpret_cast<const uint4 *>(p.F1), *b = reinterpret_cast<const uint4 *>(p.F2);
     const uint32_t na = p.f1bytes >> 4, nb = p.f2bytes >> 4;
-    int4 *none = reinterpret_cast<int4 *>(smem + p.off_none);
-    for (uint32_t i = threadIdx.x; i < kNone / 4u; i += kBlock) none[i] = make_int4(-1, -1, -1, -1);
-    fence_proxy_async_smem();  // read by bulk stores
 #pragma unroll 4
-    for (uint32_t i = threadIdx.x; i < na; i += kBlock) d[i] = __ldg(a + i);
-    for (uint32_t i = threadIdx.x; i < nb; i += kBlock) d[na + i] = __ldg(b + i);
+    for (uint32_t i = threadIdx.x; i < na; i += blockDim.x) d[i] = __ldg(a + i);
+    for (uint32_t i = threadIdx.x; i < nb; i += blockDim.x) d[na + i] = __ldg(b + i);
 }
 
 // Exclusive sum over the lanes below; total: the warp's.
@@ -372,11 +431,12 @@ __device__ __forceinline__ uint32_t codes_at(const uint32_t *packed, uint32_t i)
 
 // Whether the `need` (<= 16) bytes from text position gi on are inside the
 // text and all in keywords (cls8: the byte table).
-__device__ __forceinline__ bool bytes_known(const FilterParams &p, const uint8_t *cls8, uint64_t gi, uint32_t need) {
-    if (gi + need > p.n) return false;
+__device__ __forceinline__ bool bytes_known(const uint8_t *text, uint64_t n, const uint8_t *cls8, uint64_t gi,
+                                            uint32_t need) {
+    if (gi + need > n) return false;
     uint32_t b[16], bad = 0;
 #pragma unroll
-    for (uint32_t j = 0; j < 16; ++j) b[j] = j < need ? __ldg(p.text + gi + j) : 0u;  // all in flight together
+    for (uint32_t j = 0; j < 16; ++j) b[j] = j < need ? __ldg(text + gi + j) : 0u;  // all in flight together
 #pragma unroll
     for (uint32_t j = 0; j < 16; ++j) bad |= j < need && cls8[b[j]] == 0xFFu ? 1u : 0u;
     return bad == 0;
@@ -388,15 +448,15 @@ __device__ __forceinline__ bool bytes_known(const FilterParams &p, const uint8_t
 // text: a keyword that ends before such a byte is on the walk of the codes too,
 // so a position without a result has none; one with a result has its bytes
 // looked at, and a walk's bytes are looked at when it goes on.
-template <int MODE>
-__device__ __forceinline__ void resolve2(const StreamParams &p, WalkRoom &room, uint32_t g, uint32_t w, bool on,
-                                         int lane, uint32_t &cnt) {
+template <int MODE, bool BATCH>
+__device__ __forceinline__ void resolve2(const StreamParams &p, const Seg &sg, WalkRoom &room, uint32_t g, uint32_t w,
+                                         bool on, int lane, uint32_t &cnt) {
     const FilterParams &f = p.f;
-    const uint64_t gi = static_cast<uint64_t>(g) - p.head;  // before the text wraps
+    const uint64_t gi = text_pos(sg, g);
     bool walk = false;
     uint32_t s = 0;
     int r = -1;
-    if (on && gi < f.n) {
+    if (on && gi < sg.n) {
         const int e = __ldg(f.JK + (w & ((1u << (2u * f.k)) - 1u)));
         if (e < 0) {
             r = decode_dead(e);
@@ -413,65 +473,60 @@ __device__ __forceinline__ void resolve2(const StreamParams &p, WalkRoom &room, 
                 }
             }
         }
-        if (r >= 0 && !bytes_known(f, f.cls8g, gi, f.k + f.k2)) {
+        if (r >= 0 && !bytes_known(sg.text, sg.n, f.cls8g, gi, f.k + f.k2)) {
             walk = true;
             s = 0;
             r = -1;
         }
     }
     fill_done<MODE, false>(r >= 0, lane);
-    put_id<MODE>(f, gi, r, cnt);
-    list_walk<2, MODE>(p, room, walk, make_uint2(g, s), lane, cnt);
+    put_id<MODE>(f, sg, g, r, cnt);
+    list_walk<2, MODE, BATCH>(p, sg, room, walk, g, s, lane, cnt);
 }
 
-template <int S, int MODE>
-__global__ void __launch_bounds__(kBlock, 1) pfac_stream2(const __grid_constant__ StreamParams p) {
-    extern __shared__ __align__(128) uint8_t smem[];
+// One warp's state across its tiles: candidates or survivors waiting to be
+// resolved, its walk-list chunk, its count.
+struct WarpState {
+    uint32_t nres, cnt;
+    WalkRoom room;
+};
+
+// One warp: tiles t, t + step, ... below t_end of sg's text (tile t's loads are
+// issued); what waits in shared memory belongs to sg (BATCH: flushed at the end).
+template <int S, int MODE, bool BATCH>
+__device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uint32_t off_warp, const int32_t *none,
+                                       const Seg &sg, uint32_t t, uint32_t t_end, uint32_t step, uint64_t pol,
+                                       TileRegs &r, WarpState &ws) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t step = gridDim.x * kWarps, lt = (1u << lane) - 1u;
-    uint32_t t = static_cast<uint32_t>(warp) * gridDim.x + blockIdx.x;
-    const Loader ld{p.f.gbase + 16u * static_cast<uint32_t>(lane), policy_evict_first()};
-    TileRegs r;
-    r.look = make_uint4(0u, 0u, 0u, 0u);
-    auto load = [&](uint32_t u) {
-        ld.load<0>(p, u, lane, r);
-        ld.load<1>(p, u, lane, r);
-        ld.load<2>(p, u, lane, r);
-        ld.load<3>(p, u, lane, r);
-        ld.load<4>(p, u, lane, r);
-    };
-    if (t < p.ntiles) load(t);
-    load_filters(p, smem);
+    const uint32_t lt = (1u << lane) - 1u;
     const uint32_t *F1 = reinterpret_cast<const uint32_t *>(smem);
     const uint32_t *F2 = reinterpret_cast<const uint32_t *>(smem + p.f1bytes);
-    uint32_t *packed = reinterpret_cast<uint32_t *>(smem + p.off_warp + static_cast<uint32_t>(warp) * kWarpBytes2);
+    uint32_t *packed = reinterpret_cast<uint32_t *>(smem + off_warp + static_cast<uint32_t>(warp) * kWarpBytes2);
     uint2 *res = reinterpret_cast<uint2 *>(packed + kTile / 16 + 4);
     uint16_t *queue = reinterpret_cast<uint16_t *>(res + kRes2);
-    const int32_t *none = reinterpret_cast<const int32_t *>(smem + p.off_none);
-    WalkRoom room{0u, 0u, false};
-    uint32_t cnt = 0, nres = 0;  // candidates waiting in res: {g, codes}
+    uint32_t nres = ws.nres, cnt = ws.cnt;  // candidates waiting in res: {g, codes}
+    WalkRoom room = ws.room;
     auto flush = [&](uint32_t n) {  // resolve the last n (<= 32) of them
         __syncwarp();
         nres -= n;
         const bool on = static_cast<uint32_t>(lane) < n;
         const uint2 e = res[nres + (on ? static_cast<uint32_t>(lane) : 0u)];
-        resolve2<MODE>(p, room, e.x, e.y, on, lane, cnt);
+        resolve2<MODE, BATCH>(p, sg, room, e.x, e.y, on, lane, cnt);
         __syncwarp();
     };
-    __syncthreads();  // the filters are in place
-    for (; t < p.ntiles; t += step) {
+    for (; t < t_end; t += step) {
         // 1. codes; the registers are free for the next tile's loads
         uint32_t c[5];
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[j] = codes16(r.c[j]);
         c[4] = codes16(r.look);
-        if (t + step < p.ntiles) load(t + step);
+        if (t + step < t_end) load_tile(sg, t + step, pol, lane, r);
         __syncwarp();  // the previous tile's readers of packed and queue are done
 #pragma unroll
         for (uint32_t j = 0; j < 4; ++j) packed[32u * j + static_cast<uint32_t>(lane)] = c[j];
         if (lane == 0) packed[128] = c[4];
-        if (MODE == OUT_DENSE) fill_none<false>(p, none, t, lane);
-        if (MODE == OUT_BITS) clear_bits(p, t, lane);
+        if (MODE == OUT_DENSE) fill_none<false>(sg, none, t, lane);
+        if (MODE == OUT_BITS) clear_bits(p.f, sg, t, lane);
 
         // 2. the root filter at every S-th position: one bit each, first
         //    position highest
@@ -494,7 +549,7 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream2(const __grid_constant_
         }
         __syncwarp();  // packed is written
         constexpr int kBits = 4 * kPer / kAcc;  // bits per accumulator
-        const uint32_t g0 = t * kTile;
+        const uint32_t g0 = (t - sg.t0) * kTile;
 #pragma unroll
         for (int a = 0; a < kAcc; ++a) {
             uint32_t m = __brev(acc[a] << (32 - kBits));
@@ -523,11 +578,14 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream2(const __grid_constant_
                     const uint32_t g = g0 + sample(__ffs(m) - 1);
 #pragma unroll 1
                     for (uint32_t x = 0; x < S; ++x, ++o) {
-                        const bool in = static_cast<uint64_t>(g - x) - p.head < p.f.n;
-                        if (o < p.f.walk_cap)
-                            p.f.walks[o] = make_uint2(in ? g - x : 0xFFFFFFFFu, 0u);
-                        else if (in)
-                            settle_here<MODE>(p, g - x, 2u, cnt);
+                        const bool in = text_pos(sg, g - x) < sg.n;
+                        if (o >= p.f.walk_cap) {
+                            if (in) settle_here<MODE>(p, sg, g - x, 2u, cnt);
+                        } else if (in) {
+                            store_walk<BATCH>(p.f, sg, o, g - x, 0u);
+                        } else {
+                            blank_walk<BATCH>(p.f, o);
+                        }
                     }
                 }
                 __syncwarp();
@@ -574,9 +632,9 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream2(const __grid_constant_
         }
     }
     if (nres) flush(nres);
-    if (MODE == OUT_DENSE && lane == 0) bulk_wait_all();
-    close_room(p, room, lane);
-    add_count<MODE>(p.f, cnt, lane);
+    ws.nres = nres;
+    ws.cnt = cnt;
+    ws.room = room;
 }
 
 // ---- 8-bit codes -------------------------------------------------------------
@@ -584,14 +642,14 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream2(const __grid_constant_
 // A round of survivors (all lanes; on: this lane has one: position g, its
 // window's four bytes w and the byte c after them): the state hash, for a
 // branching state the first goto step, then out or to the walk list.
-template <int MODE>
-__device__ __forceinline__ void resolve8(const StreamParams &p, WalkRoom &room, uint32_t g, uint32_t w, uint32_t c,
-                                         bool on, int lane, uint32_t &cnt) {
+template <int MODE, bool BATCH>
+__device__ __forceinline__ void resolve8(const StreamParams &p, const Seg &sg, WalkRoom &room, uint32_t g, uint32_t w,
+                                         uint32_t c, bool on, int lane, uint32_t &cnt) {
     const FilterParams &f = p.f;
-    const uint64_t gi = static_cast<uint64_t>(g) - p.head;
+    const uint64_t gi = text_pos(sg, g);
     // windows past the text end (or before its start, which wraps) hold no keyword
-    on = on && gi < f.n && gi + f.k <= f.n;
-    bool c_ok = gi + f.k < f.n;
+    on = on && gi < sg.n && gi + f.k <= sg.n;
+    bool c_ok = gi + f.k < sg.n;
     if (on && !f.identity) {
         uint32_t x = 0, bad = 0;
 #pragma unroll
@@ -624,52 +682,39 @@ __device__ __forceinline__ void resolve8(const StreamParams &p, WalkRoom &room, 
         if (walk) r = -1;
     }
     fill_done<MODE, true>(r >= 0, lane);
-    put_id<MODE>(f, gi, r, cnt);
-    list_walk<8, MODE>(p, room, walk, make_uint2(g, s | (1u << 31)), lane, cnt);
+    put_id<MODE>(f, sg, g, r, cnt);
+    list_walk<8, MODE, BATCH>(p, sg, room, walk, g, s | (1u << 31), lane, cnt);
 }
 
-// One warp's 8-bit-code tile: its bytes, survivors and their resolution.
-template <int MODE>
-__global__ void __launch_bounds__(kBlock, 1) pfac_stream8(const __grid_constant__ StreamParams p) {
-    extern __shared__ __align__(128) uint8_t smem[];
+// As tiles2, 8-bit codes.
+template <int MODE, bool BATCH>
+__device__ __forceinline__ void tiles8(const StreamParams &p, uint8_t *smem, uint32_t off_warp, const int32_t *none,
+                                       const Seg &sg, uint32_t t, uint32_t t_end, uint32_t step, uint64_t pol,
+                                       TileRegs &r, WarpState &ws) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t step = gridDim.x * kWarps, lt = (1u << lane) - 1u;
-    uint32_t t = static_cast<uint32_t>(warp) * gridDim.x + blockIdx.x;
-    const Loader ld{p.f.gbase + 16u * static_cast<uint32_t>(lane), policy_evict_first()};
-    TileRegs r;
-    r.look = make_uint4(0u, 0u, 0u, 0u);
-    if (t < p.ntiles) {
-        ld.load<0>(p, t, lane, r);
-        ld.load<1>(p, t, lane, r);
-        ld.load<2>(p, t, lane, r);
-        ld.load<3>(p, t, lane, r);
-        ld.load<4>(p, t, lane, r);
-    }
-    load_filters(p, smem);
+    const uint32_t lt = (1u << lane) - 1u;
     const uint32_t *F1 = reinterpret_cast<const uint32_t *>(smem);
     const uint32_t *F2 = reinterpret_cast<const uint32_t *>(smem + p.f1bytes);
     const uint32_t f2words = (p.f2bytes - kStreamShortBytes) >> 2;  // only used with a second filter
     const uint32_t *FS = F2 + f2words;
-    uint32_t *stage = reinterpret_cast<uint32_t *>(smem + p.off_warp + static_cast<uint32_t>(warp) * kWarpBytes8);
+    uint32_t *stage = reinterpret_cast<uint32_t *>(smem + off_warp + static_cast<uint32_t>(warp) * kWarpBytes8);
     uint32_t *res_g = stage + kTile / 4 + 4, *res_w = res_g + kRes8;
     uint16_t *queue = reinterpret_cast<uint16_t *>(res_w + kRes8);
     uint8_t *res_c = reinterpret_cast<uint8_t *>(queue + kQueue);
-    const int32_t *none = reinterpret_cast<const int32_t *>(smem + p.off_none);
-    WalkRoom room{0u, 0u, false};
-    uint32_t cnt = 0, nres = 0;  // survivors waiting in res_*
+    uint32_t nres = ws.nres, cnt = ws.cnt;  // survivors waiting in res_*
+    WalkRoom room = ws.room;
     auto flush = [&](uint32_t n) {  // resolve the last n (<= 32) of them
         __syncwarp();
         nres -= n;
         const bool on = static_cast<uint32_t>(lane) < n;
         const uint32_t x = nres + (on ? static_cast<uint32_t>(lane) : 0u);
-        resolve8<MODE>(p, room, res_g[x], res_w[x], res_c[x], on, lane, cnt);
+        resolve8<MODE, BATCH>(p, sg, room, res_g[x], res_w[x], res_c[x], on, lane, cnt);
         __syncwarp();
     };
-    __syncthreads();  // the filters are in place
-    for (; t < p.ntiles; t += step) {
-        const bool more = t + step < p.ntiles;
-        if (MODE == OUT_DENSE) fill_none<true>(p, none, t, lane);
-        if (MODE == OUT_BITS) clear_bits(p, t, lane);
+    for (; t < t_end; t += step) {
+        const bool more = t + step < t_end;
+        if (MODE == OUT_DENSE) fill_none<true>(sg, none, t, lane);
+        if (MODE == OUT_BITS) clear_bits(p.f, sg, t, lane);
         __syncwarp();  // the previous tile's readers of stage and queue are done
         // 1. the first filter: one bit per position, first position highest;
         //    a chunk's registers take the next tile's bytes as soon as it is done
@@ -684,8 +729,8 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream8(const __grid_constant_
             *reinterpret_cast<uint4 *>(stage + J * (kChunk / 4) + 4 * lane) = cur;
             if (J == 3 && lane == 0) *reinterpret_cast<uint4 *>(stage + kTile / 4) = nxt;
             if (more) {
-                ld.load<J>(p, t + step, lane, r);
-                if (J == 3) ld.load<4>(p, t + step, lane, r);
+                load_chunk<J>(sg, t + step, pol, lane, r);
+                if (J == 3) load_chunk<4>(sg, t + step, pol, lane, r);
             }
             uint32_t win[20];
 #pragma unroll
@@ -708,7 +753,7 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream8(const __grid_constant_
         chunk(std::integral_constant<int, 2>{});
         chunk(std::integral_constant<int, 3>{});
         __syncwarp();  // stage is written
-        const uint32_t g0 = t * kTile;
+        const uint32_t g0 = (t - sg.t0) * kTile;
         // 2. survivors, at most kQueue at a time: the second filter (if any),
         //    then the state hash, 32 a round
         uint32_t m[2] = {__brev(acc[0]), __brev(acc[1])};
@@ -761,9 +806,182 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream8(const __grid_constant_
         }
     }
     if (nres) flush(nres);
-    if (MODE == OUT_DENSE && lane == 0) bulk_wait_all();
-    close_room(p, room, lane);
-    add_count<MODE>(p.f, cnt, lane);
+    ws.nres = nres;
+    ws.cnt = cnt;
+    ws.room = room;
+}
+
+// ---- the kernels -------------------------------------------------------------------
+
+// One text: tiles dealt out warp by warp over the grid.
+template <int FORM, int S, int MODE>
+__device__ __forceinline__ void stream_text(const StreamParams &p) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t step = gridDim.x * (block_of(FORM) / 32);
+    const uint32_t t = static_cast<uint32_t>(warp) * gridDim.x + blockIdx.x;
+    const uint64_t pol = policy_evict_first();
+    const Seg sg = make_seg(p.f.text, p.f.out, p.f.n);
+    const int32_t *none = reinterpret_cast<const int32_t *>(smem + p.off_none);
+    TileRegs r;
+    r.look = make_uint4(0u, 0u, 0u, 0u);
+    if (t < p.ntiles) load_tile(sg, t, pol, lane, r);
+    fill_constant(smem + p.off_none);
+    load_filters(p, smem);
+    __syncthreads();  // the filters are in place
+    WarpState ws{0u, 0u, {0u, 0u, false}};
+    if constexpr (FORM == 2)
+        tiles2<S, MODE, false>(p, smem, p.off_warp, none, sg, t, p.ntiles, step, pol, r, ws);
+    else
+        tiles8<MODE, false>(p, smem, p.off_warp, none, sg, t, p.ntiles, step, pol, r, ws);
+    if (FORM == 8 && MODE == OUT_DENSE && lane == 0) bulk_wait_all();
+    close_room<false>(p.f, ws.room, lane);
+    add_count<MODE>(p.f, ws.cnt, lane);
+}
+
+template <int S, int MODE>
+__global__ void __launch_bounds__(kBlock2, 1) pfac_stream2(const __grid_constant__ StreamParams p) {
+    stream_text<2, S, MODE>(p);
+}
+template <int MODE>
+__global__ void __launch_bounds__(kBlock8, 1) pfac_stream8(const __grid_constant__ StreamParams p) {
+    stream_text<8, 1, MODE>(p);
+}
+
+// A batch: the units (tiles) of the launch's automata, all of one form.  A CTA
+// starts with the automaton at its share of the units, so an automaton's
+// filters are loaded by about as many CTAs as its share of the work, and goes
+// on to the others in turn while they have units left; warps claim blocks of
+// consecutive units from the automaton's counter, smaller ones towards its end.
+// One launch per form: with every form in one kernel each would take the
+// registers of the largest.
+constexpr uint32_t kStreamMultiMax = 32;
+struct StreamMulti {
+    StreamParams a[kStreamMultiMax];
+    uint32_t nh;
+    uint32_t off_none, off_warp;
+};
+static_assert(sizeof(StreamMulti) <= 32764, "kernel parameters are limited to 32764 bytes");
+
+// The text of a batch that unit u belongs to, as a segment from u's tile on.
+// The planned list is searched 32 ways: its first 32 samples stay in the lanes
+// (sample_items), so up to 1,024 texts take one round of loads, which brings
+// the entries themselves.
+__device__ __forceinline__ uint32_t list_step(uint32_t n) { return n > 32u ? (n + 31u) / 32u : 1u; }
+__device__ __forceinline__ uint32_t sample_items(const Work &wk, int lane) {
+    const uint32_t i = static_cast<uint32_t>(lane) * list_step(wk.nlist);
+    return i < wk.nlist ? __ldg(&wk.list[i].first_unit) : 0xFFFFFFFFu;
+}
+template <int MODE>
+__device__ __forceinline__ Seg batch_seg(const FilterParams &f, const Work &wk, uint32_t sample, uint32_t u, int lane) {
+    uint32_t step = list_step(wk.nlist);
+    uint32_t lo = static_cast<uint32_t>(31 - __clz(__ballot_sync(kFull, sample <= u))) * step;  // list[0].first_unit == 0
+    uint32_t hi = lo + step < wk.nlist ? lo + step : wk.nlist;
+    while (hi - lo > 32u) {
+        step = (hi - lo + 31u) / 32u;
+        const uint32_t i = lo + static_cast<uint32_t>(lane) * step;
+        const bool le = i < hi && __ldg(&wk.list[i].first_unit) <= u;
+        lo += static_cast<uint32_t>(31 - __clz(__ballot_sync(kFull, le))) * step;
+        hi = lo + step < hi ? lo + step : hi;
+    }
+    const uint32_t i = lo + static_cast<uint32_t>(lane);
+    const uint4 *e = reinterpret_cast<const uint4 *>(wk.list + (i < hi ? i : lo));
+    uint4 x = __ldg(e), y = __ldg(e + 1);  // {text_off, len}, {out_off, first_unit, item}
+    const int at = 31 - __clz(__ballot_sync(kFull, i < hi && y.z <= u));
+    x.x = __shfl_sync(kFull, x.x, at);
+    x.y = __shfl_sync(kFull, x.y, at);
+    x.z = __shfl_sync(kFull, x.z, at);
+    x.w = __shfl_sync(kFull, x.w, at);
+    y.z = __shfl_sync(kFull, y.z, at);
+    uint64_t ooff = 0;
+    if (MODE == OUT_DENSE) ooff = __shfl_sync(kFull, y.x, at) | (static_cast<uint64_t>(__shfl_sync(kFull, y.y, at)) << 32);
+    Seg sg = make_seg(f.text + (x.x | (static_cast<uint64_t>(x.y) << 32)), MODE == OUT_DENSE ? f.out + ooff : nullptr,
+                      x.z | (static_cast<uint64_t>(x.w) << 32));
+    sg.t0 = u - y.z;
+    sg.unit0 = u;
+    sg.item = lo + static_cast<uint32_t>(at);
+    sg.bit0 = MODE == OUT_BITS ? (f.sl.ubase + u) * kTile : 0u;
+    return sg;
+}
+
+template <int FORM, int S, int MODE>
+__device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int lane = threadIdx.x & 31;
+    const uint64_t pol = policy_evict_first();
+    const int32_t *none = reinterpret_cast<const int32_t *>(smem + mp.off_none);
+    // (dynamic too: a kernel with static shared memory cannot take the most dynamic)
+    volatile uint32_t &start = reinterpret_cast<uint32_t *>(smem + mp.off_none)[kNone];
+    volatile uint32_t &open = reinterpret_cast<uint32_t *>(smem + mp.off_none)[kNone + 1u];
+    fill_constant(smem + mp.off_none);
+    uint64_t total = 0;
+    for (uint32_t a = 0; a < mp.nh; ++a) total += __ldg(&mp.a[a].f.batch->units);
+    if (threadIdx.x == 0) {
+        const uint64_t mine = total * (2u * blockIdx.x + 1u) / (2u * gridDim.x);
+        uint64_t sum = 0;
+        uint32_t a = 0;
+        for (; a + 1u < mp.nh; ++a) {
+            sum += __ldg(&mp.a[a].f.batch->units);
+            if (mine < sum) break;
+        }
+        start = a;
+    }
+    __syncthreads();
+    TileRegs r;
+    r.look = make_uint4(0u, 0u, 0u, 0u);
+    WarpState ws{0u, 0u, {0u, 0u, false}};
+    const uint32_t first = start;
+    for (uint32_t k = 0; k < mp.nh; ++k) {
+        const uint32_t a = (first + k) % mp.nh;
+        const StreamParams &p = mp.a[a];
+        const Work wk = load_work(p.f.batch, p.f.lists, 0u);
+        if (threadIdx.x == 0) open = *reinterpret_cast<volatile unsigned int *>(p.f.counter) < wk.units ? 1u : 0u;
+        __syncthreads();
+        const bool go = open != 0u;  // the same for every thread
+        if (go) load_filters(p, smem);
+        __syncthreads();
+        if (!go) continue;
+        // warps on this automaton, about
+        const uint32_t share = static_cast<uint32_t>(static_cast<uint64_t>(gridDim.x) * (block_of(FORM) / 32) * wk.units / total) + 1u;
+        // blocks of two units, one towards the end (bigger ones leave the last
+        // warps too much, and scatter the traffic: 64 units at first took 810
+        // us for 1,024 texts of the benchmark batch against 725); the next block is
+        // claimed while this one is matched
+        auto block = [&](uint32_t seen) { return seen < wk.units && wk.units - seen > 8u * share ? 2u : 1u; };
+        const uint32_t sample = sample_items(wk, lane);
+        uint32_t blk = block(0u), ahead = 0;
+        if (lane == 0) ahead = atomicAdd(p.f.counter, blk);
+        for (;;) {
+            uint32_t u = __shfl_sync(kFull, ahead, 0);
+            if (u >= wk.units) break;
+            const uint32_t end = wk.units - u < blk ? wk.units : u + blk;
+            blk = block(end);
+            if (lane == 0) ahead = atomicAdd(p.f.counter, blk);
+            while (u < end) {  // the block's tiles, text by text
+                const Seg sg = batch_seg<MODE>(p.f, wk, sample, u, lane);
+                const uint64_t tiles = (sg.n + sg.head + kTile - 1u) / kTile;
+                const uint32_t n = tiles - sg.t0 < end - u ? static_cast<uint32_t>(tiles - sg.t0) : end - u;
+                load_tile(sg, sg.t0, pol, lane, r);
+                if constexpr (FORM == 2)
+                    tiles2<S, MODE, true>(p, smem, mp.off_warp, none, sg, sg.t0, sg.t0 + n, 1u, pol, r, ws);
+                else
+                    tiles8<MODE, true>(p, smem, mp.off_warp, none, sg, sg.t0, sg.t0 + n, 1u, pol, r, ws);
+                u += n;
+            }
+        }
+        __syncthreads();  // every warp is done with the automaton's filters
+    }
+    if (FORM == 8 && MODE == OUT_DENSE && lane == 0) bulk_wait_all();
+    close_room<true>(mp.a[0].f, ws.room, lane);
+}
+
+template <int S, int MODE>
+__global__ void __launch_bounds__(kBlock2, 1) pfac_stream2_multi(const __grid_constant__ StreamMulti mp) {
+    stream_batch<2, S, MODE>(mp);
+}
+template <int MODE>
+__global__ void __launch_bounds__(kBlock8, 1) pfac_stream8_multi(const __grid_constant__ StreamMulti mp) {
+    stream_batch<8, 1, MODE>(mp);
 }
 
 // ---- the listed walks ----------------------------------------------------------
@@ -772,6 +990,19 @@ __global__ void __launch_bounds__(kBlock, 1) pfac_stream8(const __grid_constant_
 // at 40 registers a thread.
 constexpr int kWalkBlock = 128;
 constexpr int kWalkCtas = 12;
+
+// One listed walk of text sg: its id at position g.
+template <typename GT>
+__device__ __forceinline__ int finish_walk(const FilterParams &p, const uint8_t *cls8, const Seg &sg, uint32_t g,
+                                           uint32_t e, uint32_t B) {
+    const TileText tt = make_text(sg.text, sg.out, sg.n, 0u);
+    const uint64_t gi = text_pos(sg, g);
+    const uint32_t s = e & 0x7FFFFFFFu;
+    // 2-bit codes: the walk so far took the codes for keyword bytes'
+    if (s && (B == 8 || bytes_known(sg.text, sg.n, cls8, gi, p.k + p.k2)))
+        return filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s, p.k + p.k2 + (e >> 31));
+    return match_at<GT>(p, cls8, tt, gi, B);
+}
 
 template <int B, typename GT, int MODE>
 __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const __grid_constant__ FilterParams p) {
@@ -782,29 +1013,59 @@ __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const
     if (blockIdx.x * blockDim.x >= m) return;
     for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
     __syncthreads();
-    const uint64_t head = reinterpret_cast<uintptr_t>(p.text) & 15u;
-    const TileText tt = make_text(p.text, p.out, p.n, 0u);
+    const Seg sg = make_seg(p.text, p.out, p.n);
     uint32_t cnt = 0;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
         const uint2 e = __ldg(p.walks + j);
-        if (e.x == 0xFFFFFFFFu) continue;
-        const uint64_t gi = static_cast<uint64_t>(e.x) - head;
-        const uint32_t s = e.y & 0x7FFFFFFFu;
-        int r;
-        // 2-bit codes: the walk so far took the codes for keyword bytes'
-        if (s && (B == 8 || bytes_known(p, cls8, gi, p.k + p.k2)))
-            r = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s, p.k + p.k2 + (e.y >> 31));
-        else
-            r = match_at<GT>(p, cls8, tt, gi, B);
-        put_id<MODE>(p, gi, r, cnt);
+        if (e.x != 0xFFFFFFFFu) put_id<MODE>(p, sg, e.x, finish_walk<GT>(p, cls8, sg, e.x, e.y, B), cnt);
     }
     add_count<MODE>(p, cnt, lane);
 }
 
+// A batch's walks: the automata's parameters (a[0 .. nh), in the order of the
+// entries' automaton numbers) and byte tables in shared memory.
+struct WalkMulti {
+    FilterParams a[kStreamMultiMax];
+    uint32_t nh;
+};
+static_assert(sizeof(WalkMulti) <= 32764, "kernel parameters are limited to 32764 bytes");
+
+template <int MODE>
+__global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const __grid_constant__ WalkMulti mp) {
+    extern __shared__ __align__(16) uint8_t msm[];
+    const uint32_t listed = *reinterpret_cast<volatile const unsigned int *>(mp.a[0].list_count + 1);
+    const uint32_t m = listed < mp.a[0].walk_cap ? listed : mp.a[0].walk_cap;
+    if (blockIdx.x * blockDim.x >= m) return;
+    FilterParams *ps = reinterpret_cast<FilterParams *>(msm);
+    uint8_t *cls = msm + mp.nh * sizeof(FilterParams);
+    for (uint32_t i = threadIdx.x; i < mp.nh * static_cast<uint32_t>(sizeof(FilterParams) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(ps)[i] = reinterpret_cast<const uint32_t *>(mp.a)[i];
+    for (uint32_t i = threadIdx.x; i < mp.nh * 256u; i += blockDim.x) cls[i] = __ldg(mp.a[i >> 8].cls8g + (i & 255u));
+    __syncthreads();
+    uint32_t cnt = 0;
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
+        const uint4 e = __ldg(mp.a[0].walks4 + j);
+        if (e.x == 0xFFFFFFFFu) continue;
+        const uint32_t a = e.z >> 11, g = e.z & (kTile - 1u);
+        const FilterParams &p = ps[a];
+        const Work wk = load_work(p.batch, p.lists, 0u);
+        const uint4 *q = reinterpret_cast<const uint4 *>(wk.list + e.w);
+        const uint4 x = __ldg(q), y = __ldg(q + 1);
+        Seg sg = make_seg(p.text + (x.x | (static_cast<uint64_t>(x.y) << 32)),
+                          MODE == OUT_DENSE ? p.out + (y.x | (static_cast<uint64_t>(y.y) << 32)) : nullptr,
+                          x.z | (static_cast<uint64_t>(x.w) << 32));
+        sg.t0 = e.x - y.z;
+        sg.bit0 = MODE == OUT_BITS ? (p.sl.ubase + e.x) * kTile : 0u;
+        const int r = (p.kind & 0xFFu) == 16u ? finish_walk<int16_t>(p, cls + 256u * a, sg, g, e.y, p.kind >> 8)
+                                              : finish_walk<int32_t>(p, cls + 256u * a, sg, g, e.y, p.kind >> 8);
+        put_id<MODE>(p, sg, g, r, cnt);
+    }
+}
+
 // ---- launches --------------------------------------------------------------------
 
-template <void (*Kernel)(const StreamParams)>
-cudaError_t launch_form(const StreamParams &p, uint32_t grid, uint32_t smem, int max_smem, cudaStream_t stream) {
+template <auto Kernel, uint32_t FORM, typename P>
+cudaError_t launch_form(const P &p, uint32_t grid, uint32_t smem, int max_smem, cudaStream_t stream) {
     static std::atomic<uint64_t> configured{0};  // bit d: device d (as many as filter_device_shape knows)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -815,7 +1076,7 @@ cudaError_t launch_form(const StreamParams &p, uint32_t grid, uint32_t smem, int
         if (e != cudaSuccess) return e;
         configured.fetch_or(1ull << dev);
     }
-    Kernel<<<grid, kBlock, smem, stream>>>(p);
+    Kernel<<<grid, block_of(FORM), smem, stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -823,6 +1084,10 @@ cudaError_t launch_stream2(OutMode mode, const StreamParams &p, uint32_t step, u
                            int max_smem, cudaStream_t stream);
 cudaError_t launch_stream8(OutMode mode, const StreamParams &p, uint32_t grid, uint32_t smem, int max_smem,
                            cudaStream_t stream);
+cudaError_t launch_stream2_multi(OutMode mode, const StreamMulti &mp, uint32_t step, uint32_t grid, uint32_t smem,
+                                 int max_smem, cudaStream_t stream);
+cudaError_t launch_stream8_multi(OutMode mode, const StreamMulti &mp, uint32_t grid, uint32_t smem, int max_smem,
+                                 cudaStream_t stream);
 
 }  // namespace strm
 }  // namespace pfac

@@ -169,3 +169,49 @@ def test_list_capacity_is_kept():
                 assert np.array_equal(pos[:cap].cpu().numpy(), wpos[:cap])
                 assert np.array_equal(ids[:cap].cpu().numpy(), wids[:cap])
                 assert bool((pos[cap:] == -7).all()) and bool((ids[cap:] == -7).all())
+
+
+@pytest.mark.parametrize("names", [("dna16", "bytes4"), ("dna8", "dna4", "bytes9", "words7"),
+                                   ("dna16", "iupac", "bytes2", "bytes5", "dna1")])
+@pytest.mark.parametrize("reserve", [1 << 22, 64])
+def test_batch_streams(names, reserve):
+    """A plan with lists: automata the streaming form serves, next to ones it
+    does not; texts from 1 byte to several tiles, packed back to back (most
+    start off a 16-byte boundary), some empty; also with a walk list too small
+    for the batch."""
+    import torch
+
+    r = workloads.rng(len(names))
+    lens = [0, 1, 2, 15, 17, 2047, 2048, 2049, 4096 + 5, 70_000] + [int(x) for x in r.integers(1, 12_000, size=30)]
+    which = [int(x) for x in r.integers(0, len(names), size=len(lens))]
+    which[9] = 0
+    loads = [_workload(n, 80_000) for n in names]
+    texts = [loads[a][0][s:s + n] for a, n, s in zip(which, lens, r.integers(0, 5_000, size=len(lens)))]
+    offs = np.concatenate([[0], np.cumsum(lens)[:-1]]) + 3
+    total = int(sum(lens)) + 3
+    buf = np.zeros(total, dtype=np.uint8)
+    for t, o in zip(texts, offs):
+        buf[o:o + t.size] = t
+    autos = [api.Automaton(p) for _, p in loads]
+    try:
+        d = torch.from_numpy(buf).cuda()
+        out = torch.full((total + 8,), -7, dtype=torch.int32, device="cuda")
+        items = api.items_to_device(api.batch_items(offs, lens, offs + 1, which))
+        with api.BatchPlan([a.handle for a in autos], len(lens)) as plan:
+            plan.reserve_lists(reserve)
+            for run in range(2):
+                out.fill_(-7)
+                if run == 0:
+                    plan.run(d, items, len(lens), out)
+                else:
+                    plan.capture(d, items, len(lens), out)
+                    plan.replay()
+                got = out.cpu().numpy()
+                want = np.full(total + 8, -7, dtype=np.int32)
+                for t, o, a in zip(texts, offs, which):
+                    if t.size:
+                        want[o + 1:o + 1 + t.size] = oracle.pfac_ids(loads[a][1], t)
+                assert np.array_equal(got, want)
+    finally:
+        for a in autos:
+            a.close()
