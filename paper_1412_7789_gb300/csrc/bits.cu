@@ -73,16 +73,17 @@ __device__ __forceinline__ uint32_t list_bits(uint2 b, uint16_t *list, int lane)
     return total;
 }
 
-// One warp: tile t's part of the list, from index at on.
+// One warp: tile t's part of the list, from index at on; p0: the text position
+// of the tile's first bit (before the text wraps).
 template <bool FULL>
-__device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint2 b, unsigned long long at, uint16_t *list,
-                                         int lane) {
+__device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32_t p0, uint2 b, unsigned long long at,
+                                         uint16_t *list, int lane) {
     const uint32_t total = list_bits(b, list, lane);
     const size_t g0 = static_cast<size_t>(t) * kTile;
     for (uint32_t k0 = 0; k0 < total; k0 += 32u) {
         const uint32_t k = k0 + static_cast<uint32_t>(lane);
         const uint32_t i = k < total ? list[k] : 0u;
-        const uint32_t pos = static_cast<uint32_t>(g0) + i - p.head;
+        const uint32_t pos = p0 + i;
         if (!FULL) {
             if (k < total && at + k < p.out.cap) {
                 p.out.pos[at + k] = pos;
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
             if (w < static_cast<uint32_t>(warp)) at += own[w];
             all += own[w];
         }
-        if (t < p.ntiles) put_tile<FULL>(p, t, b, at, lists[warp], lane);
+        if (t < p.ntiles) put_tile<FULL>(p, t, t * kTile - p.head, b, at, lists[warp], lane);
         if (t0 + kWarps >= p.ntiles && threadIdx.x == 0) *p.out.count = all;
     } else {
         const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
@@ -171,11 +172,44 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
             const uint32_t c = u < p.ntiles ? __ldg(p.counts + u) : 0u;
             for (uint32_t todo = __ballot_sync(kFull, c != 0u); todo; todo &= todo - 1u) {
                 const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
-                put_tile<FULL>(p, t, tile_bits(p, t, lane), __ldg(p.prefix + t), lists[warp], lane);
+                put_tile<FULL>(p, t, t * kTile - p.head, tile_bits(p, t, lane), __ldg(p.prefix + t), lists[warp],
+                               lane);
             }
         }
         if (gw == 0 && lane == 0)
             *p.out.count = __ldg(p.prefix + p.ntiles - 1u) + __ldg(p.counts + p.ntiles - 1u);
+    }
+}
+
+// The lists of several texts (streaming form): as bits_gather, each unit's text
+// found by a 32-way search.
+__global__ void __launch_bounds__(kThreads) bits_gather_texts(BitsParams p, const BitsText *texts, uint32_t nt) {
+    __shared__ uint16_t lists[kWarps][kTile];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
+    for (uint64_t u0 = gw; u0 < p.ntiles; u0 += 32ull * nw) {
+        const uint64_t u = u0 + static_cast<uint64_t>(lane) * nw;
+        const uint32_t c = u < p.ntiles ? __ldg(p.counts + u) : 0u;
+        for (uint32_t todo = __ballot_sync(kFull, c != 0u); todo; todo &= todo - 1u) {
+            const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
+            uint32_t lo = 0, hi = nt;  // the last text whose first unit is <= t
+            while (hi - lo > 1u) {
+                const uint32_t step = hi - lo > 32u ? (hi - lo + 31u) / 32u : 1u;
+                const uint32_t i = lo + static_cast<uint32_t>(lane) * step;
+                const unsigned le = __ballot_sync(kFull, i < hi && __ldg(&texts[i].first) <= t);
+                lo += static_cast<uint32_t>(31 - __clz(le)) * step;
+                hi = lo + step < hi ? lo + step : hi;
+            }
+            const BitsText x = texts[lo];
+            p.out = x.out;
+            put_tile<false>(p, t, (t - x.first) * kTile - x.head, tile_bits(p, t, lane),
+                            __ldg(p.prefix + t) - __ldg(p.prefix + x.first), lists[warp], lane);
+        }
+    }
+    for (uint32_t i = gw * 32u + static_cast<uint32_t>(lane); i < nt; i += nw * 32u) {
+        const BitsText x = texts[i];
+        const uint32_t last = x.first + x.units - 1u;
+        *x.out.count = __ldg(p.prefix + last) + __ldg(p.counts + last) - __ldg(p.prefix + x.first);
     }
 }
 
@@ -216,6 +250,22 @@ Layout layout_of(const DevTables &t, const Tuning &tu, const uint8_t *text, uint
 
 bool bits_serve(const DevTables &t, const Tuning &tu, uint64_t n) {
     return at_serves(t, tu, n) || stream_serves(t, tu, n);
+}
+
+cudaError_t launch_bits_texts(const BitsText *texts, uint32_t nt, uint32_t units, const BitsOut &b,
+                              const unsigned long long *prefix, cudaStream_t stream) {
+    if (!texts || nt == 0 || units == 0 || !b.bits || !b.ids || !b.counts || !prefix) return cudaErrorInvalidValue;
+    BitsParams p{};
+    p.bits = b.bits;
+    p.ids = b.ids;
+    p.words = units * kWords;
+    p.ntiles = units;
+    p.counts = b.counts;
+    p.prefix = prefix;
+    const uint32_t need = (units + kWarps - 1) / kWarps, sms = device_sm_count();
+    if (sms == 0) return cudaErrorInvalidDevice;
+    bits_gather_texts<<<need < sms * 6u ? need : sms * 6u, kThreads, 0, stream>>>(p, texts, nt);
+    return cudaGetLastError();
 }
 
 size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full) {

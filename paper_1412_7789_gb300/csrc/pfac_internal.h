@@ -432,6 +432,16 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
 // (bits.cu): the short-text or the streaming form, then the lists.  Whether it
 // serves the text, its scratch, and the launches.
 bool bits_serve(const DevTables &t, const Tuning &tu, uint64_t n);
+// One text of a wave of several in OUT_BITS units (ascending first unit, none
+// empty): its units, its first byte's position in the first, where its list goes.
+struct alignas(16) BitsText {
+    CompactOut out;
+    uint32_t first, units, head, pad;
+};
+// The compacted lists of nt texts whose units' bits, ids and counts are in b
+// (b.counts[u], u < units; prefix: their exclusive sums, from any start).
+cudaError_t launch_bits_texts(const BitsText *texts, uint32_t nt, uint32_t units, const BitsOut &b,
+                              const unsigned long long *prefix, cudaStream_t stream);
 size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full);
 cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, const CompactOut &out,
                          bool full, void *scratch, size_t scratch_bytes, cudaStream_t stream);

@@ -67,6 +67,7 @@ struct ac_server_impl {
     std::vector<pfac::Tuning> tune;
     int device = 0;
     bool multi = false;          // waves match all automata in one launch (filter kernel for all)
+    std::vector<bool> streams;   // the streaming form serves the automaton's texts in large waves
     uint64_t budget = 0;         // for requests: the option's budget less the automata's tables
     uint64_t table_bytes = 0;    // the resident automata (each handle once)
     void *(*dev_alloc)(size_t, void *) = nullptr;
@@ -124,6 +125,12 @@ uint64_t units_of(const ac_server_impl *s, const ac_server_request &r) {
 // match again.)
 bool wave_lists(const ac_server_impl *s, uint32_t a) { return (s->multi || s->fifo) && s->tabs[a]->B == 8; }
 
+// Whether a wave of so many text bytes takes the streaming form for the
+// automata it serves.  Below, its launches (filters into every SM, a pass over
+// the listed walks) cost a wave more than they save.
+constexpr uint64_t kStreamWave = 4ull << 20;
+bool wave_streams(const ac_server_impl *s, uint64_t bytes) { return s->multi && bytes >= kStreamWave; }
+
 // Device bytes a request holds while admitted: its text (a host text's device
 // copy), its output and the scratch of its tiles (counts, prefix, slots,
 // dense fallback), and with 8-bit codes in one-launch waves its share of the
@@ -131,7 +138,13 @@ bool wave_lists(const ac_server_impl *s, uint32_t a) { return (s->multi || s->fi
 uint64_t request_bytes(const ac_server_impl *s, const ac_server_request &r) {
     const uint64_t per_unit = 4 + 8 + 8ull * pfac::kSlotCap + 4ull * pfac::kDenseStride;
     const uint64_t lists = wave_lists(s, r.automaton) ? 32ull * (r.n / 8) + 32 : 0;
-    return r.n + 8ull * r.cap + units_of(s, r) * per_unit + lists + 64;
+    const uint64_t own = units_of(s, r) * per_unit + lists;
+    // the streaming form, should the wave take it: count, prefix, bits and ids
+    // of each unit, 16 bytes of walk list for every eighth text byte
+    const uint64_t units = (r.n + text_head(r) + pfac::kStreamTile - 1) / pfac::kStreamTile;
+    const uint64_t other = s->streams[r.automaton] ? units * (4 + 8 + pfac::kStreamTile / 8 + 4ull * pfac::kStreamTile) + 16ull * (r.n / 8)
+                                                   : 0;
+    return r.n + 8ull * r.cap + std::max(own, other) + 64;
 }
 
 // Device scratch of a wave: from the caller's allocator (freed when the wave
@@ -233,28 +246,57 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     std::vector<uint32_t> ubase(nh, 0);
     std::vector<pfac::BatchItemDev> list(L);
     std::vector<pfac::CompactOut> outs(R);
-    uint64_t U = 0;
-    uint32_t j = 0;
-    for (uint32_t a = 0; a < nh; ++a) {
-        heads[a].offset = j;
-        heads[a].pad = 0;
-        ubase[a] = static_cast<uint32_t>(U);
-        uint64_t units = 0;
-        while (j < L && w.reqs[order[j]].r.automaton == a) {
-            const ac_server_request &r = w.reqs[order[j]].r;
-            pfac::BatchItemDev &d = list[j];
-            d.len = r.n;
-            d.out_off = 0;
-            d.first_unit = static_cast<uint32_t>(units);
-            d.item = order[j];
-            units += units_of(s, r);
-            ++j;
+    // the automata the streaming form takes in this wave
+    uint64_t wave_text = 0;
+    for (uint32_t k = 0; k < L; ++k) wave_text += w.reqs[order[k]].r.n;
+    auto streamed = [&](uint32_t a) { return s->streams[a] && wave_streams(s, wave_text); };
+    // units: the other automata's first (with slots), then the streamed ones'
+    // (with bits); the counts and their prefix are one array over both
+    std::vector<pfac::BitsText> btexts;
+    uint64_t U = 0, Uo = 0, stream_text = 0;
+    {
+        uint32_t j = 0;
+        for (uint32_t a = 0; a < nh; ++a) {
+            heads[a].offset = j;
+            heads[a].pad = 0;
+            while (j < L && w.reqs[order[j]].r.automaton == a) ++j;
+            heads[a].count = j - heads[a].offset;
         }
-        heads[a].count = j - heads[a].offset;
-        heads[a].units = static_cast<uint32_t>(units);
-        U += units;
     }
-    if (U >= 0xFFFFFFFFull) return cudaErrorInvalidValue;
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) Uo = U;
+        for (uint32_t a = 0; a < nh; ++a) {
+            if (streamed(a) != (pass == 1)) continue;
+            ubase[a] = static_cast<uint32_t>(U - Uo);
+            uint64_t units = 0;
+            for (uint32_t j = heads[a].offset; j < heads[a].offset + heads[a].count; ++j) {
+                const ac_server_request &r = w.reqs[order[j]].r;
+                pfac::BatchItemDev &d = list[j];
+                d.len = r.n;
+                d.out_off = 0;
+                d.first_unit = static_cast<uint32_t>(units);
+                d.item = order[j];
+                if (pass == 0) {
+                    units += units_of(s, r);
+                    continue;
+                }
+                const uint64_t n = (r.n + text_head(r) + pfac::kStreamTile - 1) / pfac::kStreamTile;
+                pfac::BitsText x{};
+                x.out = pfac::CompactOut{r.d_pos, r.d_ids, r.cap, reinterpret_cast<unsigned long long *>(r.d_count)};
+                x.first = static_cast<uint32_t>(ubase[a] + units);
+                x.units = static_cast<uint32_t>(n);
+                x.head = static_cast<uint32_t>(text_head(r));
+                btexts.push_back(x);
+                units += n;
+                stream_text += r.n;
+            }
+            heads[a].units = static_cast<uint32_t>(units);
+            U += units;
+        }
+    }
+    const uint64_t Us = U - Uo;
+    // (positions of the streamed units are numbered in 32 bits)
+    if (U >= 0xFFFFFFFFull || Us >= (1ull << 32) / pfac::kStreamTile) return cudaErrorInvalidValue;
     for (uint32_t i = 0; i < R; ++i) {
         const ac_server_request &r = w.reqs[i].r;
         outs[i] = pfac::CompactOut{r.d_pos, r.d_ids, r.cap, reinterpret_cast<unsigned long long *>(r.d_count)};
@@ -267,22 +309,28 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     // than slots again), the others' do (and so list nothing)
     uint64_t list_text = 0;
     for (uint32_t k = 0; k < L; ++k)
-        if (s->multi && wave_lists(s, w.reqs[order[k]].r.automaton)) list_text += w.reqs[order[k]].r.n;
+        if (s->multi && wave_lists(s, w.reqs[order[k]].r.automaton) && !streamed(w.reqs[order[k]].r.automaton))
+            list_text += w.reqs[order[k]].r.n;
     const uint32_t list_cap =
         list_text >= (4ull << 20) ? static_cast<uint32_t>(std::min<uint64_t>(list_text / 8, 0x7FFFFFF0ull)) : 0u;
     const size_t lsb = list_cap ? round256(pfac::multi_lists_bytes(list_cap)) : 0;
     auto dense_for = [&](uint32_t a, int32_t *d) -> int32_t * { return list_cap && wave_lists(s, a) ? nullptr : d; };
 
-    // device: plan (heads | list | outs) | tile counters | counts | prefix |
-    // slots | partial sums | dense fallback | host-text copies | survivor lists
+    // device: plan (heads | list | outs | streamed texts) | tile counters |
+    // counts | prefix | slots | partial sums | dense fallback | host-text copies
+    // | survivor lists | streamed units' bits | walk list | ids
     const size_t hb = sizeof(pfac::BatchHead) * nh, lb = sizeof(pfac::BatchItemDev) * L,
-                 ob = sizeof(pfac::CompactOut) * R;
-    const size_t plan_bytes = round256(hb) + round256(lb) + round256(ob);
-    const size_t cb = round256(16ull * nh), nb = round256(4 * U), pb = 8 * U, sb = 8ull * pfac::kSlotCap * U;
+                 ob = sizeof(pfac::CompactOut) * R, tb = sizeof(pfac::BitsText) * btexts.size();
+    const size_t plan_bytes = round256(hb) + round256(lb) + round256(ob) + round256(tb);
+    const size_t cb = round256(16ull * nh), nb = round256(4 * U), pb = 8 * U, sb = 8ull * pfac::kSlotCap * Uo;
     const size_t db = round256(plan_bytes + cb + nb + pb + sb + 8ull * pfac::kScanCtas);  // dense fallback: aligned
-    const size_t stb = round256(db + 4ull * pfac::kDenseStride * U);
+    const size_t stb = round256(db + 4ull * pfac::kDenseStride * Uo);
+    const uint32_t walk_cap = Us ? pfac::stream_batch_cap(stream_text) : 0u;
+    const size_t bb = round256(Us * (pfac::kStreamTile / 8)), wb = Us ? round256(pfac::stream_batch_bytes(walk_cap)) : 0,
+                 ib = 4ull * pfac::kStreamTile * Us;
+    const size_t bits_at = stb + round256(staged) + lsb;
     void *dev = nullptr;
-    e = wave_alloc(s, w, stb + round256(staged) + lsb, &dev);
+    e = wave_alloc(s, w, bits_at + bb + wb + ib, &dev);
     if (e != cudaSuccess) return e;
     uint8_t *dp = static_cast<uint8_t *>(dev);
 
@@ -306,6 +354,7 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     std::memcpy(hp, heads.data(), hb);
     std::memcpy(hp + round256(hb), list.data(), lb);
     std::memcpy(hp + round256(hb) + round256(lb), outs.data(), ob);
+    if (tb) std::memcpy(hp + round256(hb) + round256(lb) + round256(ob), btexts.data(), tb);
 
     const pfac::BatchHead *d_heads = reinterpret_cast<const pfac::BatchHead *>(dp);
     const pfac::BatchItemDev *d_list = reinterpret_cast<const pfac::BatchItemDev *>(dp + round256(hb));
@@ -314,7 +363,7 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     uint32_t *counts = reinterpret_cast<uint32_t *>(counters + cb);
     unsigned long long *prefix = reinterpret_cast<unsigned long long *>(counters + cb + nb);
     unsigned long long *slots = prefix + U;
-    unsigned long long *partials = slots + static_cast<size_t>(pfac::kSlotCap) * U;
+    unsigned long long *partials = slots + static_cast<size_t>(pfac::kSlotCap) * Uo;
     int32_t *dense = reinterpret_cast<int32_t *>(dp + db);
     void *surv_lists = list_cap ? static_cast<void *>(dp + stb + round256(staged)) : nullptr;
 
@@ -324,24 +373,48 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
         if (host_text(r)) e = cudaMemcpyAsync(const_cast<uint8_t *>(ptr[k]), r.d_text, r.n, cudaMemcpyHostToDevice,
                                               w.stream);
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(counters, 0, cb + 4 * U, w.stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counters, 0, cb + 4 * Uo, w.stream);
     if (e == cudaSuccess && surv_lists) e = cudaMemsetAsync(surv_lists, 0, 32, w.stream);
-    if (s->multi && e == cudaSuccess) {  // every automaton of the wave in one launch
-        std::vector<pfac::MatchRequest> rs(nh);
+    pfac::BitsOut bits;
+    bits.bits = reinterpret_cast<uint32_t *>(dp + bits_at);
+    bits.ids = reinterpret_cast<int32_t *>(dp + bits_at + bb + wb);
+    bits.counts = counts + Uo;
+    if (s->multi) {
+        // the wave's automata: the streamed ones in the streaming form's
+        // launches, the others in one of the filter kernel
+        std::vector<const pfac::DevTables *> ts, sts;
+        std::vector<pfac::MatchRequest> rs, srs;
         for (uint32_t a = 0; a < nh; ++a) {
-            pfac::MatchRequest &m = rs[a];
+            if (heads[a].units == 0) continue;
+            pfac::MatchRequest m;
             m.text = base;
             m.batch = d_heads + a;
             m.lists = d_list;
-            m.slots.counts = counts;
-            m.slots.slots = slots;
             m.slots.ubase = ubase[a];
-            m.slots.dense = dense_for(a, dense);
             m.scratch = counters + 16u * a;
             m.scratch_bytes = 16;
+            if (streamed(a)) {
+                m.bits = bits;
+                sts.push_back(s->tabs[a]);
+                srs.push_back(m);
+            } else {
+                m.slots.counts = counts;
+                m.slots.slots = slots;
+                m.slots.dense = dense_for(a, dense);
+                ts.push_back(s->tabs[a]);
+                rs.push_back(m);
+            }
         }
-        e = pfac::launch_filter_multi(s->tabs.data(), rs.data(), nh, pfac::OUT_SLOTS, s->tune[0].wait_ns, w.stream,
-                                      surv_lists, list_cap);
+        if (e == cudaSuccess && !ts.empty())
+            e = pfac::launch_filter_multi(ts.data(), rs.data(), static_cast<uint32_t>(ts.size()), pfac::OUT_SLOTS,
+                                          s->tune[0].wait_ns, w.stream, surv_lists, list_cap);
+        if (e == cudaSuccess && !sts.empty()) {
+            void *walks = dp + bits_at + bb;
+            e = cudaMemsetAsync(walks, 0, 32, w.stream);
+            if (e == cudaSuccess)
+                e = pfac::launch_stream_batch(sts.data(), srs.data(), static_cast<uint32_t>(sts.size()), pfac::OUT_BITS,
+                                              s->tune[0].wait_ns, walks, walk_cap, w.stream);
+        }
     }
     for (uint32_t a = 0; a < nh && e == cudaSuccess && !s->multi; ++a) {
         if (heads[a].units == 0) continue;
@@ -360,8 +433,12 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     }
     if (e == cudaSuccess)
         e = pfac::launch_compact_scan(counts, static_cast<uint32_t>(U), nullptr, prefix, partials, w.stream);
+    if (e == cudaSuccess && Us)
+        e = pfac::launch_bits_texts(
+            reinterpret_cast<const pfac::BitsText *>(dp + round256(hb) + round256(lb) + round256(ob)),
+            static_cast<uint32_t>(btexts.size()), static_cast<uint32_t>(Us), bits, prefix + Uo, w.stream);
     for (uint32_t a = 0; a < nh && e == cudaSuccess; ++a) {
-        if (heads[a].units == 0) continue;
+        if (heads[a].units == 0 || streamed(a)) continue;
         pfac::GatherRequest g;
         g.text = base;
         g.batch = d_heads + a;
@@ -551,6 +628,8 @@ ac_status ac_server_create(const ac_handle *hs, uint32_t nh, const ac_server_opt
     s->max_wave = o.max_wave ? o.max_wave : 4096u;
     s->fifo = o.fifo != 0;
     s->multi = !s->fifo && pfac::filter_multi_serves(s->tabs.data(), nh);
+    for (uint32_t a = 0; a < nh; ++a)
+        s->streams.push_back(s->multi && pfac::stream_batch_serves(*s->tabs[a], s->tune[a]));
     uint32_t nw = o.waves_in_flight ? o.waves_in_flight : 2u;
     if (nw > kMaxWaves) nw = kMaxWaves;
     if (s->fifo) nw = 1;
