@@ -23,6 +23,8 @@ namespace pfac {
 
 namespace {
 
+// (What an earlier launch wrote is read with plain loads: these kernels may
+// have started before it ended.)
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kThreads = 256;
 constexpr uint32_t kWarps = kThreads / 32;
@@ -49,8 +51,8 @@ struct BitsParams {
 __device__ __forceinline__ uint2 tile_bits(const BitsParams &p, uint32_t t, int lane) {
     const uint32_t w = t * kWords + 2u * static_cast<uint32_t>(lane);
     uint2 b = make_uint2(0u, 0u);
-    if (w < p.words) b.x = __ldg(p.bits + w);
-    if (w + 1u < p.words) b.y = __ldg(p.bits + w + 1u);
+    if (w < p.words) b.x = p.bits[w];
+    if (w + 1u < p.words) b.y = p.bits[w + 1u];
     return b;
 }
 
@@ -87,12 +89,12 @@ __device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32
         if (!FULL) {
             if (k < total && at + k < p.out.cap) {
                 p.out.pos[at + k] = pos;
-                p.out.ids[at + k] = static_cast<uint32_t>(__ldg(p.ids + g0 + i));
+                p.out.ids[at + k] = static_cast<uint32_t>(p.ids[g0 + i]);
             }
         } else {
             uint32_t id = 0, cl = 0;
             if (k < total) {
-                id = static_cast<uint32_t>(__ldg(p.ids + g0 + i));
+                id = static_cast<uint32_t>(p.ids[g0 + i]);
                 cl = chain_len(p, id);
             }
             uint32_t inc = cl;
@@ -109,13 +111,15 @@ __device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32
 
 // The occurrences of each tile's results, one warp per tile.
 __global__ void __launch_bounds__(kThreads) full_bits_count(const BitsParams p) {
+    allow_next();
+    wait_previous();
     __shared__ uint16_t lists[kWarps][kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t t = blockIdx.x * kWarps + static_cast<uint32_t>(warp); t < p.ntiles; t += gridDim.x * kWarps) {
         const uint32_t total = list_bits(tile_bits(p, t, lane), lists[warp], lane);
         uint32_t sum = 0;
         for (uint32_t k = static_cast<uint32_t>(lane); k < total; k += 32u)
-            sum += chain_len(p, static_cast<uint32_t>(__ldg(p.ids + static_cast<size_t>(t) * kTile + lists[warp][k])));
+            sum += chain_len(p, static_cast<uint32_t>(p.ids[static_cast<size_t>(t) * kTile + lists[warp][k]]));
         sum = __reduce_add_sync(kFull, sum);
         if (lane == 0) p.fcounts[t] = sum;
     }
@@ -126,6 +130,7 @@ __global__ void __launch_bounds__(kThreads) full_bits_count(const BitsParams p) 
 // prefix, and skip the empty ones by their counts.
 template <bool FULL, bool SMALL>
 __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
+    wait_previous();
     __shared__ uint16_t lists[kWarps][kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if constexpr (SMALL) {
@@ -134,11 +139,11 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
         const uint32_t t0 = blockIdx.x * kWarps, t = t0 + static_cast<uint32_t>(warp);
         unsigned long long sum = 0;
         if (FULL) {
-            for (uint32_t i = threadIdx.x; i < t0; i += kThreads) sum += __ldg(p.counts + i);
+            for (uint32_t i = threadIdx.x; i < t0; i += kThreads) sum += p.counts[i];
         } else {  // the words before the CTA's tiles, 16 bytes a thread
             const uint4 *b = reinterpret_cast<const uint4 *>(p.bits);
             for (uint32_t i = threadIdx.x; i < t0 * (kWords / 4u); i += kThreads) {
-                const uint4 v = __ldg(b + i);
+                const uint4 v = b[i];
                 sum += static_cast<uint32_t>(__popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
             }
         }
@@ -148,7 +153,7 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
         if (t < p.ntiles) b = tile_bits(p, t, lane);
         uint32_t mine = 0;
         if (FULL)
-            mine = t < p.ntiles ? __ldg(p.counts + t) : 0u;
+            mine = t < p.ntiles ? p.counts[t] : 0u;
         else
             mine = __reduce_add_sync(kFull, static_cast<uint32_t>(__popc(b.x) + __popc(b.y)));
         if (lane == 0) {
@@ -169,27 +174,28 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
         const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
         for (uint64_t u0 = gw; u0 < p.ntiles; u0 += 32ull * nw) {
             const uint64_t u = u0 + static_cast<uint64_t>(lane) * nw;
-            const uint32_t c = u < p.ntiles ? __ldg(p.counts + u) : 0u;
+            const uint32_t c = u < p.ntiles ? p.counts[u] : 0u;
             for (uint32_t todo = __ballot_sync(kFull, c != 0u); todo; todo &= todo - 1u) {
                 const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
-                put_tile<FULL>(p, t, t * kTile - p.head, tile_bits(p, t, lane), __ldg(p.prefix + t), lists[warp],
+                put_tile<FULL>(p, t, t * kTile - p.head, tile_bits(p, t, lane), p.prefix[t], lists[warp],
                                lane);
             }
         }
         if (gw == 0 && lane == 0)
-            *p.out.count = __ldg(p.prefix + p.ntiles - 1u) + __ldg(p.counts + p.ntiles - 1u);
+            *p.out.count = p.prefix[p.ntiles - 1u] + p.counts[p.ntiles - 1u];
     }
 }
 
 // The lists of several texts (streaming form): as bits_gather, each unit's text
 // found by a 32-way search.
 __global__ void __launch_bounds__(kThreads) bits_gather_texts(BitsParams p, const BitsText *texts, uint32_t nt) {
+    wait_previous();
     __shared__ uint16_t lists[kWarps][kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
     for (uint64_t u0 = gw; u0 < p.ntiles; u0 += 32ull * nw) {
         const uint64_t u = u0 + static_cast<uint64_t>(lane) * nw;
-        const uint32_t c = u < p.ntiles ? __ldg(p.counts + u) : 0u;
+        const uint32_t c = u < p.ntiles ? p.counts[u] : 0u;
         for (uint32_t todo = __ballot_sync(kFull, c != 0u); todo; todo &= todo - 1u) {
             const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
             uint32_t lo = 0, hi = nt;  // the last text whose first unit is <= t
@@ -203,13 +209,13 @@ __global__ void __launch_bounds__(kThreads) bits_gather_texts(BitsParams p, cons
             const BitsText x = texts[lo];
             p.out = x.out;
             put_tile<false>(p, t, (t - x.first) * kTile - x.head, tile_bits(p, t, lane),
-                            __ldg(p.prefix + t) - __ldg(p.prefix + x.first), lists[warp], lane);
+                            p.prefix[t] - p.prefix[x.first], lists[warp], lane);
         }
     }
     for (uint32_t i = gw * 32u + static_cast<uint32_t>(lane); i < nt; i += nw * 32u) {
         const BitsText x = texts[i];
         const uint32_t last = x.first + x.units - 1u;
-        *x.out.count = __ldg(p.prefix + last) + __ldg(p.counts + last) - __ldg(p.prefix + x.first);
+        *x.out.count = p.prefix[last] + p.counts[last] - p.prefix[x.first];
     }
 }
 
@@ -264,8 +270,7 @@ cudaError_t launch_bits_texts(const BitsText *texts, uint32_t nt, uint32_t units
     p.prefix = prefix;
     const uint32_t need = (units + kWarps - 1) / kWarps, sms = device_sm_count();
     if (sms == 0) return cudaErrorInvalidDevice;
-    bits_gather_texts<<<need < sms * 6u ? need : sms * 6u, kThreads, 0, stream>>>(p, texts, nt);
-    return cudaGetLastError();
+    return launch_next(bits_gather_texts, need < sms * 6u ? need : sms * 6u, kThreads, 0u, stream, p, texts, nt);
 }
 
 size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full) {
@@ -318,25 +323,17 @@ cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *te
     if (sms == 0) return cudaErrorInvalidDevice;
     const uint32_t grid = need < sms * 6u ? need : sms * 6u;
     if (full) {
-        full_bits_count<<<grid, kThreads, 0, stream>>>(p);
-        e = cudaGetLastError();
+        e = launch_next(full_bits_count, grid, kThreads, 0u, stream, p);
         if (e != cudaSuccess) return e;
     }
-    if (l.small) {
-        if (full)
-            bits_gather<true, true><<<need, kThreads, 0, stream>>>(p);
-        else
-            bits_gather<false, true><<<need, kThreads, 0, stream>>>(p);
-        return cudaGetLastError();
-    }
+    if (l.small)
+        return full ? launch_next(bits_gather<true, true>, need, kThreads, 0u, stream, p)
+                    : launch_next(bits_gather<false, true>, need, kThreads, 0u, stream, p);
     e = launch_compact_scan(p.counts, l.ntiles, nullptr, prefix, reinterpret_cast<unsigned long long *>(b + l.partials),
                             stream);
     if (e != cudaSuccess) return e;
-    if (full)
-        bits_gather<true, false><<<grid, kThreads, 0, stream>>>(p);
-    else
-        bits_gather<false, false><<<grid, kThreads, 0, stream>>>(p);
-    return cudaGetLastError();
+    return full ? launch_next(bits_gather<true, false>, grid, kThreads, 0u, stream, p)
+                : launch_next(bits_gather<false, false>, grid, kThreads, 0u, stream, p);
 }
 
 }  // namespace pfac

@@ -74,12 +74,14 @@ __device__ __forceinline__ uint32_t scan_units(uint32_t units, const uint32_t *u
 __global__ void __launch_bounds__(kScanThreads) compact_reduce(const uint32_t *counts, uint32_t units,
                                                                const uint32_t *units_dev,
                                                                unsigned long long *partials) {
+    allow_next();
+    wait_previous();
     const uint32_t U = scan_units(units, units_dev);
     const uint32_t R = (U + gridDim.x - 1) / gridDim.x;
     const uint64_t lo = static_cast<uint64_t>(blockIdx.x) * R;
     const uint64_t hi = lo + R < U ? lo + R : U;
     unsigned long long s = 0;
-    for (uint64_t u = lo + threadIdx.x; u < hi; u += blockDim.x) s += __ldg(counts + u);
+    for (uint64_t u = lo + threadIdx.x; u < hi; u += blockDim.x) s += counts[u];
     s = block_sum(s);
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
@@ -88,6 +90,8 @@ __global__ void __launch_bounds__(kScanThreads) compact_prefix(const uint32_t *c
                                                                const uint32_t *units_dev,
                                                                unsigned long long *prefix,
                                                                const unsigned long long *partials) {
+    allow_next();
+    wait_previous();
     const uint32_t U = scan_units(units, units_dev);
     const uint32_t R = (U + gridDim.x - 1) / gridDim.x;
     const uint64_t lo = static_cast<uint64_t>(blockIdx.x) * R;
@@ -97,7 +101,7 @@ __global__ void __launch_bounds__(kScanThreads) compact_prefix(const uint32_t *c
     base = block_sum(base);
     for (uint64_t c0 = lo; c0 < hi; c0 += blockDim.x) {
         const uint64_t u = c0 + threadIdx.x;
-        const unsigned long long v = u < hi ? __ldg(counts + u) : 0ull;
+        const unsigned long long v = u < hi ? counts[u] : 0ull;
         unsigned long long tot = 0;
         const unsigned long long ex = block_excl(v, tot);
         if (u < hi) prefix[u] = base + ex;
@@ -213,11 +217,10 @@ __global__ void __launch_bounds__(kGatherThreads) compact_gather(const GatherPar
 cudaError_t launch_compact_scan(const uint32_t *counts, uint32_t units, const uint32_t *units_dev,
                                 unsigned long long *prefix, unsigned long long *partials, cudaStream_t stream) {
     if (!counts || !prefix || !partials) return cudaErrorInvalidValue;
-    compact_reduce<<<kScanCtas, kScanThreads, 0, stream>>>(counts, units, units_dev, partials);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        launch_next(compact_reduce, kScanCtas, kScanThreads, 0u, stream, counts, units, units_dev, partials);
     if (e != cudaSuccess) return e;
-    compact_prefix<<<kScanCtas, kScanThreads, 0, stream>>>(counts, units, units_dev, prefix, partials);
-    return cudaGetLastError();
+    return launch_next(compact_prefix, kScanCtas, kScanThreads, 0u, stream, counts, units, units_dev, prefix, partials);
 }
 
 cudaError_t launch_compact_gather(const DevTables &t, const GatherRequest &g, cudaStream_t stream) {

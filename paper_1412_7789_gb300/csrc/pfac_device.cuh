@@ -9,6 +9,8 @@
 
 #include <cstdint>
 
+#include <cuda_runtime.h>
+
 #include "pfac_internal.h"
 
 namespace pfac {
@@ -17,6 +19,31 @@ namespace pfac {
 // Every bounded wait gives up after this many nanoseconds of %globaltimer
 // unless the launch names another limit (ac_set_wait_limit).
 constexpr unsigned long long kWaitNs = 2000000000ull;
+
+// Programmatic dependent launch (launch_next): the kernel may start as the CTAs
+// of the launch before it leave (allow_next lets it be scheduled early), and
+// must not go past wait_previous before that launch has ended and its writes
+// are visible.  Every kernel launched this way waits before it ends, so
+// whatever follows it follows everything before it too.  (Without the launch
+// attribute both do nothing.)
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*kernel)(P...), uint32_t grid, uint32_t block, uint32_t smem, cudaStream_t stream,
+                        const A &...args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

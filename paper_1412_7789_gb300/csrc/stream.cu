@@ -11,106 +11,146 @@ using namespace strm;
 
 namespace {
 
-// Texts up to this length take one thread per position: no filter to load
-// into every SM, no list, one launch.  4 KiB of the sweep set, where every
-// position walks to a match: 10 us a call against 70 in the filter kernel,
-// whose few tiles kept a handful of warps busy.  The line against the
-// streaming form (us a call from an idle GPU, host time included): ACGT 2 MiB
-// 30 / 32, 4 MiB 42 / 33; Zipf bytes 2 MiB 40 / 43, 4 MiB 57 / 45.
+// Texts up to this length take one lane per position: no filter to load into
+// every SM, no list, one launch.  4 KiB of the sweep set, where every position
+// walks to a match: 10 us a call against 70 in the filter kernel, whose few
+// tiles kept a handful of warps busy.  The line against the streaming form (us
+// a call from an idle GPU, host time included): ACGT 2 MiB 25 / 30, 3 MiB 29 /
+// 30; Zipf bytes 2 MiB 44 / 43, 4 MiB 57 / 40.
 constexpr uint64_t kAtMax = 2u << 20;
 constexpr int kAtBlock = 128;
 
-// One thread per position (a text this short and the tables it touches stay in
-// L2).  A warp reads its 32 bytes and the 16 after them once, one byte a lane,
-// and joins their codes into windows with log2(window) shuffles, so a position
-// costs two byte loads and one load per table level.
-template <int B, typename GT, int MODE>
+// One lane per position (a text this short and the tables it touches stay in
+// L2).  A warp reads its PER x 32 bytes and the 16 after them once, one byte a
+// lane and load, and joins their codes into windows with log2(window) shuffles,
+// so a position costs little more than a byte load and a load per table level;
+// a lane's PER positions have theirs in flight together.
+template <int B, typename GT, int MODE, int PER>
 __global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ FilterParams p) {
     __shared__ uint8_t cls8[256];
+    allow_next();  // the lists' gather
     const int lane = threadIdx.x & 31;
-    const uint64_t gi = static_cast<uint64_t>(blockIdx.x) * kAtBlock + threadIdx.x;
-    const bool in = gi < p.n, in2 = lane < 16 && gi + 32u < p.n;
-    const uint32_t b0 = in ? __ldg(p.text + gi) : 0u, b1 = in2 ? __ldg(p.text + gi + 32u) : 0u;
+    const uint64_t g0 = (static_cast<uint64_t>(blockIdx.x) * (kAtBlock / 32) + (threadIdx.x >> 5)) * (32u * PER) + lane;
+    uint32_t c[PER + 1];
+    bool in[PER + 1];
+#pragma unroll
+    for (int j = 0; j <= PER; ++j) {
+        in[j] = g0 + 32u * j < p.n && (j < PER || lane < 16);
+        c[j] = in[j] ? __ldg(p.text + g0 + 32u * j) : 0u;
+    }
     for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
     __syncthreads();
     // codes, and which positions hold none (a byte in no keyword, or the text's end)
     const bool id = B == 8 && p.identity;
-    uint32_t lo = id ? b0 : cls8[b0], hi = id ? b1 : cls8[b1];
-    const bool bad0 = !in || (!id && lo == 0xFFu), bad1 = !in2 || (!id && hi == 0xFFu);
-    const uint32_t m0 = __ballot_sync(kFull, bad0), m1 = __ballot_sync(kFull, bad1);
-    const uint32_t bad = __funnelshift_r(m0, m1, lane);  // bit j: position gi + j
-    lo &= (1u << B) - 1u;
-    hi &= (1u << B) - 1u;
-    uint32_t after = 0;  // 8-bit codes: the code after the window
+    uint32_t bad[PER + 1];  // bit i: position i of the 32
+#pragma unroll
+    for (int j = 0; j <= PER; ++j) {
+        if (!id) c[j] = cls8[c[j]];
+        bad[j] = __ballot_sync(kFull, !in[j] || (!id && c[j] == 0xFFu));
+        c[j] &= (1u << B) - 1u;
+    }
+    const uint32_t need = B == 8 ? p.k : p.k + p.k2;
+    uint32_t after[PER];  // 8-bit codes: the code after the window
     if (B == 8) {
         const uint32_t x = static_cast<uint32_t>(lane) + p.k;
-        const uint32_t y = __shfl_sync(kFull, lo, x & 31u), z = __shfl_sync(kFull, hi, x & 31u);
-        after = x < 32u ? y : z;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t y = __shfl_sync(kFull, c[j], x & 31u), z = __shfl_sync(kFull, c[j + 1], x & 31u);
+            after[j] = x < 32u ? y : z;
+        }
     }
 #pragma unroll
     for (uint32_t d = 1; d * B < 32u; d *= 2u) {  // windows of d codes -> 2 d
         const uint32_t x = static_cast<uint32_t>(lane) + d;
-        const uint32_t y = __shfl_sync(kFull, lo, x & 31u), z = __shfl_sync(kFull, hi, x & 31u);
-        lo |= (x < 32u ? y : z) << (B * d);
-        hi |= z << (B * d);  // the last lanes' are never read
-    }
-    uint32_t cnt = 0;
-    if (in) {
-        const TileText tt = make_text(p.text, p.out, p.n, 0u);
-        const uint32_t need = B == 8 ? p.k : p.k + p.k2;
-        int r = -1;
-        uint32_t s = 0, q = 0;
-        bool walk = true;
-        if (!(bad & ((1u << need) - 1u))) {
-            if (B == 8) {
-                const uint32_t w = lo & p.wmask;
-                walk = !filt::hk_outcome(p, filt::hk_find(p, w, __ldg(p.HK + filt::hk_slot(p, w))), 0u, after,
-                                         !((bad >> p.k) & 1u), r, s, q);
-            } else {
-                const int e = __ldg(p.JK + (lo & ((1u << (B * p.k)) - 1u)));
-                walk = e >= 0;
-                if (walk) {
-                    s = static_cast<uint32_t>(e);
-                    q = p.k;
-                    if (p.k2) {
-                        const int e2 = __ldg(p.J2 + ((static_cast<uint64_t>(s - p.base_k) << (B * p.k2)) |
-                                                     ((lo >> (B * p.k)) & ((1u << (B * p.k2)) - 1u))));
-                        walk = e2 >= 0;
-                        if (walk) {
-                            s = static_cast<uint32_t>(e2);
-                            q += p.k2;
-                        } else {
-                            r = decode_dead(e2);
-                        }
-                    }
-                } else {
-                    r = decode_dead(e);
-                }
-            }
-        } else if (B == 8) {
-            walk = false;  // no keyword is shorter than the state hash's window
+        uint32_t y = __shfl_sync(kFull, c[0], x & 31u);
+#pragma unroll
+        for (int j = 0; j <= PER; ++j) {  // (the last set's upper lanes are never read)
+            const uint32_t z = j < PER ? __shfl_sync(kFull, c[j < PER ? j + 1 : j], x & 31u) : y;
+            c[j] |= (x < 32u ? y : z) << (B * d);
+            y = z;
         }
-        if (walk) r = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s, q);
-        if (MODE == OUT_DENSE)
-            p.out[gi] = r;
-        else
-            cnt = r >= 0 ? 1u : 0u;
-        if (MODE == OUT_BITS && r >= 0) p.bo.ids[gi] = r;
     }
-    if (MODE == OUT_BITS) {
-        const uint32_t bits = __ballot_sync(kFull, cnt != 0u);
-        if (lane == 0 && in) p.bo.bits[gi >> 5] = bits;
+    // first loads of all the lane's positions, then the second
+    int e[PER], r[PER];
+    uint4 h[PER];
+    bool walk[PER];
+    uint32_t s[PER], q[PER], m[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        m[j] = __funnelshift_r(bad[j], bad[j + 1], lane);  // bit i: position i after this one
+        walk[j] = in[j];
+        r[j] = -1;
+        s[j] = q[j] = 0;
+        e[j] = 0;
+        h[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (m[j] & ((1u << need) - 1u)) {
+            if (B == 8) walk[j] = false;  // no keyword is shorter than the state hash's window
+            continue;
+        }
+        if (B == 8)
+            h[j] = __ldg(p.HK + filt::hk_slot(p, c[j] & p.wmask));
+        else
+            e[j] = __ldg(p.JK + (c[j] & ((1u << (B * p.k)) - 1u)));
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (m[j] & ((1u << need) - 1u)) continue;
+        if (B == 8) {
+            walk[j] = !filt::hk_outcome(p, filt::hk_find(p, c[j] & p.wmask, h[j]), 0u, after[j], !((m[j] >> p.k) & 1u),
+                                        r[j], s[j], q[j]);
+        } else if (e[j] >= 0 && p.k2) {
+            q[j] = p.k + p.k2;
+            e[j] = __ldg(p.J2 + ((static_cast<uint64_t>(static_cast<uint32_t>(e[j]) - p.base_k) << (B * p.k2)) |
+                                 ((c[j] >> (B * p.k)) & ((1u << (B * p.k2)) - 1u))));
+        } else {
+            q[j] = p.k;
+        }
+    }
+    const TileText tt = make_text(p.text, p.out, p.n, 0u);
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (B != 8 && !(m[j] & ((1u << need) - 1u))) {
+            walk[j] = e[j] >= 0;
+            s[j] = static_cast<uint32_t>(e[j]);
+            if (e[j] < 0) r[j] = decode_dead(e[j]);
+        }
+        const uint64_t gi = g0 + 32u * j;
+        if (walk[j]) r[j] = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s[j], q[j]);
+        if (MODE == OUT_DENSE) {
+            if (in[j]) p.out[gi] = r[j];
+        } else if (MODE == OUT_COUNT) {
+            cnt += in[j] && r[j] >= 0 ? 1u : 0u;
+        } else {
+            if (in[j] && r[j] >= 0) p.bo.ids[gi] = r[j];
+            const uint32_t bits = __ballot_sync(kFull, in[j] && r[j] >= 0);
+            if (lane == 0 && in[j]) p.bo.bits[gi >> 5] = bits;
+        }
     }
     add_count<MODE>(p, cnt, lane);
 }
 
+// Positions a lane from this length on: 4 (fewer CTAs, and four chains of loads
+// in flight: 1 MiB of ACGT 12.3 -> 10.5 us a call); below, 1, where the walks of
+// a text dense in matches need every warp.
+constexpr uint64_t kAtWide = 256u << 10;
+
+template <int B, typename GT, int MODE>
+void launch_at_one(const FilterParams &p, cudaStream_t stream) {
+    const uint32_t per = p.n >= kAtWide ? 4u : 1u;
+    const uint32_t grid = static_cast<uint32_t>((p.n + kAtBlock * per - 1) / (kAtBlock * per));
+    if (per == 4u)
+        pfac_at<B, GT, MODE, 4><<<grid, kAtBlock, 0, stream>>>(p);
+    else
+        pfac_at<B, GT, MODE, 1><<<grid, kAtBlock, 0, stream>>>(p);
+}
+
 template <int B, typename GT>
 cudaError_t launch_at_modes(OutMode mode, const FilterParams &p, cudaStream_t stream) {
-    const uint32_t grid = static_cast<uint32_t>((p.n + kAtBlock - 1) / kAtBlock);
     switch (mode) {
-        case OUT_DENSE: pfac_at<B, GT, OUT_DENSE><<<grid, kAtBlock, 0, stream>>>(p); break;
-        case OUT_COUNT: pfac_at<B, GT, OUT_COUNT><<<grid, kAtBlock, 0, stream>>>(p); break;
-        case OUT_BITS: pfac_at<B, GT, OUT_BITS><<<grid, kAtBlock, 0, stream>>>(p); break;
+        case OUT_DENSE: launch_at_one<B, GT, OUT_DENSE>(p, stream); break;
+        case OUT_COUNT: launch_at_one<B, GT, OUT_COUNT>(p, stream); break;
+        case OUT_BITS: launch_at_one<B, GT, OUT_BITS>(p, stream); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -119,6 +159,9 @@ cudaError_t launch_at_modes(OutMode mode, const FilterParams &p, cudaStream_t st
 template <int B, typename GT>
 cudaError_t launch_walk_modes(OutMode mode, const FilterParams &p, uint32_t sms, cudaStream_t stream) {
     const uint32_t grid = sms * kWalkCtas;
+    // (a plain launch: started early, the walks' CTAs cost the form before them
+    // more than the gap they save, 1 GiB of Zipf bytes compacted 1360 against
+    // 1155 us)
     switch (mode) {
         case OUT_DENSE: pfac_stream_walks<B, GT, OUT_DENSE><<<grid, kWalkBlock, 0, stream>>>(p); break;
         case OUT_COUNT: pfac_stream_walks<B, GT, OUT_COUNT><<<grid, kWalkBlock, 0, stream>>>(p); break;
@@ -186,10 +229,10 @@ cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mod
 
 // Shared memory of a launch: the filters, the -1 buffer (and 128 bytes for the
 // CTA), the warps' areas.
-uint32_t stream_smem(uint32_t form, uint32_t filters, uint32_t *off_none, uint32_t *off_warp) {
+uint32_t stream_smem(uint32_t form, bool batch, uint32_t filters, uint32_t *off_none, uint32_t *off_warp) {
     *off_none = (filters + 127u) & ~127u;
     *off_warp = *off_none + 4u * kNone + 128u;
-    return *off_warp + static_cast<uint32_t>(block_of(form) / 32) * (form == 2 ? kWarpBytes2 : kWarpBytes8);
+    return *off_warp + static_cast<uint32_t>(block_of(form, batch) / 32) * (form == 2 ? kWarpBytes2 : kWarpBytes8);
 }
 
 }  // namespace
@@ -204,11 +247,11 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
     StreamParams p{};
     e = stream_params(t, r, mode, tu, p);
     if (e != cudaSuccess) return e;
-    const uint64_t head = reinterpret_cast<uintptr_t>(r.text) & 15u;
-    p.ntiles = static_cast<uint32_t>((r.n + head + kTile - 1) / kTile);
-    const uint32_t smem = stream_smem(t.stream.form, p.f1bytes + p.f2bytes, &p.off_none, &p.off_warp);
+    p.sg = make_seg(r.text, r.out, r.n);
+    p.ntiles = static_cast<uint32_t>((r.n + p.sg.head + kTile - 1) / kTile);
+    const uint32_t smem = stream_smem(t.stream.form, false, p.f1bytes + p.f2bytes, &p.off_none, &p.off_warp);
     if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
-    const uint32_t nw = static_cast<uint32_t>(block_of(t.stream.form) / 32), need = (p.ntiles + nw - 1) / nw;
+    const uint32_t nw = static_cast<uint32_t>(block_of(t.stream.form, false) / 32), need = (p.ntiles + nw - 1) / nw;
     const uint32_t grid = need < static_cast<uint32_t>(sms) ? need : static_cast<uint32_t>(sms);
     e = t.stream.form == 2 ? launch_stream2(mode, p, t.stream.step, grid, smem, max_smem, stream)
                            : launch_stream8(mode, p, grid, smem, max_smem, stream);
@@ -244,6 +287,7 @@ cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *
     uint8_t *b = static_cast<uint8_t *>(walks);
     wm.nh = nh;
     // one launch per form and step, then the walks of all
+    bool next = false;  // after another of these launches
     for (uint32_t group = 0; group < 4; ++group) {
         const uint32_t form = group < 3 ? 2u : 8u, step = group < 3 ? 1u << group : 1u;
         uint32_t filters = 0;
@@ -267,20 +311,18 @@ cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *
             filters = filters > p.f1bytes + p.f2bytes ? filters : p.f1bytes + p.f2bytes;
         }
         if (mp.nh == 0) continue;
-        const uint32_t smem = stream_smem(form, filters, &mp.off_none, &mp.off_warp);
+        const uint32_t smem = stream_smem(form, true, filters, &mp.off_none, &mp.off_warp);
         if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
         const uint32_t grid = static_cast<uint32_t>(sms);
-        e = form == 2 ? launch_stream2_multi(mode, mp, step, grid, smem, max_smem, stream)
-                      : launch_stream8_multi(mode, mp, grid, smem, max_smem, stream);
+        e = form == 2 ? launch_stream2_multi(mode, mp, step, grid, smem, max_smem, stream, next)
+                      : launch_stream8_multi(mode, mp, grid, smem, max_smem, stream, next);
         if (e != cudaSuccess) return e;
+        next = true;
     }
     const uint32_t grid = static_cast<uint32_t>(sms) * 8u;
     const uint32_t smem = nh * (static_cast<uint32_t>(sizeof(FilterParams)) + 256u);
-    if (mode == OUT_DENSE)
-        pfac_stream_walks_multi<OUT_DENSE><<<grid, kWalkBlock, smem, stream>>>(wm);
-    else
-        pfac_stream_walks_multi<OUT_BITS><<<grid, kWalkBlock, smem, stream>>>(wm);
-    return cudaGetLastError();
+    return mode == OUT_DENSE ? launch_next(pfac_stream_walks_multi<OUT_DENSE>, grid, kWalkBlock, smem, stream, wm)
+                             : launch_next(pfac_stream_walks_multi<OUT_BITS>, grid, kWalkBlock, smem, stream, wm);
 }
 
 }  // namespace pfac

@@ -47,13 +47,17 @@ namespace strm {
 using filt::FilterParams;
 using filt::kFull;
 
-// Threads per CTA, one CTA per SM (GB300, 1 GiB: with 2-bit codes 640 / 768
-// threads count in 288 / 275 us; with 8-bit codes 512 / 640 / 768 write dense
-// ids in 1155 / 1064 / 1178 us, 768 spilling at 80 registers).
-constexpr int kBlock2 = 768;
-constexpr int kBlock8 = 640;
+// Threads per CTA, one CTA per SM: what runs fastest without spills, which cost
+// these loops more than the warps they buy.  GB300, 2-bit codes: 640 / 768
+// threads, 256 MiB compacted 140 / 156 us, 1 GiB counted 286 / 325 (768 with no
+// spill: 275); 8-bit codes, one text: 640 / 768, 1 GiB counted 930 / 919, dense
+// 1074 / 1050, compacted 1164 / 1114; in a batch the kernel spills at 768.
+constexpr int kBlock2 = 640;
+constexpr int kBlock8 = 768, kBlock8Multi = 640;
 constexpr int kMostWarps = (kBlock2 > kBlock8 ? kBlock2 : kBlock8) / 32;
-__host__ __device__ constexpr int block_of(uint32_t form) { return form == 2 ? kBlock2 : kBlock8; }
+__host__ __device__ constexpr int block_of(uint32_t form, bool batch) {
+    return form == 2 ? kBlock2 : (batch ? kBlock8Multi : kBlock8);
+}
 constexpr uint32_t kTile = kStreamTile;  // positions a warp takes at a time
 constexpr uint32_t kChunk = 512;         // positions per warp-wide 16-byte load
 constexpr uint32_t kQueue = 256;         // survivors of a tile kept in shared memory at a time
@@ -64,16 +68,6 @@ constexpr uint32_t kWarpBytes2 = kTile / 4 + 16 + 2 * kQueue + 8 * kRes2;
 constexpr uint32_t kWarpBytes8 = kTile + 16 + 2 * kQueue + 9 * kRes8;
 static_assert(kWarpBytes2 % 16 == 0 && kWarpBytes8 % 16 == 0, "warp areas start on 16 bytes");
 
-struct StreamParams {
-    FilterParams f;        // tables, text, outputs, walk list (walks, walk_cap, list_count[1])
-    const uint32_t *F1;    // root filter, f1bytes
-    const uint32_t *F2;    // second filter (f2bytes; 0: none), with 8-bit codes then its short-keyword part
-    uint32_t f1bytes, f2bytes;
-    uint32_t ntiles;
-    uint32_t m1, m2;       // 8-bit codes: multipliers of the window's words
-    uint32_t l2shift;      // 2-bit codes: left shift that drops the codes past the second filter's window
-    uint32_t off_none, off_warp;
-};
 
 // 16 bytes of text, read once: around L1, first to leave L2.
 __device__ __forceinline__ uint4 ldg_stream(const uint8_t *p, uint64_t pol) {
@@ -114,7 +108,7 @@ __device__ __forceinline__ uint64_t text_pos(const Seg &sg, uint32_t g) {  // be
 }
 
 // The text's part of a segment.
-__device__ __forceinline__ Seg make_seg(const uint8_t *text, int32_t *out, uint64_t n) {
+__host__ __device__ __forceinline__ Seg make_seg(const uint8_t *text, int32_t *out, uint64_t n) {
     Seg sg;
     sg.text = text;
     sg.out = out;
@@ -127,6 +121,18 @@ __device__ __forceinline__ Seg make_seg(const uint8_t *text, int32_t *out, uint6
     sg.t0 = sg.bit0 = sg.unit0 = sg.item = 0;
     return sg;
 }
+
+struct StreamParams {
+    FilterParams f;        // tables, text, outputs, walk list (walks, walk_cap, list_count[1])
+    const uint32_t *F1;    // root filter, f1bytes
+    const uint32_t *F2;    // second filter (f2bytes; 0: none), with 8-bit codes then its short-keyword part
+    uint32_t f1bytes, f2bytes;
+    uint32_t ntiles;
+    Seg sg;                // one text
+    uint32_t m1, m2;       // 8-bit codes: multipliers of the window's words
+    uint32_t l2shift;      // 2-bit codes: left shift that drops the codes past the second filter's window
+    uint32_t off_none, off_warp;
+};
 
 // A tile's registers: lane l's 16 bytes of chunks 0-3, and (lane 0) the 16
 // bytes after the tile.
@@ -818,10 +824,14 @@ template <int FORM, int S, int MODE>
 __device__ __forceinline__ void stream_text(const StreamParams &p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t step = gridDim.x * (block_of(FORM) / 32);
+    const uint32_t step = gridDim.x * (blockDim.x / 32);
     const uint32_t t = static_cast<uint32_t>(warp) * gridDim.x + blockIdx.x;
     const uint64_t pol = policy_evict_first();
-    const Seg sg = make_seg(p.f.text, p.f.out, p.f.n);
+    // 8-bit codes: from the parameters, whose values need no registers; with
+    // 2-bit codes the copy spills less
+    const Seg own = make_seg(p.f.text, p.f.out, p.f.n);
+    using SegRef = typename std::conditional<FORM == 2, const Seg, const Seg &>::type;
+    SegRef sg = FORM == 2 ? own : p.sg;
     const int32_t *none = reinterpret_cast<const int32_t *>(smem + p.off_none);
     TileRegs r;
     r.look = make_uint4(0u, 0u, 0u, 0u);
@@ -913,6 +923,9 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
     // (dynamic too: a kernel with static shared memory cannot take the most dynamic)
     volatile uint32_t &start = reinterpret_cast<uint32_t *>(smem + mp.off_none)[kNone];
     volatile uint32_t &open = reinterpret_cast<uint32_t *>(smem + mp.off_none)[kNone + 1u];
+    // the next form's launch, or the walks: neither reads what this one writes
+    // before it has ended
+    allow_next();
     fill_constant(smem + mp.off_none);
     uint64_t total = 0;
     for (uint32_t a = 0; a < mp.nh; ++a) total += __ldg(&mp.a[a].f.batch->units);
@@ -935,14 +948,22 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
         const uint32_t a = (first + k) % mp.nh;
         const StreamParams &p = mp.a[a];
         const Work wk = load_work(p.f.batch, p.f.lists, 0u);
-        if (threadIdx.x == 0) open = *reinterpret_cast<volatile unsigned int *>(p.f.counter) < wk.units ? 1u : 0u;
+        // another automaton than its own: only with units left for a good part
+        // of its warps (the filters cost some 5 us), or when too small a share
+        // of the units gave it no CTA of its own
+        if (threadIdx.x == 0) {
+            const uint32_t taken = *reinterpret_cast<volatile unsigned int *>(p.f.counter);
+            const uint32_t left = taken < wk.units ? wk.units - taken : 0u;
+            const bool owned = static_cast<uint64_t>(wk.units) * gridDim.x >= total;
+            open = left > (k > 0u && owned ? gridDim.x * (blockDim.x / 32u) / 4u : 0u) ? 1u : 0u;
+        }
         __syncthreads();
         const bool go = open != 0u;  // the same for every thread
         if (go) load_filters(p, smem);
         __syncthreads();
         if (!go) continue;
         // warps on this automaton, about
-        const uint32_t share = static_cast<uint32_t>(static_cast<uint64_t>(gridDim.x) * (block_of(FORM) / 32) * wk.units / total) + 1u;
+        const uint32_t share = static_cast<uint32_t>(static_cast<uint64_t>(gridDim.x) * (blockDim.x / 32u) * wk.units / total) + 1u;
         // blocks of two units, one towards the end (bigger ones leave the last
         // warps too much, and scatter the traffic: 64 units at first took 810
         // us for 1,024 texts of the benchmark batch against 725); the next block is
@@ -973,6 +994,7 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
     }
     if (FORM == 8 && MODE == OUT_DENSE && lane == 0) bulk_wait_all();
     close_room<true>(mp.a[0].f, ws.room, lane);
+    wait_previous();
 }
 
 template <int S, int MODE>
@@ -980,7 +1002,7 @@ __global__ void __launch_bounds__(kBlock2, 1) pfac_stream2_multi(const __grid_co
     stream_batch<2, S, MODE>(mp);
 }
 template <int MODE>
-__global__ void __launch_bounds__(kBlock8, 1) pfac_stream8_multi(const __grid_constant__ StreamMulti mp) {
+__global__ void __launch_bounds__(kBlock8Multi, 1) pfac_stream8_multi(const __grid_constant__ StreamMulti mp) {
     stream_batch<8, 1, MODE>(mp);
 }
 
@@ -1008,6 +1030,7 @@ template <int B, typename GT, int MODE>
 __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const __grid_constant__ FilterParams p) {
     __shared__ uint8_t cls8[256];
     const int lane = threadIdx.x & 31;
+    allow_next();  // the lists' scan
     const uint32_t listed = *reinterpret_cast<volatile const unsigned int *>(p.list_count + 1);
     const uint32_t m = listed < p.walk_cap ? listed : p.walk_cap;
     if (blockIdx.x * blockDim.x >= m) return;
@@ -1033,6 +1056,8 @@ static_assert(sizeof(WalkMulti) <= 32764, "kernel parameters are limited to 3276
 template <int MODE>
 __global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const __grid_constant__ WalkMulti mp) {
     extern __shared__ __align__(16) uint8_t msm[];
+    allow_next();
+    wait_previous();
     const uint32_t listed = *reinterpret_cast<volatile const unsigned int *>(mp.a[0].list_count + 1);
     const uint32_t m = listed < mp.a[0].walk_cap ? listed : mp.a[0].walk_cap;
     if (blockIdx.x * blockDim.x >= m) return;
@@ -1044,7 +1069,7 @@ __global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const _
     __syncthreads();
     uint32_t cnt = 0;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-        const uint4 e = __ldg(mp.a[0].walks4 + j);
+        const uint4 e = mp.a[0].walks4[j];
         if (e.x == 0xFFFFFFFFu) continue;
         const uint32_t a = e.z >> 11, g = e.z & (kTile - 1u);
         const FilterParams &p = ps[a];
@@ -1064,8 +1089,9 @@ __global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const _
 
 // ---- launches --------------------------------------------------------------------
 
-template <auto Kernel, uint32_t FORM, typename P>
-cudaError_t launch_form(const P &p, uint32_t grid, uint32_t smem, int max_smem, cudaStream_t stream) {
+template <auto Kernel, typename P>
+cudaError_t launch_form(const P &p, uint32_t grid, uint32_t block, uint32_t smem, int max_smem, cudaStream_t stream,
+                        bool next = false) {
     static std::atomic<uint64_t> configured{0};  // bit d: device d (as many as filter_device_shape knows)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1076,7 +1102,8 @@ cudaError_t launch_form(const P &p, uint32_t grid, uint32_t smem, int max_smem, 
         if (e != cudaSuccess) return e;
         configured.fetch_or(1ull << dev);
     }
-    Kernel<<<grid, block_of(FORM), smem, stream>>>(p);
+    if (next) return launch_next(Kernel, grid, block, smem, stream, p);
+    Kernel<<<grid, block, smem, stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -1085,9 +1112,9 @@ cudaError_t launch_stream2(OutMode mode, const StreamParams &p, uint32_t step, u
 cudaError_t launch_stream8(OutMode mode, const StreamParams &p, uint32_t grid, uint32_t smem, int max_smem,
                            cudaStream_t stream);
 cudaError_t launch_stream2_multi(OutMode mode, const StreamMulti &mp, uint32_t step, uint32_t grid, uint32_t smem,
-                                 int max_smem, cudaStream_t stream);
+                                 int max_smem, cudaStream_t stream, bool next);
 cudaError_t launch_stream8_multi(OutMode mode, const StreamMulti &mp, uint32_t grid, uint32_t smem, int max_smem,
-                                 cudaStream_t stream);
+                                 cudaStream_t stream, bool next);
 
 }  // namespace strm
 }  // namespace pfac
