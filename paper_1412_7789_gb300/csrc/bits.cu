@@ -75,18 +75,12 @@ __device__ __forceinline__ uint32_t list_bits(uint2 b, uint16_t *list, int lane)
     return total;
 }
 
-// One warp: tile t's part of the list, from index at on; p0: the text position
-// of the tile's first bit (before the text wraps).
-template <bool FULL>
-__device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32_t p0, uint2 b, unsigned long long at,
-                                         uint16_t *list, int lane) {
-    const uint32_t total = list_bits(b, list, lane);
-    const size_t g0 = static_cast<size_t>(t) * kTile;
-    // compacted: four rounds of 32 matches at a time, their ids in flight
-    // together (a tile dense in matches is one warp's work: 256 MiB of ACGT with
-    // its 4,096 matches in the first tiles 10 against 20 us; the full list's
-    // rounds wait for their chains, and took 39 against 24 us four at a time)
-    constexpr uint32_t R = FULL ? 1 : 4;
+// One warp: the `total` matches listed of the tile whose bits start at g0, from
+// index at of the list on; p0: the text position of its first bit (before the
+// text wraps).  R rounds of 32 matches at a time, their ids in flight together.
+template <uint32_t R>
+__device__ __forceinline__ void put_compact(const BitsParams &p, size_t g0, uint32_t p0, uint32_t total,
+                                            unsigned long long at, const uint16_t *list, int lane) {
     for (uint32_t k0 = 0; k0 < total; k0 += 32u * R) {
         uint32_t i[R], id[R];
 #pragma unroll
@@ -95,27 +89,53 @@ __device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32
             i[j] = k < total ? list[k] : 0u;
             id[j] = k < total ? static_cast<uint32_t>(p.ids[g0 + i[j]]) : 0u;
         }
-        if (!FULL) {
 #pragma unroll
-            for (uint32_t j = 0; j < R; ++j) {
-                const uint32_t k = k0 + 32u * j + static_cast<uint32_t>(lane);
-                if (k < total && at + k < p.out.cap) {
-                    p.out.pos[at + k] = p0 + i[j];
-                    p.out.ids[at + k] = id[j];
-                }
+        for (uint32_t j = 0; j < R; ++j) {
+            const uint32_t k = k0 + 32u * j + static_cast<uint32_t>(lane);
+            if (k < total && at + k < p.out.cap) {
+                p.out.pos[at + k] = p0 + i[j];
+                p.out.ids[at + k] = id[j];
             }
-        } else {
-            const uint32_t cl = k0 + static_cast<uint32_t>(lane) < total ? chain_len(p, id[0]) : 0u;
-            uint32_t inc = cl;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t y = __shfl_up_sync(kFull, inc, d);
-                if (lane >= d) inc += y;
-            }
-            if (k0 + static_cast<uint32_t>(lane) < total) put_chain(p, at + (inc - cl), p0 + i[0], id[0]);
-            at += __shfl_sync(kFull, inc, 31);
         }
     }
+}
+
+__device__ __forceinline__ void put_full(const BitsParams &p, size_t g0, uint32_t p0, uint32_t total,
+                                         unsigned long long at, const uint16_t *list, int lane) {
+    for (uint32_t k0 = 0; k0 < total; k0 += 32u) {
+        const uint32_t k = k0 + static_cast<uint32_t>(lane);
+        uint32_t i = 0, id = 0, cl = 0;
+        if (k < total) {
+            i = list[k];
+            id = static_cast<uint32_t>(p.ids[g0 + i]);
+            cl = chain_len(p, id);
+        }
+        uint32_t inc = cl;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (k < total) put_chain(p, at + (inc - cl), p0 + i, id);
+        at += __shfl_sync(kFull, inc, 31);
+    }
+}
+
+// One warp: tile t's part of the list.  Compacted: a tile dense in matches is
+// one warp's work, so it goes four rounds at a time (256 MiB of ACGT, its 4,096
+// matches in the first tiles: 10 against 20 us); the full list's rounds wait for
+// their chains, and took 39 against 24 us four at a time.
+template <bool FULL>
+__device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32_t p0, uint2 b, unsigned long long at,
+                                         uint16_t *list, int lane) {
+    const uint32_t total = list_bits(b, list, lane);
+    const size_t g0 = static_cast<size_t>(t) * kTile;
+    if (FULL)
+        put_full(p, g0, p0, total, at, list, lane);
+    else if (total <= 32u)
+        put_compact<1>(p, g0, p0, total, at, list, lane);
+    else
+        put_compact<4>(p, g0, p0, total, at, list, lane);
 }
 
 // The occurrences of each tile's results, one warp per tile.
