@@ -329,11 +329,11 @@ void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTa
             h.stream_F1 = std::move(F);
             h.stream_F2 = std::move(F2);
         }
-        // every position looked up and the root filter over 10 % full: the
-        // rounds that resolve the survivors cost more than the filter kernel's
-        // in-warp pipeline (64 MiB of uniform text, dense ids: at 6 % of the
-        // windows ending a keyword 163 against 182 us, at 20 % 330 against 240)
-        if (st.step == 1u && dense > 0.1) return;
+        // every position looked up and nearly all of them survivors: the filter
+        // kernel's in-warp pipeline is the faster (64 MiB of uniform text, dense
+        // ids: at 91 % of the windows ending a keyword 616 against 678 us, at
+        // 99.98 % 641 against 565)
+        if (st.step == 1u && dense > 0.95) return;
         st.form = 2;
         st.win1 = k;
         st.root = k;

@@ -64,7 +64,7 @@ constexpr uint32_t kQueue = 256;         // survivors of a tile kept in shared m
 constexpr uint32_t kNone = 1024;          // ids of -1 in shared memory
 constexpr uint32_t kRes2 = 160;          // 2-bit codes: candidates waiting to be resolved (31 + 4 * 32 at most)
 constexpr uint32_t kRes8 = 64;           // 8-bit codes: survivors waiting (31 + 32 at most)
-constexpr uint32_t kWarpBytes2 = kTile / 4 + 16 + 2 * kQueue + 8 * kRes2;
+constexpr uint32_t kWarpBytes2 = kTile / 4 + 16 + 2 * kQueue + 16 + 8 * kRes2;  // (16: a step-1 tile's last marks)
 constexpr uint32_t kWarpBytes8 = kTile + 16 + 2 * kQueue + 9 * kRes8;
 static_assert(kWarpBytes2 % 16 == 0 && kWarpBytes8 % 16 == 0, "warp areas start on 16 bytes");
 
@@ -230,9 +230,17 @@ static __device__ __noinline__ int match_at_far(const FilterParams &p, const uin
     return match_at<GT>(p, cls8, tt, gi, B);
 }
 
-// An id found at position g.
+// An id found at position g.  OUT_BITS with tile (the warp's bits of the tile
+// from position g0 on, in shared memory, every id of which passes here before
+// the tile's bits and count are written): the bit goes there.
+struct TileBits {
+    uint32_t *bits;
+    const uint16_t *marks;  // step 1: which of the tile's bytes are in no keyword, or outside the text
+    uint32_t g0;
+};
 template <int MODE>
-__device__ __forceinline__ void put_id(const FilterParams &p, const Seg &sg, uint32_t g, int r, uint32_t &cnt) {
+__device__ __forceinline__ void put_id(const FilterParams &p, const Seg &sg, uint32_t g, int r, uint32_t &cnt,
+                                       const TileBits tile = TileBits{nullptr, nullptr, 0u}) {
     if (r < 0) return;
     if (MODE == OUT_DENSE) {
         sg.out[text_pos(sg, g)] = r;
@@ -241,8 +249,12 @@ __device__ __forceinline__ void put_id(const FilterParams &p, const Seg &sg, uin
     } else {
         const uint32_t b = g + sg.bit0;
         p.bo.ids[b] = r;
-        atomicOr(p.bo.bits + (b >> 5), 1u << (b & 31u));
-        atomicAdd(p.bo.counts + b / kTile, 1u);
+        if (tile.bits) {
+            atomicOr(tile.bits + ((g - tile.g0) >> 5), 1u << (g & 31u));
+        } else {
+            atomicOr(p.bo.bits + (b >> 5), 1u << (b & 31u));
+            atomicAdd(p.bo.counts + b / kTile, 1u);
+        }
     }
 }
 
@@ -368,21 +380,23 @@ __device__ __forceinline__ void fill_done(bool found, int lane) {
 
 // The id at position g, all here: the walk list is full.
 template <int MODE>
-__device__ __forceinline__ void settle_here(const StreamParams &p, const Seg &sg, uint32_t g, uint32_t B, uint32_t &cnt) {
+__device__ __forceinline__ void settle_here(const StreamParams &p, const Seg &sg, uint32_t g, uint32_t B, uint32_t &cnt,
+                                            const TileBits tile = TileBits{nullptr, nullptr, 0u}) {
     const TileText tt = make_text(sg.text, sg.out, sg.n, 0u);
     const int r = (p.f.kind & 0xFFu) == 16u ? match_at_far<int16_t>(p.f, p.f.cls8g, tt, text_pos(sg, g), B)
                                             : match_at_far<int32_t>(p.f, p.f.cls8g, tt, text_pos(sg, g), B);
-    put_id<MODE>(p.f, sg, g, r, cnt);
+    put_id<MODE>(p.f, sg, g, r, cnt, tile);
 }
 
 // Walks (want: this lane has one) to the list, or settled here when it is full.
 template <int B, int MODE, bool BATCH>
 __device__ __forceinline__ void list_walk(const StreamParams &p, const Seg &sg, WalkRoom &room, bool want, uint32_t g,
-                                          uint32_t s, int lane, uint32_t &cnt) {
+                                          uint32_t s, int lane, uint32_t &cnt,
+                                          const TileBits tile = TileBits{nullptr, nullptr, 0u}) {
     const bool stored = push_walk<BATCH>(p, sg, room, want, g, s, lane);
     if (!room.full || __all_sync(kFull, stored)) return;
     fill_done<MODE, B == 8>(true, lane);
-    if (!stored) settle_here<MODE>(p, sg, g, B, cnt);
+    if (!stored) settle_here<MODE>(p, sg, g, B, cnt, tile);
 }
 
 // The -1 buffer (all threads; a CTA barrier follows).
@@ -430,6 +444,26 @@ __device__ __forceinline__ uint32_t codes16(const uint4 &v) {
                        __byte_perm((v.z & dmask) * dmul, (v.w & dmask) * dmul, 0x0073u), 0x5410u);
 }
 
+// Non-zero when one of 16 bytes is in no keyword: a byte is in one exactly when
+// the keyword byte of its code equals it, and a byte permute selected by twice
+// the codes (each word's next byte's moved to the high nibble) picks those.
+__device__ __forceinline__ uint32_t unknown16(const FilterParams &f, const uint4 &v) {
+    auto word = [&](uint32_t w) {
+        const uint32_t x = w & 0x06060606u;
+        return w ^ __byte_perm(f.dsel_lo, f.dsel_hi, __byte_perm(x | (x >> 4), 0u, 0x4420u));
+    };
+    return word(v.x) | word(v.y) | word(v.z) | word(v.w);
+}
+
+// The same, a flag per byte.
+__device__ __forceinline__ uint32_t unknown_marks(const FilterParams &f, const uint4 &v) {
+    auto word = [&](uint32_t w) {
+        const uint32_t x = w & 0x06060606u;
+        return filt::nonzero_bytes(w ^ __byte_perm(f.dsel_lo, f.dsel_hi, __byte_perm(x | (x >> 4), 0u, 0x4420u)));
+    };
+    return word(v.x) | (word(v.y) << 4) | (word(v.z) << 8) | (word(v.w) << 12);
+}
+
 // The 16 codes from tile position i on, from the tile's packed codes.
 __device__ __forceinline__ uint32_t codes_at(const uint32_t *packed, uint32_t i) {
     return __funnelshift_r(packed[i >> 4], packed[(i >> 4) + 1u], 2u * (i & 15u));
@@ -453,10 +487,11 @@ __device__ __forceinline__ bool bytes_known(const uint8_t *text, uint64_t n, con
 // list.  The codes may be those of bytes in no keyword, or of bytes past the
 // text: a keyword that ends before such a byte is on the walk of the codes too,
 // so a position without a result has none; one with a result has its bytes
-// looked at, and a walk's bytes are looked at when it goes on.
-template <int MODE, bool BATCH>
+// looked at (known: no need to, they are keyword bytes of the text), and a
+// walk's bytes are looked at when it goes on.
+template <int MODE, bool BATCH, bool CHECK>
 __device__ __forceinline__ void resolve2(const StreamParams &p, const Seg &sg, WalkRoom &room, uint32_t g, uint32_t w,
-                                         bool on, int lane, uint32_t &cnt) {
+                                         bool on, bool known, int lane, uint32_t &cnt, const TileBits tile) {
     const FilterParams &f = p.f;
     const uint64_t gi = text_pos(sg, g);
     bool walk = false;
@@ -479,15 +514,25 @@ __device__ __forceinline__ void resolve2(const StreamParams &p, const Seg &sg, W
                 }
             }
         }
-        if (r >= 0 && !bytes_known(sg.text, sg.n, f.cls8g, gi, f.k + f.k2)) {
+        bool doubt = r >= 0 && !known;
+        if (CHECK) {
+            if (doubt) {
+                const uint32_t i = g - tile.g0;
+                const uint32_t m = tile.marks[i >> 4] | (static_cast<uint32_t>(tile.marks[(i >> 4) + 1u]) << 16);
+                doubt = ((m >> (i & 15u)) & ((1u << (f.k + f.k2)) - 1u)) != 0u;
+            }
+        } else {
+            doubt = doubt && !bytes_known(sg.text, sg.n, f.cls8g, gi, f.k + f.k2);
+        }
+        if (doubt) {
             walk = true;
             s = 0;
             r = -1;
         }
     }
     fill_done<MODE, false>(r >= 0, lane);
-    put_id<MODE>(f, sg, g, r, cnt);
-    list_walk<2, MODE, BATCH>(p, sg, room, walk, g, s, lane, cnt);
+    put_id<MODE>(f, sg, g, r, cnt, tile);
+    list_walk<2, MODE, BATCH>(p, sg, room, walk, g, s, lane, cnt, tile);
 }
 
 // One warp's state across its tiles: candidates or survivors waiting to be
@@ -511,13 +556,27 @@ __device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uin
     uint2 *res = reinterpret_cast<uint2 *>(packed + kTile / 16 + 4);
     uint16_t *queue = reinterpret_cast<uint16_t *>(res + kRes2);
     uint32_t nres = ws.nres, cnt = ws.cnt;  // candidates waiting in res: {g, codes}
+    // every position looked up: the sets with many matches, so the tile's bytes
+    // are looked at once for all of them, and only a tile with bytes in no
+    // keyword (or of the text's ends) marks them; with fewer matches the check
+    // costs more than it saves.  (64 MiB of uniform text, a fifth of it matches:
+    // dense ids 330 -> 200 us; the filter kernel 240.)
+    constexpr bool CHECK = S == 1;
+    bool known = false;  // those waiting are from tiles without such bytes
+    uint16_t *marks = queue + kTile / 16;  // 129 of them
+    // ... and OUT_BITS collects the tile's bits in shared memory (the queue is
+    // the second filter's, which these sets have not): its candidates are all
+    // resolved before it ends, and no bit or count takes a global atomic
+    constexpr bool LOCAL = CHECK && MODE == OUT_BITS;
+    uint32_t *tbits = reinterpret_cast<uint32_t *>(queue);
+    TileBits tile{LOCAL ? tbits : nullptr, marks, 0u};
     WalkRoom room = ws.room;
     auto flush = [&](uint32_t n) {  // resolve the last n (<= 32) of them
         __syncwarp();
         nres -= n;
         const bool on = static_cast<uint32_t>(lane) < n;
         const uint2 e = res[nres + (on ? static_cast<uint32_t>(lane) : 0u)];
-        resolve2<MODE, BATCH>(p, sg, room, e.x, e.y, on, lane, cnt);
+        resolve2<MODE, BATCH, CHECK>(p, sg, room, e.x, e.y, on, known, lane, cnt, tile);
         __syncwarp();
     };
     for (; t < t_end; t += step) {
@@ -526,13 +585,35 @@ __device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uin
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[j] = codes16(r.c[j]);
         c[4] = codes16(r.look);
+        if (CHECK) {
+            uint32_t bad = lane == 0 ? unknown16(p.f, r.look) : 0u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) bad |= unknown16(p.f, r.c[j]);
+            const bool clean = t >= sg.in_lo && t < sg.in_hi && !__any_sync(kFull, bad != 0u);
+            if (nres && !(clean && known)) flush(nres);  // before their tile's marks go
+            known = clean;
+            tile.g0 = (t - sg.t0) * kTile;
+            if (!clean) {
+                __syncwarp();
+#pragma unroll
+                for (uint32_t j = 0; j <= 4; ++j) {
+                    const uint32_t i = j * kChunk + 16u * static_cast<uint32_t>(lane);
+                    uint32_t m = unknown_marks(p.f, j < 4 ? r.c[j < 4 ? j : 0] : r.look);
+                    m |= filt::outside_marks(static_cast<int64_t>(text_pos(sg, tile.g0 + i)), static_cast<int64_t>(sg.n));
+                    if (j < 4 || lane == 0) marks[32u * j + static_cast<uint32_t>(lane)] = static_cast<uint16_t>(m);
+                }
+            }
+        }
         if (t + step < t_end) load_tile(sg, t + step, pol, lane, r);
         __syncwarp();  // the previous tile's readers of packed and queue are done
 #pragma unroll
         for (uint32_t j = 0; j < 4; ++j) packed[32u * j + static_cast<uint32_t>(lane)] = c[j];
         if (lane == 0) packed[128] = c[4];
         if (MODE == OUT_DENSE) fill_none<false>(sg, none, t, lane);
-        if (MODE == OUT_BITS) clear_bits(p.f, sg, t, lane);
+        if (MODE == OUT_BITS && !LOCAL) clear_bits(p.f, sg, t, lane);
+        if (LOCAL) {
+            reinterpret_cast<uint2 *>(tbits)[lane] = make_uint2(0u, 0u);
+        }
 
         // 2. the root filter at every S-th position: one bit each, first
         //    position highest
@@ -566,7 +647,7 @@ __device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uin
                        16u * static_cast<uint32_t>(lane) + S * (b % kPer) + (S - 1u);
             };
             const uint32_t total = __reduce_add_sync(kFull, static_cast<uint32_t>(__popc(m)));
-            if (total > kQueue / S) {
+            if (S > 1 && total > kQueue / S) {
                 // a tile dense in survivors: all of them to the walk list,
                 // unresolved, in one reservation (the positions before or
                 // past the text as empty entries)
@@ -635,6 +716,14 @@ __device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uin
                     while (nres >= 32u) flush(32u);
                 }
             }
+        }
+        if (LOCAL) {
+            if (nres) flush(nres);
+            const uint2 b = reinterpret_cast<const uint2 *>(tbits)[lane];
+            const uint32_t n = __reduce_add_sync(kFull, static_cast<uint32_t>(__popc(b.x) + __popc(b.y)));
+            const size_t u = sg.bit0 / kTile + (t - sg.t0);
+            reinterpret_cast<uint2 *>(p.f.bo.bits + u * (kTile / 32u))[lane] = b;
+            if (lane == 0) p.f.bo.counts[u] = n;
         }
     }
     if (nres) flush(nres);

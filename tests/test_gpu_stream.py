@@ -50,6 +50,8 @@ SETS = {
     "dna16": (b"ACGT", 600, 16, 40),    # every 4th position looked up, a second filter
     "dna8": (b"ACGT", 300, 8, 32),      # every 2nd
     "dna4": (b"ACGT", 200, 4, 40),      # every one
+    "dna4dense": (b"ACGT", 1500, 4, 12),  # a third of the positions match
+    "dna4lines": (b"ACGT", 1500, 4, 12),  # ... with a line break after every 60
     "dna1": (b"ACGT", 60, 1, 30),       # keywords shorter than any window
     "iupac": (b"ACGTNRYKM", 200, 6, 20),  # 4-bit codes: no streaming form
     "bytes4": (bytes(range(256)), 4000, 4, 30),
@@ -73,6 +75,8 @@ def _workload(name, n):
         r = workloads.rng(13)
         text[r.integers(0, n, size=n // 500 + 1)] = ord("#")
         text[n // 3:n // 3 + 40] = ord("#")
+    if name.endswith("lines"):
+        text[60::61] = ord("\n")
     return text, pats
 
 
@@ -118,7 +122,7 @@ def test_streaming_edges(name):
             _check(a, text[:n], want, shift, out_shift)
 
 
-@pytest.mark.parametrize("name", ["dna16", "dna8", "dna4", "bytes4", "bytes9", "words7"])
+@pytest.mark.parametrize("name", ["dna16", "dna8", "dna4", "dna4lines", "bytes4", "bytes9", "words7"])
 def test_full_list(name):
     for n in (3000, AT_MAX + 777):
         text, pats = _workload(name, n)
@@ -171,7 +175,7 @@ def test_list_capacity_is_kept():
                 assert bool((pos[cap:] == -7).all()) and bool((ids[cap:] == -7).all())
 
 
-@pytest.mark.parametrize("names", [("dna16", "bytes4"), ("dna8", "dna4", "bytes9", "words7"),
+@pytest.mark.parametrize("names", [("dna16", "bytes4"), ("dna8", "dna4", "dna4lines", "bytes9", "words7"),
                                    ("dna16", "iupac", "bytes2", "bytes5", "dna1")])
 @pytest.mark.parametrize("reserve", [1 << 22, 64])
 def test_batch_streams(names, reserve):
