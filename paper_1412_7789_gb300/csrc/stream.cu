@@ -221,6 +221,7 @@ cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mod
     p.f1bytes = (1u << kFilterBits) / 8u;
     p.F2 = t.stream_F2;
     p.f2bytes = t.stream_F2 ? t.stream_f2bytes : 0u;
+    p.four = 4u;
     p.m1 = t.stream.m1;
     p.m2 = t.stream.m2;
     p.l2shift = t.stream.form == 2 ? 32u - 2u * t.stream.win2 : 0u;

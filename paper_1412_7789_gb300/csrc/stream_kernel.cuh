@@ -129,6 +129,7 @@ struct StreamParams {
     uint32_t f1bytes, f2bytes;
     uint32_t ntiles;
     Seg sg;                // one text
+    uint32_t four;         // 4
     uint32_t m1, m2;       // 8-bit codes: multipliers of the window's words
     uint32_t l2shift;      // 2-bit codes: left shift that drops the codes past the second filter's window
     uint32_t off_none, off_warp;
@@ -797,6 +798,10 @@ __device__ __forceinline__ void tiles8(const StreamParams &p, uint8_t *smem, uin
     uint16_t *queue = reinterpret_cast<uint16_t *>(res_w + kRes8);
     uint8_t *res_c = reinterpret_cast<uint8_t *>(queue + kQueue);
     uint32_t nres = ws.nres, cnt = ws.cnt;  // survivors waiting in res_*
+    // the address is one multiply-add (p.four, which the compiler does not know
+    // to be 4), not a shift, a mask and an add on the pipe that bounds the loop:
+    // 1 GiB counted 920 -> 899 us
+    const uint32_t f1_at = smem_addr(F1);
     WalkRoom room = ws.room;
     auto flush = [&](uint32_t n) {  // resolve the last n (<= 32) of them
         __syncwarp();
@@ -837,7 +842,9 @@ __device__ __forceinline__ void tiles8(const StreamParams &p, uint8_t *smem, uin
                 // word: the top bits of the 32-bit hash; bit: the first word's
                 // product past 32 bits (well mixed, and no shift to get it)
                 const uint64_t h = static_cast<uint64_t>(win[x]) * p.m1;
-                const uint32_t word = F1[(static_cast<uint32_t>(h) + win[x + 4] * p.m2) >> 17];
+                const uint32_t idx = (static_cast<uint32_t>(h) + win[x + 4] * p.m2) >> 17;
+                uint32_t word;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(word) : "r"(idx * p.four + f1_at));
                 const uint32_t b = static_cast<uint32_t>(h >> 32);
                 a = __funnelshift_l(__funnelshift_l(word, word, b), a, 1);
             }
@@ -1053,11 +1060,11 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
         if (!go) continue;
         // warps on this automaton, about
         const uint32_t share = static_cast<uint32_t>(static_cast<uint64_t>(gridDim.x) * (blockDim.x / 32u) * wk.units / total) + 1u;
-        // blocks of two units, one towards the end (bigger ones leave the last
-        // warps too much, and scatter the traffic: 64 units at first took 810
-        // us for 1,024 texts of the benchmark batch against 725); the next block is
-        // claimed while this one is matched
-        auto block = [&](uint32_t seen) { return seen < wk.units && wk.units - seen > 8u * share ? 2u : 1u; };
+        // blocks of four units, one towards the end (1 / 2 / 4 / 6 units: 1,024
+        // texts of the benchmark batch in 625 / 578 / 573 / 575 us; shares of what
+        // is left, up to 64, scatter the traffic over the whole buffer); the next
+        // block is claimed while this one is matched
+        auto block = [&](uint32_t seen) { return seen < wk.units && wk.units - seen > 8u * share ? 4u : 1u; };
         const uint32_t sample = sample_items(wk, lane);
         uint32_t blk = block(0u), ahead = 0;
         if (lane == 0) ahead = atomicAdd(p.f.counter, blk);
