@@ -264,14 +264,23 @@ namespace {
 
 using pfac::scratch_pool;
 
-// The streaming form of one long text, its walk list from the pool.
-cudaError_t run_stream(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st) {
+// `bytes` of device memory from the pool, in stream order.  Out of memory
+// leaves no error behind: the caller may have a form that takes less.
+cudaError_t pool_alloc(ac_automaton *h, size_t bytes, cudaStream_t st, void **out) {
     cudaMemPool_t pool = nullptr;
     cudaError_t e = scratch_pool(h->device, &pool);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(out, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
+// The streaming form of one long text, its walk list from the pool.  *room
+// = false: no memory for the list, and nothing was enqueued.
+cudaError_t run_stream(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st, bool *room) {
     r.walk_cap = pfac::stream_walk_cap(r.n);
     void *scratch = nullptr;
-    e = cudaMallocFromPoolAsync(&scratch, pfac::stream_bytes(r.walk_cap), pool, st);
+    cudaError_t e = pool_alloc(h, pfac::stream_bytes(r.walk_cap), st, &scratch);
+    *room = e != cudaErrorMemoryAllocation;
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(scratch, 0, 32, st);
     if (e == cudaSuccess) {
@@ -290,7 +299,11 @@ cudaError_t run_stream(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode
 // clearing of small calls.
 cudaError_t run_tiled(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st) {
     if (!r.batch && pfac::at_serves(h->dev, h->tuning, r.n)) return pfac::launch_at(h->dev, r, mode, st);
-    if (!r.batch && pfac::stream_serves(h->dev, h->tuning, r.n)) return run_stream(h, r, mode, st);
+    if (!r.batch && pfac::stream_serves(h->dev, h->tuning, r.n)) {
+        bool room = true;
+        const cudaError_t e = run_stream(h, r, mode, st, &room);
+        if (room) return e;  // else the filter kernel, which takes 16 bytes for small alphabets
+    }
     // 8-bit codes, long text: the phased form's lists after the counter
     pfac::SurvivorLists sl;
     if (!r.batch && pfac::uses_filter(h->dev, h->tuning)) sl = pfac::survivor_lists(h->dev, h->tuning, r.n);
@@ -321,15 +334,13 @@ cudaError_t run_tiled(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode,
 }
 
 // The compacted or full list of one text through the bit-per-position output,
-// its scratch from the pool.
+// its scratch from the pool.  *room as above.
 cudaError_t run_bits(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out, bool full,
-                     cudaStream_t st) {
+                     cudaStream_t st, bool *room) {
     const size_t bytes = pfac::bits_scratch_bytes(h->dev, h->tuning, text, n, full);
-    cudaMemPool_t pool = nullptr;
-    cudaError_t e = scratch_pool(h->device, &pool);
-    if (e != cudaSuccess) return e;
     void *scratch = nullptr;
-    e = cudaMallocFromPoolAsync(&scratch, bytes, pool, st);
+    cudaError_t e = pool_alloc(h, bytes, st, &scratch);
+    *room = e != cudaErrorMemoryAllocation;
     if (e != cudaSuccess) return e;
     e = pfac::enqueue_bits(h->dev, h->tuning, text, n, out, full, scratch, bytes, st);
     const cudaError_t e2 = cudaFreeAsync(scratch, st);
@@ -339,7 +350,11 @@ cudaError_t run_bits(ac_automaton *h, const uint8_t *text, uint64_t n, const pfa
 // The compacted match of one text with its scratch from the pool.
 cudaError_t run_compact(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out,
                         cudaStream_t st) {
-    if (pfac::bits_serve(h->dev, h->tuning, n)) return run_bits(h, text, n, out, false, st);
+    if (pfac::bits_serve(h->dev, h->tuning, n)) {
+        bool room = true;
+        const cudaError_t e = run_bits(h, text, n, out, false, st, &room);
+        if (room) return e;  // else by slots, which take less
+    }
     const uint32_t units = pfac::compact_units(h->dev, h->tuning, text, n);
     if (units == 0xFFFFFFFFu) return cudaErrorInvalidValue;
     // the phased form's lists instead of the dense fallback when it applies
@@ -362,7 +377,11 @@ cudaError_t run_compact(ac_automaton *h, const uint8_t *text, uint64_t n, const 
 // The full output of one text with its scratch from the pool.
 cudaError_t run_full(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out,
                      cudaStream_t st) {
-    if (pfac::bits_serve(h->dev, h->tuning, n)) return run_bits(h, text, n, out, true, st);
+    if (pfac::bits_serve(h->dev, h->tuning, n)) {
+        bool room = true;
+        const cudaError_t e = run_bits(h, text, n, out, true, st, &room);
+        if (room) return e;  // else by slots, which take less
+    }
     const uint32_t units = pfac::compact_units(h->dev, h->tuning, text, n);
     if (units == 0xFFFFFFFFu) return cudaErrorInvalidValue;
     const size_t bytes = pfac::full_scratch_bytes(h->dev, h->tuning, units, n);
@@ -1001,6 +1020,12 @@ ac_status ac_batch_reserve_lists(ac_batch b, uint64_t text_bytes) {
         const uint32_t wc = pfac::stream_batch_cap(text_bytes);
         e = cudaMalloc(&b->walks, pfac::stream_batch_bytes(wc));
         if (e == cudaSuccess) b->walk_cap = wc;
+        // no room for both lists: the filter kernel's serve every automaton
+        if (e == cudaErrorMemoryAllocation && b->lists) {
+            cudaGetLastError();
+            b->walks = nullptr;
+            e = cudaSuccess;
+        }
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -118,6 +118,11 @@ uint64_t units_of(const ac_server_impl *s, const ac_server_request &r) {
     return (r.n + text_head(r) + T - 1) / T;
 }
 
+// Work units of a request's text in the streaming form.
+uint64_t stream_units(const ac_server_request &r) {
+    return (r.n + text_head(r) + pfac::kStreamTile - 1) / pfac::kStreamTile;
+}
+
 // Whether automaton a's texts may take survivor lists for the phased form:
 // 8-bit codes in one-launch waves, or (FIFO) as ac_match_compact takes them.
 // (Small alphabets keep their dense fallback: the sets whose windows often
@@ -131,20 +136,19 @@ bool wave_lists(const ac_server_impl *s, uint32_t a) { return (s->multi || s->fi
 constexpr uint64_t kStreamWave = 4ull << 20;
 bool wave_streams(const ac_server_impl *s, uint64_t bytes) { return s->multi && bytes >= kStreamWave; }
 
-// Device bytes a request holds while admitted: its text (a host text's device
-// copy), its output and the scratch of its tiles (counts, prefix, slots,
-// dense fallback), and with 8-bit codes in one-launch waves its share of the
-// wave's survivor lists (about 4 bytes per text byte).
-uint64_t request_bytes(const ac_server_impl *s, const ac_server_request &r) {
+// Scratch a request is charged for: its tiles' (counts, prefix, slots, dense
+// fallback), and with 8-bit codes in one-launch waves its share of the wave's
+// survivor lists (about 4 bytes per text byte).
+uint64_t request_scratch(const ac_server_impl *s, const ac_server_request &r) {
     const uint64_t per_unit = 4 + 8 + 8ull * pfac::kSlotCap + 4ull * pfac::kDenseStride;
     const uint64_t lists = wave_lists(s, r.automaton) ? 32ull * (r.n / 8) + 32 : 0;
-    const uint64_t own = units_of(s, r) * per_unit + lists;
-    // the streaming form, should the wave take it: count, prefix, bits and ids
-    // of each unit, 16 bytes of walk list for every eighth text byte
-    const uint64_t units = (r.n + text_head(r) + pfac::kStreamTile - 1) / pfac::kStreamTile;
-    const uint64_t other = s->streams[r.automaton] ? units * (4 + 8 + pfac::kStreamTile / 8 + 4ull * pfac::kStreamTile) + 16ull * (r.n / 8)
-                                                   : 0;
-    return r.n + 8ull * r.cap + std::max(own, other) + 64;
+    return units_of(s, r) * per_unit + lists;
+}
+
+// Device bytes a request holds while admitted: its text (a host text's device
+// copy), its output and its scratch.
+uint64_t request_bytes(const ac_server_impl *s, const ac_server_request &r) {
+    return r.n + 8ull * r.cap + request_scratch(s, r) + 64;
 }
 
 // Device scratch of a wave: from the caller's allocator (freed when the wave
@@ -246,14 +250,29 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     std::vector<uint32_t> ubase(nh, 0);
     std::vector<pfac::BatchItemDev> list(L);
     std::vector<pfac::CompactOut> outs(R);
-    // the automata the streaming form takes in this wave
-    uint64_t wave_text = 0;
-    for (uint32_t k = 0; k < L; ++k) wave_text += w.reqs[order[k]].r.n;
-    auto streamed = [&](uint32_t a) { return s->streams[a] && wave_streams(s, wave_text); };
+    // The automata the streaming form serves take it when the wave's text is
+    // long enough, its positions can be numbered in 32 bits, and its scratch
+    // (count, prefix, bits and ids of each unit, 16 bytes per listed walk) stays
+    // within what the requests were charged: the walk list takes the rest,
+    // for every eighth text byte at most and every 64th at least (a full list
+    // only costs time: the walks past it end where they were found).
+    uint64_t wave_text = 0, stream_bytes = 0, charged = 0, needed = 0;
+    for (uint32_t k = 0; k < L; ++k) {
+        const ac_server_request &r = w.reqs[order[k]].r;
+        wave_text += r.n;
+        if (!s->streams[r.automaton]) continue;
+        stream_bytes += r.n;
+        charged += request_scratch(s, r);
+        needed += stream_units(r) * (4 + 8 + pfac::kStreamTile / 8 + 4ull * pfac::kStreamTile);
+    }
+    const uint64_t walk_room = charged > needed ? (charged - needed) / 16 : 0;
+    const bool streams = wave_streams(s, wave_text) && walk_room >= stream_bytes / 64 &&
+                         stream_bytes / pfac::kStreamTile + 2ull * L < (1ull << 32) / pfac::kStreamTile;
+    auto streamed = [&](uint32_t a) { return streams && s->streams[a]; };
     // units: the other automata's first (with slots), then the streamed ones'
     // (with bits); the counts and their prefix are one array over both
     std::vector<pfac::BitsText> btexts;
-    uint64_t U = 0, Uo = 0, stream_text = 0;
+    uint64_t U = 0, Uo = 0;
     {
         uint32_t j = 0;
         for (uint32_t a = 0; a < nh; ++a) {
@@ -280,7 +299,7 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
                     units += units_of(s, r);
                     continue;
                 }
-                const uint64_t n = (r.n + text_head(r) + pfac::kStreamTile - 1) / pfac::kStreamTile;
+                const uint64_t n = stream_units(r);
                 pfac::BitsText x{};
                 x.out = pfac::CompactOut{r.d_pos, r.d_ids, r.cap, reinterpret_cast<unsigned long long *>(r.d_count)};
                 x.first = static_cast<uint32_t>(ubase[a] + units);
@@ -288,15 +307,13 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
                 x.head = static_cast<uint32_t>(text_head(r));
                 btexts.push_back(x);
                 units += n;
-                stream_text += r.n;
             }
             heads[a].units = static_cast<uint32_t>(units);
             U += units;
         }
     }
     const uint64_t Us = U - Uo;
-    // (positions of the streamed units are numbered in 32 bits)
-    if (U >= 0xFFFFFFFFull || Us >= (1ull << 32) / pfac::kStreamTile) return cudaErrorInvalidValue;
+    if (U >= 0xFFFFFFFFull) return cudaErrorInvalidValue;
     for (uint32_t i = 0; i < R; ++i) {
         const ac_server_request &r = w.reqs[i].r;
         outs[i] = pfac::CompactOut{r.d_pos, r.d_ids, r.cap, reinterpret_cast<unsigned long long *>(r.d_count)};
@@ -325,7 +342,7 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     const size_t cb = round256(16ull * nh), nb = round256(4 * U), pb = 8 * U, sb = 8ull * pfac::kSlotCap * Uo;
     const size_t db = round256(plan_bytes + cb + nb + pb + sb + 8ull * pfac::kScanCtas);  // dense fallback: aligned
     const size_t stb = round256(db + 4ull * pfac::kDenseStride * Uo);
-    const uint32_t walk_cap = Us ? pfac::stream_batch_cap(stream_text) : 0u;
+    const uint32_t walk_cap = Us ? pfac::stream_batch_cap(std::min(stream_bytes, 8 * walk_room)) : 0u;
     const size_t bb = round256(Us * (pfac::kStreamTile / 8)), wb = Us ? round256(pfac::stream_batch_bytes(walk_cap)) : 0,
                  ib = 4ull * pfac::kStreamTile * Us;
     const size_t bits_at = stb + round256(staged) + lsb;

@@ -180,7 +180,6 @@ bool untuned(const Tuning &tu) {
 }  // namespace
 
 bool at_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
-
     return untuned(tu) && n <= kAtMax && (t.filter || (t.hashed && t.HK));
 }
 

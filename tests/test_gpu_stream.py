@@ -219,3 +219,127 @@ def test_batch_streams(names, reserve):
     finally:
         for a in autos:
             a.close()
+
+
+def _tables(autos):
+    return sum(a.info()["table_bytes"] for a in autos)
+
+
+def test_request_charge_is_kept():
+    """What a request is charged does not depend on the form its wave takes:
+    text, output and the slot form's scratch per tile of 992 positions.  A
+    budget of exactly that serves it, one byte less refuses it."""
+    import torch
+
+    n, cap = (6 << 20) + 1, 4096
+    text, pats = _workload("dna16", n)
+    wpos, wids = oracle.compact(oracle.pfac_ids(pats, text))
+    assert wpos.size <= cap
+    d = torch.from_numpy(text).cuda()
+    pos = torch.full((cap,), -7, dtype=torch.int32, device="cuda")
+    ids = torch.full((cap,), -7, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    req = np.zeros(1, dtype=api.SERVER_REQUEST)
+    for f, v in (("d_text", d.data_ptr()), ("n", n), ("d_pos", pos.data_ptr()), ("d_ids", ids.data_ptr()),
+                 ("cap", cap), ("d_count", cnt.data_ptr())):
+        req[f] = v
+    charge = n + 8 * cap + -(-n // 992) * (4 + 8 + 8 * 32 + 4 * 1024) + 64
+    with api.Automaton(pats) as a:
+        with api.Server([a.handle], hbm_budget=_tables([a]) + charge - 1) as srv:
+            with pytest.raises(api.AcError) as e:
+                srv.submit(req)
+            assert e.value.status == api.AC_ERR_BUDGET
+        with api.Server([a.handle], hbm_budget=_tables([a]) + charge) as srv:
+            srv.submit(req)
+            srv.drain()
+            assert srv.poll(4)["status"].tolist() == [api.AC_OK]
+    m = int(cnt.item())
+    assert m == wpos.size
+    assert np.array_equal(pos[:m].cpu().numpy(), wpos) and np.array_equal(ids[:m].cpu().numpy(), wids)
+
+
+def test_wave_past_32_bits_of_text():
+    """Waves that hold more text than 32 bits can number: every request is
+    served, each as ac_match_compact alone."""
+    import torch
+
+    n, cap, k = 1 << 30, 1 << 16, 8
+    letters = torch.tensor(list(b"ACGT"), dtype=torch.uint8, device="cuda")
+    torch.manual_seed(5)
+    d = letters[torch.randint(0, 4, (n,), dtype=torch.uint8, device="cuda").int()]
+    _, pats = _workload("dna16", 100_000)
+    pats = pats + [bytes(d[x:x + 20].cpu().numpy()) for x in range(0, n - 64, n // 40)]
+    new = lambda: (torch.full((cap,), -7, dtype=torch.int32, device="cuda"),
+                   torch.full((cap,), -7, dtype=torch.int32, device="cuda"),
+                   torch.zeros(1, dtype=torch.int64, device="cuda"))
+    with api.Automaton(pats) as a:
+        wpos, wids, wcnt = new()
+        api.ac_match_compact(a.handle, d, n, wpos, wids, cap, wcnt)
+        assert 0 < int(wcnt.item()) <= cap
+        bufs = [new() for _ in range(k)]
+        torch.cuda.synchronize()
+        with api.Server([a.handle], hbm_budget=64 << 30, waves_in_flight=1) as srv:
+            for pos, ids, cnt in bufs:
+                req = np.zeros(1, dtype=api.SERVER_REQUEST)
+                for f, v in (("d_text", d.data_ptr()), ("n", n), ("d_pos", pos.data_ptr()),
+                             ("d_ids", ids.data_ptr()), ("cap", cap), ("d_count", cnt.data_ptr())):
+                    req[f] = v
+                srv.submit(req)
+            srv.drain()
+            assert srv.poll(2 * k)["status"].tolist() == [api.AC_OK] * k
+        for pos, ids, cnt in bufs:
+            assert int(cnt.item()) == int(wcnt.item())
+            assert bool((pos == wpos).all()) and bool((ids == wids).all())
+
+
+_NO_ROOM = """
+import sys
+import numpy as np
+import torch
+from paper_1412_7789_gb300 import api, workloads
+kind, free_mib = sys.argv[1], int(sys.argv[2])
+n = 128 << 20
+text = np.frombuffer(b"ACGT", dtype=np.uint8)[workloads.rng(9).integers(0, 4, size=n)]
+pats = [bytes(text[x:x + 20]) for x in range(1000, n - 64, n // 300)]
+t = torch.from_numpy(text).cuda()
+out = torch.full((n if kind == "dense" else 4096,), -7, dtype=torch.int32, device="cuda")
+ids = torch.full((4096,), -7, dtype=torch.int32, device="cuda")
+cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+def call(a, m):
+    if kind == "dense":
+        api.ac_match(a.handle, t, m, out)
+    else:
+        api.ac_match_compact(a.handle, t, m, out, ids, 4096, cnt)
+    torch.cuda.synchronize()
+with api.Automaton(pats) as a, api.Automaton(pats) as b:
+    b.set_tuning(block=256)  # the filter kernel: its code is loaded before the memory goes
+    call(b, 1 << 20)
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - (free_mib << 20), dtype=torch.uint8, device="cuda")
+    call(a, n)
+    del hold
+if kind == "dense":
+    pos = torch.nonzero(out >= 0).flatten()
+    assert int((out < -1).sum()) == 0
+    val = out[pos]
+else:
+    pos, val = out[:int(cnt.item())], ids[:int(cnt.item())]
+at = list(range(1000, n - 64, n // 300))
+assert pos.tolist() == at and val.tolist() == list(range(len(pats)))
+assert api.ac_device_status() == api.AC_OK
+"""
+
+
+@pytest.mark.parametrize("kind,free_mib", [("dense", 40), ("compact", 600)])
+def test_no_room_for_the_streaming_scratch(kind, free_mib):
+    """Where the device has no room for the walk list (about a byte per text
+    byte) or the bits and ids (5.2 bytes), the call takes the form that needs
+    less (16 bytes; 4.4 per text byte) and still succeeds."""
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _NO_ROOM, kind, str(free_mib)], cwd=root, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
