@@ -32,20 +32,37 @@ METRIC = "GB/s text scanned (1 GB300) & % HBM roofline; batch/serve p50/p99 vs p
 GIB = 1 << 30
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal
 
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from an
-# ncu capture of the kernel as it stands, keyed by (workload, text bytes,
-# kernel): a capture of a 256 MiB launch of the same workload and launch
-# form, scaled by 4 to the 1 GiB launch (the traffic grows with the positions;
-# the 256 MiB capture read 343.8 MB and wrote 1020.3 MB).  Drop an entry
-# whenever its kernel changes.
+# DRAM bytes per step (dram__bytes_read.sum + dram__bytes_write.sum) from an
+# ncu capture of the kernels as they stand, keyed by (workload, text bytes,
+# kernels): a capture of a 256 MiB launch of the same workload and launch
+# form, scaled by 4 to the 1 GiB launch (the traffic grows with the
+# positions).  Drop an entry whenever its kernel changes.
 KNOWN_TRAFFIC: dict = {
-    ("sweep", GIB, "pfac_filter_pipe"): 4 * (343.750144e6 + 1020.311e6),
+    ("sweep", GIB, "pfac_stream2+pfac_stream_walks"): 4 * (304.62e6 + 1020e6 + 3.78e6),
 }
 
+AT_MAX = 2 << 20  # longest text of the short-text form
 
-def kernel_name(info: dict, out_kind: str, kernel: str, phased: bool = False) -> str:
+
+def streamed(info: dict, tun: dict) -> bool:
+    """Whether long texts take the streaming form: the tuning as built, and DNA
+    codes with a root window of 10 or bytes with keywords of at least 4 (not
+    modelled: a root filter more than 95 % full)."""
+    as_built = not any(tun[k] for k in ("block", "stages", "survivor_list")) and tun["per_thread"] != 4 \
+        and tun["halo"] <= 16
+    served = (info["code_bits"] == 2 and info["class_direct_shift"] == 1 and info["jump_depth"] == 10) or \
+        (info["code_bits"] == 8 and info["min_len"] >= 4)
+    return as_built and served
+
+
+def kernel_name(info: dict, out_kind: str, kernel: str, tun: dict, n: int, phased: bool = False) -> str:
     if kernel == "simple":
         return "pfac_simple"
+    lists = {"compact": "+compact", "full": "+full"}.get(out_kind, "")
+    if kernel == "tiled" and streamed(info, tun):
+        # the lists: the matcher with a bit per position, then scan and gather
+        name = "pfac_at" if n <= AT_MAX else "pfac_stream%d+pfac_stream_walks" % info["code_bits"]
+        return name + lists
     if info["code_bits"] <= 4 or kernel == "tiled":
         name = "pfac_filter_pipe"  # 8-bit codes: its hashed-filter form
         if phased:  # long texts: the survivor and walk steps of the phased form after it
@@ -54,7 +71,7 @@ def kernel_name(info: dict, out_kind: str, kernel: str, phased: bool = False) ->
         name = {"thread_jump": "pfac_jump8", "walk_slots": "pfac_walk8"}.get(kernel, "pfac_jump8g")
     # the compacted list: the matcher in slot mode, then scan and gather; the
     # full output: the matcher in slot mode, occurrence counts, scan, expansion
-    return name + {"compact": "+compact", "full": "+full"}.get(out_kind, "")
+    return name + lists
 
 
 def load_peaks():
@@ -291,16 +308,19 @@ def replica_gbs(bytes_per_rank: float, steps: int, world: int, t_ms: float) -> f
 # our arm
 # ----------------------------------------------------------------------------
 def matching_launches(a, n: int, kernel: str, out_kind: str) -> int:
-    """Kernels one matching call launches before any compaction: the filter
-    kernel, plus the survivor and walk steps of its phased form (single texts
-    with dense, count or compacted output: 8-bit codes from 4 MiB on unless
-    the tuning says never; 2- and 4-bit codes when the tuning asks for it or,
-    by default for dense ids and counts, when 500 per million or more of their
-    root windows end a keyword, beyond the texts whose heavy tiles are shared
-    within the CTA)."""
+    """Kernels one matching call launches before any compaction: one for texts
+    of the short-text form, two for the streaming form (the matcher and the
+    listed walks); else the filter kernel, plus the survivor and walk steps of
+    its phased form (single texts with dense, count or compacted output: 8-bit
+    codes from 4 MiB on unless the tuning says never; 2- and 4-bit codes when
+    the tuning asks for it or, by default for dense ids and counts, when 500 per
+    million or more of their root windows end a keyword, beyond the texts whose
+    heavy tiles are shared within the CTA)."""
     import torch
 
     info, tun = a.info(), a.tuning()
+    if kernel == "tiled" and streamed(info, tun):
+        return 1 if n <= AT_MAX else 2
     if kernel != "tiled" or out_kind not in ("dense", "count", "compact") or tun["filter_bytes"] == 0:
         return 1
     if n // 992 >= (1 << 22) - 1 or tun["survivor_list"] == 2:
@@ -429,14 +449,14 @@ def run_ours(args, rank: int, world: int, local_rank: int):
         legs["overlap_bound_ms"] = max(legs["h2d_ms"], legs["d2h_ms"], legs["kernel_ms"])
         e2e = {"value": replica_gbs(n, 1, world, 1e3 * e2e_s), "unit": "GB/s", "h2d_bytes_per_step": n,
                "d2h_bytes_per_step": 4 * n, "ms_per_step": 1e3 * e2e_s, "legs": legs,
-               "api": "ac_match_host (pinned host text in, ids out, 64 MiB chunks on three streams)"}
+               "api": "ac_match_host (pinned host text in, ids out, chunks of up to 64 MiB on three streams)"}
         del ht, ho
 
     peak, peak_kind = load_peaks()
     launch_ms = statistics.mean(per)
     achieved = algo_bytes / (launch_ms * 1e-3) / 1e9
     value = replica_gbs(n, args.steps, world, t_ms)
-    kname = kernel_name(info, out_kind, args.kernel, matching_launches(a, n, args.kernel, out_kind) > 1)
+    kname = kernel_name(info, out_kind, args.kernel, a.tuning(), n, matching_launches(a, n, args.kernel, out_kind) > 1)
     traffic = args.traffic
     if traffic is None:
         # the captured launch form: the default tuning only
@@ -530,7 +550,7 @@ def zipf_summary(steps: int, warmup: int) -> dict:
             "value": n / (ms * 1e-3) / 1e9, "unit": "GB/s", "ms_per_step": ms, "steps": steps, "matches": matches,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "peak_kind": peak_kind,
                          "frac": achieved / peak, "algorithmic_bytes_per_step": n + 8 * matches},
-            "kernels": "pfac_filter_pipe (hashed filter, survivors listed) + pfac_survivors + pfac_walks + scan + gather"}
+            "kernels": "pfac_stream8 (hashed filter) + pfac_stream_walks + scan + gather"}
 
 
 def extra_figures(args) -> dict:
