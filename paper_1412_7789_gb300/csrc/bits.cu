@@ -121,37 +121,127 @@ __device__ __forceinline__ void put_full(const BitsParams &p, size_t g0, uint32_
     }
 }
 
+// One warp: the occurrences of the `total` results listed of the tile whose bits
+// start at g0, four rounds of 32 in flight.
+__device__ __forceinline__ uint32_t sum_chains(const BitsParams &p, size_t g0, uint32_t total, const uint16_t *list,
+                                               int lane) {
+    uint32_t sum = 0;
+    for (uint32_t k0 = static_cast<uint32_t>(lane); k0 < total; k0 += 128u) {
+        uint32_t id[4];
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j) id[j] = k0 + 32u * j < total ? static_cast<uint32_t>(p.ids[g0 + list[k0 + 32u * j]]) : 0u;
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j)
+            if (k0 + 32u * j < total) sum += chain_len(p, id[j]);
+    }
+    return __reduce_add_sync(kFull, sum);
+}
+
+// Full output: a tile with more than kDense matches is left to the whole CTA,
+// each warp an eighth of its positions: one warp waits 64 rounds for the chains
+// of a tile where every position matches (16 MiB of ACGT, two such tiles: 200 ->
+// 115 us a call; 1 GiB 579 -> 412 with the empty tiles not read).  A CTA notes up to kNoted of them;
+// its warps do the others themselves.
+constexpr uint32_t kDense = 256, kNoted = 64;
+constexpr uint32_t kSlice = kTile / kWarps;
+static_assert(kSlice == 256, "eight positions a lane");
+struct DenseTiles {
+    uint32_t n;
+    uint32_t tile[kNoted];
+    unsigned long long at[kNoted];
+    uint32_t sum[kWarps];
+};
+__device__ __forceinline__ bool note_tile(DenseTiles &d, uint32_t t, unsigned long long at, uint32_t total, int lane) {
+    if (total <= kDense) return false;
+    uint32_t i = 0;
+    if (lane == 0) {
+        i = atomicAdd(&d.n, 1u);
+        if (i < kNoted) {
+            d.tile[i] = t;
+            d.at[i] = at;
+        }
+    }
+    return __shfl_sync(kFull, i, 0) < kNoted;
+}
+__device__ __forceinline__ uint32_t list_slice(const BitsParams &p, uint32_t t, uint32_t warp, uint16_t *list, int lane) {
+    const uint32_t w = t * kWords + warp * (kSlice / 32u) + static_cast<uint32_t>(lane) / 4u;
+    const uint32_t b = w < p.words ? (p.bits[w] >> (8u * (lane & 3))) & 0xFFu : 0u;
+    const uint32_t c = static_cast<uint32_t>(__popc(b));
+    uint32_t inc = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, inc, d);
+        if (lane >= d) inc += y;
+    }
+    uint32_t o = inc - c;
+    __syncwarp();
+    for (uint32_t m = b; m; m &= m - 1u)
+        list[o++] = static_cast<uint16_t>(warp * kSlice + 8u * lane + static_cast<uint32_t>(__ffs(m) - 1));
+    __syncwarp();
+    return __shfl_sync(kFull, inc, 31);
+}
+// The whole CTA: the occurrences of the tiles noted (WRITE: their lists).
+template <bool WRITE>
+__device__ __forceinline__ void noted_tiles(const BitsParams &p, DenseTiles &d, uint16_t *list, int lane, int warp) {
+    __syncthreads();
+    const uint32_t n = d.n < kNoted ? d.n : kNoted;
+    for (uint32_t i = 0; i < n; ++i) {
+        const uint32_t t = d.tile[i];
+        const size_t g0 = static_cast<size_t>(t) * kTile;
+        const uint32_t total = list_slice(p, t, static_cast<uint32_t>(warp), list, lane);
+        const uint32_t sum = sum_chains(p, g0, total, list, lane);
+        if (lane == 0) d.sum[warp] = sum;
+        __syncthreads();
+        unsigned long long before = 0;
+        for (uint32_t w = 0; w < (WRITE ? static_cast<uint32_t>(warp) : kWarps); ++w) before += d.sum[w];
+        if (WRITE)
+            put_full(p, g0, t * kTile - p.head, total, d.at[i] + before, list, lane);
+        else if (threadIdx.x == 0)
+            p.fcounts[t] = static_cast<uint32_t>(before);
+        __syncthreads();
+    }
+}
+
 // One warp: tile t's part of the list.  Compacted: a tile dense in matches is
 // one warp's work, so it goes four rounds at a time (256 MiB of ACGT, its 4,096
-// matches in the first tiles: 10 against 20 us); the full list's rounds wait for
-// their chains, and took 39 against 24 us four at a time.
+// matches in the first tiles: 10 against 20 us).
 template <bool FULL>
 __device__ __forceinline__ void put_tile(const BitsParams &p, uint32_t t, uint32_t p0, uint2 b, unsigned long long at,
-                                         uint16_t *list, int lane) {
+                                         uint16_t *list, int lane, DenseTiles *noted = nullptr) {
     const uint32_t total = list_bits(b, list, lane);
     const size_t g0 = static_cast<size_t>(t) * kTile;
-    if (FULL)
-        put_full(p, g0, p0, total, at, list, lane);
-    else if (total <= 32u)
+    if (FULL) {
+        if (!note_tile(*noted, t, at, total, lane)) put_full(p, g0, p0, total, at, list, lane);
+    } else if (total <= 32u)
         put_compact<1>(p, g0, p0, total, at, list, lane);
     else
         put_compact<4>(p, g0, p0, total, at, list, lane);
 }
 
-// The occurrences of each tile's results, one warp per tile.
+// The occurrences of each tile's results, one warp per tile; tiles that hold no
+// match by their counts (short texts have none) are not read.
 __global__ void __launch_bounds__(kThreads) full_bits_count(const BitsParams p) {
     allow_next();
     wait_previous();
     __shared__ uint16_t lists[kWarps][kTile];
+    __shared__ DenseTiles noted;
+    if (threadIdx.x == 0) noted.n = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t t = blockIdx.x * kWarps + static_cast<uint32_t>(warp); t < p.ntiles; t += gridDim.x * kWarps) {
-        const uint32_t total = list_bits(tile_bits(p, t, lane), lists[warp], lane);
-        uint32_t sum = 0;
-        for (uint32_t k = static_cast<uint32_t>(lane); k < total; k += 32u)
-            sum += chain_len(p, static_cast<uint32_t>(p.ids[static_cast<size_t>(t) * kTile + lists[warp][k]]));
-        sum = __reduce_add_sync(kFull, sum);
-        if (lane == 0) p.fcounts[t] = sum;
+    const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
+    for (uint64_t u0 = gw; u0 < p.ntiles; u0 += 32ull * nw) {
+        const uint64_t u = u0 + static_cast<uint64_t>(lane) * nw;
+        const bool some = u < p.ntiles && (!p.counts || p.counts[u] != 0u);
+        if (u < p.ntiles && !some) p.fcounts[u] = 0u;
+        for (uint32_t todo = __ballot_sync(kFull, some); todo; todo &= todo - 1u) {
+            const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
+            const uint32_t total = list_bits(tile_bits(p, t, lane), lists[warp], lane);
+            if (note_tile(noted, t, 0u, total, lane)) continue;
+            const uint32_t sum = sum_chains(p, static_cast<size_t>(t) * kTile, total, lists[warp], lane);
+            if (lane == 0) p.fcounts[t] = sum;
+        }
     }
+    noted_tiles<false>(p, noted, lists[warp], lane, warp);
 }
 
 // The lists.  SMALL: a CTA has kWarps consecutive tiles, one a warp, and adds
@@ -161,6 +251,11 @@ template <bool FULL, bool SMALL>
 __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
     wait_previous();
     __shared__ uint16_t lists[kWarps][kTile];
+    __shared__ DenseTiles noted;
+    if (FULL) {
+        if (threadIdx.x == 0) noted.n = 0;
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if constexpr (SMALL) {
         __shared__ unsigned long long before[kWarps];
@@ -197,7 +292,7 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
             if (w < static_cast<uint32_t>(warp)) at += own[w];
             all += own[w];
         }
-        if (t < p.ntiles) put_tile<FULL>(p, t, t * kTile - p.head, b, at, lists[warp], lane);
+        if (t < p.ntiles) put_tile<FULL>(p, t, t * kTile - p.head, b, at, lists[warp], lane, &noted);
         if (t0 + kWarps >= p.ntiles && threadIdx.x == 0) *p.out.count = all;
     } else {
         const uint32_t gw = blockIdx.x * kWarps + static_cast<uint32_t>(warp), nw = gridDim.x * kWarps;
@@ -206,13 +301,14 @@ __global__ void __launch_bounds__(kThreads) bits_gather(const BitsParams p) {
             const uint32_t c = u < p.ntiles ? p.counts[u] : 0u;
             for (uint32_t todo = __ballot_sync(kFull, c != 0u); todo; todo &= todo - 1u) {
                 const uint32_t t = static_cast<uint32_t>(u0 + static_cast<uint64_t>(__ffs(todo) - 1) * nw);
-                put_tile<FULL>(p, t, t * kTile - p.head, tile_bits(p, t, lane), p.prefix[t], lists[warp],
-                               lane);
+                put_tile<FULL>(p, t, t * kTile - p.head, tile_bits(p, t, lane), p.prefix[t], lists[warp], lane,
+                               &noted);
             }
         }
         if (gw == 0 && lane == 0)
             *p.out.count = p.prefix[p.ntiles - 1u] + p.counts[p.ntiles - 1u];
     }
+    if constexpr (FULL) noted_tiles<true>(p, noted, lists[warp], lane, warp);
 }
 
 // The lists of several texts (streaming form): as bits_gather, each unit's text
@@ -337,7 +433,7 @@ cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *te
     p.head = l.small ? 0u : static_cast<uint32_t>(reinterpret_cast<uintptr_t>(text) & 15u);
     p.words = l.small ? static_cast<uint32_t>((n + 31u) / 32u) : l.ntiles * kWords;
     p.ntiles = l.ntiles;
-    p.counts = full ? reinterpret_cast<uint32_t *>(b + l.fcounts) : r.bits.counts;
+    p.counts = r.bits.counts;
     p.fcounts = reinterpret_cast<uint32_t *>(b + l.fcounts);
     unsigned long long *prefix = reinterpret_cast<unsigned long long *>(b + l.prefix);
     p.prefix = l.small ? nullptr : prefix;
@@ -354,6 +450,7 @@ cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *te
     if (full) {
         e = launch_next(full_bits_count, grid, kThreads, 0u, stream, p);
         if (e != cudaSuccess) return e;
+        p.counts = p.fcounts;
     }
     if (l.small)
         return full ? launch_next(bits_gather<true, true>, need, kThreads, 0u, stream, p)
