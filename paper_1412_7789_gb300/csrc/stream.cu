@@ -15,10 +15,12 @@ namespace {
 // every SM, no list, one launch.  4 KiB of the sweep set, where every position
 // walks to a match: 10 us a call against 70 in the filter kernel, whose few
 // tiles kept a handful of warps busy.  The line against the streaming form (us
-// a call from an idle GPU, host time included): ACGT 2 MiB 25 / 30, 3 MiB 29 /
-// 30; Zipf bytes 2 MiB 44 / 43, 4 MiB 57 / 40.
+// a call): ACGT 2 MiB 14.5 / 15.5, 3 MiB 18.7 / 15.7; where the first 4 KiB all
+// match 18.8 / 24.0 at 2 MiB; Zipf bytes 2 MiB 25.7 / 25.5, 3 MiB 24.9 / 21.7.
 constexpr uint64_t kAtMax = 2u << 20;
-constexpr int kAtBlock = 128;
+// Threads per CTA: short texts want their positions on many SMs, longer ones
+// fewer CTAs (1 MiB of ACGT, 128 / 256 / 512: 11.8 / 10.7 / 12.4 us a call).
+__host__ __device__ constexpr int at_block(int per) { return per == 1 ? 128 : 256; }
 
 // One lane per position (a text this short and the tables it touches stay in
 // L2).  A warp reads its PER x 32 bytes and the 16 after them once, one byte a
@@ -26,11 +28,11 @@ constexpr int kAtBlock = 128;
 // so a position costs little more than a byte load and a load per table level;
 // a lane's PER positions have theirs in flight together.
 template <int B, typename GT, int MODE, int PER>
-__global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ FilterParams p) {
+__global__ void __launch_bounds__(at_block(PER)) pfac_at(const __grid_constant__ FilterParams p) {
     __shared__ uint8_t cls8[256];
     allow_next();  // the lists' gather
     const int lane = threadIdx.x & 31;
-    const uint64_t g0 = (static_cast<uint64_t>(blockIdx.x) * (kAtBlock / 32) + (threadIdx.x >> 5)) * (32u * PER) + lane;
+    const uint64_t g0 = (static_cast<uint64_t>(blockIdx.x) * (at_block(PER) / 32) + (threadIdx.x >> 5)) * (32u * PER) + lane;
     uint32_t c[PER + 1];
     bool in[PER + 1];
 #pragma unroll
@@ -73,8 +75,20 @@ __global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ Filt
     // first loads of all the lane's positions, then the second
     int e[PER], r[PER];
     uint4 h[PER];
-    bool walk[PER];
+    bool walk[PER], keep[PER];
     uint32_t s[PER], q[PER], m[PER];
+    // several positions a lane (longer texts, few of whose positions get past it):
+    // the root filter first, whose 128 KiB stay in L1, not a sector of a table
+    // in L2 for each position (2 MiB of ACGT 16.6 -> 14.7 us a call, of Zipf
+    // bytes 29.0 -> 25.8; short texts would wait for one load more)
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        keep[j] = true;
+        if (PER == 1) continue;
+        const uint32_t v = B == 8 ? ((c[j] & p.wmask) * kFilterHashMul) >> p.fshift
+                                  : c[j] & ((1u << (B * p.k)) - 1u);
+        keep[j] = (__ldg(p.Fg + (v >> 5)) << (v & 31u)) >> 31;
+    }
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         m[j] = __funnelshift_r(bad[j], bad[j + 1], lane);  // bit i: position i after this one
@@ -87,6 +101,11 @@ __global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ Filt
             if (B == 8) walk[j] = false;  // no keyword is shorter than the state hash's window
             continue;
         }
+        if (!keep[j]) {
+            walk[j] = false;
+            e[j] = -1;
+            continue;
+        }
         if (B == 8)
             h[j] = __ldg(p.HK + filt::hk_slot(p, c[j] & p.wmask));
         else
@@ -94,7 +113,7 @@ __global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ Filt
     }
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        if (m[j] & ((1u << need) - 1u)) continue;
+        if ((m[j] & ((1u << need) - 1u)) || !keep[j]) continue;
         if (B == 8) {
             walk[j] = !filt::hk_outcome(p, filt::hk_find(p, c[j] & p.wmask, h[j]), 0u, after[j], !((m[j] >> p.k) & 1u),
                                         r[j], s[j], q[j]);
@@ -130,19 +149,22 @@ __global__ void __launch_bounds__(kAtBlock) pfac_at(const __grid_constant__ Filt
     add_count<MODE>(p, cnt, lane);
 }
 
-// Positions a lane from this length on: 4 (fewer CTAs, and four chains of loads
-// in flight: 1 MiB of ACGT 12.3 -> 10.5 us a call); below, 1, where the walks of
-// a text dense in matches need every warp.
-constexpr uint64_t kAtWide = 256u << 10;
+// Positions a lane from this length on: 2 (fewer CTAs, and two chains of loads
+// in flight); below, 1, where the walks of a text dense in matches need every
+// warp.  A lane's walks run one after another, which is what counts against 4:
+// us a call, 2 / 4 positions, 1 MiB of ACGT 11.9 / 10.6, 2 MiB 14.7 / 14.0;
+// where the first 4 KiB all match 18.7 / 31.0 and 19.2 / 33.
+constexpr uint64_t kAtWide = 768u << 10;
 
 template <int B, typename GT, int MODE>
 void launch_at_one(const FilterParams &p, cudaStream_t stream) {
-    const uint32_t per = p.n >= kAtWide ? 4u : 1u;
-    const uint32_t grid = static_cast<uint32_t>((p.n + kAtBlock * per - 1) / (kAtBlock * per));
-    if (per == 4u)
-        pfac_at<B, GT, MODE, 4><<<grid, kAtBlock, 0, stream>>>(p);
+    const uint32_t per = p.n >= kAtWide ? 2u : 1u;
+    const uint32_t block = at_block(static_cast<int>(per));
+    const uint32_t grid = static_cast<uint32_t>((p.n + block * per - 1) / (block * per));
+    if (per == 2u)
+        pfac_at<B, GT, MODE, 2><<<grid, block, 0, stream>>>(p);
     else
-        pfac_at<B, GT, MODE, 1><<<grid, kAtBlock, 0, stream>>>(p);
+        pfac_at<B, GT, MODE, 1><<<grid, block, 0, stream>>>(p);
 }
 
 template <int B, typename GT>
@@ -156,18 +178,20 @@ cudaError_t launch_at_modes(OutMode mode, const FilterParams &p, cudaStream_t st
     return cudaGetLastError();
 }
 
+constexpr uint64_t kWalkEarly = 16u << 20;
 template <int B, typename GT>
 cudaError_t launch_walk_modes(OutMode mode, const FilterParams &p, uint32_t sms, cudaStream_t stream) {
     const uint32_t grid = sms * kWalkCtas;
-    // (a plain launch: started early, the walks' CTAs cost the form before them
-    // more than the gap they save, 1 GiB of Zipf bytes compacted 1360 against
-    // 1155 us)
-    switch (mode) {
-        case OUT_DENSE: pfac_stream_walks<B, GT, OUT_DENSE><<<grid, kWalkBlock, 0, stream>>>(p); break;
-        case OUT_COUNT: pfac_stream_walks<B, GT, OUT_COUNT><<<grid, kWalkBlock, 0, stream>>>(p); break;
-        case OUT_BITS: pfac_stream_walks<B, GT, OUT_BITS><<<grid, kWalkBlock, 0, stream>>>(p); break;
-        default: return cudaErrorInvalidValue;
-    }
+    auto kernel = mode == OUT_DENSE ? pfac_stream_walks<B, GT, OUT_DENSE>
+                  : mode == OUT_COUNT ? pfac_stream_walks<B, GT, OUT_COUNT>
+                                      : pfac_stream_walks<B, GT, OUT_BITS>;
+    // (started early, but with bytes for short texts only: on long ones the
+    // walks' CTAs cost the form before them more than the gap they save.  us a
+    // call, plain / early: ACGT 4 MiB 17.9 / 15.9, 64 MiB 73.6 / 70.6; Zipf bytes
+    // 4 MiB counted 28.8 / 27.0, 24 MiB 46.4 / 45.8, 64 MiB full 112 / 120, 1 GiB
+    // compacted 1155 / 1360)
+    if (B == 2 || p.n <= kWalkEarly) return launch_next(kernel, grid, kWalkBlock, 0u, stream, p);
+    kernel<<<grid, kWalkBlock, 0, stream>>>(p);
     return cudaGetLastError();
 }
 
@@ -251,7 +275,9 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
     p.ntiles = static_cast<uint32_t>((r.n + p.sg.head + kTile - 1) / kTile);
     const uint32_t smem = stream_smem(t.stream.form, false, p.f1bytes + p.f2bytes, &p.off_none, &p.off_warp);
     if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
-    const uint32_t nw = static_cast<uint32_t>(block_of(t.stream.form, false) / 32), need = (p.ntiles + nw - 1) / nw;
+    // short texts spread over the SMs, a tile to each of eight warps (3 MiB of
+    // ACGT 17.5 -> 15.7 us a call, of Zipf bytes 23.7 -> 21.7)
+    const uint32_t need = (p.ntiles + 7) / 8;
     const uint32_t grid = need < static_cast<uint32_t>(sms) ? need : static_cast<uint32_t>(sms);
     e = t.stream.form == 2 ? launch_stream2(mode, p, t.stream.step, grid, smem, max_smem, stream)
                            : launch_stream8(mode, p, grid, smem, max_smem, stream);

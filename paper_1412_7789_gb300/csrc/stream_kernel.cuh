@@ -920,6 +920,7 @@ template <int FORM, int S, int MODE>
 __device__ __forceinline__ void stream_text(const StreamParams &p) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    allow_next();  // the walks
     const uint32_t step = gridDim.x * (blockDim.x / 32);
     const uint32_t t = static_cast<uint32_t>(warp) * gridDim.x + blockIdx.x;
     const uint64_t pol = policy_evict_first();
@@ -1127,6 +1128,7 @@ __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const
     __shared__ uint8_t cls8[256];
     const int lane = threadIdx.x & 31;
     allow_next();  // the lists' scan
+    wait_previous();
     const uint32_t listed = *reinterpret_cast<volatile const unsigned int *>(p.list_count + 1);
     const uint32_t m = listed < p.walk_cap ? listed : p.walk_cap;
     if (blockIdx.x * blockDim.x >= m) return;
@@ -1135,7 +1137,7 @@ __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const
     const Seg sg = make_seg(p.text, p.out, p.n);
     uint32_t cnt = 0;
     for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-        const uint2 e = __ldg(p.walks + j);
+        const uint2 e = p.walks[j];  // (not by the read-only path: written by the launch before)
         if (e.x != 0xFFFFFFFFu) put_id<MODE>(p, sg, e.x, finish_walk<GT>(p, cls8, sg, e.x, e.y, B), cnt);
     }
     add_count<MODE>(p, cnt, lane);

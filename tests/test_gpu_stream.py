@@ -343,3 +343,16 @@ def test_no_room_for_the_streaming_scratch(kind, free_mib):
     r = subprocess.run([sys.executable, "-c", _NO_ROOM, kind, str(free_mib)], cwd=root, capture_output=True, text=True,
                        timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("name", ["dna16", "dna4", "iupac", "bytes4"])
+@pytest.mark.parametrize("part", [4, 16])
+def test_other_table_depths(name, part):
+    """Root tables rebuilt for a smaller filter: the short-text form reads them
+    at the new window, longer texts leave the streaming form."""
+    for n in (5001, AT_MAX + 5001):
+        text, pats = _workload(name, n)
+        want = oracle.pfac_ids(pats, text)
+        with api.Automaton(pats) as a:
+            a.set_tuning(filter_bytes=max(4, a.tuning()["filter_bytes"] // part))
+            _check(a, text, want, 3, 0)
