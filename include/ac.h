@@ -261,10 +261,14 @@ ac_status ac_export_jump(ac_handle h, int16_t *J, uint32_t *k, uint32_t *base_k,
  * Dense matching.  d_out_ids[i] = id of the longest keyword starting at
  * d_text[i] (within the n bytes), or -1.  d_text: n bytes, d_out_ids: n int32,
  * any alignment (16-byte aligned buffers take the vectorised path).  n = 0 is
- * a no-op.  Takes 16 bytes of scratch (the tile counter) per call from the
- * library's stream-ordered pool, except for a text short enough that each of
- * its tiles is some warp's first (no counter, no allocation).  A text that
- * takes the phased form of the filter kernel (8-bit codes from 4 MiB on; see
+ * a no-op.  With the tuning as built, texts of up to 2 MiB take no scratch, and
+ * longer ones that the streaming form serves (DNA letters with a root window
+ * of 10 codes, or 8-bit codes with keywords of 4 bytes or more) a walk list
+ * from the library's stream-ordered pool: 8 bytes for every eighth text byte
+ * and 2 MB; where the device has no room for it, the filter kernel is taken
+ * instead.  That kernel (every other automaton or tuning) takes 16 bytes (the
+ * tile counter), or none for a text short enough that each of its tiles is
+ * some warp's first; its phased form (8-bit codes from 4 MiB on; see
  * ac_tuning.survivor_list) also takes its survivor and walk lists from the
  * pool: about 3 bytes per text byte (16 per listed survivor, room for n / 8
  * of them, and 8 per walk).
@@ -276,12 +280,16 @@ ac_status ac_match(ac_handle h, const uint8_t *d_text, uint64_t n, int32_t *d_ou
  * their ids.  Writes min(total, cap) entries to d_pos / d_ids (uint32 each) and
  * the true total to *d_count (a device uint64).  The caller compares the total
  * with cap and calls again with more room when it is larger.  n must be below
- * 2^32.  Takes its scratch (per tile a match count, a prefix sum, 32 match
- * slots and a dense fallback of 4 bytes per position; for the phased form
- * the survivor and walk lists as for ac_match, and then no dense fallback:
- * the gather matches a tile with more than 32 matches again) from the
- * library's stream-ordered pool (cudaMallocFromPoolAsync) on `stream`; the
- * pool keeps the memory it grows to until the process exits.
+ * 2^32.  Takes its scratch from the library's stream-ordered pool
+ * (cudaMallocFromPoolAsync) on `stream`; the pool keeps the memory it grows to
+ * until the process exits.  With the tuning as built: a bit and an id for each
+ * position (written where it matches only), per 2,048 positions a count and a
+ * prefix sum, and the walk list of ac_match: about 5.2 bytes per text byte.
+ * The filter kernel (other tunings and automata, or no room for that): per
+ * tile a match count, a prefix sum, 32 match slots and a dense fallback of 4
+ * bytes per position, about 4.4 bytes per text byte; for its phased form the
+ * survivor and walk lists as for ac_match, and then no dense fallback: the
+ * gather matches a tile with more than 32 matches again.
  */
 ac_status ac_match_compact(ac_handle h, const uint8_t *d_text, uint64_t n, uint32_t *d_pos,
                            uint32_t *d_ids, uint64_t cap, uint64_t *d_count, void *stream);
@@ -309,7 +317,8 @@ ac_status ac_count(ac_handle h, const uint8_t *d_text, uint64_t n, uint64_t *d_c
 
 /*
  * Dense matching from and to HOST memory: copies h_text to the device, matches
- * and copies the ids back, pipelined in chunks on `stream` (chunks overlap
+ * and copies the ids back, pipelined in chunks (an eighth of the text, 4 to 64
+ * MiB) on `stream` (chunks overlap
  * copies with matching; each chunk carries a max_len halo so walks never see a
  * chunk edge).  Host buffers should be pinned (cudaHostAlloc / pin_memory) for
  * the copies to overlap.  Synchronises `stream` before returning.
@@ -321,7 +330,11 @@ ac_status ac_set_kernel(ac_handle h, ac_kernel kernel);
 
 /*
  * Launch shape of the root filter kernel (AC_KERNEL_TILED; no counterpart in
- * the paper).  Results never depend on it, only the time does.
+ * the paper).  Results never depend on it, only the time does.  With every
+ * field as built (block, stages, survivor_list 0, halo up to 16, per_thread
+ * not 4, the root tables of the compile) single texts take the short-text or
+ * the streaming form instead where those serve the automaton (ac_match); any
+ * other value keeps the filter kernel.
  *   block         threads per CTA: 0 = the kernel's choice (default): 640 for
  *                 the one-phase single-text forms of 2- and 4-bit codes (20
  *                 warps per SM, compiled at 96 registers), 512 elsewhere; or
@@ -448,7 +461,9 @@ ac_status ac_match_compact_static(ac_handle h, const uint8_t *d_text, uint64_t n
  * kernel ac_set_kernel or ac_autotune chose for its single texts (and, with a
  * plan's survivor lists, lists the survivors of its 8-bit-code automata, and
  * of those with 2- or 4-bit codes whose match_windows_ppm is 500 or more, for
- * two more launches: ac_batch_reserve_lists).  Otherwise the batch takes one
+ * two more launches: ac_batch_reserve_lists; the automata that the streaming
+ * form serves take its launches instead, one for each kind of code and one for
+ * the listed walks).  Otherwise the batch takes one
  * persistent launch per automaton.  Results are exactly
  * those of ac_match on each text alone: walks stop at the end of their own
  * text.
@@ -500,17 +515,22 @@ ac_status ac_match_batch(const ac_handle *hs, uint32_t nh, const uint8_t *d_text
  *   ac_batch_destroy frees the plan (not the handles); no work using it may be
  *                    in flight.
  *   ac_batch_reserve_lists
- *                    sizes the plan's survivor lists for the phased form of
- *                    its 8-bit-code automata (and the 2- and 4-bit ones
- *                    with match_windows_ppm of 500 or more): with the one
- *                    persistent launch,
- *                    their survivors (up to text_bytes / 8 of them per run)
- *                    are listed and resolved by two further launches at full
- *                    occupancy, as ac_match does for one long text; tiles
- *                    whose survivors no longer fit are resolved in their
- *                    warps.  Takes about 4 bytes of device memory per byte of
- *                    text_bytes (cudaMalloc); 0 frees the lists (the default:
- *                    none, every survivor is resolved in its warp).  It drops
+ *                    sizes the plan's lists for runs of up to text_bytes of
+ *                    text.  The automata (up to 32 in the plan) that the
+ *                    streaming form serves then take it, as ac_match does for
+ *                    one long text: their walks are listed (text_bytes / 8 of
+ *                    them and 4 MB) and done by one launch more; walks past
+ *                    that end where they were found.  The other
+ *                    automata's survivors (8-bit codes, and 2- and 4-bit ones
+ *                    with match_windows_ppm of 500 or more) are listed for the
+ *                    phased form of the filter kernel, up to text_bytes / 8 of
+ *                    them per run; tiles whose survivors no longer fit are
+ *                    resolved in their warps.  Takes 2 bytes of device memory
+ *                    (cudaMalloc) per byte of text_bytes for the streaming
+ *                    form and about 4 for the filter kernel's, as far as the
+ *                    plan's automata, tuned as they are then, need each (all
+ *                    in the filter kernel when both do not fit); 0 frees the
+ *                    lists (the default: none, the filter kernel alone).  It drops
  *                    a captured graph (capture again after it); no work
  *                    using the plan may be in flight.  Results do not depend
  *                    on it.
@@ -529,10 +549,11 @@ ac_status ac_batch_destroy(ac_batch b);
 /*
  * Autotuning (no counterpart in the paper): time the dense matching of handle
  * h on the device text d_sample (n bytes, at least 1 MiB is sensible; 4 MiB or
- * more for the one-thread-per-survivor step of 8-bit codes) with each
+ * more for the streaming form and the filter kernel's lists) with each
  * candidate and keep the fastest for every later call on h (single texts,
  * batches and servers).  The candidates, for an automaton with a root filter
- * (ac_tuning): the shared-table depth -- the filter as built and two smaller
+ * (ac_tuning): the tuning as built (the only one that the short-text and
+ * streaming forms serve; any other choice keeps the filter kernel); the shared-table depth -- the filter as built and two smaller
  * ones (windows of one and two codes fewer, or a hashed filter of a quarter
  * and a sixteenth of the bits) -- x threads per CTA {256, 384, 512, and 640
  * for small alphabets} x text stages {2, 3, 4} (the shapes that fit shared memory); then, at the best of
@@ -577,7 +598,10 @@ ac_status ac_autotune(ac_handle h, const uint8_t *d_sample, uint64_t n, uint32_t
  *     one persistent matching launch over the tiles of all its requests and
  *     automata (as a batch: up to 32 automata with root filters; else one
  *     launch per automaton), then one scan and a gather per automaton, so
- *     requests of any size share the launches.  In the one launch, when a
+ *     requests of any size share the launches.  When a wave holds 4 MiB or
+ *     more of text, the automata that the streaming form serves take its
+ *     launches and one gather for all of them, as far as its scratch fits in
+ *     what the requests were charged.  In the filter kernel's launch, when a
  *     wave holds 4 MiB or more of text for 8-bit-code automata, their
  *     survivors are listed and resolved by two more launches (the phased form
  *     of ac_match); their tiles then keep no dense fallback, and the gather

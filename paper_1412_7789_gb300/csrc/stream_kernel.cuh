@@ -15,9 +15,9 @@
 // What bounds it, and what it measured (GB300, 1 GiB of text): with 2-bit codes
 // dense ids are bound by DRAM writes (0.875 ms, 0.90 of the copy peak; the
 // filter kernel's own pass, 1,200 cycles of instructions a tile, took 1.065),
-// counts by instruction issue (0.29 against 0.88 ms); with 8-bit codes both by
+// counts by instruction issue (0.27 against 0.88 ms); with 8-bit codes both by
 // the filter's lookups, 16 a lane and chunk, about 8 instructions each (count
-// 0.88 against 2.15 ms, where every tenth position went through a global list).
+// 0.85 against 2.15 ms, where every tenth position went through a global list).
 //
 // 2-bit codes (pfac_stream2).  Codes come from (byte >> 1) & 3, and bytes in no
 // keyword get some code as well: the filter bit of a position with a result is
