@@ -377,7 +377,9 @@ cudaError_t run_compact(ac_automaton *h, const uint8_t *text, uint64_t n, const 
 // The full output of one text with its scratch from the pool.
 cudaError_t run_full(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out,
                      cudaStream_t st) {
-    if (pfac::bits_serve(h->dev, h->tuning, n)) {
+    // a keyword set with so many equal or nested keywords that a tile's count
+    // may pass 32 bits goes by slots, whose units are shorter
+    if (pfac::bits_serve(h->dev, h->tuning, n) && pfac::full_fits(h->dev.full_max_clen, pfac::kStreamTile)) {
         bool room = true;
         const cudaError_t e = run_bits(h, text, n, out, true, st, &room);
         if (room) return e;  // else by slots, which take less
@@ -843,9 +845,7 @@ ac_status ac_match_full(ac_handle h, const uint8_t *d_text, uint64_t n, uint32_t
     if (s != AC_OK) return s;
     if (!d_count || (cap > 0 && (!d_end || !d_ids))) return AC_ERR_INVALID_ARG;
     if (n > 0xFFFFFFFFull) return AC_ERR_INVALID_ARG;
-    // a unit's occurrence count (at most kDenseStride results, each with up to
-    // full_max_clen occurrences) must fit 32 bits
-    if (static_cast<uint64_t>(h->dev.full_max_clen) * pfac::kDenseStride > 0xFFFFFFFFull) return AC_ERR_OVERFLOW;
+    if (!pfac::full_fits(h->dev.full_max_clen, pfac::kDenseStride)) return AC_ERR_OVERFLOW;  // not even by slots
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (n == 0) return cuda_status(cudaMemsetAsync(d_count, 0, sizeof(uint64_t), st));
     if (!d_text) return AC_ERR_INVALID_ARG;

@@ -276,6 +276,12 @@ struct BitsOut {
     uint32_t *counts = nullptr;
 };
 
+// Full output: a unit's occurrences (at most `results` results, each with up
+// to max_clen of them) are counted in 32 bits.
+inline bool full_fits(uint32_t max_clen, uint32_t results) {
+    return static_cast<uint64_t>(max_clen) * results <= 0xFFFFFFFFull;
+}
+
 // Where one text's compacted list goes (ac_match_compact's arguments).
 struct CompactOut {
     uint32_t *pos;

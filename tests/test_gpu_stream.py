@@ -139,6 +139,27 @@ def test_full_list(name):
         assert np.array_equal(got[np.lexsort((got[:, 1], got[:, 0]))], want[np.lexsort((want[:, 1], want[:, 0]))])
 
 
+def test_full_counts_past_32_bits():
+    """2^21 equal keywords: a tile of 2,048 of their matches holds 2^32
+    occurrences, which only units of half a tile can count in 32 bits."""
+    import torch
+
+    copies, run = 1 << 21, 2 * 2048 + 100
+    pats = [b"A"] * copies + [b"CGTCGTCCGGTTCC"]
+    with api.Automaton(pats) as a:
+        for n in (run, AT_MAX + 4096):
+            text = _letters(n, b"CGT", 17).copy()
+            at = (n - run) // 2  # the matches: one run, two whole tiles of it at least at most offsets
+            text[at:at + run] = ord("A")
+            other = text.tobytes().count(pats[-1])
+            cap = 4
+            t = torch.from_numpy(text).cuda()
+            e, i, c = a.match_full(t, cap=cap)
+            assert int(c.item()) == run * copies + other
+            if not other:  # the first start's occurrences come first, ids ascending
+                assert e.cpu().tolist() == [at] * cap and i.cpu().tolist() == list(range(cap))
+
+
 @pytest.mark.parametrize("letters,lens", [(b"A", (16, 20, 60)), (b"A", (4, 33)), (b"x", (6, 9, 40)), (b"x", (4, 50))])
 def test_more_walks_than_listed(letters, lens):
     """A text of one letter: every position is a survivor and a long walk, far
