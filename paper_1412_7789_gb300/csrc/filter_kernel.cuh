@@ -107,7 +107,7 @@ struct FilterParams {
     unsigned long long *count;
     SlotOut sl;
     BitsOut bo;
-    uint32_t bits_head;  // OUT_BITS: text position i is position i + bits_head there
+    uint32_t walk_chunk;  // streaming form: walk-list entries a warp reserves at a time, at least
     unsigned int *counter;
     unsigned int *err;
     uint32_t off_neg1, off_warp, warp_bytes, off_packed, off_inv, off_queue, off_meta, off_help;

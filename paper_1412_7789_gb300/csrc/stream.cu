@@ -231,6 +231,14 @@ uint32_t stream_walk_cap(uint64_t n) {
 
 namespace {
 
+// Entries a warp reserves of a walk list at a time: no more than half the list
+// over all warps, so that a short list (a wave's, which stays within what its
+// requests were charged) is not used up by empty entries.
+uint32_t walk_chunk(uint32_t walk_cap) {
+    const uint32_t c = walk_cap / (2u * device_sm_count() * static_cast<uint32_t>(kMostWarps) + 1u);
+    return c < 1u ? 1u : (c < kWalkChunkEntries ? c : kWalkChunkEntries);
+}
+
 // The streaming form's parameters of one automaton, all but the places in
 // shared memory.
 cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu, StreamParams &p) {
@@ -240,6 +248,7 @@ cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mod
     p.f.walks = r.walks;
     p.f.walk_cap = r.walk_cap;
     p.f.list_count = r.list_count;
+    p.f.walk_chunk = walk_chunk(r.walk_cap);
     p.F1 = t.stream_F1 ? t.stream_F1 : t.F;
     p.f1bytes = (1u << kFilterBits) / 8u;
     p.F2 = t.stream_F2;
@@ -333,6 +342,7 @@ cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *
             p.f.list_count = reinterpret_cast<unsigned int *>(b);
             p.f.walks4 = reinterpret_cast<uint4 *>(b + 32);
             p.f.walk_cap = walk_cap;
+            p.f.walk_chunk = walk_chunk(walk_cap);
             wm.a[a] = p.f;
             filters = filters > p.f1bytes + p.f2bytes ? filters : p.f1bytes + p.f2bytes;
         }

@@ -296,10 +296,11 @@ __device__ __forceinline__ bool push_walk(const StreamParams &p, const Seg &sg, 
     if (rest < need) {
         uint32_t base = p.f.walk_cap, end = p.f.walk_cap;
         if (!room.full) {
-            if (lane == 0) base = atomicAdd(p.f.list_count + 1, kWalkChunkEntries);
+            const uint32_t chunk = need - rest > p.f.walk_chunk ? need - rest : p.f.walk_chunk;
+            if (lane == 0) base = atomicAdd(p.f.list_count + 1, chunk);
             base = __shfl_sync(kFull, base, 0);
-            room.full = base >= p.f.walk_cap || p.f.walk_cap - base <= kWalkChunkEntries;
-            end = room.full ? p.f.walk_cap : base + kWalkChunkEntries;
+            room.full = base >= p.f.walk_cap || p.f.walk_cap - base <= chunk;
+            end = room.full ? p.f.walk_cap : base + chunk;
             if (base > end) base = end;
         }
         if (rank >= rest) {

@@ -279,6 +279,63 @@ def test_request_charge_is_kept():
     assert np.array_equal(pos[:m].cpu().numpy(), wpos) and np.array_equal(ids[:m].cpu().numpy(), wids)
 
 
+@pytest.mark.parametrize("names,lens", [
+    (("dna16",), [(0, (4 << 20) + 5)]),
+    (("dna4", "dna16"), [(0, 3_000_000), (1, 5_000_001), (0, 777), (1, 2047)]),
+    (("bytes5", "dna8"), [(0, 3_000_000), (1, 4_000_001), (1, 1)]),
+    (("iupac", "dna16"), [(0, 5 << 20), (1, 40)]),  # 40 bytes of it for the streaming form
+])
+def test_wave_scratch_is_charged(names, lens):
+    """The device scratch of a wave stays within what its requests were charged
+    for their tiles (and lists), the wave's plan (a head and a counter an
+    automaton, 64 bytes a request, the scan's 256 partial sums) and a kilobyte
+    of rounding for each of its parts; every request is served."""
+    import torch
+
+    loads = [_workload(name, 5 << 20) for name in names]
+    blocks = {}
+
+    def alloc(nbytes):
+        t = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+        blocks[t.data_ptr()] = t
+        sizes.append(nbytes)
+        return t.data_ptr()
+
+    sizes, reqs, outs, charge = [], [], [], 0
+    autos = [api.Automaton(p) for _, p in loads]
+    try:
+        for a, n in lens:
+            text = loads[a][0][:n]
+            d = torch.from_numpy(text.copy()).cuda()
+            want = oracle.compact(oracle.pfac_ids(loads[a][1], text))
+            cap = max(1, want[0].size)
+            pos = torch.full((cap,), -7, dtype=torch.int32, device="cuda")
+            ids = torch.full((cap,), -7, dtype=torch.int32, device="cuda")
+            cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+            reqs.append(api.Server.request(a, d, n, pos, ids, cap, cnt))
+            outs.append((d, pos, ids, cnt, want))
+            charge += -(-n // 992) * (4 + 8 + 8 * 32 + 4 * 1024) + 64
+            if autos[a].info()["code_bits"] == 8:
+                charge += 32 * (n // 8) + 32
+        torch.cuda.synchronize()
+        with api.Server([a.handle for a in autos], waves_in_flight=1, dev_alloc=alloc,
+                        dev_free=lambda p: blocks.pop(p)) as srv:
+            srv.replay(np.concatenate(reqs), np.zeros(len(reqs)))
+            srv.drain()
+            done = srv.poll(len(reqs) + 1)
+            assert done["status"].tolist() == [api.AC_OK] * len(reqs)
+            waves = len(sizes)
+        assert waves and not blocks
+        assert sum(sizes) <= charge + waves * (32 * len(autos) + 8 * 256 + 12 * 1024), (sizes, charge)
+        for _, pos, ids, cnt, (wpos, wids) in outs:
+            m = int(cnt.item())
+            assert m == wpos.size
+            assert np.array_equal(pos[:m].cpu().numpy(), wpos) and np.array_equal(ids[:m].cpu().numpy(), wids)
+    finally:
+        for a in autos:
+            a.close()
+
+
 def test_wave_past_32_bits_of_text():
     """Waves that hold more text than 32 bits can number: every request is
     served, each as ac_match_compact alone."""
