@@ -263,10 +263,10 @@ ac_status ac_export_jump(ac_handle h, int16_t *J, uint32_t *k, uint32_t *base_k,
  * any alignment (16-byte aligned buffers take the vectorised path).  n = 0 is
  * a no-op.  With the tuning as built, texts of up to 2 MiB take no scratch, and
  * longer ones that the streaming form serves (DNA letters with a root window
- * of 10 codes, or 8-bit codes with keywords of 4 bytes or more) a walk list
- * from the library's stream-ordered pool: 8 bytes for every eighth text byte
- * and 2 MB; where the device has no room for it, the filter kernel is taken
- * instead.  That kernel (every other automaton or tuning) takes 16 bytes (the
+ * of 10 codes, or 8-bit codes with keywords of 4 bytes or more) a list of walks
+ * and one of tiles from the library's stream-ordered pool: 8 bytes for every
+ * eighth text byte, 4 for every 2,048, and 2 MB; where the device has no room
+ * for it, the filter kernel is taken instead.  That kernel (every other automaton or tuning) takes 16 bytes (the
  * tile counter), or none for a text short enough that each of its tiles is
  * some warp's first; its phased form (8-bit codes from 4 MiB on; see
  * ac_tuning.survivor_list) also takes its survivor and walk lists from the
@@ -284,7 +284,7 @@ ac_status ac_match(ac_handle h, const uint8_t *d_text, uint64_t n, int32_t *d_ou
  * (cudaMallocFromPoolAsync) on `stream`; the pool keeps the memory it grows to
  * until the process exits.  With the tuning as built: a bit and an id for each
  * position (written where it matches only), per 2,048 positions a count and a
- * prefix sum, and the walk list of ac_match: about 5.2 bytes per text byte.
+ * prefix sum, and the lists of ac_match: about 5.2 bytes per text byte.
  * The filter kernel (other tunings and automata, or no room for that): per
  * tile a match count, a prefix sum, 32 match slots and a dense fallback of 4
  * bytes per position, about 4.4 bytes per text byte; for its phased form the
@@ -519,9 +519,9 @@ ac_status ac_match_batch(const ac_handle *hs, uint32_t nh, const uint8_t *d_text
  *                    text.  The automata (up to 32 in the plan) that the
  *                    streaming form serves then take it, as ac_match does for
  *                    one long text: their walks are listed (text_bytes / 8 of
- *                    them and 4 MB) and done by one launch more; walks past
- *                    that end where they were found.  The other
- *                    automata's survivors (8-bit codes, and 2- and 4-bit ones
+ *                    them and 4 MB), tiles with many walks as a whole, and done
+ *                    by one launch more; what finds no room is done where it
+ *                    was found.  The other automata's survivors (8-bit codes, and 2- and 4-bit ones
  *                    with match_windows_ppm of 500 or more) are listed for the
  *                    phased form of the filter kernel, up to text_bytes / 8 of
  *                    them per run; tiles whose survivors no longer fit are

@@ -53,8 +53,8 @@ struct ac_batch_plan {
     void *scratch = nullptr;
     void *lists = nullptr;  // the phased form's lists (ac_batch_reserve_lists)
     uint32_t list_cap = 0;
-    void *walks = nullptr;  // the streaming form's walk list (with the lists)
-    uint32_t walk_cap = 0;
+    void *walks = nullptr;  // the streaming form's lists (with the lists)
+    pfac::StreamLists walk_lists;
     cudaStream_t capture = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -274,12 +274,14 @@ cudaError_t pool_alloc(ac_automaton *h, size_t bytes, cudaStream_t st, void **ou
     return e;
 }
 
-// The streaming form of one long text, its walk list from the pool.  *room
-// = false: no memory for the list, and nothing was enqueued.
+// The streaming form of one long text, its lists from the pool.  *room
+// = false: no memory for them, and nothing was enqueued.
 cudaError_t run_stream(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st, bool *room) {
-    r.walk_cap = pfac::stream_walk_cap(r.n);
+    const pfac::StreamLists l = pfac::stream_lists(r.n);
+    r.walk_cap = l.walk_cap;
+    r.tile_cap = l.tile_cap;
     void *scratch = nullptr;
-    cudaError_t e = pool_alloc(h, pfac::stream_bytes(r.walk_cap), st, &scratch);
+    cudaError_t e = pool_alloc(h, l.bytes(), st, &scratch);
     *room = e != cudaErrorMemoryAllocation;
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(scratch, 0, 32, st);
@@ -429,12 +431,12 @@ ac_status check_handles(const ac_handle *hs, uint32_t nh) {
 cudaError_t enqueue_batch(const ac_handle *hs, uint32_t nh, void *scratch, const uint8_t *texts,
                           const ac_batch_item *items, uint32_t nitems, int32_t *out, cudaStream_t st,
                           void *surv_lists = nullptr, uint32_t list_cap = 0, void *walks = nullptr,
-                          uint32_t walk_cap = 0) {
+                          const pfac::StreamLists &walk_lists = pfac::StreamLists{}) {
     uint8_t *base = static_cast<uint8_t *>(scratch);
     pfac::BatchHead *heads = reinterpret_cast<pfac::BatchHead *>(base);
     uint8_t *counters = base + static_cast<size_t>(nh) * 16u;
     pfac::BatchItemDev *lists = reinterpret_cast<pfac::BatchItemDev *>(base + static_cast<size_t>(nh) * 32u);
-    const bool streams = walks && walk_cap && nh <= pfac::kStreamBatchMax;
+    const bool streams = walks && walk_lists.walk_cap && nh <= pfac::kStreamBatchMax;
     std::vector<const pfac::DevTables *> ts, sts;   // the filter kernel's, the streaming form's
     std::vector<pfac::MatchRequest> rs, srs;
     std::vector<uint32_t> rest;                     // the filter kernel's automata
@@ -462,7 +464,7 @@ cudaError_t enqueue_batch(const ac_handle *hs, uint32_t nh, void *scratch, const
         e = cudaMemsetAsync(walks, 0, 32, st);
         if (e == cudaSuccess)
             e = pfac::launch_stream_batch(sts.data(), srs.data(), static_cast<uint32_t>(sts.size()), pfac::OUT_DENSE,
-                                          hs[0]->tuning.wait_ns, walks, walk_cap, st);
+                                          hs[0]->tuning.wait_ns, walks, walk_lists, st);
     }
     if (multi) {
         if (e == cudaSuccess && surv_lists && list_cap) e = cudaMemsetAsync(surv_lists, 0, 32, st);
@@ -1002,7 +1004,7 @@ ac_status ac_batch_reserve_lists(ac_batch b, uint64_t text_bytes) {
     if (b->walks) {
         cudaError_t e = cudaFree(b->walks);
         b->walks = nullptr;
-        b->walk_cap = 0;
+        b->walk_lists = pfac::StreamLists{};
         if (e != cudaSuccess) return cuda_status(e);
     }
     if (cap == 0) return AC_OK;
@@ -1017,9 +1019,9 @@ ac_status ac_batch_reserve_lists(ac_batch b, uint64_t text_bytes) {
         if (e == cudaSuccess) b->list_cap = static_cast<uint32_t>(cap);
     }
     if (e == cudaSuccess && streamed && b->hs.size() <= pfac::kStreamBatchMax) {
-        const uint32_t wc = pfac::stream_batch_cap(text_bytes);
-        e = cudaMalloc(&b->walks, pfac::stream_batch_bytes(wc));
-        if (e == cudaSuccess) b->walk_cap = wc;
+        const pfac::StreamLists l = pfac::stream_batch_lists(text_bytes, b->max_items);
+        e = cudaMalloc(&b->walks, l.batch_bytes());
+        if (e == cudaSuccess) b->walk_lists = l;
         // no room for both lists: the filter kernel's serve every automaton
         if (e == cudaErrorMemoryAllocation && b->lists) {
             cudaGetLastError();
@@ -1031,7 +1033,7 @@ ac_status ac_batch_reserve_lists(ac_batch b, uint64_t text_bytes) {
         cudaGetLastError();
         if (b->lists) cudaFree(b->lists);
         b->lists = b->walks = nullptr;  // a failed allocation leaves its pointer unset
-        b->list_cap = b->walk_cap = 0;
+        b->list_cap = 0;
         return e == cudaErrorMemoryAllocation ? AC_ERR_OOM : cuda_status(e);
     }
     return AC_OK;
@@ -1041,7 +1043,7 @@ namespace {
 ac_status batch_enqueue(ac_batch b, const uint8_t *d_texts, const ac_batch_item *d_items, uint32_t nitems,
                         int32_t *d_out, cudaStream_t st) {
     return cuda_status(enqueue_batch(b->hs.data(), static_cast<uint32_t>(b->hs.size()), b->scratch, d_texts, d_items,
-                                     nitems, d_out, st, b->lists, b->list_cap, b->walks, b->walk_cap));
+                                     nitems, d_out, st, b->lists, b->list_cap, b->walks, b->walk_lists));
 }
 
 ac_status check_plan_args(ac_batch b, const uint8_t *d_texts, const ac_batch_item *d_items, uint32_t nitems,

@@ -346,11 +346,12 @@ __global__ void __launch_bounds__(kThreads) bits_gather_texts(BitsParams p, cons
 
 inline size_t round256(size_t v) { return (v + 255u) & ~static_cast<size_t>(255u); }
 
-// Scratch: walk counters (32) | per tile: matches, occurrences (4 each),
-// prefix (8) | partial sums | bits | walk list | ids.
+// Scratch: list counters (32) | per tile: matches, occurrences (4 each),
+// prefix (8) | partial sums | bits | walk and tile list | ids.
 struct Layout {
     size_t counts, fcounts, prefix, partials, bits, walks, ids, bytes;
-    uint32_t ntiles, walk_cap;
+    uint32_t ntiles;
+    StreamLists lists;
     bool small;
 };
 
@@ -359,7 +360,7 @@ Layout layout_of(const DevTables &t, const Tuning &tu, const uint8_t *text, uint
     l.small = at_serves(t, tu, n);
     const uint64_t head = l.small ? 0u : reinterpret_cast<uintptr_t>(text) & 15u;
     l.ntiles = static_cast<uint32_t>((n + head + kTile - 1) / kTile);
-    l.walk_cap = l.small ? 0u : stream_walk_cap(n);
+    if (!l.small) l.lists = stream_lists(n);
     size_t at = 256;
     auto take = [&](size_t bytes) {
         const size_t o = at;
@@ -371,7 +372,7 @@ Layout layout_of(const DevTables &t, const Tuning &tu, const uint8_t *text, uint
     l.prefix = take(l.small ? 0 : 8ull * l.ntiles);
     l.partials = take(l.small ? 0 : 8ull * kScanCtas);
     l.bits = take(4ull * kWords * l.ntiles);
-    l.walks = take(8ull * l.walk_cap);
+    l.walks = take(l.lists.bytes());
     l.ids = take(4ull * kTile * l.ntiles);
     l.bytes = at;
     return l;
@@ -421,7 +422,8 @@ cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *te
         r.bits.counts = reinterpret_cast<uint32_t *>(b + l.counts);
         r.list_count = reinterpret_cast<unsigned int *>(b);
         r.walks = reinterpret_cast<uint2 *>(b + l.walks);
-        r.walk_cap = l.walk_cap;
+        r.walk_cap = l.lists.walk_cap;
+        r.tile_cap = l.lists.tile_cap;
         e = cudaMemsetAsync(b, 0, 32, stream);
         if (e == cudaSuccess) e = launch_stream(t, r, OUT_BITS, tu, stream);
     }

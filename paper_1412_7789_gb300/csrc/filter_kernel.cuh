@@ -108,6 +108,7 @@ struct FilterParams {
     SlotOut sl;
     BitsOut bo;
     uint32_t walk_chunk;  // streaming form: walk-list entries a warp reserves at a time, at least
+    uint32_t tile_cap;    // streaming form: entries of the tile list, which follows the walk list
     unsigned int *counter;
     unsigned int *err;
     uint32_t off_neg1, off_warp, warp_bytes, off_packed, off_inv, off_queue, off_meta, off_help;

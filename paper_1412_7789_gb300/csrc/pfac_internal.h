@@ -325,6 +325,7 @@ struct MatchRequest {
     uint32_t list_cap = 0;
     uint2 *walks = nullptr;
     uint32_t walk_cap = 0;
+    uint32_t tile_cap = 0;  // streaming form: tiles listed whole, after the walks
 };
 
 // The phased form of the filter kernel for one long text:
@@ -407,17 +408,25 @@ struct Tuning {
     int stall_help = 0;   // test aid: owners wait for one chunk more than their heavy tile has
 };
 
+// Capacities of the streaming form's lists, laid out after 32 bytes of counters:
+// walks that go on (8 bytes each, 16 in a batch), and tiles left to the walks'
+// launch as a whole (4 bytes, 16 in a batch).
+struct StreamLists {
+    uint32_t walk_cap = 0, tile_cap = 0;
+    size_t bytes() const { return 32 + 8ull * walk_cap + 4ull * tile_cap; }
+    size_t batch_bytes() const { return 32 + 16ull * walk_cap + 16ull * tile_cap; }
+};
+
 // The streaming form over a batch: whether it serves the automaton, and the
 // launches for nh (<= 32) automata it serves (rs: as launch_filter_multi's, the
-// units being tiles of kStreamTile positions).  walks: stream_batch_bytes(cap)
-// bytes whose first 32 are zeroed; walks past cap are settled where they are
-// found.
+// units being tiles of kStreamTile positions).  lists: l.batch_bytes() bytes
+// whose first 32 are zeroed; walks and tiles that find no room are settled where
+// they are found.
 bool stream_batch_serves(const DevTables &t, const Tuning &tu);
-uint32_t stream_batch_cap(uint64_t text_bytes);
-inline size_t stream_batch_bytes(uint32_t cap) { return 32 + 16ull * cap; }
+StreamLists stream_batch_lists(uint64_t text_bytes, uint32_t texts);
 constexpr uint32_t kStreamBatchMax = 32;
 cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *rs, uint32_t nh, OutMode mode,
-                                unsigned long long wait_ns, void *walks, uint32_t walk_cap, cudaStream_t stream);
+                                unsigned long long wait_ns, void *lists, const StreamLists &l, cudaStream_t stream);
 
 // One short text (dense ids or count): one thread per position, everything
 // from global memory (stream.cu).  Needs no scratch.
@@ -426,11 +435,10 @@ cudaError_t launch_at(const DevTables &t, const MatchRequest &r, OutMode mode, c
 
 // The streaming form (stream.cu) of one long text: whether it serves the text
 // with this tuning (any knob set asks for the filter kernel's own forms), the
-// room of its walk list, and the launch (r.list_count: two words, zeroed;
-// r.walks, r.walk_cap).
+// size of its lists, and the launch (r.list_count: 32 zeroed bytes; r.walks, the
+// walk list with the tile list after it; r.walk_cap, r.tile_cap).
 bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n);
-uint32_t stream_walk_cap(uint64_t n);
-inline size_t stream_bytes(uint32_t walk_cap) { return 32 + 8ull * walk_cap; }
+StreamLists stream_lists(uint64_t n);
 cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
                           cudaStream_t stream);
 

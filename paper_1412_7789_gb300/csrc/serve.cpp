@@ -252,11 +252,11 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     std::vector<pfac::CompactOut> outs(R);
     // The automata the streaming form serves take it when the wave's text is
     // long enough, its positions can be numbered in 32 bits, and its scratch
-    // (count, prefix, bits and ids of each unit, a planned text, the walk list's
-    // counters, 16 bytes per listed walk, and what rounding adds) stays
+    // (count, prefix, bits, ids and a list entry of each unit, a planned text,
+    // the lists' counters, 16 bytes per listed walk, and what rounding adds) stays
     // within what the requests were charged: the walk list takes the rest,
-    // for every eighth text byte at most and more than every 64th (a full list
-    // only costs time: the walks past it end where they were found).
+    // for every eighth text byte at most and more than every 128th (once it is
+    // full, tiles with many walks are listed whole).
     uint64_t wave_text = 0, stream_bytes = 0, charged = 0, needed = 32 + 3 * 256;
     for (uint32_t k = 0; k < L; ++k) {
         const ac_server_request &r = w.reqs[order[k]].r;
@@ -264,10 +264,11 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
         if (!s->streams[r.automaton]) continue;
         stream_bytes += r.n;
         charged += request_scratch(s, r);
-        needed += stream_units(r) * (4 + 8 + pfac::kStreamTile / 8 + 4ull * pfac::kStreamTile) + sizeof(pfac::BitsText);
+        needed += stream_units(r) * (4 + 8 + pfac::kStreamTile / 8 + 4ull * pfac::kStreamTile + 16) +
+                  sizeof(pfac::BitsText);
     }
     const uint64_t walk_room = charged > needed ? (charged - needed) / 16 : 0;
-    const bool streams = wave_streams(s, wave_text) && walk_room > stream_bytes / 64 &&
+    const bool streams = wave_streams(s, wave_text) && walk_room > stream_bytes / 128 &&
                          stream_bytes / pfac::kStreamTile + 2ull * L < (1ull << 32) / pfac::kStreamTile;
     auto streamed = [&](uint32_t a) { return streams && s->streams[a]; };
     // units: the other automata's first (with slots), then the streamed ones'
@@ -343,9 +344,13 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
     const size_t cb = round256(16ull * nh), nb = round256(4 * U), pb = 8 * U, sb = 8ull * pfac::kSlotCap * Uo;
     const size_t db = round256(plan_bytes + cb + nb + pb + sb + 8ull * pfac::kScanCtas);  // dense fallback: aligned
     const size_t stb = round256(db + 4ull * pfac::kDenseStride * Uo);
-    const uint32_t walk_cap =
-        Us ? static_cast<uint32_t>(std::min<uint64_t>(pfac::stream_batch_cap(stream_bytes), walk_room)) : 0u;
-    const size_t bb = round256(Us * (pfac::kStreamTile / 8)), wb = Us ? round256(pfac::stream_batch_bytes(walk_cap)) : 0,
+    pfac::StreamLists wl;
+    if (Us) {
+        wl.walk_cap = static_cast<uint32_t>(
+            std::min<uint64_t>(pfac::stream_batch_lists(stream_bytes, 0).walk_cap, walk_room));
+        wl.tile_cap = static_cast<uint32_t>(Us);
+    }
+    const size_t bb = round256(Us * (pfac::kStreamTile / 8)), wb = Us ? round256(wl.batch_bytes()) : 0,
                  ib = 4ull * pfac::kStreamTile * Us;
     const size_t bits_at = stb + round256(staged) + lsb;
     void *dev = nullptr;
@@ -432,7 +437,7 @@ cudaError_t launch_wave(ac_server_impl *s, WaveSlot &w) {
             e = cudaMemsetAsync(walks, 0, 32, w.stream);
             if (e == cudaSuccess)
                 e = pfac::launch_stream_batch(sts.data(), srs.data(), static_cast<uint32_t>(sts.size()), pfac::OUT_BITS,
-                                              s->tune[0].wait_ns, walks, walk_cap, w.stream);
+                                              s->tune[0].wait_ns, walks, wl, w.stream);
         }
     }
     for (uint32_t a = 0; a < nh && e == cudaSuccess && !s->multi; ++a) {

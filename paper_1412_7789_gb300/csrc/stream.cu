@@ -23,10 +23,7 @@ constexpr uint64_t kAtMax = 2u << 20;
 __host__ __device__ constexpr int at_block(int per) { return per == 1 ? 128 : 256; }
 
 // One lane per position (a text this short and the tables it touches stay in
-// L2).  A warp reads its PER x 32 bytes and the 16 after them once, one byte a
-// lane and load, and joins their codes into windows with log2(window) shuffles,
-// so a position costs little more than a byte load and a load per table level;
-// a lane's PER positions have theirs in flight together.
+// L2): match_run of 32 * PER positions a warp.
 template <int B, typename GT, int MODE, int PER>
 __global__ void __launch_bounds__(at_block(PER)) pfac_at(const __grid_constant__ FilterParams p) {
     __shared__ uint8_t cls8[256];
@@ -35,117 +32,22 @@ __global__ void __launch_bounds__(at_block(PER)) pfac_at(const __grid_constant__
     const uint64_t g0 = (static_cast<uint64_t>(blockIdx.x) * (at_block(PER) / 32) + (threadIdx.x >> 5)) * (32u * PER) + lane;
     uint32_t c[PER + 1];
     bool in[PER + 1];
-#pragma unroll
-    for (int j = 0; j <= PER; ++j) {
-        in[j] = g0 + 32u * j < p.n && (j < PER || lane < 16);
-        c[j] = in[j] ? __ldg(p.text + g0 + 32u * j) : 0u;
-    }
+    load_run<PER>(p.text, p.n, g0, lane, c, in);
     for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
     __syncthreads();
-    // codes, and which positions hold none (a byte in no keyword, or the text's end)
-    const bool id = B == 8 && p.identity;
-    uint32_t bad[PER + 1];  // bit i: position i of the 32
-#pragma unroll
-    for (int j = 0; j <= PER; ++j) {
-        if (!id) c[j] = cls8[c[j]];
-        bad[j] = __ballot_sync(kFull, !in[j] || (!id && c[j] == 0xFFu));
-        c[j] &= (1u << B) - 1u;
-    }
-    const uint32_t need = B == 8 ? p.k : p.k + p.k2;
-    uint32_t after[PER];  // 8-bit codes: the code after the window
-    if (B == 8) {
-        const uint32_t x = static_cast<uint32_t>(lane) + p.k;
-#pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const uint32_t y = __shfl_sync(kFull, c[j], x & 31u), z = __shfl_sync(kFull, c[j + 1], x & 31u);
-            after[j] = x < 32u ? y : z;
-        }
-    }
-#pragma unroll
-    for (uint32_t d = 1; d * B < 32u; d *= 2u) {  // windows of d codes -> 2 d
-        const uint32_t x = static_cast<uint32_t>(lane) + d;
-        uint32_t y = __shfl_sync(kFull, c[0], x & 31u);
-#pragma unroll
-        for (int j = 0; j <= PER; ++j) {  // (the last set's upper lanes are never read)
-            const uint32_t z = j < PER ? __shfl_sync(kFull, c[j < PER ? j + 1 : j], x & 31u) : y;
-            c[j] |= (x < 32u ? y : z) << (B * d);
-            y = z;
-        }
-    }
-    // first loads of all the lane's positions, then the second
-    int e[PER], r[PER];
-    uint4 h[PER];
-    bool walk[PER], keep[PER];
-    uint32_t s[PER], q[PER], m[PER];
-    // several positions a lane (longer texts, few of whose positions get past it):
-    // the root filter first, whose 128 KiB stay in L1, not a sector of a table
-    // in L2 for each position (2 MiB of ACGT 16.6 -> 14.7 us a call, of Zipf
-    // bytes 29.0 -> 25.8; short texts would wait for one load more)
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        keep[j] = true;
-        if (PER == 1) continue;
-        const uint32_t v = B == 8 ? ((c[j] & p.wmask) * kFilterHashMul) >> p.fshift
-                                  : c[j] & ((1u << (B * p.k)) - 1u);
-        keep[j] = (__ldg(p.Fg + (v >> 5)) << (v & 31u)) >> 31;
-    }
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        m[j] = __funnelshift_r(bad[j], bad[j + 1], lane);  // bit i: position i after this one
-        walk[j] = in[j];
-        r[j] = -1;
-        s[j] = q[j] = 0;
-        e[j] = 0;
-        h[j] = make_uint4(0u, 0u, 0u, 0u);
-        if (m[j] & ((1u << need) - 1u)) {
-            if (B == 8) walk[j] = false;  // no keyword is shorter than the state hash's window
-            continue;
-        }
-        if (!keep[j]) {
-            walk[j] = false;
-            e[j] = -1;
-            continue;
-        }
-        if (B == 8)
-            h[j] = __ldg(p.HK + filt::hk_slot(p, c[j] & p.wmask));
-        else
-            e[j] = __ldg(p.JK + (c[j] & ((1u << (B * p.k)) - 1u)));
-    }
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        if ((m[j] & ((1u << need) - 1u)) || !keep[j]) continue;
-        if (B == 8) {
-            walk[j] = !filt::hk_outcome(p, filt::hk_find(p, c[j] & p.wmask, h[j]), 0u, after[j], !((m[j] >> p.k) & 1u),
-                                        r[j], s[j], q[j]);
-        } else if (e[j] >= 0 && p.k2) {
-            q[j] = p.k + p.k2;
-            e[j] = __ldg(p.J2 + ((static_cast<uint64_t>(static_cast<uint32_t>(e[j]) - p.base_k) << (B * p.k2)) |
-                                 ((c[j] >> (B * p.k)) & ((1u << (B * p.k2)) - 1u))));
-        } else {
-            q[j] = p.k;
-        }
-    }
-    const TileText tt = make_text(p.text, p.out, p.n, 0u);
     uint32_t cnt = 0;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        if (B != 8 && !(m[j] & ((1u << need) - 1u))) {
-            walk[j] = e[j] >= 0;
-            s[j] = static_cast<uint32_t>(e[j]);
-            if (e[j] < 0) r[j] = decode_dead(e[j]);
-        }
+    match_run<B, GT, PER, (PER > 1)>(p, cls8, make_text(p.text, p.out, p.n, 0u), g0, lane, c, in, [&](int j, int r) {
         const uint64_t gi = g0 + 32u * j;
-        if (walk[j]) r[j] = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s[j], q[j]);
         if (MODE == OUT_DENSE) {
-            if (in[j]) p.out[gi] = r[j];
+            if (in[j]) p.out[gi] = r;
         } else if (MODE == OUT_COUNT) {
-            cnt += in[j] && r[j] >= 0 ? 1u : 0u;
+            cnt += r >= 0 ? 1u : 0u;
         } else {
-            if (in[j] && r[j] >= 0) p.bo.ids[gi] = r[j];
-            const uint32_t bits = __ballot_sync(kFull, in[j] && r[j] >= 0);
+            if (r >= 0) p.bo.ids[gi] = r;
+            const uint32_t bits = __ballot_sync(kFull, r >= 0);
             if (lane == 0 && in[j]) p.bo.bits[gi >> 5] = bits;
         }
-    }
+    });
     add_count<MODE>(p, cnt, lane);
 }
 
@@ -223,10 +125,12 @@ bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
     return t.stream.root == (t.stream.form == 2 ? t.k : t.fbits);
 }
 
-uint32_t stream_walk_cap(uint64_t n) {
-    // a walk for every eighth position, and each warp's last reservation
-    // (positions past that are settled where they are found)
-    return static_cast<uint32_t>(n / 8) + device_sm_count() * static_cast<uint32_t>(kMostWarps) * kWalkChunkEntries;
+StreamLists stream_lists(uint64_t n) {
+    // a walk for every eighth position, and each warp's last reservation; every tile
+    StreamLists l;
+    l.walk_cap = static_cast<uint32_t>(n / 8) + device_sm_count() * static_cast<uint32_t>(kMostWarps) * kWalkChunkEntries;
+    l.tile_cap = static_cast<uint32_t>(n / kTile) + 2u;
+    return l;
 }
 
 namespace {
@@ -247,6 +151,7 @@ cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mod
     if (mode == OUT_BITS && !r.bits.counts) return cudaErrorInvalidValue;
     p.f.walks = r.walks;
     p.f.walk_cap = r.walk_cap;
+    p.f.tile_cap = r.tile_cap;
     p.f.list_count = r.list_count;
     p.f.walk_chunk = walk_chunk(r.walk_cap);
     p.F1 = t.stream_F1 ? t.stream_F1 : t.F;
@@ -302,11 +207,15 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
 
 bool stream_batch_serves(const DevTables &t, const Tuning &tu) { return stream_serves(t, tu, 0); }
 
-uint32_t stream_batch_cap(uint64_t text_bytes) { return stream_walk_cap(text_bytes); }
+StreamLists stream_batch_lists(uint64_t text_bytes, uint32_t texts) {
+    StreamLists l = stream_lists(text_bytes);
+    l.tile_cap += 2u * texts;
+    return l;
+}
 
 cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *rs, uint32_t nh, OutMode mode,
-                                unsigned long long wait_ns, void *walks, uint32_t walk_cap, cudaStream_t stream) {
-    if (nh == 0 || nh > kStreamMultiMax || !walks || walk_cap == 0 || (mode != OUT_DENSE && mode != OUT_BITS))
+                                unsigned long long wait_ns, void *lists, const StreamLists &l, cudaStream_t stream) {
+    if (nh == 0 || nh > kStreamMultiMax || !lists || l.walk_cap == 0 || (mode != OUT_DENSE && mode != OUT_BITS))
         return cudaErrorInvalidValue;
     int sms = 0, max_smem = 0;
     cudaError_t e = filter_device_shape(&sms, &max_smem);
@@ -319,7 +228,7 @@ cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *
     std::lock_guard<std::mutex> lock(mu);
     Tuning tu;
     tu.wait_ns = wait_ns;
-    uint8_t *b = static_cast<uint8_t *>(walks);
+    uint8_t *b = static_cast<uint8_t *>(lists);
     wm.nh = nh;
     // one launch per form and step, then the walks of all
     bool next = false;  // after another of these launches
@@ -341,8 +250,9 @@ cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *
             p.f.aidx = a;
             p.f.list_count = reinterpret_cast<unsigned int *>(b);
             p.f.walks4 = reinterpret_cast<uint4 *>(b + 32);
-            p.f.walk_cap = walk_cap;
-            p.f.walk_chunk = walk_chunk(walk_cap);
+            p.f.walk_cap = l.walk_cap;
+            p.f.tile_cap = l.tile_cap;
+            p.f.walk_chunk = walk_chunk(l.walk_cap);
             wm.a[a] = p.f;
             filters = filters > p.f1bytes + p.f2bytes ? filters : p.f1bytes + p.f2bytes;
         }

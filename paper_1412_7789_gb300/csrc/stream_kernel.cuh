@@ -4,7 +4,8 @@
 //       test it against a root filter in shared memory, resolve the few
 //       positions that pass with one or two table loads, write the -1 of every
 //       other position, and list the walks that go further;
-//   pfac_stream_walks             one thread per listed walk.
+//   pfac_stream_walks             one thread per listed walk, and one lane per
+//       position of the tiles left to it as a whole (list_tile).
 //
 // Text: a warp takes tiles of 2048 positions (lane l the 16 bytes at 16 l of
 // each 512-byte chunk), with the next tile's loads issued as soon as a chunk's
@@ -231,6 +232,121 @@ static __device__ __noinline__ int match_at_far(const FilterParams &p, const uin
     return match_at<GT>(p, cls8, tt, gi, B);
 }
 
+// A warp's run of 32 * PER consecutive positions, lane l's g0, g0 + 32, ...  It
+// reads their bytes and the 16 after them once, one byte a lane and load, and
+// joins their codes into windows with log2(window) shuffles, so a position costs
+// little more than a byte load and a load per table level; a lane's PER positions
+// have theirs in flight together.  (g0 may lie before the text, and wraps then.)
+template <int PER>
+__device__ __forceinline__ void load_run(const uint8_t *text, uint64_t n, uint64_t g0, int lane, uint32_t (&c)[PER + 1],
+                                         bool (&in)[PER + 1]) {
+#pragma unroll
+    for (int j = 0; j <= PER; ++j) {
+        in[j] = g0 + 32u * j < n && (j < PER || lane < 16);
+        c[j] = in[j] ? __ldg(text + g0 + 32u * j) : 0u;
+    }
+}
+
+// put(j, id or -1) for each of the lane's positions (all lanes of the warp).
+template <int B, typename GT, int PER, bool FIRST, typename Put>
+__device__ __forceinline__ void match_run(const FilterParams &p, const uint8_t *cls8, const TileText &tt, uint64_t g0,
+                                          int lane, uint32_t (&c)[PER + 1], const bool (&in)[PER + 1], Put put) {
+    // codes, and which positions hold none (a byte in no keyword, or the text's end)
+    const bool id = B == 8 && p.identity;
+    uint32_t bad[PER + 1];  // bit i: position i of the 32
+#pragma unroll
+    for (int j = 0; j <= PER; ++j) {
+        if (!id) c[j] = cls8[c[j]];
+        bad[j] = __ballot_sync(kFull, !in[j] || (!id && c[j] == 0xFFu));
+        c[j] &= (1u << B) - 1u;
+    }
+    const uint32_t need = B == 8 ? p.k : p.k + p.k2;
+    uint32_t after[PER];  // 8-bit codes: the code after the window
+    if (B == 8) {
+        const uint32_t x = static_cast<uint32_t>(lane) + p.k;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t y = __shfl_sync(kFull, c[j], x & 31u), z = __shfl_sync(kFull, c[j + 1], x & 31u);
+            after[j] = x < 32u ? y : z;
+        }
+    }
+#pragma unroll
+    for (uint32_t d = 1; d * B < 32u; d *= 2u) {  // windows of d codes -> 2 d
+        const uint32_t x = static_cast<uint32_t>(lane) + d;
+        uint32_t y = __shfl_sync(kFull, c[0], x & 31u);
+#pragma unroll
+        for (int j = 0; j <= PER; ++j) {  // (the last set's upper lanes are never read)
+            const uint32_t z = j < PER ? __shfl_sync(kFull, c[j < PER ? j + 1 : j], x & 31u) : y;
+            c[j] |= (x < 32u ? y : z) << (B * d);
+            y = z;
+        }
+    }
+    // first loads of all the lane's positions, then the second
+    int e[PER], r[PER];
+    uint4 h[PER];
+    bool walk[PER], keep[PER];
+    uint32_t s[PER], q[PER], m[PER];
+    // FIRST (several positions a lane: longer texts, few of whose positions get
+    // past it): the root filter first, whose 128 KiB stay in L1, not a sector of a
+    // table in L2 for each position (2 MiB of ACGT 16.6 -> 14.7 us a call, of Zipf
+    // bytes 29.0 -> 25.8; short texts would wait for one load more)
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        keep[j] = true;
+        if (!FIRST) continue;
+        const uint32_t v = B == 8 ? ((c[j] & p.wmask) * kFilterHashMul) >> p.fshift
+                                  : c[j] & ((1u << (B * p.k)) - 1u);
+        keep[j] = (__ldg(p.Fg + (v >> 5)) << (v & 31u)) >> 31;
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        m[j] = __funnelshift_r(bad[j], bad[j + 1], lane);  // bit i: position i after this one
+        walk[j] = in[j];
+        r[j] = -1;
+        s[j] = q[j] = 0;
+        e[j] = 0;
+        h[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (m[j] & ((1u << need) - 1u)) {
+            if (B == 8) walk[j] = false;  // no keyword is shorter than the state hash's window
+            continue;
+        }
+        if (!keep[j]) {
+            walk[j] = false;
+            e[j] = -1;
+            continue;
+        }
+        if (B == 8)
+            h[j] = __ldg(p.HK + filt::hk_slot(p, c[j] & p.wmask));
+        else
+            e[j] = __ldg(p.JK + (c[j] & ((1u << (B * p.k)) - 1u)));
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if ((m[j] & ((1u << need) - 1u)) || !keep[j]) continue;
+        if (B == 8) {
+            walk[j] = !filt::hk_outcome(p, filt::hk_find(p, c[j] & p.wmask, h[j]), 0u, after[j], !((m[j] >> p.k) & 1u),
+                                        r[j], s[j], q[j]);
+        } else if (e[j] >= 0 && p.k2) {
+            q[j] = p.k + p.k2;
+            e[j] = __ldg(p.J2 + ((static_cast<uint64_t>(static_cast<uint32_t>(e[j]) - p.base_k) << (B * p.k2)) |
+                                 ((c[j] >> (B * p.k)) & ((1u << (B * p.k2)) - 1u))));
+        } else {
+            q[j] = p.k;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (B != 8 && !(m[j] & ((1u << need) - 1u))) {
+            walk[j] = e[j] >= 0;
+            s[j] = static_cast<uint32_t>(e[j]);
+            if (e[j] < 0) r[j] = decode_dead(e[j]);
+        }
+        if (walk[j])
+            r[j] = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(g0 + 32u * j), s[j], q[j]);
+        put(j, in[j] ? r[j] : -1);
+    }
+}
+
 // An id found at position g.  OUT_BITS with tile (the warp's bits of the tile
 // from position g0 on, in shared memory, every id of which passes here before
 // the tile's bits and count are written): the bit goes there.
@@ -284,7 +400,54 @@ __device__ __forceinline__ void blank_walk(const FilterParams &p, uint32_t slot)
 struct WalkRoom {
     uint32_t next, end;  // the warp's chunk
     bool full;           // nothing more to reserve (the counter is left alone then)
+    bool crowd;          // kSpread tiles were listed to spread them
 };
+
+// Tiles listed whole.  A tile with many candidates is not this launch's work: its
+// 20 or 24 warps an SM wait for one dependent load after another.  The walks'
+// launch takes such a tile with one lane a position (tile_run), over 48 warps an
+// SM.  Texts of 64 MiB, dense ids, ms: walks listed one by one and, where there was
+// no more room, done where they were found / these tiles listed whole / the filter
+// kernel, which keeps eight walks a lane in flight: one DNA letter 3.13 / 1.61 /
+// 2.10, one byte 3.45 / 1.75 / 2.11, a phrase of 78 bytes 3.30 / 2.50 / 2.64, a
+// repeat of 1,009 letters 4.26 / 2.20 / 2.06.  Listed are
+//   - tiles in which more than a quarter to a half of the positions looked up pass
+//     the filter (kQueue in pfac_stream2, half a tile in pfac_stream8);
+//   - once the walk list is full, tiles with more than kFew that pass (the walks of
+//     the others are settled where they are found);
+//   - in pfac_stream2 with S > 1, the first kSpread tiles with more candidates than
+//     the warp resolves in 8 rounds: a few of them in a text would each keep one
+//     warp busy long after the others have ended (5,000 keywords copied from the
+//     first 4 KiB of 16 MiB).  Where there are many (a repeat of 4,096 letters, 5 %
+//     of its positions walk) the warps resolve the rest: 64 MiB 429 us, all of them
+//     listed 850.
+constexpr uint32_t kSpread = 128;
+constexpr uint32_t kFew = 128;
+// True when tile t of sg is listed (all lanes).
+template <bool BATCH>
+__device__ __forceinline__ bool list_tile(const FilterParams &p, const Seg &sg, uint32_t t, int lane) {
+    uint32_t i = 0;
+    if (lane == 0) {
+        i = atomicAdd(p.list_count + 2, 1u);
+        if (i < p.tile_cap) {
+            if (BATCH)
+                p.walks4[p.walk_cap + i] = make_uint4(sg.unit0 + (t - sg.t0), 0u, p.aidx << 11, sg.item);
+            else
+                reinterpret_cast<uint32_t *>(p.walks + p.walk_cap)[i] = t;
+        }
+    }
+    return __shfl_sync(kFull, i, 0) < p.tile_cap;
+}
+
+// Whether kSpread tiles were listed for their few but slow candidates (all lanes).
+__device__ __forceinline__ bool crowded(const FilterParams &p, WalkRoom &room, int lane) {
+    if (!room.crowd) {
+        uint32_t i = 0;
+        if (lane == 0) i = atomicAdd(p.list_count + 3, 1u);
+        room.crowd = __shfl_sync(kFull, i, 0) >= kSpread;
+    }
+    return room.crowd;
+}
 template <bool BATCH>
 __device__ __forceinline__ bool push_walk(const StreamParams &p, const Seg &sg, WalkRoom &room, bool want, uint32_t g,
                                           uint32_t s, int lane) {
@@ -449,20 +612,17 @@ __device__ __forceinline__ uint32_t codes16(const uint4 &v) {
 // Non-zero when one of 16 bytes is in no keyword: a byte is in one exactly when
 // the keyword byte of its code equals it, and a byte permute selected by twice
 // the codes (each word's next byte's moved to the high nibble) picks those.
+__device__ __forceinline__ uint32_t unknown4(const FilterParams &f, uint32_t w) {
+    const uint32_t x = w & 0x06060606u;
+    return w ^ __byte_perm(f.dsel_lo, f.dsel_hi, __byte_perm(x | (x >> 4), 0u, 0x4420u));
+}
 __device__ __forceinline__ uint32_t unknown16(const FilterParams &f, const uint4 &v) {
-    auto word = [&](uint32_t w) {
-        const uint32_t x = w & 0x06060606u;
-        return w ^ __byte_perm(f.dsel_lo, f.dsel_hi, __byte_perm(x | (x >> 4), 0u, 0x4420u));
-    };
-    return word(v.x) | word(v.y) | word(v.z) | word(v.w);
+    return unknown4(f, v.x) | unknown4(f, v.y) | unknown4(f, v.z) | unknown4(f, v.w);
 }
 
 // The same, a flag per byte.
 __device__ __forceinline__ uint32_t unknown_marks(const FilterParams &f, const uint4 &v) {
-    auto word = [&](uint32_t w) {
-        const uint32_t x = w & 0x06060606u;
-        return filt::nonzero_bytes(w ^ __byte_perm(f.dsel_lo, f.dsel_hi, __byte_perm(x | (x >> 4), 0u, 0x4420u)));
-    };
+    auto word = [&](uint32_t w) { return filt::nonzero_bytes(unknown4(f, w)); };
     return word(v.x) | (word(v.y) << 4) | (word(v.z) << 8) | (word(v.w) << 12);
 }
 
@@ -472,15 +632,22 @@ __device__ __forceinline__ uint32_t codes_at(const uint32_t *packed, uint32_t i)
 }
 
 // Whether the `need` (<= 16) bytes from text position gi on are inside the
-// text and all in keywords (cls8: the byte table).
-__device__ __forceinline__ bool bytes_known(const uint8_t *text, uint64_t n, const uint8_t *cls8, uint64_t gi,
+// text and all in keywords: at most five aligned words, all in flight together
+// (those that hold one of the bytes), and byte permutes as in unknown16.
+__device__ __forceinline__ bool bytes_known(const FilterParams &f, const uint8_t *text, uint64_t n, uint64_t gi,
                                             uint32_t need) {
     if (gi + need > n) return false;
-    uint32_t b[16], bad = 0;
+    const uint8_t *t = text + gi;
+    const uint32_t a = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(t) & 3u), words = (a + need + 3u) >> 2;
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(t - a);
+    uint32_t x[5], bad = 0;
 #pragma unroll
-    for (uint32_t j = 0; j < 16; ++j) b[j] = j < need ? __ldg(text + gi + j) : 0u;  // all in flight together
+    for (uint32_t j = 0; j < 5; ++j) x[j] = j < words ? __ldg(w + j) : 0u;
 #pragma unroll
-    for (uint32_t j = 0; j < 16; ++j) bad |= j < need && cls8[b[j]] == 0xFFu ? 1u : 0u;
+    for (uint32_t j = 0; j < 4; ++j) {
+        const uint32_t v = __funnelshift_r(x[j], x[j + 1], 8u * a), left = need - 4u * j;
+        if (need > 4u * j) bad |= unknown4(f, v) & (left >= 4u ? 0xFFFFFFFFu : (1u << (8u * left)) - 1u);
+    }
     return bad == 0;
 }
 
@@ -524,7 +691,7 @@ __device__ __forceinline__ void resolve2(const StreamParams &p, const Seg &sg, W
                 doubt = ((m >> (i & 15u)) & ((1u << (f.k + f.k2)) - 1u)) != 0u;
             }
         } else {
-            doubt = doubt && !bytes_known(sg.text, sg.n, f.cls8g, gi, f.k + f.k2);
+            doubt = doubt && !bytes_known(f, sg.text, sg.n, gi, f.k + f.k2);
         }
         if (doubt) {
             walk = true;
@@ -638,6 +805,15 @@ __device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uin
         }
         __syncwarp();  // packed is written
         constexpr int kBits = 4 * kPer / kAcc;  // bits per accumulator
+        if (S == 1 && room.full) {
+            uint32_t found = 0;
+#pragma unroll
+            for (int a = 0; a < kAcc; ++a) found += static_cast<uint32_t>(__popc(acc[a]));
+            if (__reduce_add_sync(kFull, found) > kFew && list_tile<BATCH>(p.f, sg, t, lane)) {
+#pragma unroll
+                for (int a = 0; a < kAcc; ++a) acc[a] = 0;
+            }
+        }
         const uint32_t g0 = (t - sg.t0) * kTile;
 #pragma unroll
         for (int a = 0; a < kAcc; ++a) {
@@ -649,38 +825,10 @@ __device__ __forceinline__ void tiles2(const StreamParams &p, uint8_t *smem, uin
                        16u * static_cast<uint32_t>(lane) + S * (b % kPer) + (S - 1u);
             };
             const uint32_t total = __reduce_add_sync(kFull, static_cast<uint32_t>(__popc(m)));
-            if (S > 1 && total > kQueue / S) {
-                // a tile dense in survivors: all of them to the walk list,
-                // unresolved, in one reservation (the positions before or
-                // past the text as empty entries)
-                uint32_t base = p.f.walk_cap;
-                const uint32_t need = total * S;
-                if (!room.full) {
-                    if (lane == 0) base = atomicAdd(p.f.list_count + 1, need);
-                    base = __shfl_sync(kFull, base, 0);
-                    room.full = base >= p.f.walk_cap || p.f.walk_cap - base < need;
-                    if (base > p.f.walk_cap) base = p.f.walk_cap;
-                }
-                uint32_t all = 0, o = base + S * warp_excl(static_cast<uint32_t>(__popc(m)), all, lane);
-                fill_done<MODE, false>(true, lane);
-                for (; m; m &= m - 1u) {
-                    const uint32_t g = g0 + sample(__ffs(m) - 1);
-#pragma unroll 1
-                    for (uint32_t x = 0; x < S; ++x, ++o) {
-                        const bool in = text_pos(sg, g - x) < sg.n;
-                        if (o >= p.f.walk_cap) {
-                            if (in) settle_here<MODE>(p, sg, g - x, 2u, cnt);
-                        } else if (in) {
-                            store_walk<BATCH>(p.f, sg, o, g - x, 0u);
-                        } else {
-                            blank_walk<BATCH>(p.f, o);
-                        }
-                    }
-                }
-                __syncwarp();
+            if (S > 1 && total > kQueue / S && (total > kQueue || room.full || !crowded(p.f, room, lane)) &&
+                list_tile<BATCH>(p.f, sg, t, lane))
                 continue;
-            }
-            if (S > 1 && p.f2bytes) {
+            if (S > 1 && p.f2bytes && total <= kQueue) {
                 // 3. the second filter drops the chance hits among the samples
                 uint32_t at = 0;
                 for (; left; left = __ballot_sync(kFull, m != 0u)) {
@@ -866,7 +1014,9 @@ __device__ __forceinline__ void tiles8(const StreamParams &p, uint8_t *smem, uin
         const uint32_t mine = static_cast<uint32_t>(__popc(m[0]) + __popc(m[1]));
         uint32_t at = 0;
         if (!__any_sync(kFull, mine != 0u)) continue;
-        for (uint32_t o = warp_excl(mine, at, lane), first = 0;;) {
+        const uint32_t below = warp_excl(mine, at, lane);
+        if ((at > kTile / 2 || (room.full && at > kFew)) && list_tile<BATCH>(p.f, sg, t, lane)) continue;
+        for (uint32_t o = below, first = 0;;) {
             // the lane's survivors o, o + 1, ... of the warp's; the queue holds
             // those from `first` on
             const uint32_t end = first + kQueue;
@@ -937,7 +1087,7 @@ __device__ __forceinline__ void stream_text(const StreamParams &p) {
     fill_constant(smem + p.off_none);
     load_filters(p, smem);
     __syncthreads();  // the filters are in place
-    WarpState ws{0u, 0u, {0u, 0u, false}};
+    WarpState ws{0u, 0u, {0u, 0u, false, false}};
     if constexpr (FORM == 2)
         tiles2<S, MODE, false>(p, smem, p.off_warp, none, sg, t, p.ntiles, step, pol, r, ws);
     else
@@ -1040,7 +1190,7 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
     __syncthreads();
     TileRegs r;
     r.look = make_uint4(0u, 0u, 0u, 0u);
-    WarpState ws{0u, 0u, {0u, 0u, false}};
+    WarpState ws{0u, 0u, {0u, 0u, false, false}};
     const uint32_t first = start;
     for (uint32_t k = 0; k < mp.nh; ++k) {
         const uint32_t a = (first + k) % mp.nh;
@@ -1119,9 +1269,55 @@ __device__ __forceinline__ int finish_walk(const FilterParams &p, const uint8_t 
     const uint64_t gi = text_pos(sg, g);
     const uint32_t s = e & 0x7FFFFFFFu;
     // 2-bit codes: the walk so far took the codes for keyword bytes'
-    if (s && (B == 8 || bytes_known(sg.text, sg.n, cls8, gi, p.k + p.k2)))
+    if (s && (B == 8 || bytes_known(p, sg.text, sg.n, gi, p.k + p.k2)))
         return filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(gi), s, p.k + p.k2 + (e >> 31));
     return match_at<GT>(p, cls8, tt, gi, B);
+}
+
+// How much the launch has to do: walks, and runs of kRun positions (a warp's at a
+// time) of the tiles listed whole.
+constexpr int kRunPer = 1;
+constexpr uint32_t kRun = 32u * kRunPer, kTileRuns = kTile / kRun;
+struct Listed {
+    uint32_t m, runs;
+};
+__device__ __forceinline__ Listed listed(const FilterParams &p) {
+    const uint4 c = __ldcg(reinterpret_cast<const uint4 *>(p.list_count));  // (read once: what is compared is what is used)
+    Listed l;
+    l.m = c.y < p.walk_cap ? c.y : p.walk_cap;
+    l.runs = (c.z < p.tile_cap ? c.z : p.tile_cap) * kTileRuns;
+    return l;
+}
+
+// The first run a warp takes: a warp of each CTA first, from the CTA after those
+// that take the walks on, so that a few runs go to as many SMs, and to CTAs that
+// started early.  (16 MiB of ACGT, two tiles listed: 4 runs a CTA from the first
+// CTA on 67 us a call, one from the first / the last / this one 46.5 / 44.9 / 43.3.)
+__device__ __forceinline__ uint32_t first_run(const Listed &l) {
+    const uint32_t after = (l.m + blockDim.x - 1u) / blockDim.x % gridDim.x;
+    return (threadIdx.x / 32u) * gridDim.x + (blockIdx.x >= after ? blockIdx.x - after : blockIdx.x + gridDim.x - after);
+}
+
+// One warp: the kRun positions of a listed tile from g on (a multiple of kRun).
+template <int B, typename GT, int MODE>
+__device__ __forceinline__ void tile_run(const FilterParams &p, const uint8_t *cls8, const Seg &sg, uint32_t g,
+                                         uint32_t &cnt, int lane) {
+    const uint64_t g0 = text_pos(sg, g + static_cast<uint32_t>(lane));
+    uint32_t c[kRunPer + 1];
+    bool in[kRunPer + 1];
+    load_run<kRunPer>(sg.text, sg.n, g0, lane, c, in);
+    match_run<B, GT, kRunPer, false>(p, cls8, make_text(sg.text, sg.out, sg.n, 0u), g0, lane, c, in, [&](int j, int r) {
+        if (MODE != OUT_BITS) {
+            put_id<MODE>(p, sg, g + 32u * j + static_cast<uint32_t>(lane), r, cnt);
+            return;
+        }
+        const uint32_t b = g + 32u * j + sg.bit0, bits = __ballot_sync(kFull, r >= 0);
+        if (r >= 0) p.bo.ids[b + static_cast<uint32_t>(lane)] = r;
+        if (lane == 0 && bits) {
+            p.bo.bits[b >> 5] = bits;
+            atomicAdd(p.bo.counts + b / kTile, static_cast<uint32_t>(__popc(bits)));
+        }
+    });
 }
 
 template <int B, typename GT, int MODE>
@@ -1130,16 +1326,23 @@ __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const
     const int lane = threadIdx.x & 31;
     allow_next();  // the lists' scan
     wait_previous();
-    const uint32_t listed = *reinterpret_cast<volatile const unsigned int *>(p.list_count + 1);
-    const uint32_t m = listed < p.walk_cap ? listed : p.walk_cap;
-    if (blockIdx.x * blockDim.x >= m) return;
+    const Listed l = listed(p);
+    const uint32_t first = first_run(l), *tiles = reinterpret_cast<const uint32_t *>(p.walks + p.walk_cap);
+    if (blockIdx.x * blockDim.x >= l.m && first % gridDim.x >= l.runs) return;
+    uint32_t t = first < l.runs ? tiles[first / kTileRuns] : 0u;
     for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
     __syncthreads();
     const Seg sg = make_seg(p.text, p.out, p.n);
     uint32_t cnt = 0;
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-        const uint2 e = p.walks[j];  // (not by the read-only path: written by the launch before)
+    // (not by the read-only path: written by the launch before)
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < l.m; j += gridDim.x * blockDim.x) {
+        const uint2 e = p.walks[j];
         if (e.x != 0xFFFFFFFFu) put_id<MODE>(p, sg, e.x, finish_walk<GT>(p, cls8, sg, e.x, e.y, B), cnt);
+    }
+    for (uint32_t j = first; j < l.runs;) {
+        tile_run<B, GT, MODE>(p, cls8, sg, t * kTile + kRun * (j % kTileRuns), cnt, lane);
+        j += gridDim.x * (blockDim.x / 32u);
+        if (j < l.runs) t = tiles[j / kTileRuns];
     }
     add_count<MODE>(p, cnt, lane);
 }
@@ -1152,14 +1355,43 @@ struct WalkMulti {
 };
 static_assert(sizeof(WalkMulti) <= 32764, "kernel parameters are limited to 32764 bytes");
 
+// The segment of an entry's unit.
+template <int MODE>
+__device__ __forceinline__ Seg entry_seg(const FilterParams &p, const uint4 &e) {
+    const Work wk = load_work(p.batch, p.lists, 0u);
+    const uint4 *q = reinterpret_cast<const uint4 *>(wk.list + e.w);
+    const uint4 x = __ldg(q), y = __ldg(q + 1);
+    Seg sg = make_seg(p.text + (x.x | (static_cast<uint64_t>(x.y) << 32)),
+                      MODE == OUT_DENSE ? p.out + (y.x | (static_cast<uint64_t>(y.y) << 32)) : nullptr,
+                      x.z | (static_cast<uint64_t>(x.w) << 32));
+    sg.t0 = e.x - y.z;
+    sg.bit0 = MODE == OUT_BITS ? (p.sl.ubase + e.x) * kTile : 0u;
+    return sg;
+}
+
+// An entry's walk, and tile_run of an entry's tile: out of line, as the copies
+// for every kind of automaton would spill.
+template <typename GT, int MODE>
+static __device__ __noinline__ void entry_walk(const FilterParams &p, const uint8_t *cls8, const uint4 e, uint32_t g) {
+    uint32_t cnt = 0;
+    const Seg sg = entry_seg<MODE>(p, e);
+    put_id<MODE>(p, sg, g, finish_walk<GT>(p, cls8, sg, g, e.y, p.kind >> 8), cnt);
+}
+template <int B, typename GT, int MODE>
+static __device__ __noinline__ void entry_run(const FilterParams &p, const uint8_t *cls8, const uint4 e, uint32_t g,
+                                              int lane) {
+    uint32_t cnt = 0;
+    tile_run<B, GT, MODE>(p, cls8, entry_seg<MODE>(p, e), g, cnt, lane);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const __grid_constant__ WalkMulti mp) {
     extern __shared__ __align__(16) uint8_t msm[];
+    const int lane = threadIdx.x & 31;
     allow_next();
     wait_previous();
-    const uint32_t listed = *reinterpret_cast<volatile const unsigned int *>(mp.a[0].list_count + 1);
-    const uint32_t m = listed < mp.a[0].walk_cap ? listed : mp.a[0].walk_cap;
-    if (blockIdx.x * blockDim.x >= m) return;
+    const Listed l = listed(mp.a[0]);
+    if (blockIdx.x * blockDim.x >= l.m && first_run(l) % gridDim.x >= l.runs) return;
     FilterParams *ps = reinterpret_cast<FilterParams *>(msm);
     uint8_t *cls = msm + mp.nh * sizeof(FilterParams);
     for (uint32_t i = threadIdx.x; i < mp.nh * static_cast<uint32_t>(sizeof(FilterParams) / 4); i += blockDim.x)
@@ -1167,22 +1399,31 @@ __global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const _
     for (uint32_t i = threadIdx.x; i < mp.nh * 256u; i += blockDim.x) cls[i] = __ldg(mp.a[i >> 8].cls8g + (i & 255u));
     __syncthreads();
     uint32_t cnt = 0;
-    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
+    for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < l.m; j += gridDim.x * blockDim.x) {
         const uint4 e = mp.a[0].walks4[j];
         if (e.x == 0xFFFFFFFFu) continue;
         const uint32_t a = e.z >> 11, g = e.z & (kTile - 1u);
         const FilterParams &p = ps[a];
-        const Work wk = load_work(p.batch, p.lists, 0u);
-        const uint4 *q = reinterpret_cast<const uint4 *>(wk.list + e.w);
-        const uint4 x = __ldg(q), y = __ldg(q + 1);
-        Seg sg = make_seg(p.text + (x.x | (static_cast<uint64_t>(x.y) << 32)),
-                          MODE == OUT_DENSE ? p.out + (y.x | (static_cast<uint64_t>(y.y) << 32)) : nullptr,
-                          x.z | (static_cast<uint64_t>(x.w) << 32));
-        sg.t0 = e.x - y.z;
-        sg.bit0 = MODE == OUT_BITS ? (p.sl.ubase + e.x) * kTile : 0u;
-        const int r = (p.kind & 0xFFu) == 16u ? finish_walk<int16_t>(p, cls + 256u * a, sg, g, e.y, p.kind >> 8)
-                                              : finish_walk<int32_t>(p, cls + 256u * a, sg, g, e.y, p.kind >> 8);
-        put_id<MODE>(p, sg, g, r, cnt);
+        if ((p.kind & 0xFFu) == 16u)
+            entry_walk<int16_t, MODE>(p, cls + 256u * a, e, g);
+        else
+            entry_walk<int32_t, MODE>(p, cls + 256u * a, e, g);
+    }
+    for (uint32_t j = first_run(l); j < l.runs; j += gridDim.x * (blockDim.x / 32u)) {
+        const uint4 e = mp.a[0].walks4[mp.a[0].walk_cap + j / kTileRuns];
+        const uint32_t a = e.z >> 11, g = kRun * (j % kTileRuns);
+        const FilterParams &p = ps[a];
+        const uint8_t *cls8 = cls + 256u * a;
+        if ((p.kind >> 8) == 2u) {
+            if ((p.kind & 0xFFu) == 16u)
+                entry_run<2, int16_t, MODE>(p, cls8, e, g, lane);
+            else
+                entry_run<2, int32_t, MODE>(p, cls8, e, g, lane);
+        } else if ((p.kind & 0xFFu) == 16u) {
+            entry_run<8, int16_t, MODE>(p, cls8, e, g, lane);
+        } else {
+            entry_run<8, int32_t, MODE>(p, cls8, e, g, lane);
+        }
     }
 }
 

@@ -175,6 +175,74 @@ def test_more_walks_than_listed(letters, lens):
         _check(a, text, want, 3, 0)
 
 
+def _event_us(f):
+    """Median of five timings of three calls."""
+    import torch
+
+    f()
+    torch.cuda.synchronize()
+    out = []
+    for _ in range(5):
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        for _ in range(3):
+            f()
+        t1.record()
+        torch.cuda.synchronize()
+        out.append(t0.elapsed_time(t1) * 1000 / 3)
+    return sorted(out)[2]
+
+
+@pytest.mark.parametrize("kind,block", [("one letter", 640), ("repeat of 1009", 640), ("one byte", 512), ("phrase", 512)])
+def test_repetitive_texts_are_no_slower(kind, block):
+    """Texts where most positions walk far: as built, dense ids take no longer
+    than in the filter kernel with its own best block (a quarter more allowed
+    for the spread of the timings)."""
+    import torch
+
+    n = 8 << 20
+    if kind == "one letter":
+        unit, pats = b"A", [b"A" * m for m in (16, 20, 60)] + [b"ACGT" * 10, b"TTGACCA" * 3]
+    elif kind == "repeat of 1009":
+        unit = bytes(_letters(1009, b"ACGT", 6))
+        at = workloads.rng(2).integers(0, 1009, size=500)
+        lens = workloads.rng(3).integers(16, 65, size=500)
+        pats = [(unit * 2)[o:o + m] for o, m in zip(at.tolist(), lens.tolist())]
+    elif kind == "one byte":
+        unit, pats = b"x", [b"x" * m for m in (6, 9, 40)] + [bytes(range(40, 120)), b"xyzw" * 3]
+    else:
+        unit = b"the quick brown fox jumps over the lazy dog while the cat sleeps in the sun. "
+        at = workloads.rng(4).integers(0, len(unit), size=200)
+        lens = workloads.rng(5).integers(4, 41, size=200)
+        pats = [(unit * 2)[o:o + m] for o, m in zip(at.tolist(), lens.tolist())]
+    text = torch.from_numpy(np.tile(np.frombuffer(unit, dtype=np.uint8), n // len(unit) + 1)[:n].copy()).cuda()
+    ids = torch.empty(n, dtype=torch.int32, device="cuda")
+    with api.Automaton(pats) as a, api.Automaton(pats) as b:
+        b.set_tuning(block=block)
+        built, tuned = _event_us(lambda: a.match(text, out=ids)), _event_us(lambda: b.match(text, out=ids))
+    assert built <= 1.25 * tuned, (built, tuned)
+
+
+@pytest.mark.parametrize("letters,shortest", [(b"ACGT", 16), (b"ACGT", 8), (b"ACGT", 4),
+                                              (b"abcdefghijklmnopqrstuvwxyz", 6)])
+def test_walks_fill_the_list_part_way(letters, shortest):
+    """A repeat of 40 letters where a run of 12 starts walks 26 letters or more:
+    few enough for a tile to be resolved in its warp, and more walks than the
+    list holds, so that later tiles are listed whole (dense ids, count and the
+    compacted list; the last tile ends inside the text)."""
+    n = (12 << 20) + 1234
+    unit = bytes(_letters(40, letters, 21))
+    text = np.tile(np.frombuffer(unit, dtype=np.uint8), n // 40 + 1)[:n].copy()
+    text[(3 << 20):(3 << 20) + 3000] = ord("#")
+    pats = [(unit * 3)[o:o + 26 + o] for o in range(12)] + [b"".join(bytes([letters[(i * j) % 4]]) for i in range(shortest))
+                                                         for j in range(1, 4)]
+    want = oracle.pfac_ids(pats, text)
+    assert n // 5 < (want >= 0).sum() < n // 2
+    with api.Automaton(pats) as a:
+        assert a.info()["min_len"] == shortest
+        _check(a, text, want, 5, 1)
+
+
 def test_list_capacity_is_kept():
     """A compacted list longer than its capacity: the first entries and the
     whole count, and nothing written past the capacity."""
@@ -237,6 +305,38 @@ def test_batch_streams(names, reserve):
                     if t.size:
                         want[o + 1:o + 1 + t.size] = oracle.pfac_ids(loads[a][1], t)
                 assert np.array_equal(got, want)
+    finally:
+        for a in autos:
+            a.close()
+
+
+@pytest.mark.parametrize("reserve", [1 << 22, 1 << 13])
+def test_batch_of_texts_dense_in_walks(reserve):
+    """Texts of one letter in a plan with lists: tiles listed whole, and (the
+    smaller plan) more of them than the tile list holds."""
+    import torch
+
+    lens = [300_001, 5, 2048, 700_003, 4096 + 7]
+    sets = [[b"A" * m for m in (16, 20, 60)] + [b"ACGT" * 10], [b"A" * m for m in (4, 33)] + [b"ACGTTGCA" * 3],
+            [b"x" * m for m in (6, 9, 40)] + [bytes(range(40, 120))]]
+    which = [0, 1, 2, 2, 1, 0, 1, 2, 0, 1]
+    lens = lens + lens
+    offs = np.concatenate([[0], np.cumsum(lens)[:-1]]) + 1
+    total = int(sum(lens)) + 1
+    buf = np.zeros(total, dtype=np.uint8)
+    for o, m, a in zip(offs, lens, which):
+        buf[o:o + m] = sets[a][0][0]
+        buf[o + m // 2] = ord("C") if a < 2 else ord("y")
+    autos = [api.Automaton(p) for p in sets]
+    try:
+        out = torch.full((total,), -7, dtype=torch.int32, device="cuda")
+        items = api.items_to_device(api.batch_items(offs, lens, offs, which))
+        with api.BatchPlan([a.handle for a in autos], len(lens)) as plan:
+            plan.reserve_lists(reserve)
+            plan.run(torch.from_numpy(buf).cuda(), items, len(lens), out)
+        got = out.cpu().numpy()
+        for o, m, a in zip(offs, lens, which):
+            assert np.array_equal(got[o:o + m], oracle.pfac_ids(sets[a], buf[o:o + m]))
     finally:
         for a in autos:
             a.close()
