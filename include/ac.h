@@ -265,8 +265,9 @@ ac_status ac_export_jump(ac_handle h, int16_t *J, uint32_t *k, uint32_t *base_k,
  * longer ones that the streaming form serves (DNA letters with a root window
  * of 10 codes, or 8-bit codes with keywords of 4 bytes or more) a list of walks
  * and one of tiles from the library's stream-ordered pool: 8 bytes for every
- * eighth text byte, 4 for every 2,048, and 2 MB; where the device has no room
- * for it, the filter kernel is taken instead.  That kernel (every other automaton or tuning) takes 16 bytes (the
+ * eighth text byte (DNA letters: every sixteenth, and in a captured graph none),
+ * 4 for every 2,048, and 2 MB; where the device has no room for it, the filter
+ * kernel is taken instead.  That kernel (every other automaton or tuning) takes 16 bytes (the
  * tile counter), or none for a text short enough that each of its tiles is
  * some warp's first; its phased form (8-bit codes from 4 MiB on; see
  * ac_tuning.survivor_list) also takes its survivor and walk lists from the
@@ -284,7 +285,8 @@ ac_status ac_match(ac_handle h, const uint8_t *d_text, uint64_t n, int32_t *d_ou
  * (cudaMallocFromPoolAsync) on `stream`; the pool keeps the memory it grows to
  * until the process exits.  With the tuning as built: a bit and an id for each
  * position (written where it matches only), per 2,048 positions a count and a
- * prefix sum, and the lists of ac_match: about 5.2 bytes per text byte.
+ * prefix sum, and the lists of ac_match: about 5.2 bytes per text byte (DNA
+ * letters 4.7).
  * The filter kernel (other tunings and automata, or no room for that): per
  * tile a match count, a prefix sum, 32 match slots and a dense fallback of 4
  * bytes per position, about 4.4 bytes per text byte; for its phased form the

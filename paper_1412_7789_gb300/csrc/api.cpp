@@ -274,10 +274,21 @@ cudaError_t pool_alloc(ac_automaton *h, size_t bytes, cudaStream_t st, void **ou
     return e;
 }
 
+// Whether the stream is being captured.  (Where that cannot be told, the call
+// itself will fail.)
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return s == cudaStreamCaptureStatusActive;
+}
+
 // The streaming form of one long text, its lists from the pool.  *room
 // = false: no memory for them, and nothing was enqueued.
 cudaError_t run_stream(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode, cudaStream_t st, bool *room) {
-    const pfac::StreamLists l = pfac::stream_lists(r.n);
+    const pfac::StreamLists l = pfac::stream_lists(h->dev.stream.form, r.n, capturing(st));
     r.walk_cap = l.walk_cap;
     r.tile_cap = l.tile_cap;
     void *scratch = nullptr;
@@ -339,12 +350,13 @@ cudaError_t run_tiled(ac_automaton *h, pfac::MatchRequest r, pfac::OutMode mode,
 // its scratch from the pool.  *room as above.
 cudaError_t run_bits(ac_automaton *h, const uint8_t *text, uint64_t n, const pfac::CompactOut &out, bool full,
                      cudaStream_t st, bool *room) {
-    const size_t bytes = pfac::bits_scratch_bytes(h->dev, h->tuning, text, n, full);
+    const bool captured = capturing(st);
+    const size_t bytes = pfac::bits_scratch_bytes(h->dev, h->tuning, text, n, full, captured);
     void *scratch = nullptr;
     cudaError_t e = pool_alloc(h, bytes, st, &scratch);
     *room = e != cudaErrorMemoryAllocation;
     if (e != cudaSuccess) return e;
-    e = pfac::enqueue_bits(h->dev, h->tuning, text, n, out, full, scratch, bytes, st);
+    e = pfac::enqueue_bits(h->dev, h->tuning, text, n, out, full, captured, scratch, bytes, st);
     const cudaError_t e2 = cudaFreeAsync(scratch, st);
     return e != cudaSuccess ? e : e2;
 }

@@ -355,12 +355,12 @@ struct Layout {
     bool small;
 };
 
-Layout layout_of(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full) {
+Layout layout_of(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full, bool captured) {
     Layout l{};
     l.small = at_serves(t, tu, n);
     const uint64_t head = l.small ? 0u : reinterpret_cast<uintptr_t>(text) & 15u;
     l.ntiles = static_cast<uint32_t>((n + head + kTile - 1) / kTile);
-    if (!l.small) l.lists = stream_lists(n);
+    if (!l.small) l.lists = stream_lists(t.stream.form, n, captured);
     size_t at = 256;
     auto take = [&](size_t bytes) {
         const size_t o = at;
@@ -399,15 +399,16 @@ cudaError_t launch_bits_texts(const BitsText *texts, uint32_t nt, uint32_t units
     return launch_next(bits_gather_texts, need < sms * 6u ? need : sms * 6u, kThreads, 0u, stream, p, texts, nt);
 }
 
-size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full) {
-    return layout_of(t, tu, text, n, full).bytes;
+size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full,
+                          bool captured) {
+    return layout_of(t, tu, text, n, full, captured).bytes;
 }
 
 cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, const CompactOut &out,
-                         bool full, void *scratch, size_t scratch_bytes, cudaStream_t stream) {
+                         bool full, bool captured, void *scratch, size_t scratch_bytes, cudaStream_t stream) {
     if (!bits_serve(t, tu, n) || n == 0 || n > 0xFFFFFFFFull || !scratch || (full && (!t.full_rec || !t.full_dups)))
         return cudaErrorInvalidValue;
-    const Layout l = layout_of(t, tu, text, n, full);
+    const Layout l = layout_of(t, tu, text, n, full, captured);
     if (scratch_bytes < l.bytes) return cudaErrorInvalidValue;
     uint8_t *b = static_cast<uint8_t *>(scratch);
     MatchRequest r;

@@ -438,7 +438,7 @@ cudaError_t launch_at(const DevTables &t, const MatchRequest &r, OutMode mode, c
 // size of its lists, and the launch (r.list_count: 32 zeroed bytes; r.walks, the
 // walk list with the tile list after it; r.walk_cap, r.tile_cap).
 bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n);
-StreamLists stream_lists(uint64_t n);
+StreamLists stream_lists(uint32_t form, uint64_t n, bool captured);
 cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mode, const Tuning &tu,
                           cudaStream_t stream);
 
@@ -456,9 +456,10 @@ struct alignas(16) BitsText {
 // (b.counts[u], u < units; prefix: their exclusive sums, from any start).
 cudaError_t launch_bits_texts(const BitsText *texts, uint32_t nt, uint32_t units, const BitsOut &b,
                               const unsigned long long *prefix, cudaStream_t stream);
-size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full);
+size_t bits_scratch_bytes(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, bool full,
+                          bool captured);
 cudaError_t enqueue_bits(const DevTables &t, const Tuning &tu, const uint8_t *text, uint64_t n, const CompactOut &out,
-                         bool full, void *scratch, size_t scratch_bytes, cudaStream_t stream);
+                         bool full, bool captured, void *scratch, size_t scratch_bytes, cudaStream_t stream);
 
 // The scan and gather steps of the compacted output (compact.cu).
 //   units: launch units (host count), or, when units_dev is set, read there.

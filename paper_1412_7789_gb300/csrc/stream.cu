@@ -125,10 +125,19 @@ bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
     return t.stream.root == (t.stream.form == 2 ? t.k : t.fbits);
 }
 
-StreamLists stream_lists(uint64_t n) {
-    // a walk for every eighth position, and each warp's last reservation; every tile
+StreamLists stream_lists(uint32_t form, uint64_t n, bool captured) {
+    // Every tile; each warp's last reservation; and a walk for every eighth
+    // position, with 2-bit codes for every sixteenth: few of their windows of 14 or
+    // 16 letters go on, and the filter kernel takes no list for most of these sets.
+    // A text with more has its other tiles listed whole, which costs time only:
+    // 64 MiB, a tenth of it runs of one letter, dense ids with 8 / 4 / 2 bits of
+    // list a position 297 / 399 / 421 us (filter kernel 653), 5 % of a repeat
+    // 424 / 423 / 661 (360); bytes, prose, 285 / 461 / 700 (371).
+    // In a captured graph the memory is the graph's and no other form can step in
+    // when it is not to be had: 2-bit codes make do with the warps' reservations.
     StreamLists l;
-    l.walk_cap = static_cast<uint32_t>(n / 8) + device_sm_count() * static_cast<uint32_t>(kMostWarps) * kWalkChunkEntries;
+    const uint64_t walks = form == 2 ? (captured ? 0u : n / 16) : n / 8;
+    l.walk_cap = static_cast<uint32_t>(walks) + device_sm_count() * static_cast<uint32_t>(kMostWarps) * kWalkChunkEntries;
     l.tile_cap = static_cast<uint32_t>(n / kTile) + 2u;
     return l;
 }
@@ -208,7 +217,7 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
 bool stream_batch_serves(const DevTables &t, const Tuning &tu) { return stream_serves(t, tu, 0); }
 
 StreamLists stream_batch_lists(uint64_t text_bytes, uint32_t texts) {
-    StreamLists l = stream_lists(text_bytes);
+    StreamLists l = stream_lists(8, text_bytes, false);
     l.tile_cap += 2u * texts;
     return l;
 }

@@ -470,6 +470,70 @@ def test_wave_past_32_bits_of_text():
             assert bool((pos == wpos).all()) and bool((ids == wids).all())
 
 
+@pytest.mark.parametrize("kind", ["dense", "count", "compact"])
+def test_scratch_of_dna_texts(kind):
+    """2-bit codes: lists of half a byte per text byte (8 bytes for every
+    sixteenth, with a bit and an id a position for the compacted list: 4.7 in
+    all) and a few MB; in a captured graph, whose memory no other form could do
+    without, no more for the lists than those few MB."""
+    import torch
+
+    n, few = 128 << 20, 8 << 20
+    text = _letters(n, b"ACGT", 9)
+    pats = [bytes(text[x:x + 20]) for x in range(1000, n - 64, n // 300)]
+    t = torch.from_numpy(text).cuda()
+    m = n if kind == "dense" else 4096
+    out, ids = torch.empty(m, dtype=torch.int32, device="cuda"), torch.empty(4096, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    per_byte = 4 * (1 + 1 / 32) + 12 / 2048 if kind == "compact" else 0
+
+    def call(a, stream=None, n=n):
+        if kind == "dense":
+            api.ac_match(a.handle, t, n, out, stream)
+        elif kind == "count":
+            api.ac_count(a.handle, t, n, cnt, stream)
+        else:
+            api.ac_match_compact(a.handle, t, n, out, ids, 4096, cnt, stream)
+
+    def captured(a, n):
+        g, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(g, stream=side):
+            call(a, side, n)
+        g.replay()
+        torch.cuda.synchronize()
+        return g
+
+    def check():
+        torch.cuda.synchronize()
+        if kind == "dense":
+            at = torch.nonzero(out >= 0).flatten()
+            assert int((out < -1).sum()) == 0 and out[at].tolist() == list(range(len(pats)))
+        else:
+            assert int(cnt.item()) == len(pats)
+            at = out[:len(pats)].long() if kind == "compact" else None
+        if at is not None:
+            assert at.tolist() == list(range(1000, n - 64, n // 300))
+
+    with api.Automaton(pats) as a:
+        call(a)  # code loaded
+        torch.cuda.synchronize()
+        base, _ = api.ac_scratch_pool_usage(reset_high=True)
+        call(a)
+        check()
+        assert api.ac_scratch_pool_usage()[1] - base <= (per_byte + 0.5) * n + few
+        captured(a, AT_MAX + 1)  # what a process's first graph takes
+        out.fill_(-7)
+        cnt.zero_()
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()  # as the capture will
+        free, _ = torch.cuda.mem_get_info()
+        g = captured(a, n)
+        taken = free - torch.cuda.mem_get_info()[0]
+        check()
+        assert taken <= per_byte * n + (64 << 20)  # (mapped in pieces of up to 32 MB)
+        del g
+
+
 _NO_ROOM = """
 import sys
 import numpy as np
