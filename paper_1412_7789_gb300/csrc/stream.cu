@@ -22,8 +22,13 @@ constexpr uint64_t kAtMax = 2u << 20;
 // fewer CTAs (1 MiB of ACGT, 128 / 256 / 512: 11.8 / 10.7 / 12.4 us a call).
 __host__ __device__ constexpr int at_block(int per) { return per == 1 ? 128 : 256; }
 
-// One lane per position (a text this short and the tables it touches stay in
-// L2): match_run of 32 * PER positions a warp.
+// One lane per position (a text this short and the tables it touches stay in L2):
+// runs of 32 * PER positions a warp, whose walks are dealt out again over its
+// lanes: a warp with several positions a lane else issues as many walks one after
+// the other, for a lane or two each.  (Dense ids of 1 MiB, two positions a lane, us
+// a call: the alphabet repeated, a walk in 26 positions, 16.7 -> 12.8; words 16.0 ->
+// 14.1; where no walk is left to deal out as before.  Over the whole CTA: 12.4 and
+// 14.5, but 1 to 2 us more for every text.)
 template <int B, typename GT, int MODE, int PER>
 __global__ void __launch_bounds__(at_block(PER)) pfac_at(const __grid_constant__ FilterParams p) {
     __shared__ uint8_t cls8[256];
@@ -34,39 +39,93 @@ __global__ void __launch_bounds__(at_block(PER)) pfac_at(const __grid_constant__
     bool in[PER + 1];
     load_run<PER>(p.text, p.n, g0, lane, c, in);
     for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
-    __syncthreads();
+    const TileText tt = make_text(p.text, p.out, p.n, 0u);
     uint32_t cnt = 0;
-    match_run<B, GT, PER, (PER > 1)>(p, cls8, make_text(p.text, p.out, p.n, 0u), g0, lane, c, in, [&](int j, int r) {
-        const uint64_t gi = g0 + 32u * j;
-        if (MODE == OUT_DENSE) {
-            if (in[j]) p.out[gi] = r;
-        } else if (MODE == OUT_COUNT) {
-            cnt += r >= 0 ? 1u : 0u;
-        } else {
-            if (r >= 0) p.bo.ids[gi] = r;
-            const uint32_t bits = __ballot_sync(kFull, r >= 0);
-            if (lane == 0 && in[j]) p.bo.bits[gi >> 5] = bits;
+    if constexpr (PER == 1) {
+        __syncthreads();
+        match_run<B, GT, PER, false>(p, cls8, tt, g0, lane, c, in, [&](int, int r) {
+            if (MODE == OUT_DENSE) {
+                if (in[0]) p.out[g0] = r;
+            } else if (MODE == OUT_COUNT) {
+                cnt += r >= 0 ? 1u : 0u;
+            } else {
+                if (r >= 0) p.bo.ids[g0] = r;
+                const uint32_t bits = __ballot_sync(kFull, r >= 0);
+                if (lane == 0 && in[0]) p.bo.bits[g0 >> 5] = bits;
+            }
+        });
+    } else {
+        __shared__ uint2 walks[at_block(PER) / 32][32 * PER];  // {position in the warp's | q << 16, state}
+        __shared__ uint32_t words[at_block(PER) / 32][PER];
+        uint2 *mine = walks[threadIdx.x >> 5];
+        uint32_t *bits = words[threadIdx.x >> 5];
+        __syncthreads();
+        RunState<PER> st;
+        resolve_run<B, PER, true>(p, cls8, lane, c, in, st);
+        uint32_t n = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const bool walk = st.walk[j] && in[j], hit = in[j] && !st.walk[j] && st.r[j] >= 0;
+            const unsigned m = __ballot_sync(kFull, walk);
+            if (walk)
+                mine[n + static_cast<uint32_t>(__popc(m & ((1u << lane) - 1u)))] =
+                    make_uint2(32u * j + static_cast<uint32_t>(lane) | (st.q[j] << 16), st.s[j]);
+            n += static_cast<uint32_t>(__popc(m));
+            if (MODE == OUT_DENSE) {
+                if (in[j] && !walk) p.out[g0 + 32u * j] = st.r[j];
+            } else if (MODE == OUT_COUNT) {
+                cnt += hit ? 1u : 0u;
+            } else {
+                if (hit) p.bo.ids[g0 + 32u * j] = st.r[j];
+                const uint32_t w = __ballot_sync(kFull, hit);
+                if (lane == 0) bits[j] = w;
+            }
         }
-    });
+        __syncwarp();
+        const uint64_t w0 = g0 - static_cast<uint32_t>(lane);
+        for (uint32_t i = static_cast<uint32_t>(lane); i < n; i += 32u) {
+            const uint2 e = mine[i];
+            const uint32_t l = e.x & 0xFFFFu;
+            const int r = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(w0 + l), e.y, e.x >> 16);
+            if (MODE == OUT_DENSE) {
+                p.out[w0 + l] = r;
+            } else if (MODE == OUT_COUNT) {
+                cnt += r >= 0 ? 1u : 0u;
+            } else if (r >= 0) {
+                p.bo.ids[w0 + l] = r;
+                atomicOr(bits + (l >> 5), 1u << (l & 31u));
+            }
+        }
+        if (MODE == OUT_BITS) {
+            __syncwarp();
+            if (lane < PER && w0 + 32u * lane < p.n) p.bo.bits[(w0 >> 5) + lane] = bits[lane];
+        }
+    }
     add_count<MODE>(p, cnt, lane);
 }
 
-// Positions a lane from this length on: 2 (fewer CTAs, and two chains of loads
-// in flight); below, 1, where the walks of a text dense in matches need every
-// warp.  A lane's walks run one after another, which is what counts against 4:
-// us a call, 2 / 4 positions, 1 MiB of ACGT 11.9 / 10.6, 2 MiB 14.7 / 14.0;
-// where the first 4 KiB all match 18.7 / 31.0 and 19.2 / 33.
-constexpr uint64_t kAtWide = 768u << 10;
+// Positions a lane: 1, where the walks of a text dense in matches need every warp;
+// from kAtWide on 2 (fewer CTAs, and two chains of loads in flight); with 8-bit
+// codes from kAtWider on 4.  A lane's walks run one after another, which is what
+// counts against more with 2-bit codes.  us a call, 2 / 4 positions: 1 MiB of ACGT
+// 10.5 / 10.4, of the alphabet repeated 12.8 / 10.6, words 14.1 / 12.5, Zipf bytes
+// 14.9 / 16.5; 2 MiB 14.7 / 14.5, 22.8 / 18.1, 20.8 / 18.7, 23.0 / 22.8; where the
+// first 4 KiB of ACGT all match 18.8 / 27.
+constexpr uint64_t kAtWide = 768u << 10, kAtWider = 1u << 20;
 
+template <int B, typename GT, int MODE, int PER>
+void launch_at_per(const FilterParams &p, cudaStream_t stream) {
+    const uint64_t block = at_block(PER);
+    pfac_at<B, GT, MODE, PER><<<static_cast<uint32_t>((p.n + block * PER - 1) / (block * PER)), block, 0, stream>>>(p);
+}
 template <int B, typename GT, int MODE>
 void launch_at_one(const FilterParams &p, cudaStream_t stream) {
-    const uint32_t per = p.n >= kAtWide ? 2u : 1u;
-    const uint32_t block = at_block(static_cast<int>(per));
-    const uint32_t grid = static_cast<uint32_t>((p.n + block * per - 1) / (block * per));
-    if (per == 2u)
-        pfac_at<B, GT, MODE, 2><<<grid, block, 0, stream>>>(p);
+    if (p.n < kAtWide)
+        launch_at_per<B, GT, MODE, 1>(p, stream);
+    else if (B != 8 || p.n < kAtWider)
+        launch_at_per<B, GT, MODE, 2>(p, stream);
     else
-        pfac_at<B, GT, MODE, 1><<<grid, block, 0, stream>>>(p);
+        launch_at_per<B, GT, MODE, B == 8 ? 4 : 2>(p, stream);
 }
 
 template <int B, typename GT>

@@ -247,10 +247,17 @@ __device__ __forceinline__ void load_run(const uint8_t *text, uint64_t n, uint64
     }
 }
 
-// put(j, id or -1) for each of the lane's positions (all lanes of the warp).
-template <int B, typename GT, int PER, bool FIRST, typename Put>
-__device__ __forceinline__ void match_run(const FilterParams &p, const uint8_t *cls8, const TileText &tt, uint64_t g0,
-                                          int lane, uint32_t (&c)[PER + 1], const bool (&in)[PER + 1], Put put) {
+// A position after its first loads: its id, or the walk that is left (state s, the
+// code at position + q next).
+template <int PER>
+struct RunState {
+    int r[PER];
+    uint32_t s[PER], q[PER];
+    bool walk[PER];
+};
+template <int B, int PER, bool FIRST>
+__device__ __forceinline__ void resolve_run(const FilterParams &p, const uint8_t *cls8, int lane, uint32_t (&c)[PER + 1],
+                                            const bool (&in)[PER + 1], RunState<PER> &st) {
     // codes, and which positions hold none (a byte in no keyword, or the text's end)
     const bool id = B == 8 && p.identity;
     uint32_t bad[PER + 1];  // bit i: position i of the 32
@@ -282,14 +289,19 @@ __device__ __forceinline__ void match_run(const FilterParams &p, const uint8_t *
         }
     }
     // first loads of all the lane's positions, then the second
-    int e[PER], r[PER];
+    int e[PER];
     uint4 h[PER];
-    bool walk[PER], keep[PER];
-    uint32_t s[PER], q[PER], m[PER];
-    // FIRST (several positions a lane: longer texts, few of whose positions get
-    // past it): the root filter first, whose 128 KiB stay in L1, not a sector of a
-    // table in L2 for each position (2 MiB of ACGT 16.6 -> 14.7 us a call, of Zipf
-    // bytes 29.0 -> 25.8; short texts would wait for one load more)
+    bool keep[PER];
+    uint32_t m[PER];
+    auto &r = st.r;
+    auto &s = st.s;
+    auto &q = st.q;
+    auto &walk = st.walk;
+    // FIRST (longer texts, few of whose positions get past it): the root filter
+    // first, whose 128 KiB stay in L1, not a sector of a table in L2 for each
+    // position (2 MiB of ACGT 16.6 -> 14.7 us a call, of Zipf bytes 29.0 -> 25.8;
+    // short texts would wait for one load more, and nearly all positions of the
+    // tiles listed whole pass it)
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
         keep[j] = true;
@@ -341,9 +353,21 @@ __device__ __forceinline__ void match_run(const FilterParams &p, const uint8_t *
             s[j] = static_cast<uint32_t>(e[j]);
             if (e[j] < 0) r[j] = decode_dead(e[j]);
         }
-        if (walk[j])
-            r[j] = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(g0 + 32u * j), s[j], q[j]);
-        put(j, in[j] ? r[j] : -1);
+    }
+}
+
+// put(j, id or -1) for each of the lane's positions (all lanes of the warp), each
+// lane walking its own.
+template <int B, typename GT, int PER, bool FIRST, typename Put>
+__device__ __forceinline__ void match_run(const FilterParams &p, const uint8_t *cls8, const TileText &tt, uint64_t g0,
+                                          int lane, uint32_t (&c)[PER + 1], const bool (&in)[PER + 1], Put put) {
+    RunState<PER> st;
+    resolve_run<B, PER, FIRST>(p, cls8, lane, c, in, st);
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        if (st.walk[j])
+            st.r[j] = filt::walk_global<GT>(p, cls8, tt, static_cast<int64_t>(g0 + 32u * j), st.s[j], st.q[j]);
+        put(j, in[j] ? st.r[j] : -1);
     }
 }
 

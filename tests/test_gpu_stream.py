@@ -223,6 +223,30 @@ def test_repetitive_texts_are_no_slower(kind, block):
     assert built <= 1.25 * tuned, (built, tuned)
 
 
+@pytest.mark.parametrize("kind", ["alphabet", "words"])
+def test_short_texts_with_scattered_walks(kind):
+    """Byte texts of 1.5 MiB where a lane or two of every warp walk: dense ids
+    take no longer as built than in the filter kernel (a quarter more allowed,
+    as above), and every output is right."""
+    import torch
+
+    n = (3 << 19) + 77
+    if kind == "alphabet":
+        text, pats = workloads.paper_text(n), workloads.paper_keywords(10, 0)
+    else:
+        r = workloads.rng(31)
+        pats = [bytes(r.integers(97, 123, size=int(m)).astype(np.uint8)) for m in r.integers(4, 12, size=2000)]
+        text = np.frombuffer(b" ".join(pats[min(1999, int(x))] for x in r.zipf(1.3, size=n // 5)), dtype=np.uint8)[:n].copy()
+        assert text.size == n
+    t = torch.from_numpy(text).cuda()
+    ids = torch.empty(n, dtype=torch.int32, device="cuda")
+    with api.Automaton(pats) as a, api.Automaton(pats) as b:
+        _check(a, text, oracle.pfac_ids(pats, text), 5, 1)
+        b.set_tuning(block=512)
+        built, tuned = _event_us(lambda: a.match(t, out=ids)), _event_us(lambda: b.match(t, out=ids))
+    assert built <= 1.25 * tuned, (built, tuned)
+
+
 @pytest.mark.parametrize("letters,shortest", [(b"ACGT", 16), (b"ACGT", 8), (b"ACGT", 4),
                                               (b"abcdefghijklmnopqrstuvwxyz", 6)])
 def test_walks_fill_the_list_part_way(letters, shortest):
