@@ -139,6 +139,29 @@ def test_full_list(name):
         assert np.array_equal(got[np.lexsort((got[:, 1], got[:, 0]))], want[np.lexsort((want[:, 1], want[:, 0]))])
 
 
+def test_full_list_of_many_dense_tiles():
+    """160 MiB in which every tile has more than 256 matches: more such tiles a
+    CTA than it notes (64), so that some are done by the CTA and some by a warp.
+    The text repeats 16 letters, so the list follows from their period."""
+    import torch
+
+    unit, n = b"ACGTTGCAACCGGTTA", 160 << 20
+    pats = [unit[:4], unit[:8], unit[5:9], unit[9:13], (unit * 2)[14:19], unit[5:9]]
+    starts = [(o, len(p), i) for o in range(16) for i, p in enumerate(pats) if (unit * 3)[o:o + len(p)] == p]
+    starts.sort()
+    assert 16 // 8 < len({o for o, _, _ in starts}) and len(starts) >= 6
+    text = torch.tensor(list(unit), dtype=torch.uint8, device="cuda").repeat(n // 16)
+    first = torch.arange(0, n, 16, dtype=torch.int64, device="cuda")
+    ends = (first[:, None] + torch.tensor([o + m - 1 for o, m, _ in starts], device="cuda")[None, :]).flatten()
+    ids = torch.tensor([i for _, _, i in starts], dtype=torch.int32, device="cuda").repeat(n // 16)
+    inside = ends < n
+    ends, ids = ends[inside].int(), ids[inside]
+    with api.Automaton(pats) as a:
+        e, i, c = a.match_full(text, cap=ends.numel())
+        assert int(c.item()) == ends.numel()
+        assert bool((e.int() == ends).all()) and bool((i.int() == ids).all())
+
+
 def test_full_counts_past_32_bits():
     """2^21 equal keywords: a tile of 2,048 of their matches holds 2^32
     occurrences, which only units of half a tile can count in 32 bits."""
