@@ -302,7 +302,7 @@ void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTa
         const double dense = bits_of(h.F);
         double best = 7.0 + 225.0 * dense;
         for (uint32_t step : {2u, 4u}) {
-            if (h.minlen < step + 4u) continue;  // at most 4^6 completions a window
+            if (h.minlen < step + 4u) continue;  // at most 4^5 completions a window
             std::vector<uint32_t> F(kWords, 0u), F2;
             for (uint32_t id = 0; id < h.nkw; ++id)
                 for (uint32_t o = 0; o < step; ++o) {
@@ -335,7 +335,6 @@ void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTa
         // 99.98 % 641 against 565)
         if (st.step == 1u && dense > 0.95) return;
         st.form = 2;
-        st.win1 = k;
         st.root = k;
     } else if (h.hashed && h.minlen >= kHashWindow && h.fbits == kFilterBits) {
         st.form = 8;
@@ -351,7 +350,6 @@ void stream_filters(const uint8_t *const *patterns, const uint32_t *lens, HostTa
                 bits += 8u * lens[id] > win ? 1u : 1ull << (win + 1u - 8u * lens[id]);
             if (bits > kMostBits) break;
         }
-        st.win1 = win;
         st.m1 = kFilterHashMul;
         st.m2 = win > 32u ? kStreamMul2 << (64u - win) : 0u;
         auto bytes4 = [&](uint32_t id, uint32_t o) {  // 4 bytes from offset o, zero past the end

@@ -46,10 +46,9 @@ constexpr uint32_t kHashWindow = 4;  // codes per hashed window (at most)
 constexpr uint32_t kHkBranch = 0xFFFFFFFFu;
 
 // The streaming form for one long text (stream_kernel.cuh): positions a warp
-// takes at a time, positions per unit of a walk-list entry, multiplier of a
-// window's second word, and the short-keyword part of the second filter.
+// takes at a time, multiplier of a window's second word, and the short-keyword
+// part of the second filter.
 constexpr uint32_t kStreamTile = 2048;
-constexpr uint32_t kStreamUnit = 1024;
 constexpr uint32_t kStreamMul2 = 0xC2B2AE35u;
 constexpr uint32_t kStreamShortBytes = 4096;
 
@@ -85,14 +84,14 @@ struct RawBytes {
 //     (all completions where the keyword ends inside it); F2 (none when empty)
 //     that of every window of win2 codes there, hashed.
 //   form 8 (8-bit codes, no keyword shorter than 4): F1 the hashed windows of
-//     every keyword's first win1 bits (all completions where the keyword ends
-//     inside them); F2 (none when empty) those of its first 6 bytes, then, in
+//     every keyword's first bits, as many as m2 is shifted for (all completions
+//     where the keyword ends inside them); F2 (none when empty) those of its first 6 bytes, then, in
 //     its last kStreamShortBytes, the first 4 bytes of the keywords shorter
 //     than 6.
 struct StreamTables {
     uint32_t form = 0;
     uint32_t step = 1;             // form 2: every step-th position is looked up
-    uint32_t win1 = 0, win2 = 0;   // windows in codes (form 2); win1 in bits (form 8)
+    uint32_t win2 = 0;             // the second filter's window: codes (form 2), bytes (form 8)
     uint32_t m1 = 0, m2 = 0;       // form 8: multipliers of the window's words
     uint32_t root = 0;             // the root tables' depth it was built with (k, or the filter's bits)
 };
@@ -428,8 +427,9 @@ constexpr uint32_t kStreamBatchMax = 32;
 cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *rs, uint32_t nh, OutMode mode,
                                 unsigned long long wait_ns, void *lists, const StreamLists &l, cudaStream_t stream);
 
-// One short text (dense ids or count): one thread per position, everything
-// from global memory (stream.cu).  Needs no scratch.
+// One short text (dense ids, count, or OUT_BITS for a list): a lane for every one,
+// two or four positions, everything from global memory (stream.cu).  Needs no
+// scratch.
 bool at_serves(const DevTables &t, const Tuning &tu, uint64_t n);
 cudaError_t launch_at(const DevTables &t, const MatchRequest &r, OutMode mode, cudaStream_t stream);
 

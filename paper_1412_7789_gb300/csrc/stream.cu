@@ -11,15 +11,19 @@ using namespace strm;
 
 namespace {
 
-// Texts up to this length take one lane per position: no filter to load into
-// every SM, no list, one launch.  4 KiB of the sweep set, where every position
-// walks to a match: 10 us a call against 70 in the filter kernel, whose few
-// tiles kept a handful of warps busy.  The line against the streaming form (us
-// a call): ACGT 2 MiB 14.5 / 15.5, 3 MiB 18.7 / 15.7; where the first 4 KiB all
-// match 18.8 / 24.0 at 2 MiB; Zipf bytes 2 MiB 25.7 / 25.5, 3 MiB 24.9 / 21.7.
+// Texts up to this length take a lane for every position or few: no filter to load
+// into every SM, no list, one launch.  4 KiB of the sweep set, where every position
+// walks to a match: 10 us a call against 70 in the filter kernel, whose few tiles
+// kept a handful of warps busy.  The line against the streaming form, us a call,
+// short-text / streaming form at 2 MiB: dense ids of ACGT 14.7 / 21.5 (100 keywords)
+// and 16.6 / 17.3 (3,000), Zipf bytes 22.8 / 25.6, the alphabet repeated 18.1 /
+// 21.3; lists, which both make in a second pass, 29.0 / 31.3, 30.8 / 25.1, 38.5 /
+// 33.0 and 32.0 / 35.8.  At 3 MiB dense ids 18.8 / 22.1, 20.8 / 17.9, 29.5 / 25.9
+// and 24.8 / 22.5, lists 38.6 / 31.3, 40.9 / 25.9, 51.6 / 35.6 and 44.0 / 41.0.
 constexpr uint64_t kAtMax = 2u << 20;
-// Threads per CTA: short texts want their positions on many SMs, longer ones
-// fewer CTAs (1 MiB of ACGT, 128 / 256 / 512: 11.8 / 10.7 / 12.4 us a call).
+// Threads per CTA: a lane's worth a position, 64 / 128 / 256 take the same within a
+// microsecond; with more a lane, 128 / 256 / 512: ACGT, 3,000 keywords, 1 MiB 11.5 /
+// 10.7 / 12.4 us a call, Zipf bytes 2 MiB 22.9 / 22.9 / 24.9.
 __host__ __device__ constexpr int at_block(int per) { return per == 1 ? 128 : 256; }
 
 // One lane per position (a text this short and the tables it touches stay in L2):
@@ -146,11 +150,12 @@ cudaError_t launch_walk_modes(OutMode mode, const FilterParams &p, uint32_t sms,
     auto kernel = mode == OUT_DENSE ? pfac_stream_walks<B, GT, OUT_DENSE>
                   : mode == OUT_COUNT ? pfac_stream_walks<B, GT, OUT_COUNT>
                                       : pfac_stream_walks<B, GT, OUT_BITS>;
-    // (started early, but with bytes for short texts only: on long ones the
-    // walks' CTAs cost the form before them more than the gap they save.  us a
-    // call, plain / early: ACGT 4 MiB 17.9 / 15.9, 64 MiB 73.6 / 70.6; Zipf bytes
-    // 4 MiB counted 28.8 / 27.0, 24 MiB 46.4 / 45.8, 64 MiB full 112 / 120, 1 GiB
-    // compacted 1155 / 1360)
+    // (started early, but with bytes for short texts only: on long ones the walks'
+    // CTAs cost the form before them more than the gap they save.  us a call, plain /
+    // early: ACGT 4 MiB 17.9 / 15.9, 64 MiB 73.6 / 70.6; 20,000 keywords in Zipf
+    // bytes, counted 4 MiB 29.2 / 28.8, 16 MiB 41.5 / 39.8, 24 MiB 48.3 / 47.5, 32
+    // MiB 54.9 / 57.0, 64 MiB 81.0 / 86.9; dense 16 MiB 45.2 / 44.4, 24 MiB 54.9 /
+    // 56.4; compacted 16 MiB 52.3 / 50.2, 24 MiB 58.2 / 58.5, 64 MiB 97.8 / 105.2)
     if (B == 2 || p.n <= kWalkEarly) return launch_next(kernel, grid, kWalkBlock, 0u, stream, p);
     kernel<<<grid, kWalkBlock, 0, stream>>>(p);
     return cudaGetLastError();
@@ -180,7 +185,8 @@ cudaError_t launch_at(const DevTables &t, const MatchRequest &r, OutMode mode, c
 }
 
 bool stream_serves(const DevTables &t, const Tuning &tu, uint64_t n) {
-    if (!t.stream.form || !untuned(tu) || n / kStreamUnit >= (1ull << 22) - 2) return false;
+    // (positions, and what rounds a text up to whole tiles, are numbered in 32 bits)
+    if (!t.stream.form || !untuned(tu) || n >= (1ull << 32) - kTile) return false;
     return t.stream.root == (t.stream.form == 2 ? t.k : t.fbits);
 }
 
@@ -233,11 +239,11 @@ cudaError_t stream_params(const DevTables &t, const MatchRequest &r, OutMode mod
     return cudaSuccess;
 }
 
-// Shared memory of a launch: the filters, the -1 buffer (and 128 bytes for the
-// CTA), the warps' areas.
-uint32_t stream_smem(uint32_t form, bool batch, uint32_t filters, uint32_t *off_none, uint32_t *off_warp) {
-    *off_none = (filters + 127u) & ~127u;
-    *off_warp = *off_none + 4u * kNone + 128u;
+// Shared memory of a launch: the filters, 128 bytes for the CTA, the -1 buffer
+// (where it has bulk stores), the warps' areas.
+uint32_t stream_smem(uint32_t form, OutMode mode, bool batch, uint32_t filters, uint32_t *off_cta, uint32_t *off_warp) {
+    *off_cta = (filters + 127u) & ~127u;
+    *off_warp = *off_cta + 128u + (has_bulk(form, mode) ? 4u * kNone : 0u);
     return *off_warp + static_cast<uint32_t>(block_of(form, batch) / 32) * (form == 2 ? kWarpBytes2 : kWarpBytes8);
 }
 
@@ -255,7 +261,7 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
     if (e != cudaSuccess) return e;
     p.sg = make_seg(r.text, r.out, r.n);
     p.ntiles = static_cast<uint32_t>((r.n + p.sg.head + kTile - 1) / kTile);
-    const uint32_t smem = stream_smem(t.stream.form, false, p.f1bytes + p.f2bytes, &p.off_none, &p.off_warp);
+    const uint32_t smem = stream_smem(t.stream.form, mode, false, p.f1bytes + p.f2bytes, &p.off_cta, &p.off_warp);
     if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
     // short texts spread over the SMs, a tile to each of eight warps (3 MiB of
     // ACGT 17.5 -> 15.7 us a call, of Zipf bytes 23.7 -> 21.7)
@@ -325,7 +331,7 @@ cudaError_t launch_stream_batch(const DevTables *const *ts, const MatchRequest *
             filters = filters > p.f1bytes + p.f2bytes ? filters : p.f1bytes + p.f2bytes;
         }
         if (mp.nh == 0) continue;
-        const uint32_t smem = stream_smem(form, true, filters, &mp.off_none, &mp.off_warp);
+        const uint32_t smem = stream_smem(form, mode, true, filters, &mp.off_cta, &mp.off_warp);
         if (static_cast<int>(smem) > max_smem) return cudaErrorInvalidConfiguration;
         const uint32_t grid = static_cast<uint32_t>(sms);
         e = form == 2 ? launch_stream2_multi(mode, mp, step, grid, smem, max_smem, stream, next)

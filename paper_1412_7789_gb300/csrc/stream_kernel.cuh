@@ -62,7 +62,9 @@ __host__ __device__ constexpr int block_of(uint32_t form, bool batch) {
 constexpr uint32_t kTile = kStreamTile;  // positions a warp takes at a time
 constexpr uint32_t kChunk = 512;         // positions per warp-wide 16-byte load
 constexpr uint32_t kQueue = 256;         // survivors of a tile kept in shared memory at a time
-constexpr uint32_t kNone = 1024;          // ids of -1 in shared memory
+constexpr uint32_t kNone = 1024;          // ids of -1 in shared memory, for bulk stores
+// Whether the kernel writes its tiles of -1 by bulk stores (fill_none).
+__host__ __device__ constexpr bool has_bulk(uint32_t form, int mode) { return form == 8 && mode == OUT_DENSE; }
 constexpr uint32_t kRes2 = 160;          // 2-bit codes: candidates waiting to be resolved (31 + 4 * 32 at most)
 constexpr uint32_t kRes8 = 64;           // 8-bit codes: survivors waiting (31 + 32 at most)
 constexpr uint32_t kWarpBytes2 = kTile / 4 + 16 + 2 * kQueue + 16 + 8 * kRes2;  // (16: a step-1 tile's last marks)
@@ -133,7 +135,7 @@ struct StreamParams {
     uint32_t four;         // 4
     uint32_t m1, m2;       // 8-bit codes: multipliers of the window's words
     uint32_t l2shift;      // 2-bit codes: left shift that drops the codes past the second filter's window
-    uint32_t off_none, off_warp;
+    uint32_t off_cta, off_warp;
 };
 
 // A tile's registers: lane l's 16 bytes of chunks 0-3, and (lane 0) the 16
@@ -675,6 +677,12 @@ __device__ __forceinline__ bool bytes_known(const FilterParams &f, const uint8_t
     return bad == 0;
 }
 
+// ... those of a window: out of line for the matcher, which asks for the few
+// results of sets with windows of several positions (inlined: 96 registers for 90).
+static __device__ __noinline__ bool bytes_known_far(const FilterParams &f, const uint8_t *text, uint64_t n, uint64_t gi) {
+    return bytes_known(f, text, n, gi, f.k + f.k2);
+}
+
 // A round of candidates (all lanes; on: this lane has one: position g and the
 // 16 codes w from it): window table, stride table, then out or to the walk
 // list.  The codes may be those of bytes in no keyword, or of bytes past the
@@ -715,7 +723,7 @@ __device__ __forceinline__ void resolve2(const StreamParams &p, const Seg &sg, W
                 doubt = ((m >> (i & 15u)) & ((1u << (f.k + f.k2)) - 1u)) != 0u;
             }
         } else {
-            doubt = doubt && !bytes_known(f, sg.text, sg.n, gi, f.k + f.k2);
+            doubt = doubt && !bytes_known_far(f, sg.text, sg.n, gi);
         }
         if (doubt) {
             walk = true;
@@ -1104,11 +1112,11 @@ __device__ __forceinline__ void stream_text(const StreamParams &p) {
     const Seg own = make_seg(p.f.text, p.f.out, p.f.n);
     using SegRef = typename std::conditional<FORM == 2, const Seg, const Seg &>::type;
     SegRef sg = FORM == 2 ? own : p.sg;
-    const int32_t *none = reinterpret_cast<const int32_t *>(smem + p.off_none);
+    const int32_t *none = reinterpret_cast<const int32_t *>(smem + p.off_cta + 128u);
     TileRegs r;
     r.look = make_uint4(0u, 0u, 0u, 0u);
     if (t < p.ntiles) load_tile(sg, t, pol, lane, r);
-    fill_constant(smem + p.off_none);
+    if (has_bulk(FORM, MODE)) fill_constant(smem + p.off_cta + 128u);
     load_filters(p, smem);
     __syncthreads();  // the filters are in place
     WarpState ws{0u, 0u, {0u, 0u, false, false}};
@@ -1116,7 +1124,7 @@ __device__ __forceinline__ void stream_text(const StreamParams &p) {
         tiles2<S, MODE, false>(p, smem, p.off_warp, none, sg, t, p.ntiles, step, pol, r, ws);
     else
         tiles8<MODE, false>(p, smem, p.off_warp, none, sg, t, p.ntiles, step, pol, r, ws);
-    if (FORM == 8 && MODE == OUT_DENSE && lane == 0) bulk_wait_all();
+    if (has_bulk(FORM, MODE) && lane == 0) bulk_wait_all();
     close_room<false>(p.f, ws.room, lane);
     add_count<MODE>(p.f, ws.cnt, lane);
 }
@@ -1141,7 +1149,7 @@ constexpr uint32_t kStreamMultiMax = 32;
 struct StreamMulti {
     StreamParams a[kStreamMultiMax];
     uint32_t nh;
-    uint32_t off_none, off_warp;
+    uint32_t off_cta, off_warp;
 };
 static_assert(sizeof(StreamMulti) <= 32764, "kernel parameters are limited to 32764 bytes");
 
@@ -1191,14 +1199,14 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     const uint64_t pol = policy_evict_first();
-    const int32_t *none = reinterpret_cast<const int32_t *>(smem + mp.off_none);
+    const int32_t *none = reinterpret_cast<const int32_t *>(smem + mp.off_cta + 128u);
     // (dynamic too: a kernel with static shared memory cannot take the most dynamic)
-    volatile uint32_t &start = reinterpret_cast<uint32_t *>(smem + mp.off_none)[kNone];
-    volatile uint32_t &open = reinterpret_cast<uint32_t *>(smem + mp.off_none)[kNone + 1u];
+    volatile uint32_t &start = reinterpret_cast<uint32_t *>(smem + mp.off_cta)[0];
+    volatile uint32_t &open = reinterpret_cast<uint32_t *>(smem + mp.off_cta)[1];
     // the next form's launch, or the walks: neither reads what this one writes
     // before it has ended
     allow_next();
-    fill_constant(smem + mp.off_none);
+    if (has_bulk(FORM, MODE)) fill_constant(smem + mp.off_cta + 128u);
     uint64_t total = 0;
     for (uint32_t a = 0; a < mp.nh; ++a) total += __ldg(&mp.a[a].f.batch->units);
     if (threadIdx.x == 0) {
@@ -1264,7 +1272,7 @@ __device__ __forceinline__ void stream_batch(const StreamMulti &mp) {
         }
         __syncthreads();  // every warp is done with the automaton's filters
     }
-    if (FORM == 8 && MODE == OUT_DENSE && lane == 0) bulk_wait_all();
+    if (has_bulk(FORM, MODE) && lane == 0) bulk_wait_all();
     close_room<true>(mp.a[0].f, ws.room, lane);
     wait_previous();
 }
