@@ -282,8 +282,10 @@ cudaError_t launch_stream(const DevTables &t, const MatchRequest &r, OutMode mod
 bool stream_batch_serves(const DevTables &t, const Tuning &tu) { return stream_serves(t, tu, 0); }
 
 StreamLists stream_batch_lists(uint64_t text_bytes, uint32_t texts) {
+    // a text's two ragged tiles too, as far as they are long enough to be listed
     StreamLists l = stream_lists(8, text_bytes, false);
-    l.tile_cap += 2u * texts;
+    const uint64_t ragged = 2ull * texts, most = text_bytes / kFew;
+    l.tile_cap += static_cast<uint32_t>(ragged < most ? ragged : most);
     return l;
 }
 
