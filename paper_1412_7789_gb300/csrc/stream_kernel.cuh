@@ -1359,9 +1359,13 @@ __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const
     allow_next();  // the lists' scan
     wait_previous();
     const Listed l = listed(p);
-    const uint32_t first = first_run(l), *tiles = reinterpret_cast<const uint32_t *>(p.walks + p.walk_cap);
-    if (blockIdx.x * blockDim.x >= l.m && first % gridDim.x >= l.runs) return;
-    uint32_t t = first < l.runs ? tiles[first / kTileRuns] : 0u;
+    const bool idle = blockIdx.x * blockDim.x >= l.m;
+    if (idle && l.runs == 0u) return;
+    const uint32_t first = l.runs ? first_run(l) : 0u, *tiles = reinterpret_cast<const uint32_t *>(p.walks + p.walk_cap);
+    if (idle && first % gridDim.x >= l.runs) return;
+    // (2-bit codes: the first tile's number is on its way meanwhile; with 8-bit
+    // codes it would cost the walks' loop spills)
+    uint32_t t = B == 2 && first < l.runs ? tiles[first / kTileRuns] : 0u;
     for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) cls8[i] = __ldg(p.cls8g + i);
     __syncthreads();
     const Seg sg = make_seg(p.text, p.out, p.n);
@@ -1372,9 +1376,10 @@ __global__ void __launch_bounds__(kWalkBlock, kWalkCtas) pfac_stream_walks(const
         if (e.x != 0xFFFFFFFFu) put_id<MODE>(p, sg, e.x, finish_walk<GT>(p, cls8, sg, e.x, e.y, B), cnt);
     }
     for (uint32_t j = first; j < l.runs;) {
+        if (B != 2) t = tiles[j / kTileRuns];
         tile_run<B, GT, MODE>(p, cls8, sg, t * kTile + kRun * (j % kTileRuns), cnt, lane);
         j += gridDim.x * (blockDim.x / 32u);
-        if (j < l.runs) t = tiles[j / kTileRuns];
+        if (B == 2 && j < l.runs) t = tiles[j / kTileRuns];
     }
     add_count<MODE>(p, cnt, lane);
 }
@@ -1423,7 +1428,8 @@ __global__ void __launch_bounds__(kWalkBlock, 8) pfac_stream_walks_multi(const _
     allow_next();
     wait_previous();
     const Listed l = listed(mp.a[0]);
-    if (blockIdx.x * blockDim.x >= l.m && first_run(l) % gridDim.x >= l.runs) return;
+    const bool idle = blockIdx.x * blockDim.x >= l.m;
+    if (idle && (l.runs == 0u || first_run(l) % gridDim.x >= l.runs)) return;
     FilterParams *ps = reinterpret_cast<FilterParams *>(msm);
     uint8_t *cls = msm + mp.nh * sizeof(FilterParams);
     for (uint32_t i = threadIdx.x; i < mp.nh * static_cast<uint32_t>(sizeof(FilterParams) / 4); i += blockDim.x)
